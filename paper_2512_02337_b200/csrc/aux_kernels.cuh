@@ -14,6 +14,7 @@ struct SummaryParams {
     void* kmin;
     void* workspace;
     int layer0, batch, Hkv, bs, d, max_blocks, n_pages, A_max;
+    int aligned;  // set by the launcher: kmax and kmin take 16-byte stores
 };
 
 struct ScoreParams {

@@ -186,6 +186,39 @@ def test_commit_appends_and_updates_summaries():
     assert torch.equal(kmax[:, :, :, :nb], kmax2[:, :, :, :nb]) and torch.equal(kmin[:, :, :, :nb], kmin2[:, :, :, :nb])
 
 
+@pytest.mark.parametrize("dtype,Hkv,d,bs,shift", [("bf16", 1, 64, 16, 0), ("bf16", 8, 128, 64, 0), ("bf16", 9, 128, 32, 1),
+                                                  ("fp32", 3, 64, 64, 0), ("fp32", 12, 128, 16, 1)])
+def test_summaries_of_ragged_blocks_are_exact(dtype, Hkv, d, bs, shift):
+    """Eq. 1 with one token up to a whole block valid, head counts around the eight a CTA takes, NaN and signed zeros among
+    the keys, summaries that start off a 16-byte boundary (``shift`` elements): bit-exact, max and min are."""
+    dt, dev, L = wl.torch_dtype(dtype), "cuda", 2
+    lens = [1, bs - 1, bs * 3, bs * 5 + 1]
+    g = torch.Generator().manual_seed(Hkv + d)
+    mb = 6
+    k = torch.randn((L, mb * len(lens), Hkv, bs, d), generator=g)
+    k[torch.rand(k.shape, generator=g) < 0.01] = float("nan")
+    k[torch.rand(k.shape, generator=g) < 0.05] = -0.0
+    k = k.to(dt).to(dev)
+    table = torch.randperm(mb * len(lens), generator=g).to(torch.int32).view(len(lens), mb).to(dev)
+    cache = B.Cache(k, k, table, torch.tensor(lens, dtype=torch.int32, device=dev), mb * bs)
+    cfg = B.make_config(L, Hkv, Hkv, d, bs, dtype, 1, 1, 3, bs)
+    n = L * len(lens) * Hkv * mb * d
+    flat = [torch.full((n + 8,), 5.0, dtype=dt, device=dev)[shift:shift + n] for _ in range(2)]
+    kmax, kmin = (f.view(L, len(lens), Hkv, mb, d) for f in flat)
+    ws = torch.zeros(4096, dtype=torch.uint8, device=dev)
+    B.specpv_update_block_summaries(cfg, 0, L, cache, None, mb, kmax, kmin, ws)
+    util.sync_status(ws)
+    for b, n_tok in enumerate(lens):
+        nb = (n_tok + bs - 1) // bs
+        keys = k[:, table[b, :nb].long()].permute(0, 2, 1, 3, 4).float().reshape(L, Hkv, nb * bs, d)[:, :, :n_tok]
+        for i in range(nb):
+            blk = keys[:, :, i * bs:(i + 1) * bs]
+            hi = torch.where(blk.isnan(), torch.full_like(blk, -float("inf")), blk).amax(2)
+            lo = torch.where(blk.isnan(), torch.full_like(blk, float("inf")), blk).amin(2)
+            assert torch.equal(kmax[:, b, :, i].float(), hi) and torch.equal(kmin[:, b, :, i].float(), lo)
+        assert torch.all(kmax[:, b, :, nb:].float() == 5.0) and torch.all(kmin[:, b, :, nb:].float() == 5.0)
+
+
 def test_commit_in_layer_groups_matches_the_oracle():
     """A step's commit issued in two layer groups, in ascending order: every group writes its rows at the lengths as
     they stand and the lengths advance with the group that holds the model's last layer."""
