@@ -79,7 +79,7 @@ StagingPlan plan_staging(const Geometry& g, int n_layers_per_call, int batch, in
 WorkspacePlan plan_workspace(const Geometry& g, int n_layers_per_call, int max_batch, int M_max) {
     WorkspacePlan w{};
     const size_t base = (size_t)g.Hkv * n_layers_per_call * max_batch;
-    const size_t R_pad = round_up((size_t)M_max * g.G, 256);
+    const size_t R_pad = packed_rows(M_max, g.G);
     w.counter_off = kStatusBytes;
     w.counter_bytes = kHeaderBytes - kStatusBytes;
     w.partial_off = kHeaderBytes;

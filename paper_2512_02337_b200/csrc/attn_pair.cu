@@ -832,7 +832,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1) att
 // costs it clock: measured inside the benchmark step it is 8-10 % slower (4.56 against 4.12-4.23 ms for 32 layers at
 // 128K), and its set-up and merge tail make it slower on single-layer calls (33 against 21 us for a 4096-token cache).
 bool attention_pair_wanted(const AttnArgs& a) {
-    if (a.M_max * a.g.G <= 128) return false;
+    if (a.g.d != 128 || 128 % a.g.G != 0 || a.M_max * a.g.G <= 128) return false;
     const char* v = getenv("SPECPV_ATTN_KERNEL");
     return v != nullptr && strcmp(v, "pair") == 0;
 }

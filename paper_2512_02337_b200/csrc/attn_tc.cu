@@ -1,16 +1,22 @@
-// Tensor-core verification attention for B200 (sm_100a): bfloat16, head_dim 128, pages of 16, 32 or 64 tokens.
+// Tensor-core verification attention for B200 (sm_100a): bfloat16, head_dim 64 or 128, pages of 16, 32 or 64 tokens.
 // Tree-masked GQA attention of the step's tokens over a paged cache (paper Section 3.2-3.3,
 // Algorithm 1 "TreeDecode"), used for both the partial and the full cache.
 //
-// One CTA owns one (layer, sequence, KV head, KV split, row group).  All G query heads of the KV
-// head times up to 2*(128/G) step tokens are packed into two 128-row tiles, so QK^T and PV are
-// dense 128x128x128 contractions:
+// One CTA owns one (layer, sequence, KV head, KV split, row group).  All G query heads of the KV head times
+// floor(128/G) step tokens are packed into a 128-row tile, so QK^T and PV are dense 128x128xd and 128xdx128
+// contractions.  Two streams of tiles run through the CTA in ping-pong, so that the contractions of one hide behind
+// the softmax of the other:
+//   two row tiles   stream t is row tile t; both streams walk the same K/V tiles
+//   one row tile    stream t takes every other K/V tile of the one row tile, each stream with its own running maximum,
+//                   sum and accumulator; the two meet in shared memory at the end.  (One stream alone leaves the tensor
+//                   pipe idle during its softmax: 64K tokens x 36 layers, 32 query rows per head, 1715 -> 1457 us = the
+//                   copy rate.)
 //   warp 0      TMA producer: Q once, then K and V tiles of 128 tokens (2, 4 or 8 pages, one copy per page
-//               and 64-channel half, each issued by its own lane) through the block table into a ring of
-//               32 KB shared-memory slots (128-byte swizzle)
+//               and 64-channel part, each issued by its own lane) through the block table into a ring of
+//               shared-memory slots (128-byte swizzle)
 //   warp 1      MMA issuer: tcgen05.mma  S_t = Q_t K^T  (both operands in shared memory) and
 //               O_t += P_t V (P read from tensor memory, V MN-major from shared memory)
-//   warps 4-7   softmax of row tile 0, warps 8-11 of row tile 1: one thread per row reads S from
+//   warps 4-7   softmax of stream 0, warps 8-11 of stream 1: one thread per row reads S from
 //               tensor memory, keeps the running max / sum of an online softmax in the log2
 //               domain, writes P (bfloat16) over S, rescales O only when the max grew by > 2^8,
 //               and finally normalises O and writes it out
@@ -24,26 +30,35 @@ namespace specpv {
 namespace {
 
 constexpr int kThreadsTc = 384;          // 12 warps
-constexpr int kSlotBytes = 32768;        // one K or V tile: [2 d-halves][128 tokens][64 d] bf16
-constexpr int kStages = 5;
-constexpr int kQBytes = 2 * 32768;       // two row tiles
-constexpr int kSmemBytes = 1024 + kQBytes + kStages * kSlotBytes;
+
+// Shared memory by head size: a K or V tile is [d/64 parts][128 tokens][64 d] bf16, a Q tile [d/64 parts][128 rows][64 d].
+template <int D>
+struct Shape {
+    static constexpr int kParts = D / 64;
+    static constexpr int kSlotBytes = kTileTokens * D * 2;
+    static constexpr int kStages = D == 128 ? 5 : 10;
+    static constexpr int kQTileBytes = 128 * D * 2;
+    static constexpr int kQBytes = 2 * kQTileBytes;
+    static constexpr int kSmemBytes = 1024 + kQBytes + kStages * kSlotBytes;
+};
+constexpr int kMaxStages = 10;
 
 using namespace tc;
 
-// Instruction descriptor, kind::f16: D = f32, A = B = bf16, M = 128, N = 128.
+// Instruction descriptors, kind::f16: accumulator f32, A = B = bf16, M = 128, N = 128 tokens (QK) or D channels (PV).
 constexpr uint32_t kIdescQK = make_idesc(128, false);
-constexpr uint32_t kIdescPV = make_idesc(128, true);  // B (= V) is MN-major
+template <int D>
+constexpr uint32_t kIdescPV = make_idesc(D, true);  // B (= V) is MN-major
 
 struct __align__(8) Barriers {
     uint64_t q_full;
-    uint64_t kv_full[kStages];  // a K or V tile has landed in its slot
-    uint64_t kv_empty[kStages]; // every contraction that reads the slot has completed (one barrier per slot: a barrier
-                                // shared by all slots could run two phases ahead of the producer, which a parity
-                                // wait cannot tell from none)
-    uint64_t s_full[2];         // phase j: S_t(j) = Q_t K_j^T is complete
-    uint64_t p_full[2];         // phase j: the four softmax warps of row tile t have stored P_t(j)
-    uint64_t o_done[2];         // the last PV of row tile t has completed
+    uint64_t kv_full[kMaxStages];   // a K or V tile has landed in its slot
+    uint64_t kv_empty[kMaxStages];  // every contraction that reads the slot has completed (one barrier per slot: a barrier
+                                    // shared by all slots could run two phases ahead of the producer, which a parity
+                                    // wait cannot tell from none)
+    uint64_t s_full[2];         // phase j: the j-th S of stream t is complete
+    uint64_t p_full[2];         // phase j: the four softmax warps of stream t have stored their j-th P
+    uint64_t o_done[2];         // the last PV of stream t has completed
     uint64_t v_need;            // MMA issuer -> warp 2: this V tile has landed and needs its tail rows zeroed
     uint64_t v_fixed;           // warp 2 -> MMA issuer: done
     uint64_t drain;             // completion of the contractions issued before a wait gave up
@@ -51,49 +66,575 @@ struct __align__(8) Barriers {
     int abort_flag;
 };
 
+// What every role of a CTA knows about its work.
+struct Job {
+    uint8_t* smem;
+    uint32_t q_smem, tmem;
+    int split, rg, h, lb, b, l;
+    int seq_len, M, tok_per_tile, tile_rows, tok0;
+    int tile_begin, n_ctx_tiles, n_tiles, first_fix;
+};
+
+// The roles.  kOne: the row group is one row tile and the streams take alternate K/V tiles.
+// K/V tiles go through the ring in the order in which the issuer releases them: V(i - lag), then K(i), where lag is the
+// number of S buffers that a row tile has (two row tiles: one each, lag 1; one row tile: both, lag 2).
+
+// =========================== TMA producer ================================================
+template <int D>
+__device__ __forceinline__ void copy_q(const TcParams& p, const Job& c, Barriers& bars, bool one, int lane) {
+    using Sh = Shape<D>;
+    const uint32_t qbar = smem_u32(&bars.q_full);
+    const int n_q_tiles = one ? 1 : 2;
+    if (lane == 0) {
+        mbar_expect_tx(qbar, (uint32_t)(n_q_tiles * Sh::kParts * c.tile_rows * 128));
+        for (int t = 0; t < n_q_tiles; ++t)
+            for (int part = 0; part < Sh::kParts; ++part)
+                tma_load_3d(c.q_smem + t * Sh::kQTileBytes + part * 16384, &p.tm_q, part * 64, c.h * p.G,
+                            c.lb * p.M_max + c.tok0 + t * c.tok_per_tile, qbar);
+    }
+    __syncwarp();
+}
+
+// Pool row coordinate of a page of context tile j (128 / page size of them).  Lane kParts pg + part looks page pg
+// up and later issues the copy of that page's 64-channel part, so that a tile's copies leave in one pass of
+// the warp; the table is read one tile ahead so that its latency hides behind the wait for a free slot.
+template <int D>
+__device__ __forceinline__ int page_row(const TcParams& p, const Job& c, int j, int lane) {
+    constexpr int kParts = Shape<D>::kParts;
+    const int ppt = kTileTokens / p.bs, my_pg = lane / kParts;
+    int row = (int)p.pool_rows;  // out of range: the copy engine fills zeros
+    const int blk = (c.tile_begin + j) * ppt + my_pg;
+    if (my_pg < ppt && j < c.n_ctx_tiles && (long long)blk * p.bs < c.seq_len && blk < p.max_blocks) {
+        const int page = p.block_table[(size_t)c.b * p.max_blocks + blk];
+        if (page < 0 || page >= p.n_pages) {
+            if (lane % kParts == 0) record_fault(p.workspace, SPECPV_ERR_BAD_BLOCK_TABLE, c.b, blk, page, c.l);
+        } else {
+            row = (int)((((long long)(p.layer0 + c.l) * p.n_pages + page) * p.Hkv + c.h) * p.bs);
+        }
+    }
+    return row;
+}
+
+// The whole warp runs the loop (a lone lane of a diverged warp runs slowly).
+template <int D>
+__device__ __forceinline__ void produce(const TcParams& p, const Job& c, Barriers& bars, bool one, int first_row, int lane) {
+    using Sh = Shape<D>;
+    constexpr int kStages = Sh::kStages, kParts = Sh::kParts, kSlotBytes = Sh::kSlotBytes;
+    const int lag = one ? 2 : 1;
+    volatile int* abort_flag = &bars.abort_flag;
+    const uint32_t kv_smem = c.q_smem + Sh::kQBytes;
+    const int ppt = kTileTokens / p.bs;
+    const int my_pg = lane / kParts, my_part = lane % kParts;
+    bool ok = true;
+    int row_k = 0, row_v1 = 0, row_v2 = 0, row_next = first_row;  // rows of tiles i, i - 1, i - 2, i + 1
+    uint32_t slot = 0, par = 1, use = 0;  // ring position of the next use; parity of the release that frees its slot
+    for (int i = 0; i < c.n_tiles + lag; ++i) {
+        row_v2 = row_v1;
+        row_v1 = row_k;
+        row_k = row_next;
+        row_next = page_row<D>(p, c, i + 1, lane);
+        for (int kv = 1; kv >= 0; --kv) {  // 1: V tile, 0: K tile
+            const int j = kv ? i - lag : i;
+            if (j < 0 || j >= c.n_tiles) continue;
+            const uint32_t full = smem_u32(&bars.kv_full[slot]), empty = smem_u32(&bars.kv_empty[slot]);
+            if (use >= (uint32_t)kStages) ok = mbar_wait(empty, par, abort_flag, p.workspace, 1);
+            if (!ok) break;  // a wait gave up: nothing more is copied
+            const uint32_t dst = kv_smem + slot * kSlotBytes + my_part * 16384;
+            if (lane == 0) mbar_expect_tx(full, kSlotBytes);
+            if (j >= c.n_ctx_tiles) {  // the step's own tokens: two boxes of 64 rows per part
+                if (my_pg < 2)
+                    tma_load_3d(dst + my_pg * 8192, kv ? &p.tm_vnew : &p.tm_knew, my_part * 64, c.h,
+                                c.lb * p.M_max + my_pg * 64, full);
+            } else if (my_pg < ppt) {
+                tma_load_2d(dst + my_pg * p.bs * 128, kv ? &p.tm_vpool : &p.tm_kpool, my_part * 64,
+                            kv ? (one ? row_v2 : row_v1) : row_k, full);
+            }
+            __syncwarp();
+            ++use;
+            if (++slot == kStages) { slot = 0; par ^= 1; }
+        }
+        if (!ok) break;
+    }
+}
+
+// =========================== MMA issuer ==================================================
+// One warp issues every contraction (issuing from two warps serialises the tensor pipe).  Issue
+// order (ping-pong of the two streams): QK(0,0) QK(0,1) | PV(0,0) QK(1,0) PV(0,1) QK(1,1) | ...
+// Barrier instructions do not overlap with queued MMAs (each costs the pipe 30-100 idle cycles),
+// so the loop keeps them to four waits per KV tile, without votes, and four commits behind MMAs.  The whole
+// warp runs the loop, lane 0 issues.
+template <int D, bool kOne>
+__device__ __forceinline__ void issue(const TcParams& p, const Job& c, Barriers& bars, int lane) {
+    using Sh = Shape<D>;
+    constexpr int kStages = Sh::kStages;
+    constexpr uint32_t kSlotWords = Sh::kSlotBytes >> 4, kQTileWords = Sh::kQTileBytes >> 4;  // 16-byte units of descriptors
+    volatile int* abort_flag = &bars.abort_flag;
+    const uint32_t kv_smem = c.q_smem + Sh::kQBytes, tmem = c.tmem;
+    const int n_tiles = c.n_tiles, first_fix = c.first_fix;
+    bool ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.q_full), 0, abort_flag, p.workspace, 2));
+    // Shared-memory descriptors: the upper word (stride between 8-row groups, version, swizzle) is
+    // constant; the lower word is the 16-byte address plus the leading-dimension offset.
+    const uint32_t desc_hi = (uint32_t)((1024u >> 4) | (1u << 14) | (2u << 29));
+    const uint32_t q_lo = ((c.q_smem >> 4) & 0x3FFFu) | ((16u >> 4) << 16);
+    const uint32_t k_lo0 = ((kv_smem >> 4) & 0x3FFFu) | ((16u >> 4) << 16);
+    const uint32_t v_lo0 = ((kv_smem >> 4) & 0x3FFFu) | ((16384u >> 4) << 16);
+    const uint32_t full0 = smem_u32(&bars.kv_full[0]), empty0 = smem_u32(&bars.kv_empty[0]);
+    const uint32_t sfull0 = smem_u32(&bars.s_full[0]), pfull0 = smem_u32(&bars.p_full[0]);
+    auto issue_pv = [&](int t, uint32_t vb_lo, bool first) {  // O_t (+)= P_t V
+        const uint32_t a = tmem + t * 128, d = tmem + 256 + t * 128;
+#pragma unroll
+        for (int kk = 0; kk < 8; ++kk)  // 16 tokens per instruction: two 8-row K groups of 1024 bytes
+            mma_ts_lohi(d, a + kk * 8, vb_lo + (uint32_t)kk * (2048u >> 4), desc_hi, kIdescPV<D>, (!first || kk > 0) ? 1u : 0u);
+    };
+    auto issue_qk = [&](int t, uint32_t a_lo, uint32_t kb_lo) {  // S_t = Q K^T
+        const uint32_t d = tmem + t * 128;
+#pragma unroll
+        for (int kk = 0; kk < D / 16; ++kk) {  // 16 channels per instruction
+            const uint32_t off = (uint32_t)((kk >> 2) * 16384 + (kk & 3) * 32) >> 4;
+            mma_ss_lohi(d, a_lo + off, kb_lo + off, desc_hi, kIdescQK, kk > 0 ? 1u : 0u);
+        }
+    };
+    // Ring uses: K0 | V0 K1 | V1 K2 | .. with two row tiles, K0 | K1 | V0 K2 | V1 K3 | .. with one.
+    // A wait that gives up raises the abort flag, which makes the later waits of this tile return at once; the
+    // loop ends after this tile, so at most one tile's contractions are issued past the failed wait.  (One exit
+    // per tile: an exit after every wait costs the issuing thread 7 % of the kernel.)
+    if (!kOne) {
+        uint32_t k_slot = 0, k_par = 0, v_slot = 1, v_par = 0;  // slot and phase parity of the next K and V tile
+        for (int j = 0; j <= n_tiles; ++j) {
+            const int jp = j - 1;
+            if (j < n_tiles) ok &= mbar_wait(full0 + k_slot * 8, k_par, abort_flag, p.workspace, 3);
+            if (j > 0) {
+                ok &= mbar_wait(full0 + v_slot * 8, v_par, abort_flag, p.workspace, 4);
+                // a ragged or tree tile: warp 2 zeroes the rows of V past the valid tokens first
+                if (jp >= first_fix) {
+                    if (lane == 0) mbar_arrive(smem_u32(&bars.v_need));
+                    ok &= mbar_wait(smem_u32(&bars.v_fixed), (jp - first_fix) & 1, abort_flag, p.workspace, 9);
+                }
+            }
+            const uint32_t kb_lo = launder(k_lo0 + k_slot * kSlotWords);
+            const uint32_t vb_lo = launder(v_lo0 + v_slot * kSlotWords);
+            for (int t = 0; t < 2; ++t) {
+                if (j > 0) {
+                    ok &= mbar_wait(pfull0 + t * 8, jp & 1, abort_flag, p.workspace, 5);
+                    tc_fence_after();
+                }
+                if (lane == 0) {
+                    if (j > 0) {
+                        issue_pv(t, vb_lo, jp == 0);
+                        if (t == 1) tc_commit(empty0 + v_slot * 8);
+                        if (j == n_tiles) tc_commit(smem_u32(&bars.o_done[t]));
+                    }
+                    if (j < n_tiles) {
+                        issue_qk(t, launder(q_lo + (uint32_t)t * kQTileWords), kb_lo);
+                        tc_commit(sfull0 + t * 8);
+                        if (t == 1) tc_commit(empty0 + k_slot * 8);
+                    }
+                }
+                __syncwarp();
+            }
+            if (!ok) break;
+            if (j < n_tiles) { k_slot += 2; if (k_slot >= kStages) { k_slot -= kStages; k_par ^= 1; } }
+            if (j > 0) { v_slot += 2; if (v_slot >= kStages) { v_slot -= kStages; v_par ^= 1; } }
+        }
+    } else {
+        uint32_t slot = 0, par = 0;
+        auto advance = [&] { if (++slot == kStages) { slot = 0; par ^= 1; } };
+        for (int i = 0; i < n_tiles + 2; ++i) {
+            const int t = i & 1, jv = i - 2;
+            uint32_t k_slot = 0, v_slot = 0;
+            if (jv >= 0) {
+                v_slot = slot;
+                ok &= mbar_wait(full0 + slot * 8, par, abort_flag, p.workspace, 4);
+                advance();
+                if (jv >= first_fix) {
+                    if (lane == 0) mbar_arrive(smem_u32(&bars.v_need));
+                    ok &= mbar_wait(smem_u32(&bars.v_fixed), (jv - first_fix) & 1, abort_flag, p.workspace, 9);
+                }
+                ok &= mbar_wait(pfull0 + t * 8, (jv >> 1) & 1, abort_flag, p.workspace, 5);
+            }
+            if (i < n_tiles) {
+                k_slot = slot;
+                ok &= mbar_wait(full0 + slot * 8, par, abort_flag, p.workspace, 3);
+                advance();
+            }
+            tc_fence_after();
+            if (lane == 0) {
+                if (jv >= 0) {
+                    issue_pv(t, launder(v_lo0 + v_slot * kSlotWords), jv < 2);
+                    tc_commit(empty0 + v_slot * 8);
+                    if (i >= n_tiles) tc_commit(smem_u32(&bars.o_done[t]));
+                }
+                if (i < n_tiles) {
+                    issue_qk(t, q_lo, launder(k_lo0 + k_slot * kSlotWords));
+                    tc_commit(sfull0 + t * 8);
+                    tc_commit(empty0 + k_slot * 8);
+                }
+            }
+            __syncwarp();
+            if (!ok) break;
+        }
+    }
+    if (!ok && lane == 0) {
+        // after a give-up: wait (bounded) until the contractions that WERE issued have completed, so that the
+        // tensor memory is not freed under them
+        tc_commit(smem_u32(&bars.drain));
+        const uint64_t t0 = global_ns();
+        while (!mbar_try_wait(smem_u32(&bars.drain), 0) && global_ns() - t0 < 100000000ull) {}
+    }
+    __syncwarp();
+}
+
+// =========================== V fixer =====================================================
+// Rows of a V tile past its valid tokens may hold anything (stale shared memory, rows of other
+// sequences' steps): zero them so that 0 * garbage cannot produce NaN.  Only the last context
+// tile (when ragged) and the tile of the step's own tokens can need it.
+template <int D, bool kOne>
+__device__ __forceinline__ void fix_v(const TcParams& p, const Job& c, Barriers& bars, int lane) {
+    using Sh = Shape<D>;
+    for (int jp = c.first_fix; jp < c.n_tiles; ++jp) {
+        const int use = kOne && jp < c.n_tiles - 1 ? 2 * jp + 2 : 2 * jp + 1;  // the ring use of V(jp)
+        // the request arrives once the tile has landed (a wait on the slot's own barrier this far
+        // ahead of the pipeline could match an earlier phase of the same parity)
+        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.v_need), (jp - c.first_fix) & 1, &bars.abort_flag, p.workspace, 10)))
+            break;
+        const int n_valid = jp >= c.n_ctx_tiles ? c.M : min(kTileTokens, c.seq_len - (c.tile_begin + jp) * kTileTokens);
+        uint8_t* v = c.smem + Sh::kQBytes + (size_t)(use % Sh::kStages) * Sh::kSlotBytes;
+        const int n_rows = kTileTokens - n_valid;
+        for (int i = lane; i < n_rows * Sh::kParts * 8; i += 32) {
+            const int chunk = i & 7, part = (i >> 3) % Sh::kParts, r = n_valid + (i >> 3) / Sh::kParts;
+            *reinterpret_cast<uint4*>(v + part * 16384 + r * 128 + chunk * 16) = make_uint4(0, 0, 0, 0);
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&bars.v_fixed));
+    }
+}
+
+// =========================== softmax / correction / epilogue ==============================
+template <int D, bool kOne>
+__device__ __forceinline__ void softmax(const TcParams& p, const Job& c, Barriers& bars, int warp, int lane) {
+    using Sh = Shape<D>;
+    volatile int* abort_flag = &bars.abort_flag;
+    const int t = (warp - 4) >> 2;           // stream of this warpgroup
+    const int q = warp & 3;                  // TMEM lane quarter this warp may access
+    const int row_in_tile = q * 32 + lane;
+    const int n_tiles = c.n_tiles;
+    constexpr int step = kOne ? 2 : 1;
+    const int first_tile = kOne ? t : 0;     // K/V tiles of this stream: first_tile, first_tile + step, ..
+    if (first_tile >= n_tiles) return;
+    const int row_tile = kOne ? 0 : t;
+    const int row = row_tile * 128 + row_in_tile;                              // row within the row group
+    const int tok = c.tok0 + row_tile * c.tok_per_tile + row_in_tile / p.G;    // step token of this row
+    const int g = row_in_tile % p.G;
+    const bool row_valid = row_in_tile < c.tile_rows && tok < c.M;
+    const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
+    const uint32_t s_addr = c.tmem + lane_addr + t * 128;
+    const uint32_t o_addr = c.tmem + lane_addr + 256 + t * 128;
+    uint64_t mask_lo = 0, mask_hi = 0;
+    if (row_valid) {
+        const uint64_t* mrow = p.tree_mask + ((size_t)c.b * p.M_max + tok) * p.mask_words;
+        mask_lo = mrow[0];
+        if (p.mask_words > 1) mask_hi = mrow[1];
+    }
+    float m_run = -INFINITY, l_run = 0.f;
+    bool ok = true;
+    const float2 sc2 = make_float2(p.scale_log2, p.scale_log2);
+    // One row tile (the form of short calls): the first pass of the loop is a dry run over zeros by the stream whose S comes
+    // last, while Q and the first K tile are still on their way: it brings the loop's code (some 20 KB, straight-line) into
+    // the instruction cache.  In a model's layer other kernels have run since the last call, and with cold code the first
+    // tile took 4.6-5 us from S to P instead of 1.5.  (The form with two row tiles walks long contexts, where its loop
+    // ran 8 % slower with the dry run in it.)
+    const bool warm_up = kOne && (t == 1 || n_tiles == 1);
+    uint32_t s_par = warm_up ? 1 : 0;
+    for (int j = warm_up ? first_tile - step : first_tile; j < n_tiles && ok; j += step, s_par ^= 1) {
+        const bool dry = kOne && j < first_tile;
+        const bool is_new = j >= c.n_ctx_tiles;
+        const int n_valid = is_new ? c.M : min(kTileTokens, c.seq_len - (c.tile_begin + j) * kTileTokens);
+        const bool masked = is_new || n_valid < kTileTokens;
+        uint64_t vis_lo = ~0ull, vis_hi = ~0ull;  // visibility of the tile's 128 columns for this row
+        if (masked) {
+            if (is_new) {
+                vis_lo = mask_lo;
+                vis_hi = mask_hi;
+            }
+            if (n_valid < 64) {
+                vis_lo &= (n_valid <= 0) ? 0ull : (~0ull >> (64 - n_valid));
+                vis_hi = 0;
+            } else if (n_valid < 128) {
+                vis_hi &= (n_valid == 64) ? 0ull : (~0ull >> (128 - n_valid));
+            }
+        }
+        // the whole row of S (128 columns) goes to registers in one round trip
+        uint32_t v[128];
+        auto load_s = [&] {
+            TMEM_LD32(s_addr, v);
+            TMEM_LD32(s_addr + 32, (v + 32));
+            TMEM_LD32(s_addr + 64, (v + 64));
+            TMEM_LD32(s_addr + 96, (v + 96));
+            tmem_wait_ld();
+        };
+        if (!dry) {
+            ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.s_full[t]), s_par, abort_flag, p.workspace, 6));
+            if (!ok) break;
+            tc_fence_after();
+            load_s();
+        } else {
+#pragma unroll
+            for (int i = 0; i < 128; ++i) v[i] = 0;
+        }
+        // P = 2^(s*scale - m) as bf16 pairs, packed in place: word i of P (columns 2i, 2i+1) overwrites
+        // v[i], whose own value was consumed by an earlier pair, so no second register array is needed.
+        // The row sum is taken over the ROUNDED weights the tensor core will use, so that O / l is an
+        // exact weighted average of V rows (the rounding error of a dominant weight cancels instead of
+        // scaling the output).
+        auto exp_row = [&](float m_use) {
+            const float2 nm2 = make_float2(-m_use, -m_use);
+            float2 sum2[4];  // independent partial sums: one chain of 64 dependent adds would outlast the exponentials
+#pragma unroll
+            for (int e = 0; e < 4; ++e) sum2[e] = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int i = 0; i < 64; ++i) {
+                const float2 x = __ffma2_rn(make_float2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1])),
+                                            sc2, nm2);
+                const uint32_t w = pack_bf16(ex2(x.x), ex2(x.y));
+                v[i] = w;
+                add_bf16_pair(sum2[i & 3], w);
+            }
+            const float2 s01 = __fadd2_rn(sum2[0], sum2[1]), s23 = __fadd2_rn(sum2[2], sum2[3]);
+            return (s01.x + s23.x) + (s01.y + s23.y);
+        };
+        // Fast path (every full context tile after the stream's first): keep the reference m_run of the row as it
+        // is and skip the row maximum.  Weights may then exceed 1; float32 sums and bf16 weights keep
+        // their relative precision whatever the exponent, so only overflow has to be ruled out: if a
+        // row sum leaves the safe range (or a row has no reference yet), the warp takes the tile again
+        // from tensor memory on the general path, which brings m_run up to date.  (The dry run, without a reference,
+        // passes through both paths.)
+        float l_add = 0.f;
+        bool general = !dry && (j == first_tile || masked);
+        if (!general) {
+            l_add = exp_row(m_run);
+            const bool bad = !(l_add < kSafeRowSum) || m_run == -INFINITY;
+            if (__any_sync(0xffffffffu, bad)) {
+                general = true;
+                if (!dry) load_s();  // S_t is still intact: P has not been stored yet
+            }
+        }
+        if (general) {
+            if (masked) {  // ragged or tree-masked tile: invisible columns become -inf (at most two tiles per CTA)
+#pragma unroll
+                for (int i = 0; i < 128; ++i) {
+                    const uint64_t word = i < 64 ? vis_lo : vis_hi;
+                    if (!((word >> (i & 63)) & 1ull)) v[i] = 0xff800000u;
+                }
+            }
+            float mx0 = __uint_as_float(v[0]), mx1 = __uint_as_float(v[1]), mx2 = __uint_as_float(v[2]),
+                  mx3 = __uint_as_float(v[3]);
+#pragma unroll
+            for (int i = 4; i < 124; i += 8) {  // three-input max: two new values per instruction
+                mx0 = fmax3(mx0, __uint_as_float(v[i]), __uint_as_float(v[i + 1]));
+                mx1 = fmax3(mx1, __uint_as_float(v[i + 2]), __uint_as_float(v[i + 3]));
+                mx2 = fmax3(mx2, __uint_as_float(v[i + 4]), __uint_as_float(v[i + 5]));
+                mx3 = fmax3(mx3, __uint_as_float(v[i + 6]), __uint_as_float(v[i + 7]));
+            }
+            mx0 = fmax3(mx0, __uint_as_float(v[124]), __uint_as_float(v[125]));
+            mx1 = fmax3(mx1, __uint_as_float(v[126]), __uint_as_float(v[127]));
+            const float mx = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3));
+            const float m_tile = mx * p.scale_log2;
+            // lazy rescale: keep the old reference max unless the new one is more than 2^8 larger.
+            // The decision is per row, the tensor-memory traffic is warp-wide: if any row of the
+            // warp rescales, all 32 rows pass through it (with a factor of 1 where nothing changes).
+            bool need = false;
+            if (j <= first_tile) {
+                m_run = m_tile;
+            } else {
+                need = m_tile > m_run + kRescaleThreshold || (m_run == -INFINITY && m_tile > -INFINITY);
+            }
+            if (__any_sync(0xffffffffu, need)) {
+                const float factor = !need ? 1.f : (m_run == -INFINITY ? 0.f : ex2(m_run - m_tile));
+                // O_t already holds every earlier PV of this stream: the tensor pipe runs in order, and S_t, issued
+                // after them, is complete
+#pragma unroll (kOne ? 1 : D / 32)
+                for (int cc = 0; cc < D / 32; ++cc) {
+                    uint32_t o[32];
+                    TMEM_LD32(o_addr + cc * 32, o);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * factor);
+                    TMEM_ST32(o_addr + cc * 32, o);
+                }
+                if (need) {
+                    l_run *= factor;
+                    m_run = m_tile;
+                }
+            }
+            l_add = exp_row(m_run == -INFINITY ? 0.f : m_run);
+        }
+        if (dry) {
+            l_run = l_add < 0.f ? l_add : 0.f;  // never negative: zero again, and the dry run's sums are not dead code
+            continue;
+        }
+        TMEM_ST32(s_addr, v);
+        TMEM_ST32(s_addr + 32, (v + 32));
+        l_run += l_add;
+        tmem_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&bars.p_full[t]));
+    }
+    // ---- epilogue: wait for the last PV, normalise, write out ---------------------------
+    if (ok) ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.o_done[t]), 0, abort_flag, p.workspace, 8));
+    // One row tile, both streams in use: stream t finishes channels [t D/2, (t+1) D/2) and leaves the other half of
+    // its accumulator in the ring (every copy has been consumed, and the other stream's contractions have read it
+    // too), channel-major so that a warp's rows are adjacent.
+    const bool meet = kOne && n_tiles > 1;
+    constexpr int kHalfD = D / 2;
+    float* xo = reinterpret_cast<float*>(c.smem + Sh::kQBytes);  // [2][D/2][128]
+    float* xml = xo + 2 * kHalfD * 128;                          // [2][2][128]: reference maximum, row sum
+    if (meet) {
+        if (ok) ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.o_done[1 - t]), 0, abort_flag, p.workspace, 8));
+        if (ok) {
+            tc_fence_after();
+#pragma unroll 1
+            for (int cc = 0; cc < kHalfD / 32; ++cc) {
+                uint32_t v[32];
+                TMEM_LD32(o_addr + (1 - t) * kHalfD + cc * 32, v);
+                tmem_wait_ld();
+#pragma unroll
+                for (int i = 0; i < 32; ++i) xo[(t * kHalfD + cc * 32 + i) * 128 + row_in_tile] = __uint_as_float(v[i]);
+            }
+            xml[t * 256 + row_in_tile] = m_run;
+            xml[t * 256 + 128 + row_in_tile] = l_run;
+        }
+        asm volatile("bar.sync 1, 256;" ::: "memory");  // both streams' warps come here, whatever their waits returned
+        if (*abort_flag) ok = false;
+    }
+    if (!ok) return;
+    tc_fence_after();
+    float w_mine = 1.f, w_other = 0.f;  // weights of the two streams relative to their common maximum
+    if (meet) {
+        const float m_o = xml[(1 - t) * 256 + row_in_tile], l_o = xml[(1 - t) * 256 + 128 + row_in_tile];
+        const float m_all = fmaxf(m_run, m_o);
+        w_mine = m_run == -INFINITY ? 0.f : ex2(m_run - m_all);
+        w_other = m_o == -INFINITY ? 0.f : ex2(m_o - m_all);
+        l_run = l_run * w_mine + l_o * w_other;
+        m_run = m_all;
+    }
+    const bool direct = p.n_splits == 1;
+    const float inv = direct ? 1.f / l_run : 1.f;
+    w_mine *= inv;
+    w_other *= inv;
+    const size_t out_row = ((size_t)c.lb * p.M_max + tok) * p.Hq + c.h * p.G + g;
+    const size_t prow = (((size_t)c.lb * p.Hkv + c.h) * p.n_splits + c.split) * p.R_pad + c.rg * p.rg_tiles * 128 + row;
+    const int c_begin = meet ? t * kHalfD : 0, c_end = meet ? c_begin + kHalfD : D;
+    const float* other = xo + (1 - t) * kHalfD * 128 + row_in_tile;
+#pragma unroll (kOne ? 1 : D / 32)
+    for (int c0 = c_begin; c0 < c_end; c0 += 32) {
+        uint32_t v[32];
+        TMEM_LD32(o_addr + c0, v);
+        tmem_wait_ld();
+        if (!row_valid) continue;
+        if (meet) {
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+                v[i] = __float_as_uint(__uint_as_float(v[i]) * w_mine + other[(c0 - c_begin + i) * 128] * w_other);
+        } else if (direct) {
+#pragma unroll
+            for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) * inv);
+        }
+        if (!direct) {
+            // a thread's row is contiguous: 32-byte stores fill whole sectors, half as many
+            // memory transactions as 16-byte ones for this one-row-per-lane pattern
+            float* dst = p.part_o + prow * D + c0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + 8 * i),
+                             "r"(v[8 * i]), "r"(v[8 * i + 1]), "r"(v[8 * i + 2]), "r"(v[8 * i + 3]), "r"(v[8 * i + 4]),
+                             "r"(v[8 * i + 5]), "r"(v[8 * i + 6]), "r"(v[8 * i + 7])
+                             : "memory");
+        } else if (p.out_f32) {  // the caller's buffer: 16-byte aligned
+            uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<float*>(p.out) + out_row * D + c0);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) dst[i] = make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+        } else {
+            uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(p.out) + out_row * D + c0);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                uint4 w;
+                w.x = pack_bf16(__uint_as_float(v[8 * i]), __uint_as_float(v[8 * i + 1]));
+                w.y = pack_bf16(__uint_as_float(v[8 * i + 2]), __uint_as_float(v[8 * i + 3]));
+                w.z = pack_bf16(__uint_as_float(v[8 * i + 4]), __uint_as_float(v[8 * i + 5]));
+                w.w = pack_bf16(__uint_as_float(v[8 * i + 6]), __uint_as_float(v[8 * i + 7]));
+                dst[i] = w;
+            }
+        }
+    }
+    if (row_valid && (!meet || t == 0)) {
+        if (direct) {
+            if (p.lse) p.lse[out_row] = m_run * kLn2 + logf(l_run);
+        } else {
+            p.part_ml[prow * 2] = m_run * kLn2;  // natural-log units for the merge
+            p.part_ml[prow * 2 + 1] = l_run;
+        }
+    }
+}
+
 // =================================================================================================
+// kForm: the row groups a launch can meet (a kernel with both forms has twice the code, which a call that follows other
+// kernels pays for in instruction-cache misses).
+enum { kOneTile, kTwoTiles, kBoth };
+template <int D, int kForm>
 __global__ void __launch_bounds__(kThreadsTc, 1) attn_tc_kernel(const __grid_constant__ TcParams p) {
+    using Sh = Shape<D>;
     extern __shared__ uint8_t smem_raw[];
-    // 1024-byte alignment for the 128-byte swizzle atoms
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     __shared__ Barriers bars;
-
+    Job c;
+    // 1024-byte alignment for the 128-byte swizzle atoms
+    c.smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int split = blockIdx.x % p.n_splits, rg = blockIdx.x / p.n_splits;
-    const int h = blockIdx.y, lb = blockIdx.z;
-    const int b = lb % p.batch, l = lb / p.batch;
+    // CTA order: all full row groups first (those of a head side by side, they read the same K/V), then the row groups of
+    // one tile, which are shorter and fill the machine's tail
+    c.split = blockIdx.x % p.n_splits;
+    int unit = blockIdx.x / p.n_splits;
+    if (unit < p.n_full_units) {
+        c.rg = unit % p.n_full_groups;
+        unit /= p.n_full_groups;
+    } else {
+        c.rg = p.n_full_groups;
+        unit -= p.n_full_units;
+    }
+    c.h = unit % p.Hkv;
+    c.lb = unit / p.Hkv;
+    c.b = c.lb % p.batch;
+    c.l = c.lb / p.batch;
 
-    const int seq_len = max(p.seq_lens[b], 0);
-    int M = p.q_lens ? p.q_lens[b] : p.M_max;
-    M = min(max(M, 0), p.M_max);
-    const int tok_per_tile = 128 / p.G;               // step tokens per 128-row tile
-    const int tok0 = rg * 2 * tok_per_tile;           // first step token of this row group
-    if (tok0 >= M) return;                            // nothing to do (uniform for the CTA)
-    const int n_q_tiles = (M - tok0 > tok_per_tile) ? 2 : 1;
+    c.seq_len = max(p.seq_lens[c.b], 0);
+    c.M = p.q_lens ? p.q_lens[c.b] : p.M_max;
+    c.M = min(max(c.M, 0), p.M_max);
+    c.tok_per_tile = 128 / p.G;                  // step tokens per 128-row tile
+    c.tile_rows = c.tok_per_tile * p.G;          // rows of a tile in use (all 128 when G divides 128)
+    c.tok0 = c.rg * p.rg_tiles * c.tok_per_tile; // first step token of this row group
+    if (c.tok0 >= c.M) return;                   // nothing to do (uniform for the CTA)
+    const bool one = kForm == kOneTile || (kForm == kBoth && c.M - c.tok0 <= c.tok_per_tile);  // one row tile
 
-    // KV range of this split: whole 128-token tiles, split evenly over the sequence's tiles
-    const int total_tiles = (seq_len + kTileTokens - 1) / kTileTokens;
-    const int tiles_per_split = (total_tiles + p.n_splits - 1) / p.n_splits;
-    const int tile_begin = min(split * tiles_per_split, total_tiles);
-    const int tile_end = min(tile_begin + tiles_per_split, total_tiles);
-    const bool last_split = split == p.n_splits - 1;
-    const int n_ctx_tiles = tile_end - tile_begin;
-    const int n_tiles = n_ctx_tiles + (last_split ? 1 : 0);  // the last split also attends the step's own tokens
+    // KV range of this split: an equal share of the sequence's 128-token tiles and the tile of the step's own tokens,
+    // which comes last
+    const int total_tiles = (c.seq_len + kTileTokens - 1) / kTileTokens;
+    c.tile_begin = (int)((long long)(total_tiles + 1) * c.split / p.n_splits);
+    c.n_tiles = (int)((long long)(total_tiles + 1) * (c.split + 1) / p.n_splits) - c.tile_begin;
+    const bool last_split = c.split == p.n_splits - 1;
+    c.n_ctx_tiles = c.n_tiles - (last_split ? 1 : 0);
+    const int tile_end = c.tile_begin + c.n_ctx_tiles;
     // first tile whose V rows need zeroing past the valid tokens: a ragged last context tile, else the
     // tile of the step's own tokens (fewer than 128), else none
-    const bool ragged_ctx = n_ctx_tiles > 0 && tile_end == total_tiles && (seq_len % kTileTokens) != 0;
-    const int first_fix = ragged_ctx ? n_ctx_tiles - 1 : ((last_split && M < kTileTokens) ? n_ctx_tiles : n_tiles);
+    const bool ragged_ctx = c.n_ctx_tiles > 0 && tile_end == total_tiles && (c.seq_len % kTileTokens) != 0;
+    c.first_fix = ragged_ctx ? c.n_ctx_tiles - 1 : ((last_split && c.M < kTileTokens) ? c.n_ctx_tiles : c.n_tiles);
 
-    const uint32_t q_smem = smem_u32(smem);
-    const uint32_t kv_smem = q_smem + kQBytes;
-    volatile int* abort_flag = &bars.abort_flag;
-
-    if (n_tiles == 0) {
+    if (c.n_tiles == 0) {
         // an empty split: publish (m = -inf, l = 0) so that the merge ignores it
-        for (int r = threadIdx.x; r < 256; r += kThreadsTc) {
-            const int row = rg * 256 + r;
+        for (int r = threadIdx.x; r < p.rg_tiles * 128; r += kThreadsTc) {
+            const int row = c.rg * p.rg_tiles * 128 + r;
             if (row < p.R_pad) {
-                const size_t prow = (((size_t)lb * p.Hkv + h) * p.n_splits + split) * p.R_pad + row;
+                const size_t prow = (((size_t)c.lb * p.Hkv + c.h) * p.n_splits + c.split) * p.R_pad + row;
                 p.part_ml[prow * 2] = -INFINITY;
                 p.part_ml[prow * 2 + 1] = 0.f;
             }
@@ -102,22 +643,37 @@ __global__ void __launch_bounds__(kThreadsTc, 1) attn_tc_kernel(const __grid_con
     }
 
     // ---- set-up ------------------------------------------------------------------------------
-    if (threadIdx.x == 0) {
-        mbar_init(smem_u32(&bars.q_full), 1);
-        for (int s = 0; s < kStages; ++s) {
-            mbar_init(smem_u32(&bars.kv_full[s]), 1);
-            mbar_init(smem_u32(&bars.kv_empty[s]), 1);
+    // Warp 0 initialises the barriers, starts the copy of Q and looks the first tile's pages up while the tensor memory is
+    // allocated: the first K tile is two dependent loads (lengths, block table) and a copy away.
+    c.q_smem = smem_u32(c.smem);
+    int first_row = 0;
+    if (warp == 0) {
+        if (lane == 0) {
+            mbar_init(smem_u32(&bars.q_full), 1);
+            for (int s = 0; s < Sh::kStages; ++s) {
+                mbar_init(smem_u32(&bars.kv_full[s]), 1);
+                mbar_init(smem_u32(&bars.kv_empty[s]), 1);
+            }
+            for (int t = 0; t < 2; ++t) {
+                mbar_init(smem_u32(&bars.s_full[t]), 1);
+                mbar_init(smem_u32(&bars.p_full[t]), 4);  // one arrival per softmax warp
+                mbar_init(smem_u32(&bars.o_done[t]), 1);
+            }
+            mbar_init(smem_u32(&bars.v_need), 1);
+            mbar_init(smem_u32(&bars.v_fixed), 1);
+            mbar_init(smem_u32(&bars.drain), 1);
+            bars.abort_flag = 0;
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         }
-        for (int t = 0; t < 2; ++t) {
-            mbar_init(smem_u32(&bars.s_full[t]), 1);
-            mbar_init(smem_u32(&bars.p_full[t]), 4);  // one arrival per softmax warp
-            mbar_init(smem_u32(&bars.o_done[t]), 1);
-        }
-        mbar_init(smem_u32(&bars.v_need), 1);
-        mbar_init(smem_u32(&bars.v_fixed), 1);
-        mbar_init(smem_u32(&bars.drain), 1);
-        bars.abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        __syncwarp();
+        copy_q<D>(p, c, bars, one, lane);
+        first_row = page_row<D>(p, c, 0, lane);
+    }
+    if (c.tile_rows < 128) {  // rows past the packed ones are never copied: finite values, so that their softmax stays quiet
+        const int n = (128 - c.tile_rows) * 8;
+        for (int i = threadIdx.x; i < 2 * Sh::kParts * n; i += kThreadsTc)
+            *reinterpret_cast<uint4*>(c.smem + (i / n) * 16384 + c.tile_rows * 128 + (i % n) * 16) = make_uint4(0, 0, 0, 0);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     if (warp == 1) {
@@ -128,370 +684,25 @@ __global__ void __launch_bounds__(kThreadsTc, 1) attn_tc_kernel(const __grid_con
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = bars.tmem_base;
+    c.tmem = bars.tmem_base;
     // tensor-memory columns: S_t at t*128, O_t at 256 + t*128; P_t aliases S_t (64 columns of bf16 pairs)
 
-    // Register budget: the control warpgroup (warps 0-3) gives registers to the two softmax warpgroups.
+    // Register budget: the control warpgroup (warps 0-3) gives registers to the two softmax warpgroups: 128 x 56 +
+    // 256 x 224 = the 384 x 168 of the launch.
     if (warp == 0) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
-        // =========================== TMA producer ================================================
-        // The whole warp runs the loop (a lone lane of a diverged warp runs slowly); lane 0 issues the copies.
-        const uint32_t qbar = smem_u32(&bars.q_full);
-        if (lane == 0) {
-            mbar_expect_tx(qbar, (uint32_t)(n_q_tiles * 32768));
-            for (int t = 0; t < n_q_tiles; ++t)
-                for (int half = 0; half < 2; ++half)
-                    tma_load_3d(q_smem + t * 32768 + half * 16384, &p.tm_q, half * 64, h * p.G,
-                                lb * p.M_max + tok0 + t * tok_per_tile, qbar);
-        }
-        __syncwarp();
-        const int32_t* table = p.block_table + (size_t)b * p.max_blocks;
-        const long long layer_row0 = (long long)(p.layer0 + l) * p.n_pages;
-        bool ok = true;
-        // Pool row coordinate of a context tile's pages (128 / page size of them).  Lane 2 pg + half looks page pg
-        // up and later issues the copy of that page's 64-channel half, so that a tile's copies leave in one pass of
-        // the warp; the table is read one tile ahead so that its latency hides behind the wait for a free slot.
-        const int ppt = kTileTokens / p.bs;
-        const int my_pg = lane >> 1, my_half = lane & 1;
-        auto page_row = [&](int j) {
-            int row = (int)p.pool_rows;  // out of range: the copy engine fills zeros
-            const int blk = (tile_begin + j) * ppt + my_pg;
-            if (my_pg < ppt && j < n_ctx_tiles && (long long)blk * p.bs < seq_len && blk < p.max_blocks) {
-                const int page = table[blk];
-                if (page < 0 || page >= p.n_pages) {
-                    if (my_half == 0) record_fault(p.workspace, SPECPV_ERR_BAD_BLOCK_TABLE, b, blk, page, l);
-                } else {
-                    row = (int)(((layer_row0 + page) * p.Hkv + h) * p.bs);
-                }
-            }
-            return row;
-        };
-        int row_next = page_row(0);
-        uint32_t slot = 0, par = 1;  // ring position of the next use; parity of the release that frees its slot
-        for (int j = 0; j < n_tiles; ++j) {
-            const bool is_new = j >= n_ctx_tiles;
-            const int row_mine = row_next;
-            row_next = page_row(j + 1);
-            for (int kv = 0; kv < 2; ++kv) {  // 0: K tile, 1: V tile
-                const uint32_t full = smem_u32(&bars.kv_full[slot]), empty = smem_u32(&bars.kv_empty[slot]);
-                if (2 * j + kv >= kStages) ok = mbar_wait(empty, par, abort_flag, p.workspace, 1);
-                if (!ok) break;  // a wait gave up: nothing more is copied
-                const uint32_t dst = kv_smem + slot * kSlotBytes + my_half * 16384;
-                if (lane == 0) mbar_expect_tx(full, kSlotBytes);
-                if (is_new) {  // the step's own tokens: two boxes of 64 rows per half
-                    if (lane < 4)
-                        tma_load_3d(dst + my_pg * 8192, kv ? &p.tm_vnew : &p.tm_knew, my_half * 64, h, lb * p.M_max + my_pg * 64,
-                                    full);
-                } else if (my_pg < ppt) {
-                    tma_load_2d(dst + my_pg * p.bs * 128, kv ? &p.tm_vpool : &p.tm_kpool, my_half * 64, row_mine, full);
-                }
-                __syncwarp();
-                if (++slot == kStages) { slot = 0; par ^= 1; }
-            }
-            if (!ok) break;
-        }
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+        produce<D>(p, c, bars, one, first_row, lane);
     } else if (warp == 1) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
-        // =========================== MMA issuer ==================================================
-        // One warp issues every contraction (issuing from two warps serialises the tensor pipe).  Issue
-        // order (ping-pong of the two row tiles): QK(0,0) QK(0,1) | PV(0,0) QK(1,0) PV(0,1) QK(1,1) | ...
-        // Barrier instructions do not overlap with queued MMAs (each costs the pipe 30-100 idle cycles),
-        // so the loop keeps them to four waits per KV tile, without votes, and four commits behind MMAs.  The whole
-        // warp runs the loop, lane 0 issues.
-        bool ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.q_full), 0, abort_flag, p.workspace, 2));
-        // Shared-memory descriptors: the upper word (stride between 8-row groups, version, swizzle) is
-        // constant; the lower word is the 16-byte address plus the leading-dimension offset.
-        const uint32_t desc_hi = (uint32_t)((1024u >> 4) | (1u << 14) | (2u << 29));
-        const uint32_t q_lo = ((q_smem >> 4) & 0x3FFFu) | ((16u >> 4) << 16);
-        const uint32_t k_lo0 = ((kv_smem >> 4) & 0x3FFFu) | ((16u >> 4) << 16);
-        const uint32_t v_lo0 = ((kv_smem >> 4) & 0x3FFFu) | ((16384u >> 4) << 16);
-        const uint32_t full0 = smem_u32(&bars.kv_full[0]), empty0 = smem_u32(&bars.kv_empty[0]);
-        const uint32_t sfull0 = smem_u32(&bars.s_full[0]), pfull0 = smem_u32(&bars.p_full[0]);
-        // ring position of K tile j (use 2j) and of V tile j-1 (use 2j-1): slot and phase parity
-        uint32_t k_slot = 0, k_par = 0, v_slot = 1, v_par = 0;
-        for (int j = 0; j <= n_tiles; ++j) {
-            const int jp = j - 1;
-            // A wait that gives up raises the abort flag, which makes the later waits of this tile return at once; the
-            // loop ends after this tile, so at most one tile's contractions are issued past the failed wait.  (One exit
-            // per tile: an exit after every wait costs the issuing thread 7 % of the kernel.)
-            if (j < n_tiles) ok &= mbar_wait(full0 + k_slot * 8, k_par, abort_flag, p.workspace, 3);
-            if (j > 0) {
-                ok &= mbar_wait(full0 + v_slot * 8, v_par, abort_flag, p.workspace, 4);
-                // a ragged or tree tile: warp 2 zeroes the rows of V past the valid tokens first
-                if (jp >= first_fix) {
-                    if (lane == 0) mbar_arrive(smem_u32(&bars.v_need));
-                    ok &= mbar_wait(smem_u32(&bars.v_fixed), (jp - first_fix) & 1, abort_flag, p.workspace, 9);
-                }
-            }
-            const uint32_t kb_lo = launder(k_lo0 + k_slot * (kSlotBytes >> 4));
-            const uint32_t vb_lo = launder(v_lo0 + v_slot * (kSlotBytes >> 4));
-            for (int t = 0; t < n_q_tiles; ++t) {
-                if (j > 0) {
-                    ok &= mbar_wait(pfull0 + t * 8, jp & 1, abort_flag, p.workspace, 5);
-                    tc_fence_after();
-                }
-                if (lane == 0) {
-                    if (j > 0) {  // O_t += P_t V_{j-1}
-                        const uint32_t a = tmem + t * 128, d = tmem + 256 + t * 128;
-#pragma unroll
-                        for (int kk = 0; kk < 8; ++kk)  // 16 tokens per instruction: two 8-row K groups of 1024 bytes
-                            mma_ts_lohi(d, a + kk * 8, vb_lo + (uint32_t)kk * (2048u >> 4), desc_hi, kIdescPV,
-                                        (jp > 0 || kk > 0) ? 1u : 0u);
-                        if (t == n_q_tiles - 1) tc_commit(empty0 + v_slot * 8);
-                        if (j == n_tiles) tc_commit(smem_u32(&bars.o_done[t]));
-                    }
-                    if (j < n_tiles) {  // S_t = Q_t K_j^T
-                        const uint32_t a_lo = launder(q_lo + (uint32_t)t * (32768u >> 4));
-                        const uint32_t d = tmem + t * 128;
-#pragma unroll
-                        for (int kk = 0; kk < 8; ++kk) {  // 16 channels of d per instruction
-                            const uint32_t off = (uint32_t)((kk >> 2) * 16384 + (kk & 3) * 32) >> 4;
-                            mma_ss_lohi(d, a_lo + off, kb_lo + off, desc_hi, kIdescQK, kk > 0 ? 1u : 0u);
-                        }
-                        tc_commit(sfull0 + t * 8);
-                        if (t == n_q_tiles - 1) tc_commit(empty0 + k_slot * 8);
-                    }
-                }
-                __syncwarp();
-            }
-            if (!ok) break;
-            if (j < n_tiles) { k_slot += 2; if (k_slot >= kStages) { k_slot -= kStages; k_par ^= 1; } }
-            if (j > 0) { v_slot += 2; if (v_slot >= kStages) { v_slot -= kStages; v_par ^= 1; } }
-        }
-        if (!ok && lane == 0) {
-            // after a give-up: wait (bounded) until the contractions that WERE issued have completed, so that the
-            // tensor memory is not freed under them
-            tc_commit(smem_u32(&bars.drain));
-            const uint64_t t0 = global_ns();
-            while (!mbar_try_wait(smem_u32(&bars.drain), 0) && global_ns() - t0 < 100000000ull) {}
-        }
-        __syncwarp();
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+        one ? issue<D, true>(p, c, bars, lane) : issue<D, false>(p, c, bars, lane);
     } else if (warp == 2) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
-        // =========================== V fixer =====================================================
-        // Rows of a V tile past its valid tokens may hold anything (stale shared memory, rows of other
-        // sequences' steps): zero them so that 0 * garbage cannot produce NaN.  Only the last context
-        // tile (when ragged) and the tile of the step's own tokens can need it.
-        for (int jp = first_fix; jp < n_tiles; ++jp) {
-            const int use = 2 * jp + 1;
-            // the request arrives once the tile has landed (a wait on the slot's own barrier this far
-            // ahead of the pipeline could match an earlier phase of the same parity)
-            if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.v_need), (jp - first_fix) & 1, abort_flag, p.workspace, 10)))
-                break;
-            const int n_valid = jp >= n_ctx_tiles ? M : min(kTileTokens, seq_len - (tile_begin + jp) * kTileTokens);
-            uint8_t* v = smem + kQBytes + (size_t)(use % kStages) * kSlotBytes;
-            const int n_rows = kTileTokens - n_valid;
-            for (int i = lane; i < n_rows * 2 * 8; i += 32) {
-                const int chunk = i & 7, half = (i >> 3) & 1, r = n_valid + (i >> 4);
-                *reinterpret_cast<uint4*>(v + half * 16384 + r * 128 + chunk * 16) = make_uint4(0, 0, 0, 0);
-            }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&bars.v_fixed));
-        }
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+        one ? fix_v<D, true>(p, c, bars, lane) : fix_v<D, false>(p, c, bars, lane);
     } else if (warp == 3) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
-        // =========================== softmax / correction / epilogue ==============================
-        const int t = (warp - 4) >> 2;           // row tile of this warpgroup
-        const int q = warp & 3;                  // TMEM lane quarter this warp may access
-        const int row_in_tile = q * 32 + lane;
-        if (t < n_q_tiles) {
-            const int row = t * 128 + row_in_tile;                 // row within the row group
-            const int tok = tok0 + row / p.G;                      // step token of this row
-            const int g = row % p.G;
-            const bool row_valid = tok < M;
-            const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
-            const uint32_t s_addr = tmem + lane_addr + t * 128;
-            const uint32_t o_addr = tmem + lane_addr + 256 + t * 128;
-            uint64_t mask_lo = 0, mask_hi = 0;
-            if (row_valid) {
-                const uint64_t* mrow = p.tree_mask + ((size_t)b * p.M_max + tok) * p.mask_words;
-                mask_lo = mrow[0];
-                if (p.mask_words > 1) mask_hi = mrow[1];
-            }
-            float m_run = -INFINITY, l_run = 0.f;
-            bool ok = true;
-            const float2 sc2 = make_float2(p.scale_log2, p.scale_log2);
-            for (int j = 0; j < n_tiles && ok; ++j) {
-                const bool is_new = j >= n_ctx_tiles;
-                const int n_valid = is_new ? M : min(kTileTokens, seq_len - (tile_begin + j) * kTileTokens);
-                const bool masked = is_new || n_valid < kTileTokens;
-                uint64_t vis_lo = ~0ull, vis_hi = ~0ull;  // visibility of the tile's 128 columns for this row
-                if (masked) {
-                    if (is_new) {
-                        vis_lo = mask_lo;
-                        vis_hi = mask_hi;
-                    }
-                    if (n_valid < 64) {
-                        vis_lo &= (n_valid <= 0) ? 0ull : (~0ull >> (64 - n_valid));
-                        vis_hi = 0;
-                    } else if (n_valid < 128) {
-                        vis_hi &= (n_valid == 64) ? 0ull : (~0ull >> (128 - n_valid));
-                    }
-                }
-                ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.s_full[t]), j & 1, abort_flag, p.workspace, 6));
-                if (!ok) break;
-                tc_fence_after();
-                // the whole row of S (128 columns) goes to registers in one round trip
-                uint32_t v[128];
-                TMEM_LD32(s_addr, v);
-                TMEM_LD32(s_addr + 32, (v + 32));
-                TMEM_LD32(s_addr + 64, (v + 64));
-                TMEM_LD32(s_addr + 96, (v + 96));
-                tmem_wait_ld();
-                // P = 2^(s*scale - m) as bf16 pairs, packed in place: word i of P (columns 2i, 2i+1) overwrites
-                // v[i], whose own value was consumed by an earlier pair, so no second register array is needed.
-                // The row sum is taken over the ROUNDED weights the tensor core will use, so that O / l is an
-                // exact weighted average of V rows (the rounding error of a dominant weight cancels instead of
-                // scaling the output).
-                auto exp_row = [&](float m_use) {
-                    const float2 nm2 = make_float2(-m_use, -m_use);
-                    float2 sum2[4];  // independent partial sums: one chain of 64 dependent adds would outlast the exponentials
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) sum2[e] = make_float2(0.f, 0.f);
-#pragma unroll
-                    for (int i = 0; i < 64; ++i) {
-                        const float2 x = __ffma2_rn(make_float2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1])),
-                                                    sc2, nm2);
-                        const uint32_t w = pack_bf16(ex2(x.x), ex2(x.y));
-                        v[i] = w;
-                        add_bf16_pair(sum2[i & 3], w);
-                    }
-                    const float2 s01 = __fadd2_rn(sum2[0], sum2[1]), s23 = __fadd2_rn(sum2[2], sum2[3]);
-                    return (s01.x + s23.x) + (s01.y + s23.y);
-                };
-                // Fast path (every full context tile after the first): keep the reference m_run of the row as it
-                // is and skip the row maximum.  Weights may then exceed 1; float32 sums and bf16 weights keep
-                // their relative precision whatever the exponent, so only overflow has to be ruled out: if a
-                // row sum leaves the safe range (or a row has no reference yet), the warp takes the tile again
-                // from tensor memory on the general path, which brings m_run up to date.
-                float l_add = 0.f;
-                bool general = j == 0 || masked;
-                if (!general) {
-                    l_add = exp_row(m_run);
-                    const bool bad = !(l_add < kSafeRowSum) || m_run == -INFINITY;
-                    if (__any_sync(0xffffffffu, bad)) {
-                        general = true;  // S_t is still intact: P has not been stored yet
-                        TMEM_LD32(s_addr, v);
-                        TMEM_LD32(s_addr + 32, (v + 32));
-                        TMEM_LD32(s_addr + 64, (v + 64));
-                        TMEM_LD32(s_addr + 96, (v + 96));
-                        tmem_wait_ld();
-                    }
-                }
-                if (general) {
-                    if (masked) {  // ragged or tree-masked tile: invisible columns become -inf (at most two tiles per CTA)
-#pragma unroll
-                        for (int i = 0; i < 128; ++i) {
-                            const uint64_t word = i < 64 ? vis_lo : vis_hi;
-                            if (!((word >> (i & 63)) & 1ull)) v[i] = 0xff800000u;
-                        }
-                    }
-                    float mx0 = __uint_as_float(v[0]), mx1 = __uint_as_float(v[1]), mx2 = __uint_as_float(v[2]),
-                          mx3 = __uint_as_float(v[3]);
-#pragma unroll
-                    for (int i = 4; i < 124; i += 8) {  // three-input max: two new values per instruction
-                        mx0 = fmax3(mx0, __uint_as_float(v[i]), __uint_as_float(v[i + 1]));
-                        mx1 = fmax3(mx1, __uint_as_float(v[i + 2]), __uint_as_float(v[i + 3]));
-                        mx2 = fmax3(mx2, __uint_as_float(v[i + 4]), __uint_as_float(v[i + 5]));
-                        mx3 = fmax3(mx3, __uint_as_float(v[i + 6]), __uint_as_float(v[i + 7]));
-                    }
-                    mx0 = fmax3(mx0, __uint_as_float(v[124]), __uint_as_float(v[125]));
-                    mx1 = fmax3(mx1, __uint_as_float(v[126]), __uint_as_float(v[127]));
-                    const float mx = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3));
-                    const float m_tile = mx * p.scale_log2;
-                    // lazy rescale: keep the old reference max unless the new one is more than 2^8 larger.
-                    // The decision is per row, the tensor-memory traffic is warp-wide: if any row of the
-                    // warp rescales, all 32 rows pass through it (with a factor of 1 where nothing changes).
-                    bool need = false;
-                    if (j == 0) {
-                        m_run = m_tile;
-                    } else {
-                        need = m_tile > m_run + kRescaleThreshold || (m_run == -INFINITY && m_tile > -INFINITY);
-                    }
-                    if (__any_sync(0xffffffffu, need)) {
-                        const float factor = !need ? 1.f : (m_run == -INFINITY ? 0.f : ex2(m_run - m_tile));
-                        // O_t already holds every earlier PV: the tensor pipe runs in order, and S_t(j), issued
-                        // after PV(j-1,t), is complete
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            uint32_t o[32];
-                            TMEM_LD32(o_addr + c * 32, o);
-                            tmem_wait_ld();
-#pragma unroll
-                            for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * factor);
-                            TMEM_ST32(o_addr + c * 32, o);
-                        }
-                        if (need) {
-                            l_run *= factor;
-                            m_run = m_tile;
-                        }
-                    }
-                    l_add = exp_row((m_run == -INFINITY) ? 0.f : m_run);
-                }
-                TMEM_ST32(s_addr, v);
-                TMEM_ST32(s_addr + 32, (v + 32));
-                l_run += l_add;
-                tmem_wait_st();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&bars.p_full[t]));
-            }
-            // ---- epilogue: wait for the last PV, normalise, write out ---------------------------
-            if (ok) ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.o_done[t]), 0, abort_flag, p.workspace, 8));
-            if (ok) {
-                tc_fence_after();
-                const bool direct = p.n_splits == 1;
-                const float inv = direct ? 1.f / l_run : 1.f;
-                const size_t out_row = ((size_t)lb * p.M_max + tok) * p.Hq + h * p.G + g;
-                const size_t prow = (((size_t)lb * p.Hkv + h) * p.n_splits + split) * p.R_pad + rg * 256 + row;
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    uint32_t v[32];
-                    TMEM_LD32(o_addr + c * 32, v);
-                    tmem_wait_ld();
-                    if (!row_valid) continue;
-                    if (!direct) {
-                        // a thread's row is 512 contiguous bytes: 32-byte stores fill whole sectors, half as many
-                        // memory transactions as 16-byte ones for this one-row-per-lane pattern
-                        float* dst = p.part_o + prow * kD + c * 32;
-#pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + 8 * i),
-                                         "r"(v[8 * i]), "r"(v[8 * i + 1]), "r"(v[8 * i + 2]), "r"(v[8 * i + 3]), "r"(v[8 * i + 4]),
-                                         "r"(v[8 * i + 5]), "r"(v[8 * i + 6]), "r"(v[8 * i + 7])
-                                         : "memory");
-                    } else if (p.out_f32) {
-                        float4* dst = reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + out_row * kD + c * 32);
-#pragma unroll
-                        for (int i = 0; i < 8; ++i)
-                            dst[i] = make_float4(__uint_as_float(v[4 * i]) * inv, __uint_as_float(v[4 * i + 1]) * inv,
-                                                 __uint_as_float(v[4 * i + 2]) * inv, __uint_as_float(v[4 * i + 3]) * inv);
-                    } else {
-                        uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(p.out) + out_row * kD + c * 32);
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            uint4 w;
-                            w.x = pack_bf16(__uint_as_float(v[8 * i]) * inv, __uint_as_float(v[8 * i + 1]) * inv);
-                            w.y = pack_bf16(__uint_as_float(v[8 * i + 2]) * inv, __uint_as_float(v[8 * i + 3]) * inv);
-                            w.z = pack_bf16(__uint_as_float(v[8 * i + 4]) * inv, __uint_as_float(v[8 * i + 5]) * inv);
-                            w.w = pack_bf16(__uint_as_float(v[8 * i + 6]) * inv, __uint_as_float(v[8 * i + 7]) * inv);
-                            dst[i] = w;
-                        }
-                    }
-                }
-                if (row_valid) {
-                    if (direct) {
-                        if (p.lse) p.lse[out_row] = m_run * kLn2 + logf(l_run);
-                    } else {
-                        p.part_ml[prow * 2] = m_run * kLn2;  // natural-log units for the merge
-                        p.part_ml[prow * 2 + 1] = l_run;
-                    }
-                }
-            }
-        }
+        one ? softmax<D, true>(p, c, bars, warp, lane) : softmax<D, false>(p, c, bars, warp, lane);
     }
 
     // ---- teardown ----------------------------------------------------------------------------
@@ -499,75 +710,138 @@ __global__ void __launch_bounds__(kThreadsTc, 1) attn_tc_kernel(const __grid_con
     __syncthreads();
     if (warp == 1) {
         // after a give-up no new copy was issued; the few in flight (at most a ring of them) land within microseconds
-        if (*abort_flag) __nanosleep(1000000);
+        if (*(volatile int*)&bars.abort_flag) __nanosleep(1000000);
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(c.tmem) : "memory");
     }
 }
 
-// Log-sum-exp merge of the KV splits: one warp per output row (a thread owns four channels), eight rows per
-// CTA; grid = (row groups, Hkv, layers x seqs).
-constexpr int kMergeRows = 8;
-__global__ void __launch_bounds__(32 * kMergeRows) merge_tc_kernel(TcParams p) {
-    const int r = blockIdx.x * kMergeRows + (threadIdx.x >> 5), h = blockIdx.y, lb = blockIdx.z, lane = threadIdx.x & 31;
+// Log-sum-exp merge of the KV splits: D/4 threads per row, each owning four channels.  Bound by latency: the partial rows
+// come from L2, so kMergeAhead of them are in flight per thread, requested before the splits' maxima are known, and a
+// row's threads fetch the maxima and sums of as many splits side by side (one layer, 60 rows x 4 heads, 9 splits: 3.8 ->
+// 2.3 us against four loads in flight behind a serial pass over the maxima).  Splits are added in order.
+constexpr int kMergeThreads = 128;
+constexpr int kMergeAhead = 8;
+template <int D>
+__global__ void __launch_bounds__(kMergeThreads) merge_tc_kernel(const __grid_constant__ TcParams p) {
+    constexpr int kRowThreads = D / 4;
+    const int row_in_head = blockIdx.x * (kMergeThreads / kRowThreads) + threadIdx.x / kRowThreads;  // step token * G + query head
+    const int h = blockIdx.y, lb = blockIdx.z, lane = threadIdx.x % kRowThreads;
     const int b = lb % p.batch;
     int M = p.q_lens ? p.q_lens[b] : p.M_max;
     M = min(max(M, 0), p.M_max);
-    if (r >= M * p.G) return;
-    const size_t base = ((size_t)lb * p.Hkv + h) * p.n_splits;
-    const float2* ml = reinterpret_cast<const float2*>(p.part_ml);
+    if (row_in_head >= M * p.G) return;
+    const unsigned members = kRowThreads == 32 ? 0xffffffffu : 0xffffu << (threadIdx.x & 16);  // the row's lanes
+    const int j = row_in_head / p.G, g = row_in_head % p.G;
+    const int tok_per_tile = 128 / p.G;
+    const int r = j / tok_per_tile * 128 + j % tok_per_tile * p.G + g;  // its place in the packed row tiles
+    const size_t row0 = ((size_t)lb * p.Hkv + h) * p.n_splits * p.R_pad + r;
+    const float4* po = reinterpret_cast<const float4*>(p.part_o + row0 * D) + lane;
+    const float2* ml = reinterpret_cast<const float2*>(p.part_ml) + row0;
+    const size_t po_stride = (size_t)p.R_pad * kRowThreads;
+    float4 buf[kMergeAhead];
+#pragma unroll
+    for (int u = 0; u < kMergeAhead; ++u)
+        if (u < p.n_splits) buf[u] = po[u * po_stride];
     float m_all = -INFINITY;
-    for (int s = 0; s < p.n_splits; ++s) m_all = fmaxf(m_all, ml[(base + s) * p.R_pad + r].x);
+    for (int s = lane; s < p.n_splits; s += kRowThreads) m_all = fmaxf(m_all, ml[(size_t)s * p.R_pad].x);
+#pragma unroll
+    for (int o = kRowThreads / 2; o > 0; o >>= 1) m_all = fmaxf(m_all, __shfl_xor_sync(members, m_all, o));
     float l_all = 0.f;
     float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-    // four splits at a time, their loads in flight together (added in split order, so the result does not depend on
-    // the batching); an empty split's partial O was never written and is not read
-    for (int s0 = 0; s0 < p.n_splits; s0 += 4) {
-        float2 m_l[4];
-        float4 po[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const size_t prow = (base + min(s0 + u, p.n_splits - 1)) * p.R_pad + r;
-            m_l[u] = ml[prow];
-            if (s0 + u >= p.n_splits) m_l[u].x = -INFINITY;
+    for (int c0 = 0; c0 < p.n_splits; c0 += kRowThreads) {  // a lane per split of this chunk
+        float w_mine = 0.f, l_mine = 0.f;
+        if (c0 + lane < p.n_splits) {
+            const float2 v = ml[(size_t)(c0 + lane) * p.R_pad];
+            if (v.x != -INFINITY) {  // an empty split's partial O was never written: weight 0, not used
+                w_mine = __expf(v.x - m_all);
+                l_mine = v.y * w_mine;
+            }
         }
+        for (int s0 = c0; s0 < min(c0 + kRowThreads, p.n_splits); s0 += kMergeAhead) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const size_t prow = (base + min(s0 + u, p.n_splits - 1)) * p.R_pad + r;
-            po[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (m_l[u].x != -INFINITY) po[u] = __ldg(reinterpret_cast<const float4*>(p.part_o + prow * kD) + lane);
-        }
+            for (int u = 0; u < kMergeAhead; ++u) {
+                const float w = __shfl_sync(members, w_mine, s0 - c0 + u, kRowThreads);
+                l_all += __shfl_sync(members, l_mine, s0 - c0 + u, kRowThreads);
+                if (s0 + u >= p.n_splits) break;
+                if (w != 0.f) {
+                    o.x = fmaf(buf[u].x, w, o.x);
+                    o.y = fmaf(buf[u].y, w, o.y);
+                    o.z = fmaf(buf[u].z, w, o.z);
+                    o.w = fmaf(buf[u].w, w, o.w);
+                }
+            }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            if (m_l[u].x == -INFINITY) continue;
-            const float w = __expf(m_l[u].x - m_all);
-            l_all = fmaf(m_l[u].y, w, l_all);
-            o.x = fmaf(po[u].x, w, o.x);
-            o.y = fmaf(po[u].y, w, o.y);
-            o.z = fmaf(po[u].z, w, o.z);
-            o.w = fmaf(po[u].w, w, o.w);
+            for (int u = 0; u < kMergeAhead; ++u)
+                if (s0 + kMergeAhead + u < p.n_splits) buf[u] = po[(size_t)(s0 + kMergeAhead + u) * po_stride];
         }
     }
-    const int j = r / p.G, g = r % p.G;
     const size_t row = ((size_t)lb * p.M_max + j) * p.Hq + h * p.G + g;
     const float inv = 1.f / l_all;
     o.x *= inv; o.y *= inv; o.z *= inv; o.w *= inv;
     if (p.out_f32) {
-        reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + row * kD)[lane] = o;
+        reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + row * D)[lane] = o;
     } else {
         uint2 w2;
         w2.x = pack_bf16(o.x, o.y);
         w2.y = pack_bf16(o.z, o.w);
-        reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.out) + row * kD)[lane] = w2;
+        reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.out) + row * D)[lane] = w2;
     }
     if (p.lse && lane == 0) p.lse[row] = m_all + logf(l_all);
+}
+
+template <int D, int kForm>
+specpv_status launch_form(const TcParams& p, int n_lb, cudaStream_t stream) {
+    using Sh = Shape<D>;
+    if (!set_smem_limit_once(reinterpret_cast<const void*>(attn_tc_kernel<D, kForm>), Sh::kSmemBytes)) return SPECPV_ERR_CUDA;
+    attn_tc_kernel<D, kForm><<<p.n_splits * p.n_row_groups * p.Hkv * n_lb, kThreadsTc, Sh::kSmemBytes, stream>>>(p);
+    if (cudaGetLastError() != cudaSuccess) return SPECPV_ERR_CUDA;
+    count_launch();
+    return SPECPV_OK;
+}
+
+template <int D>
+specpv_status launch_kernels(const TcParams& p, int n_lb, cudaStream_t stream) {
+    // per-sequence row counts, or a last row group of one tile, can bring both forms into one launch
+    const bool both = p.rg_tiles == 2 && (p.q_lens || p.n_full_groups < p.n_row_groups);
+    const specpv_status st = p.rg_tiles == 1 ? launch_form<D, kOneTile>(p, n_lb, stream)
+                             : both          ? launch_form<D, kBoth>(p, n_lb, stream)
+                                             : launch_form<D, kTwoTiles>(p, n_lb, stream);
+    if (st != SPECPV_OK) return st;
+    if (p.n_splits > 1) {
+        constexpr int rows = kMergeThreads / (D / 4);
+        merge_tc_kernel<D><<<dim3((p.M_max * p.G + rows - 1) / rows, p.Hkv, n_lb), kMergeThreads, 0, stream>>>(p);
+        if (cudaGetLastError() != cudaSuccess) return SPECPV_ERR_CUDA;
+        count_launch();
+    }
+    return SPECPV_OK;
+}
+
+// Time until `n_short` CTAs of `t_short` each, started behind `n_long` of `t_long`, are done on 148 SMs of one CTA each.
+double cta_makespan(long long n_long, double t_long, long long n_short, double t_short) {
+    constexpr long long kSms = 148;
+    const long long q = n_long / kSms, more = n_long % kSms;  // `more` SMs take one long CTA more than the others
+    const double early = q * t_long, late = early + (more ? t_long : 0.0);
+    if (n_short == 0) return late;
+    double end = 1e300;
+    for (int on_early = 0; on_early < 2; ++on_early)  // the last short CTA ends on one kind of SM or the other
+        for (long long k = 1; k <= n_short / kSms + (long long)(t_long / t_short) + 2; ++k) {
+            const double t = (on_early ? early : late) + k * t_short;
+            const long long done = more * (t >= late ? (long long)((t - late) / t_short + 1e-9) : 0) +
+                                   (kSms - more) * (t >= early ? (long long)((t - early) / t_short + 1e-9) : 0);
+            if (done < n_short) continue;
+            const double all = t > late ? t : late;
+            end = all < end ? all : end;
+            break;
+        }
+    return end;
 }
 
 }  // namespace
 
 bool attention_tc_supported(const AttnArgs& a) {
-    if (a.g.dtype != SPECPV_DTYPE_BF16 || a.g.d != 128 || (a.g.bs != 64 && a.g.bs != 32 && a.g.bs != 16)) return false;
-    if (a.g.G > 128 || (128 % a.g.G) != 0) return false;
+    if (a.g.dtype != SPECPV_DTYPE_BF16 || (a.g.d != 128 && a.g.d != 64) || (a.g.bs != 64 && a.g.bs != 32 && a.g.bs != 16)) return false;
+    if (a.g.G > 128) return false;
     if (a.M_max > kMaxQTokens) return false;
     // row coordinates of the pool tensor map must fit in a positive int32
     const unsigned long long rows = (unsigned long long)a.g.n_layers * a.n_pages * a.g.Hkv * (unsigned long long)a.g.bs;
@@ -575,35 +849,28 @@ bool attention_tc_supported(const AttnArgs& a) {
     return get_encode_fn() != nullptr;
 }
 
-specpv_status launch_merge_tc(const TcParams& p, int R_max, int n_lb, cudaStream_t stream) {
-    dim3 mgrid((R_max + kMergeRows - 1) / kMergeRows, p.Hkv, n_lb);
-    merge_tc_kernel<<<mgrid, 32 * kMergeRows, 0, stream>>>(p);
-    if (cudaGetLastError() != cudaSuccess) return SPECPV_ERR_CUDA;
-    count_launch();
-    return SPECPV_OK;
-}
-
 specpv_status launch_attention_tc(const AttnArgs& a, cudaStream_t stream) {
     TcParams p{};
     const int G = a.g.G, Hq = a.g.Hq, Hkv = a.g.Hkv;
+    const uint64_t d = (uint64_t)a.g.d;
     const uint64_t step_tokens = (uint64_t)a.n_layers * a.batch * a.M_max;
     {
-        uint64_t dims[3] = {128, (uint64_t)Hq, step_tokens};
-        uint64_t strides[2] = {256, (uint64_t)Hq * 256};
+        uint64_t dims[3] = {d, (uint64_t)Hq, step_tokens};
+        uint64_t strides[2] = {2 * d, (uint64_t)Hq * 2 * d};
         uint32_t box[3] = {64, (uint32_t)G, (uint32_t)(128 / G)};
         if (!encode_map(&p.tm_q, a.q, 3, dims, strides, box)) return SPECPV_ERR_CUDA;
     }
     {
-        uint64_t dims[3] = {128, (uint64_t)Hkv, step_tokens};
-        uint64_t strides[2] = {256, (uint64_t)Hkv * 256};
+        uint64_t dims[3] = {d, (uint64_t)Hkv, step_tokens};
+        uint64_t strides[2] = {2 * d, (uint64_t)Hkv * 2 * d};
         uint32_t box[3] = {64, 1, 64};
         if (!encode_map(&p.tm_knew, a.k_new, 3, dims, strides, box)) return SPECPV_ERR_CUDA;
         if (!encode_map(&p.tm_vnew, a.v_new, 3, dims, strides, box)) return SPECPV_ERR_CUDA;
     }
     const uint64_t pool_rows = (uint64_t)a.g.n_layers * a.n_pages * Hkv * (uint64_t)a.g.bs;
     {
-        uint64_t dims[2] = {128, pool_rows};
-        uint64_t strides[1] = {256};
+        uint64_t dims[2] = {d, pool_rows};
+        uint64_t strides[1] = {2 * d};
         uint32_t box[2] = {64, (uint32_t)a.g.bs};
         if (!encode_map(&p.tm_kpool, a.k_pool, 2, dims, strides, box)) return SPECPV_ERR_CUDA;
         if (!encode_map(&p.tm_vpool, a.v_pool, 2, dims, strides, box)) return SPECPV_ERR_CUDA;
@@ -617,45 +884,53 @@ specpv_status launch_attention_tc(const AttnArgs& a, cudaStream_t stream) {
     p.pool_rows = (uint32_t)pool_rows;
     p.scale_log2 = a.g.scale * kLog2e;
 
-    const int R_max = a.M_max * G;
-    p.n_row_groups = (R_max + 255) / 256;
-    p.R_pad = p.n_row_groups * 256;
-    if (attention_pair_wanted(a)) return launch_attention_pair(p, a, stream);
-
-    if (!set_smem_limit_once(reinterpret_cast<const void*>(attn_tc_kernel), kSmemBytes)) return SPECPV_ERR_CUDA;
-    // KV splits: fill the 148 SMs (one CTA each) in whole waves as evenly as the workspace allows
-    const int base = Hkv * a.n_layers * a.batch * p.n_row_groups;
-    const int max_tiles = (a.max_seq_len + kTileTokens - 1) / kTileTokens;
-    const size_t per_split = (size_t)Hkv * a.n_layers * a.batch * p.R_pad * (kD + 2) * sizeof(float);
-    // Choose the split count with a small cost model (microseconds): whole waves of one CTA per SM,
-    // each CTA paying a fixed set-up/drain cost plus its tiles; splitting adds the partial-result
-    // round trip through the workspace and the merge launch.
-    int best = 1;
+    if (attention_pair_wanted(a)) {
+        p.n_row_groups = (a.M_max * G + 255) / 256;
+        p.R_pad = p.n_row_groups * 256;
+        return launch_attention_pair(p, a, stream);
+    }
+    // Row tiles per CTA and KV splits, by a cost model in microseconds (one CTA per SM).  A tile costs 0.9 with one row tile
+    // per CTA (alternate streams) and 1.5 with two (the same contractions for half the K/V traffic); with 16-token pages the
+    // copy engine's 32 boxes per tile cost nearly the latter in either form (61440 tokens x 16 layers: 2.0 and 2.3 us per
+    // tile under the power limit).  A CTA pays 7 for set-up, first tile and drain; splitting adds the partial results (1.5 / 4 per CTA, and their bytes) and the merge launch.
+    // Two row tiles are the better form when there are CTAs enough; one row tile gives twice the CTAs where a launch
+    // cannot fill the SMs otherwise (one layer, 8 KV heads, 60 rows x 4: 4096 tokens 20.0 -> 18.6 us, 16384 tokens
+    // 32.5 -> 29.2 us).  Down to one tile per CTA pays (24 rows x 4, 2048 tokens: 15.8 / 15.1 / 14.2 us at 6 / 9 / 18
+    // splits).  A last row group of one tile makes shorter CTAs, which come last in the grid (64K tokens x 36 layers,
+    // 90 rows x 4: 4100 -> 3690 us).
+    const int tok_per_tile = 128 / G, row_tiles = (a.M_max + tok_per_tile - 1) / tok_per_tile;
+    const int n_units = Hkv * a.n_layers * a.batch;
+    const int positions = (a.max_seq_len + kTileTokens - 1) / kTileTokens + 1;  // context tiles + the tile of the step's own tokens
+    const double row_bytes = (double)n_units * a.M_max * G * (a.g.d + 2) * sizeof(float);  // partial results of a split
+    const double tile_bytes = (double)n_units * 128 * (a.g.d + 2) * sizeof(float);
+    const double tile1 = a.g.bs == 16 ? 1.4 : 0.9;
     double best_cost = 1e30;
-    const double t_tile = 1.3, t_cta = 6.0, t_partial = 3.0, t_merge_launch = 6.0;
-    const double avg_tiles = max_tiles + 1.0;  // context tiles + the tile of the step's own tokens
-    for (int s = 1; s <= 64; ++s) {
-        if (s > 1 && (s > max_tiles / 2 || per_split * s > a.partial_bytes)) break;  // at least two tiles per CTA
-        const long long ctas = (long long)base * s;
-        const double waves = (double)((ctas + 147) / 148);
-        double cost = waves * (t_cta + t_tile * (avg_tiles / s + (s > 1 ? 0.5 : 0.0)));
-        if (s > 1) cost += waves * t_partial + t_merge_launch + (double)per_split * s * 2.0 / 4.0e6;  // bytes / (4 TB/s) in us
-        if (cost < best_cost * 0.97) {
-            best_cost = cost;
-            best = s;
+    for (int rg_tiles = row_tiles > 1 ? 2 : 1; rg_tiles >= 1; --rg_tiles) {
+        const int groups = (row_tiles + rg_tiles - 1) / rg_tiles, full = row_tiles / rg_tiles;
+        for (int s = 1; s <= 64 && s <= positions; ++s) {
+            if (s > 1 && tile_bytes * s * groups * rg_tiles > (double)a.partial_bytes) break;
+            const int tiles = (positions + s - 1) / s;
+            const double t1 = 7.0 + tile1 * tiles + (s > 1 ? 1.5 : 0.0), t2 = 7.0 + 1.5 * tiles + (s > 1 ? 4.0 : 0.0);
+            const long long n_long = (long long)n_units * s * full, n_short = (long long)n_units * s * (groups - full);
+            double cost = cta_makespan(n_long, rg_tiles == 2 ? t2 : t1, n_short, t1);
+            if (s > 1) cost += 3.0 + row_bytes * s * 2.0 / 5.3e6;  // written and read through L2 at 5.3 TB/s
+            if (cost < best_cost) {
+                best_cost = cost;
+                p.n_splits = s;
+                p.rg_tiles = rg_tiles;
+            }
         }
     }
-    p.n_splits = best;
+    p.n_row_groups = (row_tiles + p.rg_tiles - 1) / p.rg_tiles;
+    p.n_full_groups = row_tiles / p.rg_tiles;
+    p.n_full_units = n_units * p.n_full_groups;
+    p.R_pad = p.n_row_groups * p.rg_tiles * 128;
     char* ws = reinterpret_cast<char*>(a.workspace) + a.partial_off;
     p.part_o = reinterpret_cast<float*>(ws);
-    p.part_ml = reinterpret_cast<float*>(ws + (size_t)Hkv * a.n_layers * a.batch * p.n_splits * p.R_pad * kD * sizeof(float));
+    p.part_ml = reinterpret_cast<float*>(ws + (size_t)n_units * p.n_splits * p.R_pad * a.g.d * sizeof(float));
 
-    dim3 grid(p.n_splits * p.n_row_groups, Hkv, a.n_layers * a.batch);
-    attn_tc_kernel<<<grid, kThreadsTc, kSmemBytes, stream>>>(p);
-    if (cudaGetLastError() != cudaSuccess) return SPECPV_ERR_CUDA;
-    count_launch();
-    if (p.n_splits > 1) return launch_merge_tc(p, R_max, a.n_layers * a.batch, stream);
-    return SPECPV_OK;
+    const int n_lb = a.n_layers * a.batch;
+    return a.g.d == 128 ? launch_kernels<128>(p, n_lb, stream) : launch_kernels<64>(p, n_lb, stream);
 }
 
 }  // namespace specpv

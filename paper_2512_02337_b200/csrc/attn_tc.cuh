@@ -13,7 +13,7 @@ constexpr float kRescaleThreshold = 8.0f;  // log2 units
 constexpr float kSafeRowSum = 1.1529215e18f;  // 2^60: a tile's row sum below this cannot overflow the float32 sums
 
 struct TcParams {
-    CUtensorMap tm_q;      // (d, Hq, tokens)          box (64, G, 128/G)
+    CUtensorMap tm_q;      // (d, Hq, tokens)          box (64, G, floor(128/G))
     CUtensorMap tm_knew;   // (d, Hkv, tokens)         box (64, 1, 64)
     CUtensorMap tm_vnew;
     CUtensorMap tm_kpool;  // (d, rows)                box (64, page size)
@@ -24,7 +24,7 @@ struct TcParams {
     const int32_t* seq_lens;
     void* out;
     float* lse;
-    float* part_o;   // [lb][Hkv][splits][R_pad][128]  (pair kernel: [pair][2][256][128])
+    float* part_o;   // [lb][Hkv][splits][R_pad][d]  (pair kernel: [pair][2][256][128])
     float* part_ml;  // [lb][Hkv][splits][R_pad][2]    (pair kernel: [pair][2][256][2])
     int32_t* counters;  // pair kernel: arrival counters of shared units, [unit][CTA rank], zero between launches
     void* workspace;
@@ -32,6 +32,9 @@ struct TcParams {
     int pairs_per_unit;  // pair kernel: > 0 = every unit has this many pairs of its own; 0 = pairs take equal shares of all tiles
     int layer0, batch, M_max, mask_words, Hq, Hkv, G, max_blocks, n_pages;
     int n_splits, n_row_groups, R_pad, out_f32;
+    int rg_tiles;        // 128-row tiles per row group (1 or 2)
+    int n_full_groups;   // row groups of rg_tiles tiles at M_max rows; one group of a single tile may follow
+    int n_full_units;    // (layer, sequence, KV head, full row group) units of the launch
     int bs;          // tokens per page (16, 32 or 64)
     uint32_t pool_rows;  // rows of the pool tensor map (an out-of-range row coordinate reads zeros)
     float scale_log2;
@@ -77,8 +80,7 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
 }
 
 
-// launchers: the split merge (attn_tc.cu) and the CTA-pair attention kernel (attn_pair.cu)
-specpv_status launch_merge_tc(const TcParams& p, int R_max, int n_lb, cudaStream_t stream);
+// the CTA-pair attention kernel (attn_pair.cu)
 bool attention_pair_wanted(const AttnArgs& a);
 specpv_status launch_attention_pair(TcParams& p, const AttnArgs& a, cudaStream_t stream);
 

@@ -48,6 +48,15 @@ struct Geometry {
 specpv_status validate_config(const specpv_config* cfg, Geometry* g);
 specpv_status validate_kv(const Geometry& g, const specpv_paged_kv* kv);
 
+// Rows of the attention kernels' packed 128-row tiles (floor(128 / G) step tokens each, two tiles per row group).
+inline size_t packed_rows(int M_max, int G) {
+    const size_t rows = ((size_t)M_max * G + 255) / 256 * 256;
+    if (G > 128) return rows;
+    const int tok = 128 / G;
+    const size_t tiled = (size_t)(M_max + 2 * tok - 1) / (2 * tok) * 256;
+    return tiled > rows ? tiled : rows;
+}
+
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 inline size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -96,7 +105,7 @@ struct AttnArgs {
 };
 
 specpv_status launch_attention_simt(const AttnArgs& a, cudaStream_t stream);
-specpv_status launch_attention_tc(const AttnArgs& a, cudaStream_t stream);  // bf16, d = 128, bs = 64
+specpv_status launch_attention_tc(const AttnArgs& a, cudaStream_t stream);  // bf16
 bool attention_tc_supported(const AttnArgs& a);
 
 }  // namespace specpv

@@ -117,6 +117,26 @@ def test_maximum_rows_and_long_split_context(dtype):
     run_case(dtype, 8, 2, 128, 64, ctx=[64 * 300 + 63], Ms=[128], depth=8, branch=4, seed=5)
 
 
+@pytest.mark.parametrize("Hq,Hkv,d", [(10, 2, 128), (12, 2, 64), (7, 1, 128), (8, 2, 64), (24, 2, 128)])
+@pytest.mark.parametrize("bs,ctx,Ms,n_chain", [
+    (64, [0, 127, 128, 129], [1, 25, 24, 9], 0),      # one row tile; none, one, one and two context tiles
+    (16, [128 * 2, 128 * 3 + 1], [26, 10], 0),         # an even and an odd number of tiles between the two streams
+    (32, [128 * 5 - 1], [33], 20),                     # two and three row tiles
+])
+def test_packed_rows_and_alternating_streams(Hq, Hkv, d, bs, ctx, Ms, n_chain):
+    """Group sizes that do not divide 128 (rows of a tile left over), head size 64, and sequences of one row tile,
+    whose two streams take alternate K/V tiles: 0 to 5 context tiles, ragged last tiles, row counts at the tile edge."""
+    run_case("bf16", Hq, Hkv, d, bs, ctx=ctx, Ms=Ms, n_chain=n_chain, seed=Hq + d + len(ctx))
+
+
+@pytest.mark.parametrize("M,n_layers", [(60, 20), (90, 12), (26, 24)])
+def test_many_layers_and_one_layer_agree_with_the_oracle(M, n_layers):
+    """The row tiles per CTA and the KV splits depend on how many CTAs a launch has: two row tiles without splits, a last
+    row group of one tile behind the full ones, and one row tile with splits, on the same ragged context."""
+    run_case("bf16", 32, 8, 128, 64, ctx=[128 * 6 + 70], Ms=[M], n_layers=n_layers, seed=M)
+    run_case("bf16", 32, 8, 128, 64, ctx=[128 * 6 + 70], Ms=[M], n_layers=1, seed=M + 1)
+
+
 def test_partial_entry_point_multi_layer_bf16():
     run_case("bf16", 32, 8, 128, 64, ctx=[64 * 64 + 20, 64 * 70], Ms=[60, 33], depth=6, branch=4, n_layers=3,
              seed=6, partial_entry=True)
