@@ -40,6 +40,7 @@ struct SimtParams {
     void* workspace;
     int layer0, batch, M_max, mask_words, Hq, Hkv, G, bs, max_blocks, n_pages;
     int n_splits, chunk;
+    int pdl;  // set by launch_pdl_if
     float scale;
 };
 
@@ -56,6 +57,7 @@ __device__ __forceinline__ float warp_sum(float v) {
 
 template <typename T, typename TO, int D>
 __global__ void __launch_bounds__(kThreads) attn_simt_kernel(SimtParams p) {
+    pdl_begin(p.pdl);
     constexpr int CPL = D / 32;  // channels per lane
     extern __shared__ float smem[];
     float* Ks = smem;                       // [kTile][D + 1]
@@ -219,6 +221,7 @@ __global__ void __launch_bounds__(kThreads) attn_simt_kernel(SimtParams p) {
 // one thread per channel.
 template <typename TO, int D>
 __global__ void __launch_bounds__(D) merge_splits_kernel(SimtParams p) {
+    pdl_begin(p.pdl);
     const int r = blockIdx.x, h = blockIdx.y, lb = blockIdx.z, c = threadIdx.x;
     const int b = lb % p.batch;
     int M = p.q_lens ? p.q_lens[b] : p.M_max;
@@ -249,13 +252,11 @@ specpv_status launch_typed(const AttnArgs& a, SimtParams& p, cudaStream_t stream
     cudaError_t e = cudaFuncSetAttribute(attn_simt_kernel<T, TO, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return SPECPV_ERR_CUDA;
     dim3 grid(p.n_splits, a.g.Hkv, a.n_layers * a.batch);
-    attn_simt_kernel<T, TO, D><<<grid, kThreads, smem, stream>>>(p);
-    if (cudaGetLastError() != cudaSuccess) return SPECPV_ERR_CUDA;
+    if (launch_pdl_if(attn_simt_kernel<T, TO, D>, grid, kThreads, smem, stream, p) != cudaSuccess) return SPECPV_ERR_CUDA;
     count_launch();
     if (p.n_splits > 1) {
         dim3 mgrid(a.M_max * a.g.G, a.g.Hkv, a.n_layers * a.batch);
-        merge_splits_kernel<TO, D><<<mgrid, D, 0, stream>>>(p);
-        if (cudaGetLastError() != cudaSuccess) return SPECPV_ERR_CUDA;
+        if (launch_pdl_if(merge_splits_kernel<TO, D>, mgrid, D, 0, stream, p) != cudaSuccess) return SPECPV_ERR_CUDA;
         count_launch();
     }
     return SPECPV_OK;

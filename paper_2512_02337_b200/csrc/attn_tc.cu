@@ -117,7 +117,7 @@ __device__ __forceinline__ int page_row(const TcParams& p, const Job& c, int j, 
 
 // The whole warp runs the loop (a lone lane of a diverged warp runs slowly).
 template <int D>
-__device__ __forceinline__ void produce(const TcParams& p, const Job& c, Barriers& bars, bool one, int first_row, int lane) {
+__device__ __forceinline__ void produce(const TcParams& p, const Job& c, Barriers& bars, bool one, int lane) {
     using Sh = Shape<D>;
     constexpr int kStages = Sh::kStages, kParts = Sh::kParts, kSlotBytes = Sh::kSlotBytes;
     const int lag = one ? 2 : 1;
@@ -126,7 +126,7 @@ __device__ __forceinline__ void produce(const TcParams& p, const Job& c, Barrier
     const int ppt = kTileTokens / p.bs;
     const int my_pg = lane / kParts, my_part = lane % kParts;
     bool ok = true;
-    int row_k = 0, row_v1 = 0, row_v2 = 0, row_next = first_row;  // rows of tiles i, i - 1, i - 2, i + 1
+    int row_k = 0, row_v1 = 0, row_v2 = 0, row_next = page_row<D>(p, c, 0, lane);  // rows of tiles i, i - 1, i - 2, i + 1
     uint32_t slot = 0, par = 1, use = 0;  // ring position of the next use; parity of the release that frees its slot
     for (int i = 0; i < c.n_tiles + lag; ++i) {
         row_v2 = row_v1;
@@ -607,68 +607,32 @@ __global__ void __launch_bounds__(kThreadsTc, 1) attn_tc_kernel(const __grid_con
     c.b = c.lb % p.batch;
     c.l = c.lb / p.batch;
 
-    c.seq_len = max(p.seq_lens[c.b], 0);
-    c.M = p.q_lens ? p.q_lens[c.b] : p.M_max;
-    c.M = min(max(c.M, 0), p.M_max);
     c.tok_per_tile = 128 / p.G;                  // step tokens per 128-row tile
     c.tile_rows = c.tok_per_tile * p.G;          // rows of a tile in use (all 128 when G divides 128)
     c.tok0 = c.rg * p.rg_tiles * c.tok_per_tile; // first step token of this row group
-    if (c.tok0 >= c.M) return;                   // nothing to do (uniform for the CTA)
-    const bool one = kForm == kOneTile || (kForm == kBoth && c.M - c.tok0 <= c.tok_per_tile);  // one row tile
 
-    // KV range of this split: an equal share of the sequence's 128-token tiles and the tile of the step's own tokens,
-    // which comes last
-    const int total_tiles = (c.seq_len + kTileTokens - 1) / kTileTokens;
-    c.tile_begin = (int)((long long)(total_tiles + 1) * c.split / p.n_splits);
-    c.n_tiles = (int)((long long)(total_tiles + 1) * (c.split + 1) / p.n_splits) - c.tile_begin;
-    const bool last_split = c.split == p.n_splits - 1;
-    c.n_ctx_tiles = c.n_tiles - (last_split ? 1 : 0);
-    const int tile_end = c.tile_begin + c.n_ctx_tiles;
-    // first tile whose V rows need zeroing past the valid tokens: a ragged last context tile, else the
-    // tile of the step's own tokens (fewer than 128), else none
-    const bool ragged_ctx = c.n_ctx_tiles > 0 && tile_end == total_tiles && (c.seq_len % kTileTokens) != 0;
-    c.first_fix = ragged_ctx ? c.n_ctx_tiles - 1 : ((last_split && c.M < kTileTokens) ? c.n_ctx_tiles : c.n_tiles);
-
-    if (c.n_tiles == 0) {
-        // an empty split: publish (m = -inf, l = 0) so that the merge ignores it
-        for (int r = threadIdx.x; r < p.rg_tiles * 128; r += kThreadsTc) {
-            const int row = c.rg * p.rg_tiles * 128 + r;
-            if (row < p.R_pad) {
-                const size_t prow = (((size_t)c.lb * p.Hkv + c.h) * p.n_splits + c.split) * p.R_pad + row;
-                p.part_ml[prow * 2] = -INFINITY;
-                p.part_ml[prow * 2 + 1] = 0.f;
-            }
-        }
-        return;
-    }
-
-    // ---- set-up ------------------------------------------------------------------------------
-    // Warp 0 initialises the barriers, starts the copy of Q and looks the first tile's pages up while the tensor memory is
-    // allocated: the first K tile is two dependent loads (lengths, block table) and a copy away.
+    // ---- set-up (nothing here depends on earlier work on the stream) ----------------------------
     c.q_smem = smem_u32(c.smem);
-    int first_row = 0;
-    if (warp == 0) {
-        if (lane == 0) {
-            mbar_init(smem_u32(&bars.q_full), 1);
-            for (int s = 0; s < Sh::kStages; ++s) {
-                mbar_init(smem_u32(&bars.kv_full[s]), 1);
-                mbar_init(smem_u32(&bars.kv_empty[s]), 1);
-            }
-            for (int t = 0; t < 2; ++t) {
-                mbar_init(smem_u32(&bars.s_full[t]), 1);
-                mbar_init(smem_u32(&bars.p_full[t]), 4);  // one arrival per softmax warp
-                mbar_init(smem_u32(&bars.o_done[t]), 1);
-            }
-            mbar_init(smem_u32(&bars.v_need), 1);
-            mbar_init(smem_u32(&bars.v_fixed), 1);
-            mbar_init(smem_u32(&bars.drain), 1);
-            bars.abort_flag = 0;
-            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (threadIdx.x == 0) {
+        mbar_init(smem_u32(&bars.q_full), 1);
+        for (int s = 0; s < Sh::kStages; ++s) {
+            mbar_init(smem_u32(&bars.kv_full[s]), 1);
+            mbar_init(smem_u32(&bars.kv_empty[s]), 1);
         }
-        __syncwarp();
-        copy_q<D>(p, c, bars, one, lane);
-        first_row = page_row<D>(p, c, 0, lane);
+        for (int t = 0; t < 2; ++t) {
+            mbar_init(smem_u32(&bars.s_full[t]), 1);
+            mbar_init(smem_u32(&bars.p_full[t]), 4);  // one arrival per softmax warp
+            mbar_init(smem_u32(&bars.o_done[t]), 1);
+        }
+        mbar_init(smem_u32(&bars.v_need), 1);
+        mbar_init(smem_u32(&bars.v_fixed), 1);
+        mbar_init(smem_u32(&bars.drain), 1);
+        bars.abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        prefetch_map(&p.tm_q);
+        prefetch_map(&p.tm_kpool);
+        prefetch_map(&p.tm_vpool);
     }
     if (c.tile_rows < 128) {  // rows past the packed ones are never copied: finite values, so that their softmax stays quiet
         const int n = (128 - c.tile_rows) * 8;
@@ -685,29 +649,65 @@ __global__ void __launch_bounds__(kThreadsTc, 1) attn_tc_kernel(const __grid_con
     __syncthreads();
     tc_fence_after();
     c.tmem = bars.tmem_base;
+    if (p.n_splits == 1) pdl_trigger();
+    pdl_wait();
     // tensor-memory columns: S_t at t*128, O_t at 256 + t*128; P_t aliases S_t (64 columns of bf16 pairs)
 
-    // Register budget: the control warpgroup (warps 0-3) gives registers to the two softmax warpgroups: 128 x 56 +
-    // 256 x 224 = the 384 x 168 of the launch.
-    if (warp == 0) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
-        produce<D>(p, c, bars, one, first_row, lane);
-    } else if (warp == 1) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
-        one ? issue<D, true>(p, c, bars, lane) : issue<D, false>(p, c, bars, lane);
-    } else if (warp == 2) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
-        one ? fix_v<D, true>(p, c, bars, lane) : fix_v<D, false>(p, c, bars, lane);
-    } else if (warp == 3) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
-    } else {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
-        one ? softmax<D, true>(p, c, bars, warp, lane) : softmax<D, false>(p, c, bars, warp, lane);
+    c.seq_len = max(p.seq_lens[c.b], 0);
+    c.M = p.q_lens ? p.q_lens[c.b] : p.M_max;
+    c.M = min(max(c.M, 0), p.M_max);
+    bool work = c.tok0 < c.M;                    // (uniform for the CTA)
+    const bool one = kForm == kOneTile || (kForm == kBoth && c.M - c.tok0 <= c.tok_per_tile);  // one row tile
+
+    // KV range of this split: an equal share of the sequence's 128-token tiles and the tile of the step's own tokens,
+    // which comes last
+    const int total_tiles = (c.seq_len + kTileTokens - 1) / kTileTokens;
+    const uint32_t positions = (uint32_t)total_tiles + 1;  // at most 2^24 + 1, and at most 64 splits
+    c.tile_begin = (int)(positions * (uint32_t)c.split / (uint32_t)p.n_splits);
+    c.n_tiles = (int)(positions * (uint32_t)(c.split + 1) / (uint32_t)p.n_splits) - c.tile_begin;
+    const bool last_split = c.split == p.n_splits - 1;
+    c.n_ctx_tiles = c.n_tiles - (last_split ? 1 : 0);
+    const int tile_end = c.tile_begin + c.n_ctx_tiles;
+    // first tile whose V rows need zeroing past the valid tokens: a ragged last context tile, else the
+    // tile of the step's own tokens (fewer than 128), else none
+    const bool ragged_ctx = c.n_ctx_tiles > 0 && tile_end == total_tiles && (c.seq_len % kTileTokens) != 0;
+    c.first_fix = ragged_ctx ? c.n_ctx_tiles - 1 : ((last_split && c.M < kTileTokens) ? c.n_ctx_tiles : c.n_tiles);
+
+    if (work && c.n_tiles == 0) {
+        // an empty split: publish (m = -inf, l = 0) so that the merge ignores it
+        for (int r = threadIdx.x; r < p.rg_tiles * 128; r += kThreadsTc) {
+            const size_t prow = (((size_t)c.lb * p.Hkv + c.h) * p.n_splits + c.split) * p.R_pad + c.rg * p.rg_tiles * 128 + r;
+            p.part_ml[prow * 2] = -INFINITY;
+            p.part_ml[prow * 2 + 1] = 0.f;
+        }
+        work = false;
+    }
+
+    if (work) {
+        // Register budget: the control warpgroup (warps 0-3) gives registers to the two softmax warpgroups: 128 x 56 +
+        // 256 x 224 = the 384 x 168 of the launch.
+        if (warp == 0) {
+            asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+            copy_q<D>(p, c, bars, one, lane);
+            produce<D>(p, c, bars, one, lane);
+        } else if (warp == 1) {
+            asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+            one ? issue<D, true>(p, c, bars, lane) : issue<D, false>(p, c, bars, lane);
+        } else if (warp == 2) {
+            asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+            one ? fix_v<D, true>(p, c, bars, lane) : fix_v<D, false>(p, c, bars, lane);
+        } else if (warp == 3) {
+            asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+        } else {
+            asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
+            one ? softmax<D, true>(p, c, bars, warp, lane) : softmax<D, false>(p, c, bars, warp, lane);
+        }
     }
 
     // ---- teardown ----------------------------------------------------------------------------
     tc_fence_before();
     __syncthreads();
+    if (p.n_splits > 1) pdl_trigger();
     if (warp == 1) {
         // after a give-up no new copy was issued; the few in flight (at most a ring of them) land within microseconds
         if (*(volatile int*)&bars.abort_flag) __nanosleep(1000000);
@@ -720,10 +720,11 @@ __global__ void __launch_bounds__(kThreadsTc, 1) attn_tc_kernel(const __grid_con
 // come from L2, so kMergeAhead of them are in flight per thread, requested before the splits' maxima are known, and a
 // row's threads fetch the maxima and sums of as many splits side by side (one layer, 60 rows x 4 heads, 9 splits: 3.8 ->
 // 2.3 us against four loads in flight behind a serial pass over the maxima).  Splits are added in order.
-constexpr int kMergeThreads = 128;
+constexpr int kMergeThreads = 512;
 constexpr int kMergeAhead = 8;
 template <int D>
 __global__ void __launch_bounds__(kMergeThreads) merge_tc_kernel(const __grid_constant__ TcParams p) {
+    pdl_begin(p.pdl);
     constexpr int kRowThreads = D / 4;
     const int row_in_head = blockIdx.x * (kMergeThreads / kRowThreads) + threadIdx.x / kRowThreads;  // step token * G + query head
     const int h = blockIdx.y, lb = blockIdx.z, lane = threadIdx.x % kRowThreads;
@@ -794,8 +795,9 @@ template <int D, int kForm>
 specpv_status launch_form(const TcParams& p, int n_lb, cudaStream_t stream) {
     using Sh = Shape<D>;
     if (!set_smem_limit_once(reinterpret_cast<const void*>(attn_tc_kernel<D, kForm>), Sh::kSmemBytes)) return SPECPV_ERR_CUDA;
-    attn_tc_kernel<D, kForm><<<p.n_splits * p.n_row_groups * p.Hkv * n_lb, kThreadsTc, Sh::kSmemBytes, stream>>>(p);
-    if (cudaGetLastError() != cudaSuccess) return SPECPV_ERR_CUDA;
+    if (launch_pdl(attn_tc_kernel<D, kForm>, p.n_splits * p.n_row_groups * p.Hkv * n_lb, kThreadsTc, Sh::kSmemBytes, stream, p) !=
+        cudaSuccess)
+        return SPECPV_ERR_CUDA;
     count_launch();
     return SPECPV_OK;
 }
@@ -810,8 +812,9 @@ specpv_status launch_kernels(const TcParams& p, int n_lb, cudaStream_t stream) {
     if (st != SPECPV_OK) return st;
     if (p.n_splits > 1) {
         constexpr int rows = kMergeThreads / (D / 4);
-        merge_tc_kernel<D><<<dim3((p.M_max * p.G + rows - 1) / rows, p.Hkv, n_lb), kMergeThreads, 0, stream>>>(p);
-        if (cudaGetLastError() != cudaSuccess) return SPECPV_ERR_CUDA;
+        const dim3 grid((p.M_max * p.G + rows - 1) / rows, p.Hkv, n_lb);
+        if (launch_pdl_if(merge_tc_kernel<D>, grid, kMergeThreads, 0, stream, p) != cudaSuccess)
+            return SPECPV_ERR_CUDA;
         count_launch();
     }
     return SPECPV_OK;

@@ -32,6 +32,7 @@ struct TcParams {
     int pairs_per_unit;  // pair kernel: > 0 = every unit has this many pairs of its own; 0 = pairs take equal shares of all tiles
     int layer0, batch, M_max, mask_words, Hq, Hkv, G, max_blocks, n_pages;
     int n_splits, n_row_groups, R_pad, out_f32;
+    int pdl;             // merge kernel: set by launch_pdl_if
     int rg_tiles;        // 128-row tiles per row group (1 or 2)
     int n_full_groups;   // row groups of rg_tiles tiles at M_max rows; one group of a single tile may follow
     int n_full_units;    // (layer, sequence, KV head, full row group) units of the launch

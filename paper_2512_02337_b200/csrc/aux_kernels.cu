@@ -41,6 +41,7 @@ __device__ __forceinline__ uint32_t packed_min(uint32_t a, uint32_t b, float) {
 
 template <typename T>
 __global__ void __launch_bounds__(32 * kSumWarps) summaries_kernel(SummaryParams p) {
+    pdl_begin(p.pdl);
     constexpr uint32_t kNegInf = sizeof(T) == 2 ? 0xFF80FF80u : 0xFF800000u;
     constexpr uint32_t kPosInf = kNegInf & (sizeof(T) == 2 ? 0x7FFF7FFFu : 0x7FFFFFFFu);
     const int lane = threadIdx.x & 31;
@@ -118,6 +119,7 @@ constexpr int kScoreRowTile = 4;
 
 template <typename T, int D>
 __global__ void __launch_bounds__(32 * kScoreWarps) scores_simt_kernel(ScoreParams p) {
+    pdl_begin(p.pdl);
     extern __shared__ float smem[];
     float* Smax = smem;                                   // [blocks][D + 1]
     float* Smin = Smax + kScoreBlocksPerCta * (D + 1);    // [blocks][D + 1]
@@ -228,6 +230,7 @@ __device__ __forceinline__ uint64_t select_key(float score, int index) {
 }
 
 __global__ void __launch_bounds__(kSelectThreads) select_kernel(SelectParams p) {
+    pdl_begin(p.pdl);
     __shared__ unsigned int hist[256];
     __shared__ uint64_t s_prefix;
     __shared__ int s_remaining;
@@ -380,6 +383,7 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(SelectParams p) 
 // block's K and V (16-byte vectors) into the partial cache.
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(128) gather_kernel(GatherParams p) {
+    pdl_begin(p.pdl);
     const int s = blockIdx.x, h = blockIdx.y, lb = blockIdx.z;
     const int b = lb % p.batch, l = lb / p.batch;
     const int count = p.count[b];
@@ -438,6 +442,7 @@ __global__ void __launch_bounds__(128) gather_kernel(GatherParams p) {
 // Commit: grid = (A_max, Hkv, layers x seqs); a CTA appends one accepted token's K and V row.
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(32) commit_rows_kernel(CommitParams p) {
+    pdl_begin(p.pdl);
     const int a = blockIdx.x, h = blockIdx.y, lb = blockIdx.z;
     const int b = lb % p.batch, l = lb / p.batch;
     const int n = min(max(p.n_accepted[b], 0), p.A_max);
@@ -473,6 +478,8 @@ __global__ void __launch_bounds__(32) commit_rows_kernel(CommitParams p) {
 
 __global__ void commit_lens_kernel(int32_t* seq_lens, const int32_t* n_accepted, int batch, int A_max,
                                    int capacity_tokens) {
+    pdl_trigger();
+    pdl_wait();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= batch) return;
     const int n = min(max(n_accepted[b], 0), A_max);
@@ -484,10 +491,10 @@ __global__ void commit_lens_kernel(int32_t* seq_lens, const int32_t* n_accepted,
 // ---------------------------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------------------------
-#define SPECPV_CHECK_LAUNCH()                                     \
-    do {                                                          \
-        if (cudaGetLastError() != cudaSuccess) return SPECPV_ERR_CUDA; \
-        count_launch();                                           \
+#define SPECPV_LAUNCH(...)                                                     \
+    do {                                                                       \
+        if (launch_pdl_if(__VA_ARGS__) != cudaSuccess) return SPECPV_ERR_CUDA; \
+        count_launch();                                                        \
     } while (0)
 
 specpv_status launch_summaries(const SummaryParams& params, int n_layers, int blocks_touched, int dtype,
@@ -497,9 +504,7 @@ specpv_status launch_summaries(const SummaryParams& params, int n_layers, int bl
     p.aligned = aligned16(p.kmax) && aligned16(p.kmin);
     const int warps = p.Hkv < kSumWarps ? p.Hkv : kSumWarps;
     dim3 grid(blocks_touched, (p.Hkv + kSumWarps - 1) / kSumWarps, n_layers * p.batch);
-    if (dtype == SPECPV_DTYPE_F32) summaries_kernel<float><<<grid, 32 * warps, 0, stream>>>(p);
-    else summaries_kernel<__nv_bfloat16><<<grid, 32 * warps, 0, stream>>>(p);
-    SPECPV_CHECK_LAUNCH();
+    SPECPV_LAUNCH(dtype == SPECPV_DTYPE_F32 ? summaries_kernel<float> : summaries_kernel<__nv_bfloat16>, grid, 32 * warps, 0, stream, p);
     return SPECPV_OK;
 }
 
@@ -509,8 +514,7 @@ static specpv_status launch_scores_typed(const ScoreParams& p, int n_layers, int
     if (cudaFuncSetAttribute(scores_simt_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return SPECPV_ERR_CUDA;
     dim3 grid((max_nb + kScoreBlocksPerCta - 1) / kScoreBlocksPerCta, p.Hkv, n_layers * p.batch);
-    scores_simt_kernel<T, D><<<grid, 32 * kScoreWarps, smem, stream>>>(p);
-    SPECPV_CHECK_LAUNCH();
+    SPECPV_LAUNCH(scores_simt_kernel<T, D>, grid, 32 * kScoreWarps, smem, stream, p);
     return SPECPV_OK;
 }
 
@@ -529,23 +533,20 @@ specpv_status launch_scores(const ScoreParams& p, int n_layers, int max_nb, int 
 specpv_status launch_select(const SelectParams& p, int n_layers, cudaStream_t stream) {
     if (n_layers <= 0 || p.batch <= 0) return SPECPV_OK;
     dim3 grid(p.Hkv, p.batch, n_layers);
-    select_kernel<<<grid, kSelectThreads, 0, stream>>>(p);
-    SPECPV_CHECK_LAUNCH();
+    SPECPV_LAUNCH(select_kernel, grid, kSelectThreads, 0, stream, p);
     return SPECPV_OK;
 }
 
 specpv_status launch_gather(const GatherParams& p, int n_layers, cudaStream_t stream) {
     dim3 grid(p.budget_blocks, p.Hkv, n_layers * p.batch);
-    gather_kernel<<<grid, 128, 0, stream>>>(p);
-    SPECPV_CHECK_LAUNCH();
+    SPECPV_LAUNCH(gather_kernel, grid, 128, 0, stream, p);
     return SPECPV_OK;
 }
 
 specpv_status launch_commit(const CommitParams& p, int n_layers, int32_t* seq_lens, cudaStream_t stream) {
     if (p.A_max > 0 && n_layers > 0) {
         dim3 grid(p.A_max, p.Hkv, n_layers * p.batch);
-        commit_rows_kernel<<<grid, 32, 0, stream>>>(p);
-        SPECPV_CHECK_LAUNCH();
+        SPECPV_LAUNCH(commit_rows_kernel, grid, 32, 0, stream, p);
     }
     (void)seq_lens;
     return SPECPV_OK;
@@ -553,8 +554,9 @@ specpv_status launch_commit(const CommitParams& p, int n_layers, int32_t* seq_le
 
 specpv_status launch_commit_lens(int32_t* seq_lens, const int32_t* n_accepted, int batch, int A_max,
                                  int capacity_tokens, cudaStream_t stream) {
-    commit_lens_kernel<<<(batch + 63) / 64, 64, 0, stream>>>(seq_lens, n_accepted, batch, A_max, capacity_tokens);
-    SPECPV_CHECK_LAUNCH();
+    if (launch_pdl(commit_lens_kernel, (batch + 63) / 64, 64, 0, stream, seq_lens, n_accepted, batch, A_max, capacity_tokens) != cudaSuccess)
+        return SPECPV_ERR_CUDA;
+    count_launch();
     return SPECPV_OK;
 }
 

@@ -15,6 +15,7 @@ struct SummaryParams {
     void* workspace;
     int layer0, batch, Hkv, bs, d, max_blocks, n_pages, A_max;
     int aligned;  // set by the launcher: kmax and kmin take 16-byte stores
+    int pdl;      // set by launch_pdl_if
 };
 
 struct ScoreParams {
@@ -27,6 +28,7 @@ struct ScoreParams {
     float* scores;
     void* workspace;
     int layer0, batch, M_max, Hq, Hkv, G, bs, max_blocks, reduce;
+    int pdl;         // set by launch_pdl_if
     int score_mode;  // 0: max of the two full dot products (Eq. 2 as printed), 1: maximum per channel
 };
 
@@ -36,6 +38,7 @@ struct SelectParams {
     int32_t* idx;
     int32_t* count;
     int batch, Hkv, bs, max_blocks, sink_blocks, local_blocks, budget_blocks;
+    int pdl;          // set by launch_pdl_if
     int share_heads;  // 1: every KV head of a layer keeps the blocks chosen on the mean of the heads' scores
 };
 
@@ -52,6 +55,7 @@ struct GatherParams {
     int32_t* partial_lens;
     void* workspace;
     int batch, Hkv, bs, d, es, budget_blocks, full_max_blocks, full_pages, part_max_blocks, part_pages;
+    int pdl;  // set by launch_pdl_if
 };
 
 struct CommitParams {
@@ -65,6 +69,7 @@ struct CommitParams {
     const int32_t* seq_lens;
     void* workspace;
     int layer0, batch, M_max, A_max, Hkv, bs, d, es, max_blocks, n_pages;
+    int pdl;  // set by launch_pdl_if
 };
 
 specpv_status launch_summaries(const SummaryParams& p, int n_layers, int blocks_touched, int dtype, cudaStream_t stream);

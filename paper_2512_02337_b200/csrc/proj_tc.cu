@@ -37,7 +37,7 @@ struct ProjTcParams {
     float* partials;
     void* workspace;
     ProjSegment seg[3];
-    int n_seg, layer0, n_tiles, n_out, tokens, n_pad, ksteps, splits, stages, group;
+    int n_seg, layer0, n_tiles, n_out, tokens, n_pad, ksteps, splits, stages, group, pdl;
 };
 
 struct __align__(8) ProjBarriers {
@@ -113,11 +113,16 @@ __global__ void __launch_bounds__(kProjThreads, 2) proj_tc_kernel(const __grid_c
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = bars.tmem_base;
+    pdl_trigger();
 
     if (warp == 0) {
         // ---- producer: the whole warp walks the ring, lane 0 issues the copies ----------------------------
         const int w_row = (p.layer0 + l) * p.n_out + tile * kFeatTile;
         const int x_row = l * p.tokens + tok0;
+        // the weights do not wait for the previous kernel: they start on their way to L2 while it ends
+        for (int i = lane; i < n_k; i += 32) tma_prefetch_2d(&p.tm_w, (kb + i) * 64, w_row);
+        __syncwarp();
+        pdl_wait();
         bool ok = true;
         // The copies of p.group consecutive stages are issued together: a weight row is 128 contiguous bytes
         // per stage, and DRAM serves the same row's neighbouring chunks far better when they are asked for at
@@ -145,6 +150,7 @@ __global__ void __launch_bounds__(kProjThreads, 2) proj_tc_kernel(const __grid_c
         const uint32_t idesc = make_idesc((uint32_t)p.n_pad, false);
         const uint32_t desc_hi = (uint32_t)((1024u >> 4) | (1u << 14) | (2u << 29));
         bool ok = true;
+        pdl_wait();  // (nothing to read here, but the limits of the waits below start to run)
         for (int i = 0; i < n_k; ++i) {
             const int slot = i % p.stages;
             ok &= mbar_wait(smem_u32(&bars.full[slot]), (i / p.stages) & 1, abort_flag, p.workspace, 31);
@@ -166,6 +172,7 @@ __global__ void __launch_bounds__(kProjThreads, 2) proj_tc_kernel(const __grid_c
         // ---- epilogue: thread <-> output feature (tensor-memory lane), then thread <-> (row, channel pairs) ---
         const int q = warp & 3;
         const int f = q * 32 + lane;
+        pdl_wait();
         const bool ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.d_full), 0, abort_flag, p.workspace, 32));
         tc_fence_after();
         float* stage = reinterpret_cast<float*>(smem);  // [n_pad][128]; every copy into the ring has been consumed
@@ -209,6 +216,7 @@ __global__ void __launch_bounds__(kProjThreads, 2) proj_tc_kernel(const __grid_c
 // Adds the partial sums of a tile's input-feature ranges in range order and finishes the rows: a CTA takes four rows
 // of one tile, a thread one row's channels (2j, 2j+1, 64+2j, 64+2j+1), so that all its loads are in flight together.
 __global__ void __launch_bounds__(128) proj_reduce_kernel(const __grid_constant__ ProjTcParams p, int n_chunks) {
+    pdl_begin(p.pdl);
     const int tile = blockIdx.x, l = blockIdx.z / n_chunks, chunk = blockIdx.z % n_chunks;
     const int tok0 = chunk * kMaxTokTile;
     const int valid = min(p.n_pad, p.tokens - tok0);
@@ -239,11 +247,12 @@ struct ProjSimtParams {
     const float* cos_sin;
     const void* residual;
     ProjSegment seg[3];
-    int n_seg, layer0, n_out, n_in, tokens, tile;
+    int n_seg, layer0, n_out, n_in, tokens, tile, pdl;
 };
 
 template <typename T>
 __global__ void __launch_bounds__(128) proj_simt_kernel(const __grid_constant__ ProjSimtParams p) {
+    pdl_begin(p.pdl);
     extern __shared__ float vals[];  // one output tile of one row
     const int tok = blockIdx.x, tile = blockIdx.y, l = blockIdx.z;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -286,6 +295,8 @@ __global__ void __launch_bounds__(128) proj_simt_kernel(const __grid_constant__ 
 __global__ void rope_table_kernel(const uint64_t* __restrict__ tree_mask, const int32_t* __restrict__ q_lens,
                                   const int32_t* __restrict__ base_pos, int M_max, int d, double theta,
                                   float* __restrict__ cos_sin) {
+    pdl_trigger();
+    pdl_wait();
     const int row = blockIdx.x, b = row / M_max, j = row % M_max;
     const int W = (M_max + 63) / 64, half = d / 2;
     int M = q_lens ? q_lens[b] : M_max;
@@ -357,12 +368,14 @@ specpv_status launch_proj_tc(const ProjArgs& a, cudaStream_t stream) {
     p.splits = splits;
     p.partials = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(a.workspace) + a.scratch_off);
     dim3 grid(p.n_tiles * splits, n_chunks, a.n_layers_call);
-    proj_tc_kernel<<<grid, kProjThreads, 1024 + ring_bytes, stream>>>(p);
-    if (cudaGetLastError() != cudaSuccess) return SPECPV_ERR_CUDA;
+    if (launch_pdl(proj_tc_kernel, grid, kProjThreads, 1024 + ring_bytes, stream, p) != cudaSuccess) return SPECPV_ERR_CUDA;
     count_launch();
     if (splits > 1) {
-        proj_reduce_kernel<<<dim3(p.n_tiles, (p.n_pad + 3) / 4, a.n_layers_call * n_chunks), 128, 0, stream>>>(p, n_chunks);
-        if (cudaGetLastError() != cudaSuccess) return SPECPV_ERR_CUDA;
+        const dim3 rgrid(p.n_tiles, (p.n_pad + 3) / 4, a.n_layers_call * n_chunks);
+        p.pdl = pdl_pays(rgrid);
+        if ((p.pdl ? launch_pdl(proj_reduce_kernel, rgrid, 128, 0, stream, p, n_chunks)
+                   : launch_plain(proj_reduce_kernel, rgrid, 128, 0, stream, p, n_chunks)) != cudaSuccess)
+            return SPECPV_ERR_CUDA;
         count_launch();
     }
     return SPECPV_OK;
@@ -377,19 +390,20 @@ specpv_status launch_proj_simt(const ProjArgs& a, cudaStream_t stream) {
     p.layer0 = a.layer0; p.n_out = a.n_out; p.n_in = a.n_in; p.tokens = a.tokens; p.tile = a.tile;
     dim3 grid(a.tokens, a.n_out / a.tile, a.n_layers_call);
     const size_t smem = (size_t)a.tile * sizeof(float);
+    cudaError_t st;
     if (a.dtype == SPECPV_DTYPE_F32)
-        proj_simt_kernel<float><<<grid, 128, smem, stream>>>(p);
+        st = launch_pdl_if(proj_simt_kernel<float>, grid, 128, smem, stream, p);
     else
-        proj_simt_kernel<__nv_bfloat16><<<grid, 128, smem, stream>>>(p);
-    if (cudaGetLastError() != cudaSuccess) return SPECPV_ERR_CUDA;
+        st = launch_pdl_if(proj_simt_kernel<__nv_bfloat16>, grid, 128, smem, stream, p);
+    if (st != cudaSuccess) return SPECPV_ERR_CUDA;
     count_launch();
     return SPECPV_OK;
 }
 
 specpv_status launch_rope_table(const uint64_t* tree_mask, const int32_t* q_lens, const int32_t* base_pos, int batch,
                                 int M_max, int d, double theta, float* cos_sin, cudaStream_t stream) {
-    rope_table_kernel<<<batch * M_max, 64, 0, stream>>>(tree_mask, q_lens, base_pos, M_max, d, theta, cos_sin);
-    if (cudaGetLastError() != cudaSuccess) return SPECPV_ERR_CUDA;
+    if (launch_pdl(rope_table_kernel, batch * M_max, 64, 0, stream, tree_mask, q_lens, base_pos, M_max, d, theta, cos_sin) != cudaSuccess)
+        return SPECPV_ERR_CUDA;
     count_launch();
     return SPECPV_OK;
 }

@@ -165,6 +165,8 @@ __global__ void __launch_bounds__(kScoreThreads, 1) scores_tc_kernel(const __gri
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = bars.tmem_base;
+    pdl_trigger();
+    pdl_wait();
     const int tok_per_tile = 128 / p.G;
 
     // Register budget: 384 threads start with 168 registers each; the control warps keep 48, which is what lets the
@@ -509,11 +511,9 @@ specpv_status launch_scores_tc(const ScoreParams& sp, int n_layers_call, int n_l
         p.tok_n = sp.M_max - tok0 < tok_per_pass ? sp.M_max - tok0 : tok_per_pass;
         p.accumulate = tok0 > 0;
         p.n_cols = p.tok_n * sp.G <= 128 ? 128 : 256;  // accumulator columns, padded to whole 128-row Q tiles
-        if (sp.score_mode == 1)
-            scores_tc_kernel<true><<<grid, kScoreThreads, kScoreSmem, stream>>>(p);
-        else
-            scores_tc_kernel<false><<<grid, kScoreThreads, kScoreSmem, stream>>>(p);
-        if (cudaGetLastError() != cudaSuccess) return SPECPV_ERR_CUDA;
+        if (launch_pdl(sp.score_mode == 1 ? scores_tc_kernel<true> : scores_tc_kernel<false>, grid, kScoreThreads, kScoreSmem, stream,
+                       p) != cudaSuccess)
+            return SPECPV_ERR_CUDA;
         count_launch();
     }
     return SPECPV_OK;
