@@ -7,7 +7,7 @@ fallback: if the shared library is missing, importing the symbols fails loudly.
 from __future__ import annotations
 
 import ctypes
-from ctypes import POINTER, c_float, c_int, c_int32, c_size_t, c_void_p
+from ctypes import POINTER, byref, c_double, c_float, c_int, c_int32, c_size_t, c_void_p
 from dataclasses import dataclass
 from pathlib import Path
 
@@ -58,6 +58,20 @@ class PagedKV(ctypes.Structure):
                 ("n_pages", c_int32), ("max_seq_len", c_int32)]
 
 
+# Argument kinds of the calls (P pointer, i int32, z size_t, d double): declared, so that plain Python numbers can be passed.
+# A call of the step is a few microseconds of device work, and wrapping every argument in a ctypes object cost as much.
+_SIGNATURES = {
+    "specpv_poll_status": "PPP", "specpv_build_tree_mask": "PiiPi", "specpv_select_mode": "iiiiii",
+    "specpv_update_block_summaries": "PiiPPiPPPzP", "specpv_score_blocks": "PiiPPiPPPPPPzP",
+    "specpv_select_partial_kv": "PiPPiiPPPzP", "specpv_refresh_partial": "PPPPPPPzP",
+    "specpv_verify_partial": "PiiPPPPPiPPPPzP", "specpv_verify_full": "PiiPPPPPiPPPPzP",
+    "specpv_verify_host": "PiiiPPPPiPPPPzP", "specpv_commit_accepted": "PiiPPiPPiPPPPzP",
+    "specpv_verify_partial_static": "PiiPPPPPiPPPPP", "specpv_rope_table": "PPPPiidPP",
+    "specpv_qkv_rope": "PiiPiPPiiPPPPzP", "specpv_o_proj": "PiiPPiPiiPPzP",
+    "specpv_verify_full_offloaded": "PiiPPPPPiPPPPzPP", "specpv_selftest_wait_timeout": "PziPP",
+}
+_KINDS = {"P": c_void_p, "i": c_int, "z": c_size_t, "d": c_double}
+
 _lib = None
 
 
@@ -75,25 +89,33 @@ def lib() -> ctypes.CDLL:
         _lib.specpv_kernel_launches.restype = ctypes.c_uint64
         for name in EXPORTS[3:] + SELFTEST_EXPORTS:
             getattr(_lib, name).restype = c_int
+            getattr(_lib, name).argtypes = [_KINDS[k] for k in _SIGNATURES[name]]
     return _lib
 
 
-def _ptr(t) -> c_void_p:
+def _ptr(t) -> int | None:
     if t is None:
-        return c_void_p(0)
+        return None
     if isinstance(t, torch.Tensor):
         assert t.is_contiguous(), "tensors passed to the C ABI must be contiguous"
-        return c_void_p(t.data_ptr())
+        return t.data_ptr()
     if isinstance(t, np.ndarray):
         assert t.flags.c_contiguous
-        return c_void_p(t.ctypes.data)
+        return t.ctypes.data
     raise TypeError(type(t))
 
 
-def _stream(stream) -> c_void_p:
+# the current stream's handle without building a torch.cuda.Stream (3 us of a call's host time)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_get_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
+def _stream(stream) -> int:
     if stream is None:
+        if _raw_stream is not None and _get_device is not None:
+            return _raw_stream(_get_device())
         stream = torch.cuda.current_stream()
-    return c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def _check(status: int, where: str):
@@ -118,9 +140,9 @@ class Cache:
     max_seq_len: int
 
     def desc(self) -> PagedKV:
-        batch, max_blocks = self.block_table.shape
-        return PagedKV(self.k_pool.data_ptr(), self.v_pool.data_ptr(), self.block_table.data_ptr(),
-                       self.seq_lens.data_ptr(), batch, max_blocks, self.k_pool.shape[1], int(self.max_seq_len))
+        k, table = self.k_pool, self.block_table
+        return PagedKV(k.data_ptr(), self.v_pool.data_ptr(), table.data_ptr(), self.seq_lens.data_ptr(), table.size(0),
+                       table.size(1), k.size(1), int(self.max_seq_len))
 
 
 def specpv_status_string(status: int) -> str:
@@ -128,7 +150,7 @@ def specpv_status_string(status: int) -> str:
 
 
 def specpv_workspace_bytes(cfg: Config, n_layers_per_call: int, max_batch: int, max_seq_len: int, M_max: int) -> int:
-    return int(lib().specpv_workspace_bytes(ctypes.byref(cfg), n_layers_per_call, max_batch, max_seq_len, M_max))
+    return int(lib().specpv_workspace_bytes(byref(cfg), n_layers_per_call, max_batch, max_seq_len, M_max))
 
 
 def specpv_kernel_launches() -> int:
@@ -170,32 +192,32 @@ def specpv_select_mode(ctx_len, budget_tokens, n_partially_verified, n_candidate
 def specpv_update_block_summaries(cfg, layer0, n_layers, kv: Cache, tok_begin, max_blocks_touched, kmax, kmin,
                                   workspace, stream=None):
     d = kv.desc()
-    _check(lib().specpv_update_block_summaries(ctypes.byref(cfg), layer0, n_layers, ctypes.byref(d), _ptr(tok_begin),
+    _check(lib().specpv_update_block_summaries(byref(cfg), layer0, n_layers, byref(d), _ptr(tok_begin),
                                                max_blocks_touched, _ptr(kmax), _ptr(kmin), _ptr(workspace),
-                                               c_size_t(workspace.numel()), _stream(stream)),
+                                               workspace.numel(), _stream(stream)),
            "specpv_update_block_summaries")
 
 
 def specpv_score_blocks(cfg, layer0, n_layers, q, q_lens, M_max, last_query, kmax, kmin, kv: Cache, scores,
                         workspace, stream=None):
     d = kv.desc()
-    _check(lib().specpv_score_blocks(ctypes.byref(cfg), layer0, n_layers, _ptr(q), _ptr(q_lens), M_max,
-                                     _ptr(last_query), _ptr(kmax), _ptr(kmin), ctypes.byref(d), _ptr(scores),
-                                     _ptr(workspace), c_size_t(workspace.numel()), _stream(stream)),
+    _check(lib().specpv_score_blocks(byref(cfg), layer0, n_layers, _ptr(q), _ptr(q_lens), M_max,
+                                     _ptr(last_query), _ptr(kmax), _ptr(kmin), byref(d), _ptr(scores),
+                                     _ptr(workspace), workspace.numel(), _stream(stream)),
            "specpv_score_blocks")
 
 
 def specpv_select_partial_kv(cfg, n_layers, scores, seq_lens, batch, max_blocks, idx, count, workspace, stream=None):
-    _check(lib().specpv_select_partial_kv(ctypes.byref(cfg), n_layers, _ptr(scores), _ptr(seq_lens), batch,
+    _check(lib().specpv_select_partial_kv(byref(cfg), n_layers, _ptr(scores), _ptr(seq_lens), batch,
                                           max_blocks, _ptr(idx), _ptr(count), _ptr(workspace),
-                                          c_size_t(workspace.numel()), _stream(stream)),
+                                          workspace.numel(), _stream(stream)),
            "specpv_select_partial_kv")
 
 
 def specpv_refresh_partial(cfg, full: Cache, idx, count, partial: Cache, partial_lens, workspace, stream=None):
     fd, pd = full.desc(), partial.desc()
-    _check(lib().specpv_refresh_partial(ctypes.byref(cfg), ctypes.byref(fd), _ptr(idx), _ptr(count), ctypes.byref(pd),
-                                        _ptr(partial_lens), _ptr(workspace), c_size_t(workspace.numel()),
+    _check(lib().specpv_refresh_partial(byref(cfg), byref(fd), _ptr(idx), _ptr(count), byref(pd),
+                                        _ptr(partial_lens), _ptr(workspace), workspace.numel(),
                                         _stream(stream)),
            "specpv_refresh_partial")
 
@@ -203,9 +225,9 @@ def specpv_refresh_partial(cfg, full: Cache, idx, count, partial: Cache, partial
 def _verify(fn_name, cfg, layer0, n_layers, q, k_new, v_new, tree_mask, q_lens, M_max, kv: Cache, out, lse,
             workspace, stream):
     d = kv.desc()
-    _check(getattr(lib(), fn_name)(ctypes.byref(cfg), layer0, n_layers, _ptr(q), _ptr(k_new), _ptr(v_new),
-                                   _ptr(tree_mask), _ptr(q_lens), M_max, ctypes.byref(d), _ptr(out), _ptr(lse),
-                                   _ptr(workspace), c_size_t(workspace.numel()), _stream(stream)), fn_name)
+    _check(getattr(lib(), fn_name)(byref(cfg), layer0, n_layers, _ptr(q), _ptr(k_new), _ptr(v_new),
+                                   _ptr(tree_mask), _ptr(q_lens), M_max, byref(d), _ptr(out), _ptr(lse),
+                                   _ptr(workspace), workspace.numel(), _stream(stream)), fn_name)
 
 
 def specpv_verify_partial(cfg, layer0, n_layers, q, k_new, v_new, tree_mask, q_lens, M_max, partial: Cache, out,
@@ -224,8 +246,8 @@ def specpv_verify_partial_static(cfg, layer0, n_layers, q, k_new, v_new, tree_ma
     call allocates nothing (for callers whose device memory is all spoken for).  ``device_status`` is an
     optional int32 device tensor of 5 words that receives the call's device-side status."""
     d = partial.desc()
-    _check(lib().specpv_verify_partial_static(ctypes.byref(cfg), layer0, n_layers, _ptr(q), _ptr(k_new), _ptr(v_new),
-                                              _ptr(tree_mask), _ptr(q_lens), M_max, ctypes.byref(d), _ptr(out),
+    _check(lib().specpv_verify_partial_static(byref(cfg), layer0, n_layers, _ptr(q), _ptr(k_new), _ptr(v_new),
+                                              _ptr(tree_mask), _ptr(q_lens), M_max, byref(d), _ptr(out),
                                               _ptr(lse), _ptr(device_status), _stream(stream)),
            "specpv_verify_partial_static")
 
@@ -233,7 +255,7 @@ def specpv_verify_partial_static(cfg, layer0, n_layers, q, k_new, v_new, tree_ma
 def specpv_selftest_wait_timeout(workspace, limit_us: int, observed_ns=None, stream=None):
     """Self-test (include/specpv_selftest.h): a bounded barrier wait that runs out after ``limit_us`` microseconds and
     records SPECPV_ERR_TIMEOUT in the workspace's status word.  ``observed_ns``: optional uint64/int64 device tensor."""
-    _check(lib().specpv_selftest_wait_timeout(_ptr(workspace), c_size_t(workspace.numel() * workspace.element_size()),
+    _check(lib().specpv_selftest_wait_timeout(_ptr(workspace), workspace.numel() * workspace.element_size(),
                                               int(limit_us), _ptr(observed_ns), _stream(stream)),
            "specpv_selftest_wait_timeout")
 
@@ -247,39 +269,39 @@ def specpv_verify_full(cfg, layer0, n_layers, q, k_new, v_new, tree_mask, q_lens
 def specpv_verify_host(cfg, mode, layer0, n_layers, q_host, k_new_host, v_new_host, tree_mask_host, M_max,
                        kv: Cache, out_host, lse_host, workspace, stream=None):
     d = kv.desc()
-    _check(lib().specpv_verify_host(ctypes.byref(cfg), mode, layer0, n_layers, _ptr(q_host), _ptr(k_new_host),
-                                    _ptr(v_new_host), _ptr(tree_mask_host), M_max, ctypes.byref(d), _ptr(out_host),
-                                    _ptr(lse_host), _ptr(workspace), c_size_t(workspace.numel()), _stream(stream)),
+    _check(lib().specpv_verify_host(byref(cfg), mode, layer0, n_layers, _ptr(q_host), _ptr(k_new_host),
+                                    _ptr(v_new_host), _ptr(tree_mask_host), M_max, byref(d), _ptr(out_host),
+                                    _ptr(lse_host), _ptr(workspace), workspace.numel(), _stream(stream)),
            "specpv_verify_host")
 
 
 def specpv_commit_accepted(cfg, layer0, n_layers, k_new, v_new, M_max, accepted, n_accepted, A_max, dst: Cache,
                            kmax, kmin, workspace, stream=None):
     d = dst.desc()
-    _check(lib().specpv_commit_accepted(ctypes.byref(cfg), layer0, n_layers, _ptr(k_new), _ptr(v_new), M_max,
-                                        _ptr(accepted), _ptr(n_accepted), A_max, ctypes.byref(d), _ptr(kmax),
-                                        _ptr(kmin), _ptr(workspace), c_size_t(workspace.numel()), _stream(stream)),
+    _check(lib().specpv_commit_accepted(byref(cfg), layer0, n_layers, _ptr(k_new), _ptr(v_new), M_max,
+                                        _ptr(accepted), _ptr(n_accepted), A_max, byref(d), _ptr(kmax),
+                                        _ptr(kmin), _ptr(workspace), workspace.numel(), _stream(stream)),
            "specpv_commit_accepted")
 
 
 # ---- the linear maps either side of the attention ---------------------------------------------------------------
 def specpv_rope_table(cfg, tree_mask, q_lens, base_pos, batch, M_max, rope_theta, cos_sin, stream=None):
-    _check(lib().specpv_rope_table(ctypes.byref(cfg), _ptr(tree_mask), _ptr(q_lens), _ptr(base_pos), batch, M_max,
-                                   ctypes.c_double(rope_theta), _ptr(cos_sin), _stream(stream)),
+    _check(lib().specpv_rope_table(byref(cfg), _ptr(tree_mask), _ptr(q_lens), _ptr(base_pos), batch, M_max,
+                                   rope_theta, _ptr(cos_sin), _stream(stream)),
            "specpv_rope_table")
 
 
 def specpv_qkv_rope(cfg, layer0, n_layers, x, hidden, w_qkv, cos_sin, batch, M_max, q, k_new, v_new, workspace,
                     stream=None):
-    _check(lib().specpv_qkv_rope(ctypes.byref(cfg), layer0, n_layers, _ptr(x), hidden, _ptr(w_qkv), _ptr(cos_sin),
+    _check(lib().specpv_qkv_rope(byref(cfg), layer0, n_layers, _ptr(x), hidden, _ptr(w_qkv), _ptr(cos_sin),
                                  batch, M_max, _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(workspace),
-                                 c_size_t(workspace.numel()), _stream(stream)),
+                                 workspace.numel(), _stream(stream)),
            "specpv_qkv_rope")
 
 
 def specpv_o_proj(cfg, layer0, n_layers, attn, w_o, hidden, residual, batch, M_max, y, workspace, stream=None):
-    _check(lib().specpv_o_proj(ctypes.byref(cfg), layer0, n_layers, _ptr(attn), _ptr(w_o), hidden, _ptr(residual),
-                               batch, M_max, _ptr(y), _ptr(workspace), c_size_t(workspace.numel()), _stream(stream)),
+    _check(lib().specpv_o_proj(byref(cfg), layer0, n_layers, _ptr(attn), _ptr(w_o), hidden, _ptr(residual),
+                               batch, M_max, _ptr(y), _ptr(workspace), workspace.numel(), _stream(stream)),
            "specpv_o_proj")
 
 
@@ -317,8 +339,8 @@ class OffloadedCache:
 def specpv_verify_full_offloaded(cfg, layer0, n_layers, q, k_new, v_new, tree_mask, q_lens, M_max,
                                  full: OffloadedCache, out, lse, workspace, stream=None, copy_stream=None):
     d = full.desc()
-    _check(lib().specpv_verify_full_offloaded(ctypes.byref(cfg), layer0, n_layers, _ptr(q), _ptr(k_new), _ptr(v_new),
-                                              _ptr(tree_mask), _ptr(q_lens), M_max, ctypes.byref(d), _ptr(out),
-                                              _ptr(lse), _ptr(workspace), c_size_t(workspace.numel()),
+    _check(lib().specpv_verify_full_offloaded(byref(cfg), layer0, n_layers, _ptr(q), _ptr(k_new), _ptr(v_new),
+                                              _ptr(tree_mask), _ptr(q_lens), M_max, byref(d), _ptr(out),
+                                              _ptr(lse), _ptr(workspace), workspace.numel(),
                                               _stream(stream), _stream(copy_stream)),
            "specpv_verify_full_offloaded")
