@@ -11,9 +11,9 @@
 //                   sum and accumulator; the two meet in shared memory at the end.  (One stream alone leaves the tensor
 //                   pipe idle during its softmax: 64K tokens x 36 layers, 32 query rows per head, 1715 -> 1457 us = the
 //                   copy rate.)
-//   warp 0      TMA producer: Q once, then K and V tiles of 128 tokens (2, 4 or 8 pages, one copy per page
-//               and 64-channel part, each issued by its own lane) through the block table into a ring of
-//               shared-memory slots (128-byte swizzle)
+//   warp 0      TMA producer: Q once, then K and V tiles of 128 tokens (2, 4 or 8 pages, one copy per page,
+//               each issued by its own lane) through the block table into a ring of shared-memory slots
+//               (128-byte swizzle)
 //   warp 1      MMA issuer: tcgen05.mma  S_t = Q_t K^T  (both operands in shared memory) and
 //               O_t += P_t V (P read from tensor memory, V MN-major from shared memory)
 //   warps 4-7   softmax of stream 0, warps 8-11 of stream 1: one thread per row reads S from
@@ -31,12 +31,17 @@ namespace {
 
 constexpr int kThreadsTc = 384;          // 12 warps
 
-// Shared memory by head size: a K or V tile is [d/64 parts][128 tokens][64 d] bf16, a Q tile [d/64 parts][128 rows][64 d].
+// Shared memory by head size: a Q tile is [d/64 parts][128 rows][64 d] bf16, a K or V tile [16 groups of 8 tokens][d/64 parts]
+// [8 tokens][64 d], so that a page is contiguous and arrives in ONE copy of all its channels (a tensor map with the tokens
+// split into groups of eight).  (The copy engine spends some 60 ns per box whatever it carries, and a copy per page and part
+// made 16-token pages wait for it: 61440 tokens x 16 layers, 32 rows,
+// 834 -> 675 us; a copy of half a page or a quarter is no faster.)
 template <int D>
 struct Shape {
     static constexpr int kParts = D / 64;
     static constexpr int kSlotBytes = kTileTokens * D * 2;
     static constexpr int kStages = D == 128 ? 5 : 10;
+    static constexpr int kGroupBytes = 8 * D * 2;  // eight tokens of a K or V tile
     static constexpr int kQTileBytes = 128 * D * 2;
     static constexpr int kQBytes = 2 * kQTileBytes;
     static constexpr int kSmemBytes = 1024 + kQBytes + kStages * kSlotBytes;
@@ -95,24 +100,21 @@ __device__ __forceinline__ void copy_q(const TcParams& p, const Job& c, Barriers
     __syncwarp();
 }
 
-// Pool row coordinate of a page of context tile j (128 / page size of them).  Lane kParts pg + part looks page pg
-// up and later issues the copy of that page's 64-channel part, so that a tile's copies leave in one pass of
-// the warp; the table is read one tile ahead so that its latency hides behind the wait for a free slot.
-template <int D>
-__device__ __forceinline__ int page_row(const TcParams& p, const Job& c, int j, int lane) {
-    constexpr int kParts = Shape<D>::kParts;
-    const int ppt = kTileTokens / p.bs, my_pg = lane / kParts;
-    int row = (int)p.pool_rows;  // out of range: the copy engine fills zeros
-    const int blk = (c.tile_begin + j) * ppt + my_pg;
-    if (my_pg < ppt && j < c.n_ctx_tiles && (long long)blk * p.bs < c.seq_len && blk < p.max_blocks) {
+// Pool group coordinate (eight tokens each) of page `lane` of context tile j (128 / page size of them).  The lane that looks
+// a page up later issues its copy, so that a tile's copies leave in one pass of the warp; the table is read one tile
+// ahead so that its latency hides behind the wait for a free slot.
+__device__ __forceinline__ int page_group(const TcParams& p, const Job& c, int j, int lane) {
+    const int ppt = kTileTokens / p.bs;
+    int group = (int)(p.pool_rows / 8);  // out of range: the copy engine fills zeros
+    const int blk = (c.tile_begin + j) * ppt + lane;
+    if (lane < ppt && j < c.n_ctx_tiles && (long long)blk * p.bs < c.seq_len && blk < p.max_blocks) {
         const int page = p.block_table[(size_t)c.b * p.max_blocks + blk];
-        if (page < 0 || page >= p.n_pages) {
-            if (lane % kParts == 0) record_fault(p.workspace, SPECPV_ERR_BAD_BLOCK_TABLE, c.b, blk, page, c.l);
-        } else {
-            row = (int)((((long long)(p.layer0 + c.l) * p.n_pages + page) * p.Hkv + c.h) * p.bs);
-        }
+        if (page < 0 || page >= p.n_pages)
+            record_fault(p.workspace, SPECPV_ERR_BAD_BLOCK_TABLE, c.b, blk, page, c.l);
+        else
+            group = (int)((((long long)(p.layer0 + c.l) * p.n_pages + page) * p.Hkv + c.h) * (p.bs / 8));
     }
-    return row;
+    return group;
 }
 
 // The whole warp runs the loop (a lone lane of a diverged warp runs slowly).
@@ -124,30 +126,32 @@ __device__ __forceinline__ void produce(const TcParams& p, const Job& c, Barrier
     volatile int* abort_flag = &bars.abort_flag;
     const uint32_t kv_smem = c.q_smem + Sh::kQBytes;
     const int ppt = kTileTokens / p.bs;
-    const int my_pg = lane / kParts, my_part = lane % kParts;
+    const uint32_t page_off = lane * (p.bs / 8) * Sh::kGroupBytes;
+    const int new_groups = (c.M + 7) / 8;  // groups of the step's own tokens
     bool ok = true;
-    int row_k = 0, row_v1 = 0, row_v2 = 0, row_next = page_row<D>(p, c, 0, lane);  // rows of tiles i, i - 1, i - 2, i + 1
+    int at_k = 0, at_v1 = 0, at_v2 = 0, at_next = page_group(p, c, 0, lane);  // of tiles i, i - 1, i - 2, i + 1
     uint32_t slot = 0, par = 1, use = 0;  // ring position of the next use; parity of the release that frees its slot
     for (int i = 0; i < c.n_tiles + lag; ++i) {
-        row_v2 = row_v1;
-        row_v1 = row_k;
-        row_k = row_next;
-        row_next = page_row<D>(p, c, i + 1, lane);
+        at_v2 = at_v1;
+        at_v1 = at_k;
+        at_k = at_next;
+        at_next = page_group(p, c, i + 1, lane);
         for (int kv = 1; kv >= 0; --kv) {  // 1: V tile, 0: K tile
             const int j = kv ? i - lag : i;
             if (j < 0 || j >= c.n_tiles) continue;
             const uint32_t full = smem_u32(&bars.kv_full[slot]), empty = smem_u32(&bars.kv_empty[slot]);
             if (use >= (uint32_t)kStages) ok = mbar_wait(empty, par, abort_flag, p.workspace, 1);
             if (!ok) break;  // a wait gave up: nothing more is copied
-            const uint32_t dst = kv_smem + slot * kSlotBytes + my_part * 16384;
-            if (lane == 0) mbar_expect_tx(full, kSlotBytes);
-            if (j >= c.n_ctx_tiles) {  // the step's own tokens: two boxes of 64 rows per part
-                if (my_pg < 2)
-                    tma_load_3d(dst + my_pg * 8192, kv ? &p.tm_vnew : &p.tm_knew, my_part * 64, c.h,
-                                c.lb * p.M_max + my_pg * 64, full);
-            } else if (my_pg < ppt) {
-                tma_load_2d(dst + my_pg * p.bs * 128, kv ? &p.tm_vpool : &p.tm_kpool, my_part * 64,
-                            kv ? (one ? row_v2 : row_v1) : row_k, full);
+            const uint32_t dst = kv_smem + slot * kSlotBytes;
+            if (j >= c.n_ctx_tiles) {  // the step's own tokens, a copy per group and part; the rest of the slot is masked or zeroed
+                if (lane == 0) mbar_expect_tx(full, new_groups * Sh::kGroupBytes);
+                if (lane < new_groups * kParts)
+                    tma_load_3d(dst + lane * 1024, kv ? &p.tm_vnew : &p.tm_knew, lane % kParts * 64, c.h,
+                                c.lb * p.M_max + lane / kParts * 8, full);
+            } else {
+                if (lane == 0) mbar_expect_tx(full, kSlotBytes);
+                if (lane < ppt)
+                    tma_load_4d(dst + page_off, kv ? &p.tm_vpool : &p.tm_kpool, 0, 0, 0, kv ? (one ? at_v2 : at_v1) : at_k, full);
             }
             __syncwarp();
             ++use;
@@ -173,25 +177,26 @@ __device__ __forceinline__ void issue(const TcParams& p, const Job& c, Barriers&
     const int n_tiles = c.n_tiles, first_fix = c.first_fix;
     bool ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.q_full), 0, abort_flag, p.workspace, 2));
     // Shared-memory descriptors: the upper word (stride between 8-row groups, version, swizzle) is
-    // constant; the lower word is the 16-byte address plus the leading-dimension offset.
-    const uint32_t desc_hi = (uint32_t)((1024u >> 4) | (1u << 14) | (2u << 29));
+    // constant; the lower word is the 16-byte address plus the leading-dimension offset (V: to the next 64 channels).
+    const uint32_t q_hi = (uint32_t)((1024u >> 4) | (1u << 14) | (2u << 29));
+    const uint32_t kv_hi = (uint32_t)((Sh::kGroupBytes >> 4) | (1u << 14) | (2u << 29));
     const uint32_t q_lo = ((c.q_smem >> 4) & 0x3FFFu) | ((16u >> 4) << 16);
     const uint32_t k_lo0 = ((kv_smem >> 4) & 0x3FFFu) | ((16u >> 4) << 16);
-    const uint32_t v_lo0 = ((kv_smem >> 4) & 0x3FFFu) | ((16384u >> 4) << 16);
+    const uint32_t v_lo0 = ((kv_smem >> 4) & 0x3FFFu) | ((1024u >> 4) << 16);
     const uint32_t full0 = smem_u32(&bars.kv_full[0]), empty0 = smem_u32(&bars.kv_empty[0]);
     const uint32_t sfull0 = smem_u32(&bars.s_full[0]), pfull0 = smem_u32(&bars.p_full[0]);
     auto issue_pv = [&](int t, uint32_t vb_lo, bool first) {  // O_t (+)= P_t V
         const uint32_t a = tmem + t * 128, d = tmem + 256 + t * 128;
 #pragma unroll
-        for (int kk = 0; kk < 8; ++kk)  // 16 tokens per instruction: two 8-row K groups of 1024 bytes
-            mma_ts_lohi(d, a + kk * 8, vb_lo + (uint32_t)kk * (2048u >> 4), desc_hi, kIdescPV<D>, (!first || kk > 0) ? 1u : 0u);
+        for (int kk = 0; kk < 8; ++kk)  // 16 tokens per instruction: two groups
+            mma_ts_lohi(d, a + kk * 8, vb_lo + (uint32_t)kk * (2 * Sh::kGroupBytes >> 4), kv_hi, kIdescPV<D>, (!first || kk > 0) ? 1u : 0u);
     };
     auto issue_qk = [&](int t, uint32_t a_lo, uint32_t kb_lo) {  // S_t = Q K^T
         const uint32_t d = tmem + t * 128;
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk) {  // 16 channels per instruction
-            const uint32_t off = (uint32_t)((kk >> 2) * 16384 + (kk & 3) * 32) >> 4;
-            mma_ss_lohi(d, a_lo + off, kb_lo + off, desc_hi, kIdescQK, kk > 0 ? 1u : 0u);
+            const uint32_t q_off = (uint32_t)((kk >> 2) * 16384 + (kk & 3) * 32) >> 4, k_off = (uint32_t)((kk >> 2) * 1024 + (kk & 3) * 32) >> 4;
+            mma_ss_lohi(d, a_lo + q_off, q_hi, kb_lo + k_off, kv_hi, kIdescQK, kk > 0 ? 1u : 0u);
         }
     };
     // Ring uses: K0 | V0 K1 | V1 K2 | .. with two row tiles, K0 | K1 | V0 K2 | V1 K3 | .. with one.
@@ -299,11 +304,13 @@ __device__ __forceinline__ void fix_v(const TcParams& p, const Job& c, Barriers&
             break;
         const int n_valid = jp >= c.n_ctx_tiles ? c.M : min(kTileTokens, c.seq_len - (c.tile_begin + jp) * kTileTokens);
         uint8_t* v = c.smem + Sh::kQBytes + (size_t)(use % Sh::kStages) * Sh::kSlotBytes;
-        const int n_rows = kTileTokens - n_valid;
-        for (int i = lane; i < n_rows * Sh::kParts * 8; i += 32) {
-            const int chunk = i & 7, part = (i >> 3) % Sh::kParts, r = n_valid + (i >> 3) / Sh::kParts;
-            *reinterpret_cast<uint4*>(v + part * 16384 + r * 128 + chunk * 16) = make_uint4(0, 0, 0, 0);
-        }
+        // a lane keeps its 16-byte column, the warp takes 32 / (8 kParts) rows at a time (the last split of a short call
+        // waits for this: with the row and column worked out per store it took a microsecond longer)
+        constexpr int kRowsAtOnce = 32 / (8 * Sh::kParts);
+        v += lane / 8 % Sh::kParts * 1024 + lane % 8 * 16;
+#pragma unroll 4
+        for (int r = n_valid + lane / (8 * Sh::kParts); r < kTileTokens; r += kRowsAtOnce)
+            *reinterpret_cast<uint4*>(v + (r >> 3) * Sh::kGroupBytes + (r & 7) * 128) = make_uint4(0, 0, 0, 0);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&bars.v_fixed));
@@ -863,20 +870,27 @@ specpv_status launch_attention_tc(const AttnArgs& a, cudaStream_t stream) {
         uint32_t box[3] = {64, (uint32_t)G, (uint32_t)(128 / G)};
         if (!encode_map(&p.tm_q, a.q, 3, dims, strides, box)) return SPECPV_ERR_CUDA;
     }
+    const bool pair = attention_pair_wanted(a);
     {
         uint64_t dims[3] = {d, (uint64_t)Hkv, step_tokens};
         uint64_t strides[2] = {2 * d, (uint64_t)Hkv * 2 * d};
-        uint32_t box[3] = {64, 1, 64};
+        uint32_t box[3] = {64, 1, pair ? 64u : 8u};
         if (!encode_map(&p.tm_knew, a.k_new, 3, dims, strides, box)) return SPECPV_ERR_CUDA;
         if (!encode_map(&p.tm_vnew, a.v_new, 3, dims, strides, box)) return SPECPV_ERR_CUDA;
     }
     const uint64_t pool_rows = (uint64_t)a.g.n_layers * a.n_pages * Hkv * (uint64_t)a.g.bs;
-    {
+    if (pair) {
         uint64_t dims[2] = {d, pool_rows};
         uint64_t strides[1] = {2 * d};
         uint32_t box[2] = {64, (uint32_t)a.g.bs};
         if (!encode_map(&p.tm_kpool, a.k_pool, 2, dims, strides, box)) return SPECPV_ERR_CUDA;
         if (!encode_map(&p.tm_vpool, a.v_pool, 2, dims, strides, box)) return SPECPV_ERR_CUDA;
+    } else {  // (64 channels, 8 tokens, parts, groups of 8 tokens): a page's box lands group by group, its parts side by side
+        uint64_t dims[4] = {64, 8, d / 64, pool_rows / 8};
+        uint64_t strides[3] = {2 * d, 128, 16 * d};
+        uint32_t box[4] = {64, 8, (uint32_t)d / 64, (uint32_t)a.g.bs / 8};
+        if (!encode_map(&p.tm_kpool, a.k_pool, 4, dims, strides, box)) return SPECPV_ERR_CUDA;
+        if (!encode_map(&p.tm_vpool, a.v_pool, 4, dims, strides, box)) return SPECPV_ERR_CUDA;
     }
     p.tree_mask = a.tree_mask; p.q_lens = a.q_lens; p.block_table = a.block_table; p.seq_lens = a.seq_lens;
     p.out = a.out; p.lse = a.lse; p.workspace = a.workspace;
@@ -887,15 +901,14 @@ specpv_status launch_attention_tc(const AttnArgs& a, cudaStream_t stream) {
     p.pool_rows = (uint32_t)pool_rows;
     p.scale_log2 = a.g.scale * kLog2e;
 
-    if (attention_pair_wanted(a)) {
+    if (pair) {
         p.n_row_groups = (a.M_max * G + 255) / 256;
         p.R_pad = p.n_row_groups * 256;
         return launch_attention_pair(p, a, stream);
     }
     // Row tiles per CTA and KV splits, by a cost model in microseconds (one CTA per SM).  A tile costs 0.9 with one row tile
-    // per CTA (alternate streams) and 1.5 with two (the same contractions for half the K/V traffic); with 16-token pages the
-    // copy engine's 32 boxes per tile cost nearly the latter in either form (61440 tokens x 16 layers: 2.0 and 2.3 us per
-    // tile under the power limit).  A CTA pays 7 for set-up, first tile and drain; splitting adds the partial results (1.5 / 4 per CTA, and their bytes) and the merge launch.
+    // per CTA (alternate streams) and 1.5 with two (the same contractions for half the K/V traffic).  A CTA pays 7 for
+    // set-up, first tile and drain; splitting adds the partial results (1.5 / 4 per CTA, and their bytes) and the merge launch.
     // Two row tiles are the better form when there are CTAs enough; one row tile gives twice the CTAs where a launch
     // cannot fill the SMs otherwise (one layer, 8 KV heads, 60 rows x 4: 4096 tokens 20.0 -> 18.6 us, 16384 tokens
     // 32.5 -> 29.2 us).  Down to one tile per CTA pays (24 rows x 4, 2048 tokens: 15.8 / 15.1 / 14.2 us at 6 / 9 / 18
@@ -906,14 +919,13 @@ specpv_status launch_attention_tc(const AttnArgs& a, cudaStream_t stream) {
     const int positions = (a.max_seq_len + kTileTokens - 1) / kTileTokens + 1;  // context tiles + the tile of the step's own tokens
     const double row_bytes = (double)n_units * a.M_max * G * (a.g.d + 2) * sizeof(float);  // partial results of a split
     const double tile_bytes = (double)n_units * 128 * (a.g.d + 2) * sizeof(float);
-    const double tile1 = a.g.bs == 16 ? 1.4 : 0.9;
     double best_cost = 1e30;
     for (int rg_tiles = row_tiles > 1 ? 2 : 1; rg_tiles >= 1; --rg_tiles) {
         const int groups = (row_tiles + rg_tiles - 1) / rg_tiles, full = row_tiles / rg_tiles;
         for (int s = 1; s <= 64 && s <= positions; ++s) {
             if (s > 1 && tile_bytes * s * groups * rg_tiles > (double)a.partial_bytes) break;
             const int tiles = (positions + s - 1) / s;
-            const double t1 = 7.0 + tile1 * tiles + (s > 1 ? 1.5 : 0.0), t2 = 7.0 + 1.5 * tiles + (s > 1 ? 4.0 : 0.0);
+            const double t1 = 7.0 + 0.9 * tiles + (s > 1 ? 1.5 : 0.0), t2 = 7.0 + 1.5 * tiles + (s > 1 ? 4.0 : 0.0);
             const long long n_long = (long long)n_units * s * full, n_short = (long long)n_units * s * (groups - full);
             double cost = cta_makespan(n_long, rg_tiles == 2 ? t2 : t1, n_short, t1);
             if (s > 1) cost += 3.0 + row_bytes * s * 2.0 / 5.3e6;  // written and read through L2 at 5.3 TB/s

@@ -14,9 +14,9 @@ constexpr float kSafeRowSum = 1.1529215e18f;  // 2^60: a tile's row sum below th
 
 struct TcParams {
     CUtensorMap tm_q;      // (d, Hq, tokens)          box (64, G, floor(128/G))
-    CUtensorMap tm_knew;   // (d, Hkv, tokens)         box (64, 1, 64)
+    CUtensorMap tm_knew;   // (d, Hkv, tokens)         box (64, 1, 8)  (pair kernel: 64)
     CUtensorMap tm_vnew;
-    CUtensorMap tm_kpool;  // (d, rows)                box (64, page size)
+    CUtensorMap tm_kpool;  // (64, 8, d/64, rows/8)    box (64, 8, d/64, page size / 8)  (pair kernel: (d, rows), box (64, page size))
     CUtensorMap tm_vpool;
     const uint64_t* tree_mask;
     const int32_t* q_lens;
@@ -41,15 +41,15 @@ struct TcParams {
     float scale_log2;
 };
 
-// tcgen05.mma with the shared-memory descriptors given as (low word, common high word); `acc` = 0
+// tcgen05.mma with the shared-memory descriptors given as (low word, high word); `acc` = 0
 // overwrites D, anything else accumulates.
-__device__ __forceinline__ void mma_ss_lohi(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc,
-                                            uint32_t acc) {
+__device__ __forceinline__ void mma_ss_lohi(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
+                                            uint32_t idesc, uint32_t acc) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
-        "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\tsetp.ne.b32 p, %5, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(acc)
+        "mov.b64 da, {%1, %2};\n\tmov.b64 db, {%3, %4};\n\tsetp.ne.b32 p, %6, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(acc)
         : "memory");
 }
 __device__ __forceinline__ void mma_ts_lohi(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t hi, uint32_t idesc,
