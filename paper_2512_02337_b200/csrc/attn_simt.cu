@@ -3,25 +3,35 @@
 // size) with float32 arithmetic and accurate expf; it is the path for float32 caches and the
 // on-device second opinion for the tensor-core kernel.
 //
-// Work split: grid = (KV splits, KV heads, layers x sequences).  A CTA walks its token range in
-// 32-token tiles staged in shared memory; warp w owns 4 query rows per pass (lane <-> token for the
-// logits, lane <-> channel for the PV product) and keeps the running (max, sum, accumulator) of an
-// online softmax.  The last split also attends the step's own tokens under the tree mask.  With
-// more than one split the unnormalised partial results go to the workspace and merge_splits_kernel
-// combines them with a log-sum-exp merge.
+// Work split: one CTA per (layer, sequence, KV head, KV split, tile of 64 query rows).  A CTA walks its share of the
+// 64-token tiles (the tiles of the step's own tokens come last, under the tree mask): Q, K and V are staged in shared memory
+// as float32 (Q and K channel-major), a thread owns four rows and four tokens of S and four rows and D/16 channels of O, so
+// both products are register-tiled, and the running (max, sum, accumulator) of the online softmax stay in registers.
+// With more than one split the unnormalised partial results go to the workspace and merge_splits_kernel combines them with
+// a log-sum-exp merge.
+// Short calls are bound by latency: the form before this one (a warp per four rows, a lane per token, 256 tokens per CTA)
+// left a 2048-token call on 16 CTAs.  8 query heads of 64, 2 KV heads, 16 rows, float32: 2048 tokens 119 -> 18 us.
+// Larger ones are bound by shared-memory reads, two 16-byte loads per 16 multiplications (32 rows, 8192 tokens x 4 layers:
+// 283 -> 108 us).
 #include <math.h>
 
 #include "common.cuh"
+#include "tc_common.cuh"
 
 namespace specpv {
 
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kWarps = kThreads / 32;
-constexpr int kTile = 32;         // tokens per tile (one per lane)
-constexpr int kRowsPerWarp = 4;   // query rows a warp carries per pass
-constexpr int kRowsPerPass = kWarps * kRowsPerWarp;
+constexpr int kTok = 64;          // tokens per tile
+constexpr int kRows = 64;         // query rows per CTA
+constexpr int kPitch = kTok + 4;  // row pitch of the staged tiles (keeps float4 alignment)
+
+// dynamic shared memory: Q [D][kPitch], K [D][kPitch] (both channel-major), V [kTok][D], P [kRows][kPitch]
+template <int D>
+constexpr size_t simt_smem() {
+    return (size_t)(2 * D * kPitch + kTok * D + kRows * kPitch) * sizeof(float);
+}
 
 struct SimtParams {
     const void* q;
@@ -39,46 +49,55 @@ struct SimtParams {
     float* part_ml;  // [lb][Hkv][splits][R_max][2]
     void* workspace;
     int layer0, batch, M_max, mask_words, Hq, Hkv, G, bs, max_blocks, n_pages;
-    int n_splits, chunk;
+    int n_splits, row_tiles;
     int pdl;  // set by launch_pdl_if
     float scale;
 };
 
-__device__ __forceinline__ float warp_max(float v) {
+// reductions over the 16 lanes that share a row
+__device__ __forceinline__ float row_max(float v) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    for (int o = 8; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
 }
-__device__ __forceinline__ float warp_sum(float v) {
+__device__ __forceinline__ float row_sum(float v) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
+}
+// four consecutive values as float32 (16-byte aligned for float32, 8-byte for bfloat16)
+__device__ __forceinline__ float4 load4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
+    const uint2 w = *reinterpret_cast<const uint2*>(p);
+    return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xFFFF0000u), __uint_as_float(w.y << 16),
+                       __uint_as_float(w.y & 0xFFFF0000u));
 }
 
 template <typename T, typename TO, int D>
 __global__ void __launch_bounds__(kThreads) attn_simt_kernel(SimtParams p) {
     pdl_begin(p.pdl);
-    constexpr int CPL = D / 32;  // channels per lane
+    constexpr int CPT = D / 16;   // output channels per thread
+    constexpr int kLoads = D / 16;  // float4 loads per thread of a 64 x D tile
     extern __shared__ float smem[];
-    float* Ks = smem;                       // [kTile][D + 1]
-    float* Vs = Ks + kTile * (D + 1);       // [kTile][D]
-    float* Qs = Vs + kTile * D;             // [kRowsPerPass][D]
-    __shared__ int s_tile_valid;
+    float* Qt = smem;
+    float* Kt = Qt + D * kPitch;
+    float* Vs = Kt + D * kPitch;
+    float* Ps = Vs + kTok * D;
+    __shared__ uint64_t s_mask[kRows][2];  // step tokens each row sees
 
-    const int split = blockIdx.x, h = blockIdx.y, lb = blockIdx.z;
+    const int split = blockIdx.x % p.n_splits, row0 = blockIdx.x / p.n_splits * kRows;
+    const int h = blockIdx.y, lb = blockIdx.z;
     const int b = lb % p.batch, l = lb / p.batch;
-    const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
-    const int seq_len = p.seq_lens[b];
+    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
+    const int seq_len = max(p.seq_lens[b], 0);
     int M = p.q_lens ? p.q_lens[b] : p.M_max;
     M = min(max(M, 0), p.M_max);
-    const int R = M * p.G;
-    const int R_max = p.M_max * p.G;
+    const int R = M * p.G, R_max = p.M_max * p.G;
+    if (row0 >= R) return;
 
-    const bool last_split = split == p.n_splits - 1;
-    const int ctx_begin = min(split * p.chunk, seq_len);
-    const int ctx_end = last_split ? seq_len : min((split + 1) * p.chunk, seq_len);
-    const int n_ctx_tiles = (ctx_end - ctx_begin + kTile - 1) / kTile;
-    const int n_new_tiles = last_split ? (M + kTile - 1) / kTile : 0;
+    const int ctx_tiles = (seq_len + kTok - 1) / kTok, positions = ctx_tiles + (M + kTok - 1) / kTok;
+    const int tile_begin = (int)((long long)positions * split / p.n_splits);
+    const int tile_end = (int)((long long)positions * (split + 1) / p.n_splits);
 
     const T* q = reinterpret_cast<const T*>(p.q) + (size_t)lb * p.M_max * p.Hq * D;
     const T* k_new = reinterpret_cast<const T*>(p.k_new) + (size_t)lb * p.M_max * p.Hkv * D;
@@ -89,174 +108,266 @@ __global__ void __launch_bounds__(kThreads) attn_simt_kernel(SimtParams p) {
     const int32_t* table = p.block_table + (size_t)b * p.max_blocks;
     const uint64_t* mask = p.tree_mask + (size_t)b * p.M_max * p.mask_words;
 
-    for (int pass_row0 = 0; pass_row0 < R; pass_row0 += kRowsPerPass) {
+    // staging: a thread takes row or token tid % 64, and of it the 16-byte pieces tid / 64, + 4, ..
+    const int st = tid % kTok, sc = tid / kTok;
+    {
+        const int r = row0 + st;
+        const T* src = q + ((size_t)(r / p.G) * p.Hq + h * p.G + r % p.G) * D;
+#pragma unroll
+        for (int i = 0; i < kLoads; ++i) {
+            const int c = (sc + 4 * i) * 4;
+            const float4 v = r < R ? load4(src + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+            Qt[(c + 0) * kPitch + st] = v.x;
+            Qt[(c + 1) * kPitch + st] = v.y;
+            Qt[(c + 2) * kPitch + st] = v.z;
+            Qt[(c + 3) * kPitch + st] = v.w;
+        }
+        if (tid < kRows) {
+            const uint64_t* m = mask + (size_t)(r / p.G) * p.mask_words;
+            s_mask[tid][0] = r < R ? m[0] : 0ull;
+            s_mask[tid][1] = r < R && p.mask_words > 1 ? m[1] : 0ull;
+        }
+    }
+    // K and V rows of tile `tile` for this thread's token, in flight while the previous tile is worked on
+    float4 kbuf[kLoads], vbuf[kLoads];
+    auto fetch = [&](int tile) {
+        const T *ks = nullptr, *vs = nullptr;
+        if (tile < ctx_tiles) {
+            const int t = tile * kTok + st;
+            if (t < seq_len) {
+                const int page = table[t / p.bs];
+                if (page >= 0 && page < p.n_pages) {
+                    const size_t off = (((size_t)page * p.Hkv + h) * p.bs + t % p.bs) * D;
+                    ks = k_pool + off;
+                    vs = v_pool + off;
+                }
+            }
+        } else if ((tile - ctx_tiles) * kTok + st < M) {
+            const size_t off = ((size_t)((tile - ctx_tiles) * kTok + st) * p.Hkv + h) * D;
+            ks = k_new + off;
+            vs = v_new + off;
+        }
+#pragma unroll
+        for (int i = 0; i < kLoads; ++i) {
+            const int c = (sc + 4 * i) * 4;
+            kbuf[i] = ks ? load4(ks + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+            vbuf[i] = vs ? load4(vs + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    };
+    float m_run[4], l_run[4], acc[4][CPT];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        m_run[i] = -INFINITY;
+        l_run[i] = 0.f;
+#pragma unroll
+        for (int c = 0; c < CPT; ++c) acc[i][c] = 0.f;
+    }
+    if (tile_begin < tile_end) fetch(tile_begin);
+    for (int tile = tile_begin; tile < tile_end; ++tile) {
+        const bool is_new = tile >= ctx_tiles;
+        const int tok0 = (is_new ? tile - ctx_tiles : tile) * kTok;
+        __syncthreads();  // the previous tile has been read
+#pragma unroll
+        for (int i = 0; i < kLoads; ++i) {
+            const int c = (sc + 4 * i) * 4;
+            Kt[(c + 0) * kPitch + st] = kbuf[i].x;
+            Kt[(c + 1) * kPitch + st] = kbuf[i].y;
+            Kt[(c + 2) * kPitch + st] = kbuf[i].z;
+            Kt[(c + 3) * kPitch + st] = kbuf[i].w;
+            *reinterpret_cast<float4*>(Vs + st * D + c) = vbuf[i];
+        }
         __syncthreads();
-        // stage this pass's query rows (row r = token j * G + head g of the group)
-        for (int e = tid; e < kRowsPerPass * D; e += kThreads) {
-            int r = pass_row0 + e / D, c = e % D;
-            float v = 0.f;
-            if (r < R) {
-                int j = r / p.G, g = r % p.G;
-                v = to_float(q[((size_t)j * p.Hq + h * p.G + g) * D + c]);
+        if (tile + 1 < tile_end) fetch(tile + 1);
+        // S = Q K^T: rows 4 ty .. + 3, tokens 4 tx .. + 3.  Channels are summed in runs of 16, the runs then added: the
+        // rounding of a long serial sum would show in the weights of the largest logits.
+        float sv[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) sv[i][j] = 0.f;
+#pragma unroll 1
+        for (int c0 = 0; c0 < D; c0 += 16) {
+            float part[4][4];
+#pragma unroll
+            for (int cc = 0; cc < 16; ++cc) {
+                const float4 a = *reinterpret_cast<const float4*>(Qt + (c0 + cc) * kPitch + 4 * ty);
+                const float4 k4 = *reinterpret_cast<const float4*>(Kt + (c0 + cc) * kPitch + 4 * tx);
+                const float av[4] = {a.x, a.y, a.z, a.w}, kv[4] = {k4.x, k4.y, k4.z, k4.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) part[i][j] = cc == 0 ? av[i] * kv[j] : fmaf(av[i], kv[j], part[i][j]);
             }
-            Qs[e] = v;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) sv[i][j] += part[i][j];
         }
-        float m_run[kRowsPerWarp], l_run[kRowsPerWarp], acc[kRowsPerWarp][CPL];
+        // which of the thread's tokens exist (a token behind a bad page id is skipped)
+        unsigned exists = 0;
 #pragma unroll
-        for (int i = 0; i < kRowsPerWarp; ++i) {
-            m_run[i] = -INFINITY;
-            l_run[i] = 0.f;
-#pragma unroll
-            for (int c = 0; c < CPL; ++c) acc[i][c] = 0.f;
+        for (int j = 0; j < 4; ++j) {
+            const int t = tok0 + 4 * tx + j;
+            bool ok = t < (is_new ? M : seq_len);
+            if (ok && !is_new) {
+                const int page = table[t / p.bs];
+                ok = page >= 0 && page < p.n_pages;
+                if (!ok && ty == 0 && row0 == 0) record_fault(p.workspace, SPECPV_ERR_BAD_BLOCK_TABLE, b, t / p.bs, page, l);
+            }
+            exists |= (unsigned)ok << j;
         }
-
-        for (int tile = 0; tile < n_ctx_tiles + n_new_tiles; ++tile) {
-            const bool is_new = tile >= n_ctx_tiles;
-            const int tok0 = is_new ? (tile - n_ctx_tiles) * kTile : ctx_begin + tile * kTile;
-            const int tok_end = is_new ? M : ctx_end;
-            __syncthreads();
-            if (tid == 0) s_tile_valid = 1;
-            __syncthreads();
-            // stage K and V of the tile as float32
-            for (int e = tid; e < kTile * D; e += kThreads) {
-                int tt = e / D, c = e % D;
-                int t = tok0 + tt;
-                float kv = 0.f, vv = 0.f;
-                if (t < tok_end) {
-                    if (is_new) {
-                        size_t off = ((size_t)t * p.Hkv + h) * D + c;
-                        kv = to_float(k_new[off]);
-                        vv = to_float(v_new[off]);
-                    } else {
-                        int page = table[t / p.bs];
-                        if (page < 0 || page >= p.n_pages) {
-                            if (c == 0) record_fault(p.workspace, SPECPV_ERR_BAD_BLOCK_TABLE, b, t / p.bs, page, l);
-                            s_tile_valid = 0;
-                        } else {
-                            size_t off = (((size_t)page * p.Hkv + h) * p.bs + t % p.bs) * D + c;
-                            kv = to_float(k_pool[off]);
-                            vv = to_float(v_pool[off]);
-                        }
-                    }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            unsigned vis = exists;
+            if (is_new) vis &= (unsigned)(s_mask[4 * ty + i][(tok0 + 4 * tx) >> 6] >> ((4 * tx) & 63)) & 15u;
+            float mx = -INFINITY;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                sv[i][j] = (vis >> j) & 1u ? sv[i][j] * p.scale : -INFINITY;
+                mx = fmaxf(mx, sv[i][j]);
+            }
+            const float m_new = fmaxf(m_run[i], row_max(mx));
+            const float m_safe = m_new == -INFINITY ? 0.f : m_new;
+            float sum = 0.f;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                sv[i][j] = expf(sv[i][j] - m_safe);  // exp(-inf) = 0 for masked keys
+                sum += sv[i][j];
+            }
+            const float corr = expf(m_run[i] - m_safe);  // 0 while nothing has been seen
+            l_run[i] = l_run[i] * corr + row_sum(sum);
+            m_run[i] = m_new;
+#pragma unroll
+            for (int c = 0; c < CPT; ++c) acc[i][c] *= corr;
+            *reinterpret_cast<float4*>(Ps + (4 * ty + i) * kPitch + 4 * tx) = make_float4(sv[i][0], sv[i][1], sv[i][2], sv[i][3]);
+        }
+        __syncwarp();  // the rows a thread reads below were written by its own half warp
+        // O += P V: channels CPT tx .. + CPT - 1
+#pragma unroll 2
+        for (int t = 0; t < kTok; t += 4) {
+            float4 pr[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) pr[i] = *reinterpret_cast<const float4*>(Ps + (4 * ty + i) * kPitch + t);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                float vv[CPT];
+#pragma unroll
+                for (int c = 0; c < CPT; c += 4) {
+                    const float4 v4 = *reinterpret_cast<const float4*>(Vs + (t + u) * D + c * 16 + 4 * tx);
+                    vv[c] = v4.x; vv[c + 1] = v4.y; vv[c + 2] = v4.z; vv[c + 3] = v4.w;
                 }
-                Ks[tt * (D + 1) + c] = kv;
-                Vs[tt * D + c] = vv;
-            }
-            __syncthreads();
-            const bool tile_ok = s_tile_valid != 0;  // a tile reached through a bad page id is skipped
-            const int t_lane = tok0 + lane;
-            // logits of this lane's token against the warp's rows
-            float s[kRowsPerWarp];
 #pragma unroll
-            for (int i = 0; i < kRowsPerWarp; ++i) s[i] = 0.f;
-            const float* krow = Ks + lane * (D + 1);
-            const float* qrow = Qs + warp * kRowsPerWarp * D;
-#pragma unroll 8
-            for (int c = 0; c < D; ++c) {
-                float kc = krow[c];
+                for (int i = 0; i < 4; ++i) {
+                    const float w = u == 0 ? pr[i].x : u == 1 ? pr[i].y : u == 2 ? pr[i].z : pr[i].w;
 #pragma unroll
-                for (int i = 0; i < kRowsPerWarp; ++i) s[i] = fmaf(qrow[i * D + c], kc, s[i]);
-            }
-#pragma unroll
-            for (int i = 0; i < kRowsPerWarp; ++i) {
-                const int r = pass_row0 + warp * kRowsPerWarp + i;
-                bool visible = tile_ok && t_lane < tok_end && r < R;
-                if (visible && is_new) {
-                    int j = r / p.G;
-                    visible = (mask[(size_t)j * p.mask_words + t_lane / 64] >> (t_lane % 64)) & 1ull;
-                }
-                float logit = visible ? s[i] * p.scale : -INFINITY;
-                float m_new = fmaxf(m_run[i], warp_max(logit));
-                float m_safe = m_new == -INFINITY ? 0.f : m_new;
-                float pr = expf(logit - m_safe);       // exp(-inf) = 0 for masked keys
-                float corr = expf(m_run[i] - m_safe);  // 0 while nothing has been seen
-                l_run[i] = l_run[i] * corr + warp_sum(pr);
-                m_run[i] = m_new;
-#pragma unroll
-                for (int c = 0; c < CPL; ++c) acc[i][c] *= corr;
-                s[i] = pr;
-            }
-            // PV: lane <-> channel
-#pragma unroll 4
-            for (int tt = 0; tt < kTile; ++tt) {
-                float vv[CPL];
-#pragma unroll
-                for (int c = 0; c < CPL; ++c) vv[c] = Vs[tt * D + lane + 32 * c];
-#pragma unroll
-                for (int i = 0; i < kRowsPerWarp; ++i) {
-                    float pr = __shfl_sync(0xffffffffu, s[i], tt);
-#pragma unroll
-                    for (int c = 0; c < CPL; ++c) acc[i][c] = fmaf(pr, vv[c], acc[i][c]);
+                    for (int c = 0; c < CPT; ++c) acc[i][c] = fmaf(w, vv[c], acc[i][c]);
                 }
             }
         }
-
-        // write this pass's rows
+    }
+    // acc[i][c .. c + 3] are channels 16 c + 4 tx .. + 3 of row 4 ty + i
 #pragma unroll
-        for (int i = 0; i < kRowsPerWarp; ++i) {
-            const int r = pass_row0 + warp * kRowsPerWarp + i;
-            if (r >= R) continue;
-            if (p.n_splits == 1) {
-                const int j = r / p.G, g = r % p.G;
-                const size_t row = ((size_t)lb * p.M_max + j) * p.Hq + h * p.G + g;
-                TO* o = reinterpret_cast<TO*>(p.out) + row * D;
-                float inv = 1.f / l_run[i];
+    for (int i = 0; i < 4; ++i) {
+        const int r = row0 + 4 * ty + i;
+        if (r >= R) continue;
+        if (p.n_splits == 1) {
+            const int j = r / p.G, g = r % p.G;
+            const size_t row = ((size_t)lb * p.M_max + j) * p.Hq + h * p.G + g;
+            TO* o = reinterpret_cast<TO*>(p.out) + row * D;
+            const float inv = 1.f / l_run[i];
 #pragma unroll
-                for (int c = 0; c < CPL; ++c) o[lane + 32 * c] = from_float<TO>(acc[i][c] * inv);
-                if (p.lse && lane == 0) p.lse[row] = m_run[i] + logf(l_run[i]);
-            } else {
-                const size_t prow = (((size_t)lb * p.Hkv + h) * p.n_splits + split) * R_max + r;
+            for (int c = 0; c < CPT; ++c) o[c / 4 * 64 + 4 * tx + c % 4] = from_float<TO>(acc[i][c] * inv);
+            if (p.lse && tx == 0) p.lse[row] = m_run[i] + logf(l_run[i]);
+        } else {
+            const size_t prow = (((size_t)lb * p.Hkv + h) * p.n_splits + split) * R_max + r;
 #pragma unroll
-                for (int c = 0; c < CPL; ++c) p.part_o[prow * D + lane + 32 * c] = acc[i][c];
-                if (lane == 0) {
-                    p.part_ml[prow * 2] = m_run[i];
-                    p.part_ml[prow * 2 + 1] = l_run[i];
-                }
+            for (int c = 0; c < CPT; c += 4)
+                *reinterpret_cast<float4*>(p.part_o + prow * D + c / 4 * 64 + 4 * tx) =
+                    make_float4(acc[i][c], acc[i][c + 1], acc[i][c + 2], acc[i][c + 3]);
+            if (tx == 0) {
+                p.part_ml[prow * 2] = m_run[i];
+                p.part_ml[prow * 2 + 1] = l_run[i];
             }
         }
     }
 }
 
-// Log-sum-exp merge of the per-split partial results: grid = (R_max rows, KV heads, layers x seqs),
-// one thread per channel.
+// Log-sum-exp merge of the per-split partial results: D/4 threads per row, four channels each, eight partial rows in flight
+// per thread; grid = (row groups, KV heads, layers x seqs).
+constexpr int kMergeThreads = 128;
+constexpr int kMergeAhead = 8;
 template <typename TO, int D>
-__global__ void __launch_bounds__(D) merge_splits_kernel(SimtParams p) {
+__global__ void __launch_bounds__(kMergeThreads) merge_splits_kernel(SimtParams p) {
     pdl_begin(p.pdl);
-    const int r = blockIdx.x, h = blockIdx.y, lb = blockIdx.z, c = threadIdx.x;
+    constexpr int kRowThreads = D / 4;
+    const int r = blockIdx.x * (kMergeThreads / kRowThreads) + threadIdx.x / kRowThreads;
+    const int h = blockIdx.y, lb = blockIdx.z, lane = threadIdx.x % kRowThreads;
     const int b = lb % p.batch;
     int M = p.q_lens ? p.q_lens[b] : p.M_max;
     M = min(max(M, 0), p.M_max);
     if (r >= M * p.G) return;
+    const unsigned members = kRowThreads == 32 ? 0xffffffffu : 0xffffu << (threadIdx.x & 16);
     const int R_max = p.M_max * p.G;
-    const size_t base = ((size_t)lb * p.Hkv + h) * p.n_splits;
+    const size_t row0 = ((size_t)lb * p.Hkv + h) * p.n_splits * R_max + r;
+    const float4* po = reinterpret_cast<const float4*>(p.part_o + row0 * D) + lane;
+    const float2* ml = reinterpret_cast<const float2*>(p.part_ml) + row0;
+    const size_t po_stride = (size_t)R_max * kRowThreads;
     float m_all = -INFINITY;
-    for (int s = 0; s < p.n_splits; ++s) m_all = fmaxf(m_all, p.part_ml[((base + s) * R_max + r) * 2]);
-    float l_all = 0.f, o = 0.f;
-    for (int s = 0; s < p.n_splits; ++s) {
-        const size_t prow = (base + s) * R_max + r;
-        float m_s = p.part_ml[prow * 2];
-        if (m_s == -INFINITY) continue;  // an empty split
-        float w = expf(m_s - m_all);
-        l_all = fmaf(p.part_ml[prow * 2 + 1], w, l_all);
-        o = fmaf(p.part_o[prow * D + c], w, o);
+    for (int s = lane; s < p.n_splits; s += kRowThreads) m_all = fmaxf(m_all, ml[(size_t)s * R_max].x);
+#pragma unroll
+    for (int o = kRowThreads / 2; o > 0; o >>= 1) m_all = fmaxf(m_all, __shfl_xor_sync(members, m_all, o));
+    float l_all = 0.f;
+    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int c0 = 0; c0 < p.n_splits; c0 += kRowThreads) {  // a lane per split of this chunk
+        const int n = min(kRowThreads, p.n_splits - c0);
+        float w_mine = 0.f, l_mine = 0.f;
+        if (lane < n) {
+            const float2 v = ml[(size_t)(c0 + lane) * R_max];
+            if (v.x != -INFINITY) {  // a split that saw no token weighs nothing
+                w_mine = expf(v.x - m_all);
+                l_mine = v.y * w_mine;
+            }
+        }
+        for (int s0 = 0; s0 < n; s0 += kMergeAhead) {
+            float4 buf[kMergeAhead];
+#pragma unroll
+            for (int u = 0; u < kMergeAhead; ++u) buf[u] = po[(size_t)(c0 + min(s0 + u, n - 1)) * po_stride];
+#pragma unroll
+            for (int u = 0; u < kMergeAhead; ++u) {
+                // lanes past the last split hold weight 0; beyond the row's lanes the shuffle would wrap
+                const float w = __shfl_sync(members, w_mine, min(s0 + u, kRowThreads - 1), kRowThreads);
+                const float lw = __shfl_sync(members, l_mine, min(s0 + u, kRowThreads - 1), kRowThreads);
+                if (s0 + u >= n || w == 0.f) continue;
+                l_all += lw;
+                o.x = fmaf(buf[u].x, w, o.x);
+                o.y = fmaf(buf[u].y, w, o.y);
+                o.z = fmaf(buf[u].z, w, o.z);
+                o.w = fmaf(buf[u].w, w, o.w);
+            }
+        }
     }
     const int j = r / p.G, g = r % p.G;
     const size_t row = ((size_t)lb * p.M_max + j) * p.Hq + h * p.G + g;
-    reinterpret_cast<TO*>(p.out)[row * D + c] = from_float<TO>(o / l_all);
-    if (p.lse && c == 0) p.lse[row] = m_all + logf(l_all);
+    TO* dst = reinterpret_cast<TO*>(p.out) + row * D + lane * 4;
+    const float inv = 1.f / l_all;
+    dst[0] = from_float<TO>(o.x * inv);
+    dst[1] = from_float<TO>(o.y * inv);
+    dst[2] = from_float<TO>(o.z * inv);
+    dst[3] = from_float<TO>(o.w * inv);
+    if (p.lse && lane == 0) p.lse[row] = m_all + logf(l_all);
 }
 
 template <typename T, typename TO, int D>
 specpv_status launch_typed(const AttnArgs& a, SimtParams& p, cudaStream_t stream) {
-    const size_t smem = (size_t)(kTile * (D + 1) + kTile * D + kRowsPerPass * D) * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(attn_simt_kernel<T, TO, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return SPECPV_ERR_CUDA;
-    dim3 grid(p.n_splits, a.g.Hkv, a.n_layers * a.batch);
+    constexpr size_t smem = simt_smem<D>();
+    if (!tc::set_smem_limit_once(reinterpret_cast<const void*>(attn_simt_kernel<T, TO, D>), (int)smem)) return SPECPV_ERR_CUDA;
+    dim3 grid(p.n_splits * p.row_tiles, a.g.Hkv, a.n_layers * a.batch);
     if (launch_pdl_if(attn_simt_kernel<T, TO, D>, grid, kThreads, smem, stream, p) != cudaSuccess) return SPECPV_ERR_CUDA;
     count_launch();
     if (p.n_splits > 1) {
-        dim3 mgrid(a.M_max * a.g.G, a.g.Hkv, a.n_layers * a.batch);
-        if (launch_pdl_if(merge_splits_kernel<TO, D>, mgrid, D, 0, stream, p) != cudaSuccess) return SPECPV_ERR_CUDA;
+        constexpr int rows = kMergeThreads / (D / 4);
+        dim3 mgrid((a.M_max * a.g.G + rows - 1) / rows, a.g.Hkv, a.n_layers * a.batch);
+        if (launch_pdl_if(merge_splits_kernel<TO, D>, mgrid, kMergeThreads, 0, stream, p) != cudaSuccess) return SPECPV_ERR_CUDA;
         count_launch();
     }
     return SPECPV_OK;
@@ -273,20 +384,20 @@ specpv_status launch_attention_simt(const AttnArgs& a, cudaStream_t stream) {
     p.Hq = a.g.Hq; p.Hkv = a.g.Hkv; p.G = a.g.G; p.bs = a.g.bs; p.max_blocks = a.max_blocks; p.n_pages = a.n_pages;
     p.scale = a.g.scale;
 
-    // split the KV range so that the launch has about two CTAs per SM, as far as the workspace allows
+    // split the KV range so that the launch has about two CTAs per SM, down to one tile per CTA (a tile takes some 3 us, a
+    // partial result a fraction of one), as far as the workspace allows
     constexpr int kTargetCtas = 2 * 148;
     const int base = a.g.Hkv * a.n_layers * a.batch;
     const int R_max = a.M_max * a.g.G;
-    int n_splits = (kTargetCtas + base - 1) / base;
-    const int max_by_len = (a.max_seq_len + 255) / 256;
-    if (n_splits > max_by_len) n_splits = max_by_len;
+    p.row_tiles = (R_max + kRows - 1) / kRows;
+    const int positions = (a.max_seq_len + kTok - 1) / kTok + (a.M_max + kTok - 1) / kTok;
+    int n_splits = kTargetCtas / (base * p.row_tiles);
+    if (n_splits > positions) n_splits = positions;
+    if (n_splits > 64) n_splits = 64;
     const size_t per_split = (size_t)base * R_max * (a.g.d + 2) * sizeof(float);
     if (n_splits > 1 && per_split * n_splits > a.partial_bytes) n_splits = (int)(a.partial_bytes / per_split);
     if (n_splits < 1) n_splits = 1;
     p.n_splits = n_splits;
-    int chunk = (a.max_seq_len + n_splits - 1) / n_splits;
-    p.chunk = (chunk + kTile - 1) / kTile * kTile;
-    if (p.chunk < kTile) p.chunk = kTile;
     char* ws = reinterpret_cast<char*>(a.workspace) + a.partial_off;
     p.part_o = reinterpret_cast<float*>(ws);
     p.part_ml = reinterpret_cast<float*>(ws + (size_t)base * n_splits * R_max * a.g.d * sizeof(float));

@@ -5,6 +5,7 @@
 
 #include "common.cuh"
 #include "aux_kernels.cuh"
+#include "tc_common.cuh"
 
 namespace specpv {
 
@@ -109,12 +110,13 @@ __global__ void __launch_bounds__(32 * kSumWarps) summaries_kernel(SummaryParams
 }
 
 // ---------------------------------------------------------------------------------------------
-// Eq. 2-3 (SIMT form): lane <-> block, the CTA's 32*warps blocks' summaries staged in shared
-// memory as float32, the group's query rows read as broadcasts.  grid = (block groups, Hkv,
-// layers x seqs).
+// Eq. 2-3 (SIMT form): lane <-> block, the CTA's 32 blocks' summaries staged in shared memory as float32; the warps share
+// the group's query rows out in turns of kScoreRowTile rows, which they read as broadcasts, and their partial results are
+// added in warp order.  Bound by latency on the small shapes it serves (2048 tokens, 64 rows: 40 -> 6 us against a warp
+// per 32 blocks that took all rows by itself).  grid = (block groups, Hkv, layers x seqs).
 // ---------------------------------------------------------------------------------------------
-constexpr int kScoreWarps = 4;
-constexpr int kScoreBlocksPerCta = 32 * kScoreWarps;
+constexpr int kScoreWarps = 8;
+constexpr int kScoreBlocksPerCta = 32;
 constexpr int kScoreRowTile = 4;
 
 template <typename T, int D>
@@ -123,8 +125,9 @@ __global__ void __launch_bounds__(32 * kScoreWarps) scores_simt_kernel(ScorePara
     extern __shared__ float smem[];
     float* Smax = smem;                                   // [blocks][D + 1]
     float* Smin = Smax + kScoreBlocksPerCta * (D + 1);    // [blocks][D + 1]
-    float* Qs = Smin + kScoreBlocksPerCta * (D + 1);      // [kScoreRowTile][D]
-    const int h = blockIdx.y, lb = blockIdx.z, tid = threadIdx.x;
+    __shared__ float s_q[kScoreWarps][kScoreRowTile][D];
+    __shared__ float s_red[kScoreWarps][32];
+    const int h = blockIdx.y, lb = blockIdx.z, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = lb % p.batch, l = lb / p.batch;
     const int seq_len = p.seq_lens[b];
     const int nb = (seq_len + p.bs - 1) / p.bs;
@@ -154,21 +157,23 @@ __global__ void __launch_bounds__(32 * kScoreWarps) scores_simt_kernel(ScorePara
         Smin[bi * (D + 1) + c] = vmin;
     }
     const T* q = reinterpret_cast<const T*>(p.q) + (size_t)lb * p.M_max * p.Hq * D;
-    const float* my_max = Smax + tid * (D + 1);
-    const float* my_min = Smin + tid * (D + 1);
+    __syncthreads();
+    const float* my_max = Smax + lane * (D + 1);
+    const float* my_min = Smin + lane * (D + 1);
     float red = p.reduce == SPECPV_REDUCE_MAX ? -INFINITY : 0.f;
-    for (int r0 = row_begin; r0 < row_end; r0 += kScoreRowTile) {
-        __syncthreads();
-        for (int e = tid; e < kScoreRowTile * D; e += blockDim.x) {
+    for (int r0 = row_begin + warp * kScoreRowTile; r0 < row_end; r0 += kScoreWarps * kScoreRowTile) {
+        __syncwarp();
+        float (*Qs)[D] = s_q[warp];
+        for (int e = lane; e < kScoreRowTile * D; e += 32) {
             int r = r0 + e / D, c = e % D;
             float v = 0.f;
             if (r < row_end) {
                 int j = r / p.G, g = r % p.G;
                 v = to_float(q[((size_t)j * p.Hq + h * p.G + g) * D + c]);
             }
-            Qs[e] = v;
+            Qs[e / D][c] = v;
         }
-        __syncthreads();
+        __syncwarp();
         float dmax[kScoreRowTile], dmin[kScoreRowTile];
 #pragma unroll
         for (int i = 0; i < kScoreRowTile; ++i) dmax[i] = dmin[i] = 0.f;
@@ -178,7 +183,7 @@ __global__ void __launch_bounds__(32 * kScoreWarps) scores_simt_kernel(ScorePara
                 float a = my_max[c], bb = my_min[c];
 #pragma unroll
                 for (int i = 0; i < kScoreRowTile; ++i) {
-                    float qc = Qs[i * D + c];
+                    float qc = Qs[i][c];
                     dmax[i] = fmaf(qc, a, dmax[i]);
                     dmin[i] = fmaf(qc, bb, dmin[i]);
                 }
@@ -191,7 +196,7 @@ __global__ void __launch_bounds__(32 * kScoreWarps) scores_simt_kernel(ScorePara
                 float a = my_max[c], bb = my_min[c];
 #pragma unroll
                 for (int i = 0; i < kScoreRowTile; ++i) {
-                    float qc = Qs[i * D + c];
+                    float qc = Qs[i][c];
                     dmax[i] = fmaf(qc, qc < 0.f ? bb : a, dmax[i]);
                 }
             }
@@ -205,8 +210,13 @@ __global__ void __launch_bounds__(32 * kScoreWarps) scores_simt_kernel(ScorePara
             red = p.reduce == SPECPV_REDUCE_MAX ? fmaxf(red, s) : red + s;
         }
     }
+    s_red[warp][lane] = red;
+    __syncthreads();
     const int i = blk0 + tid;
-    if (i < nb) {
+    if (tid < 32 && i < nb) {
+        red = s_red[0][tid];
+#pragma unroll
+        for (int w = 1; w < kScoreWarps; ++w) red = p.reduce == SPECPV_REDUCE_MAX ? fmaxf(red, s_red[w][tid]) : red + s_red[w][tid];
         if (p.reduce != SPECPV_REDUCE_MAX) red /= (float)(row_end - row_begin);
         p.scores[(((size_t)lb * p.Hkv + h) * p.max_blocks) + i] = red;
     }
@@ -510,9 +520,8 @@ specpv_status launch_summaries(const SummaryParams& params, int n_layers, int bl
 
 template <typename T, int D>
 static specpv_status launch_scores_typed(const ScoreParams& p, int n_layers, int max_nb, cudaStream_t stream) {
-    const size_t smem = (size_t)(2 * kScoreBlocksPerCta * (D + 1) + kScoreRowTile * D) * sizeof(float);
-    if (cudaFuncSetAttribute(scores_simt_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return SPECPV_ERR_CUDA;
+    const size_t smem = (size_t)(2 * kScoreBlocksPerCta * (D + 1)) * sizeof(float);
+    if (!tc::set_smem_limit_once(reinterpret_cast<const void*>(scores_simt_kernel<T, D>), (int)smem)) return SPECPV_ERR_CUDA;
     dim3 grid((max_nb + kScoreBlocksPerCta - 1) / kScoreBlocksPerCta, p.Hkv, n_layers * p.batch);
     SPECPV_LAUNCH(scores_simt_kernel<T, D>, grid, 32 * kScoreWarps, smem, stream, p);
     return SPECPV_OK;

@@ -129,6 +129,17 @@ def test_packed_rows_and_alternating_streams(Hq, Hkv, d, bs, ctx, Ms, n_chain):
     run_case("bf16", Hq, Hkv, d, bs, ctx=ctx, Ms=Ms, n_chain=n_chain, seed=Hq + d + len(ctx))
 
 
+@pytest.mark.parametrize("Hq,Hkv,d", [(8, 2, 64), (5, 1, 128)])
+@pytest.mark.parametrize("bs,ctx,Ms,n_chain", [
+    (64, [0, 1, 63, 64], [16, 1, 13, 12], 0),         # no context to one 64-token tile, row counts around 64
+    (16, [65, 64 * 9], [65, 17], 0),                   # the step's own tokens in two tiles
+    (32, [64 * 40 + 33], [60], 68),                    # 128 step tokens, several row tiles, many splits
+])
+def test_float32_kernel_tile_edges(Hq, Hkv, d, bs, ctx, Ms, n_chain):
+    """The plain kernel's 64-row and 64-token tiles at their edges, one and many KV splits."""
+    run_case("fp32", Hq, Hkv, d, bs, ctx=ctx, Ms=Ms, n_chain=n_chain, seed=Hq + bs)
+
+
 @pytest.mark.parametrize("M,n_layers", [(60, 20), (90, 12), (26, 24)])
 def test_many_layers_and_one_layer_agree_with_the_oracle(M, n_layers):
     """The row tiles per CTA and the KV splits depend on how many CTAs a launch has: two row tiles without splits, a last
