@@ -26,7 +26,7 @@ constexpr int kWTileBytes = kFeatTile * 128;  // 128 features x 64 input feature
 constexpr int kProjDataBytes = 192 * 1024;
 constexpr int kProjSmem = 1024 + kProjDataBytes;
 constexpr int kProjMaxStages = 8;
-constexpr int kIssueGroup = 2;             // stages whose copies are issued together
+constexpr int kIssueGroup = 2;             // stages whose copies are issued together (one range per tile)
 constexpr int kMaxTokTile = 256;           // rows per CTA (accumulator columns)
 
 struct ProjTcParams {
@@ -48,29 +48,47 @@ struct __align__(8) ProjBarriers {
     int abort_flag;
 };
 
-// Channels (2j, 2j+1) = lo and (64+2j, 64+2j+1) = hi of feature tile `tile`, row `tok` of layer-in-call `l`.
-__device__ __forceinline__ void proj_finish(const ProjTcParams& p, int tile, int l, int tok, int j, float2 lo, float2 hi) {
+// Where channels (2j, 2j+1) and (64+2j, 64+2j+1) of feature tile `tile`, row `tok` of layer-in-call `l` go, and what they
+// are rotated by and added to: asked for ahead of the sums, so that the two latencies overlap.
+struct ProjTarget {
+    __nv_bfloat16* dst;
+    float4 cs;         // cos, sin, cos, sin
+    uint32_t res[2];   // residual of the two channel pairs
+    bool rope, add;
+};
+__device__ __forceinline__ ProjTarget proj_target(const ProjTcParams& p, int tile, int l, int tok, int j) {
     int s = 0;
     for (int i = 1; i < p.n_seg; ++i)
         if (tile >= p.seg[i].first_tile) s = i;
     const ProjSegment& sg = p.seg[s];
-    if (sg.rope) {
-        const float4 cs = __ldg(reinterpret_cast<const float4*>(p.cos_sin + ((size_t)tok * 64 + 2 * j) * 2));  // cos, sin, cos, sin
+    ProjTarget t;
+    t.rope = sg.rope;
+    t.add = p.residual && s == 0;
+    t.cs = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (t.rope) t.cs = __ldg(reinterpret_cast<const float4*>(p.cos_sin + ((size_t)tok * 64 + 2 * j) * 2));
+    const size_t off = ((size_t)l * p.tokens + tok) * sg.row_stride + (size_t)(tile - sg.first_tile) * kFeatTile + 2 * j;
+    t.res[0] = t.res[1] = 0;
+    if (t.add) {
+        t.res[0] = __ldg(reinterpret_cast<const uint32_t*>(p.residual + off));
+        t.res[1] = __ldg(reinterpret_cast<const uint32_t*>(p.residual + off + 64));
+    }
+    t.dst = reinterpret_cast<__nv_bfloat16*>(sg.base) + off;
+    return t;
+}
+__device__ __forceinline__ void proj_finish(const ProjTarget& t, float2 lo, float2 hi) {
+    if (t.rope) {
+        const float4 cs = t.cs;
         const float2 rl = make_float2(lo.x * cs.x - hi.x * cs.y, lo.y * cs.z - hi.y * cs.w);
         const float2 rh = make_float2(hi.x * cs.x + lo.x * cs.y, hi.y * cs.z + lo.y * cs.w);
         lo = rl;
         hi = rh;
     }
-    const size_t off = ((size_t)l * p.tokens + tok) * sg.row_stride + (size_t)(tile - sg.first_tile) * kFeatTile + 2 * j;
-    if (p.residual && s == 0) {
-        const uint32_t a = __ldg(reinterpret_cast<const uint32_t*>(p.residual + off));
-        const uint32_t b = __ldg(reinterpret_cast<const uint32_t*>(p.residual + off + 64));
-        lo.x += __uint_as_float(a << 16); lo.y += __uint_as_float(a & 0xFFFF0000u);
-        hi.x += __uint_as_float(b << 16); hi.y += __uint_as_float(b & 0xFFFF0000u);
+    if (t.add) {
+        lo.x += __uint_as_float(t.res[0] << 16); lo.y += __uint_as_float(t.res[0] & 0xFFFF0000u);
+        hi.x += __uint_as_float(t.res[1] << 16); hi.y += __uint_as_float(t.res[1] & 0xFFFF0000u);
     }
-    __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(sg.base) + off;
-    *reinterpret_cast<uint32_t*>(dst) = pack_bf16(lo.x, lo.y);
-    *reinterpret_cast<uint32_t*>(dst + 64) = pack_bf16(hi.x, hi.y);
+    *reinterpret_cast<uint32_t*>(t.dst) = pack_bf16(lo.x, lo.y);
+    *reinterpret_cast<uint32_t*>(t.dst + 64) = pack_bf16(hi.x, hi.y);
 }
 
 __device__ __forceinline__ size_t partial_base(const ProjTcParams& p, int l, int chunk, int n_chunks, int tile, int split) {
@@ -198,7 +216,7 @@ __global__ void __launch_bounds__(kProjThreads, 2) proj_tc_kernel(const __grid_c
                     *reinterpret_cast<float2*>(part + (size_t)t * kFeatTile + 2 * j) = lo;
                     *reinterpret_cast<float2*>(part + (size_t)t * kFeatTile + 64 + 2 * j) = hi;
                 } else {
-                    proj_finish(p, tile, l, tok0 + t, j, lo, hi);
+                    proj_finish(proj_target(p, tile, l, tok0 + t, j), lo, hi);
                 }
             }
         }
@@ -224,6 +242,7 @@ __global__ void __launch_bounds__(128) proj_reduce_kernel(const __grid_constant_
     if (t >= valid) return;
     const float* part = p.partials + partial_base(p, l, chunk, n_chunks, tile, 0) + (size_t)t * kFeatTile + 2 * j;
     const size_t split_stride = (size_t)p.n_pad * kFeatTile;
+    const ProjTarget target = proj_target(p, tile, l, tok0 + t, j);
     float2 a[8], b[8];
 #pragma unroll
     for (int s = 0; s < 8; ++s)
@@ -237,7 +256,7 @@ __global__ void __launch_bounds__(128) proj_reduce_kernel(const __grid_constant_
         if (s < p.splits) {
             lo.x += a[s].x; lo.y += a[s].y; hi.x += b[s].x; hi.y += b[s].y;
         }
-    proj_finish(p, tile, l, tok0 + t, j, lo, hi);
+    proj_finish(target, lo, hi);
 }
 
 // ---- plain kernel: any dtype / head size ---------------------------------------------------------------------
@@ -353,7 +372,6 @@ specpv_status launch_proj_tc(const ProjArgs& a, cudaStream_t stream) {
     const int ring_bytes = small_ring ? kProjDataBytes / 2 : kProjDataBytes;
     p.stages = ring_bytes / stage_bytes;
     if (p.stages > kProjMaxStages) p.stages = kProjMaxStages;
-    p.group = kIssueGroup <= p.stages / 2 ? kIssueGroup : (p.stages / 2 > 0 ? p.stages / 2 : 1);
     // enough CTAs to fill every SM's slots: split the input features while the tiles alone cannot
     const long long units = (long long)a.n_layers_call * n_chunks * p.n_tiles;
     const int slots = small_ring ? 2 * 148 : 148;
@@ -366,6 +384,9 @@ specpv_status launch_proj_tc(const ProjArgs& a, cudaStream_t stream) {
         while (splits > 1 && per_split * splits > a.scratch_bytes) --splits;
     }
     p.splits = splits;
+    // With several ranges a CTA's share is short and its weights are on their way to L2 before the first copy, which leaves
+    // nothing to gain from copies in pairs (one layer, 24 rows: the block 37.8 -> 36.6 us with single ones).
+    p.group = splits > 1 || p.stages < 4 ? 1 : kIssueGroup;
     p.partials = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(a.workspace) + a.scratch_off);
     dim3 grid(p.n_tiles * splits, n_chunks, a.n_layers_call);
     if (launch_pdl(proj_tc_kernel, grid, kProjThreads, 1024 + ring_bytes, stream, p) != cudaSuccess) return SPECPV_ERR_CUDA;
