@@ -241,9 +241,9 @@ SPECPV_EXPORT specpv_status specpv_update_block_summaries(const specpv_config* c
     if (max_blocks_touched > kv->max_blocks) max_blocks_touched = kv->max_blocks;
     SummaryParams p{};
     p.k_pool = kv->k_pool; p.block_table = kv->block_table; p.seq_lens = kv->seq_lens; p.tok_begin = tok_begin;
-    p.n_appended = nullptr; p.kmax = kmax; p.kmin = kmin; p.workspace = workspace;
+    p.kmax = kmax; p.kmin = kmin; p.workspace = workspace;
     p.layer0 = layer0; p.batch = kv->batch; p.Hkv = g.Hkv; p.bs = g.bs; p.d = g.d; p.max_blocks = kv->max_blocks;
-    p.n_pages = kv->n_pages; p.A_max = 0;
+    p.n_pages = kv->n_pages;
     return launch_summaries(p, n_layers, max_blocks_touched, g.dtype, reinterpret_cast<cudaStream_t>(stream));
 }
 
@@ -506,24 +506,12 @@ SPECPV_EXPORT specpv_status specpv_commit_accepted(const specpv_config* cfg, int
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     CommitParams p{};
     p.k_new = k_new; p.v_new = v_new; p.accepted = accepted; p.n_accepted = n_accepted; p.k_pool = dst->k_pool;
-    p.v_pool = dst->v_pool; p.block_table = dst->block_table; p.seq_lens = dst->seq_lens; p.workspace = workspace;
+    p.v_pool = dst->v_pool; p.block_table = dst->block_table; p.seq_lens = const_cast<int32_t*>(dst->seq_lens);
+    p.kmax = kmax; p.kmin = kmin; p.workspace = workspace;
     p.layer0 = layer0; p.batch = dst->batch; p.M_max = M_max; p.A_max = A_max; p.Hkv = g.Hkv; p.bs = g.bs; p.d = g.d;
-    p.es = g.es; p.max_blocks = dst->max_blocks; p.n_pages = dst->n_pages;
-    st = launch_commit(p, n_layers, nullptr, s);
-    if (st != SPECPV_OK) return st;
-    if (kmax) {
-        SummaryParams sp{};
-        sp.k_pool = dst->k_pool; sp.block_table = dst->block_table; sp.seq_lens = dst->seq_lens;
-        sp.tok_begin = dst->seq_lens; sp.n_appended = n_accepted; sp.kmax = kmax; sp.kmin = kmin; sp.workspace = workspace;
-        sp.layer0 = layer0; sp.batch = dst->batch; sp.Hkv = g.Hkv; sp.bs = g.bs; sp.d = g.d; sp.max_blocks = dst->max_blocks;
-        sp.n_pages = dst->n_pages; sp.A_max = A_max;
-        st = launch_summaries(sp, n_layers, (A_max + g.bs - 1) / g.bs + 1, g.dtype, s);
-        if (st != SPECPV_OK) return st;
-    }
-    if (layer0 + n_layers == g.n_layers)
-        return launch_commit_lens(const_cast<int32_t*>(dst->seq_lens), n_accepted, dst->batch, A_max,
-                                  dst->max_blocks * g.bs, s);
-    return SPECPV_OK;
+    p.max_blocks = dst->max_blocks; p.n_pages = dst->n_pages;
+    p.advance = layer0 + n_layers == g.n_layers;
+    return launch_commit(p, n_layers, g.dtype, s);
 }
 
 // ---- the linear maps either side of the attention --------------------------------------------------------------

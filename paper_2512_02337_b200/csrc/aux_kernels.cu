@@ -40,19 +40,52 @@ __device__ __forceinline__ uint32_t packed_min(uint32_t a, uint32_t b, float) {
     return __float_as_uint(fminf(__uint_as_float(a), __uint_as_float(b)));
 }
 
+// A lane's running maximum and minimum of one 16-byte chunk of channels.
+template <typename T>
+struct SummaryAcc {
+    static constexpr uint32_t kNegInf = sizeof(T) == 2 ? 0xFF80FF80u : 0xFF800000u;
+    static constexpr uint32_t kPosInf = kNegInf & (sizeof(T) == 2 ? 0x7FFF7FFFu : 0x7FFFFFFFu);
+    uint32_t mx[4] = {kNegInf, kNegInf, kNegInf, kNegInf}, mn[4] = {kPosInf, kPosInf, kPosInf, kPosInf};
+    __device__ __forceinline__ void take(const uint4& v) {
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            mx[e] = packed_max(mx[e], w[e], T());
+            mn[e] = packed_min(mn[e], w[e], T());
+        }
+    }
+    __device__ __forceinline__ void combine(int chunks) {  // over the lanes that hold the same chunk
+        for (int o = 16; o >= chunks; o >>= 1) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                mx[e] = packed_max(mx[e], __shfl_xor_sync(0xffffffffu, mx[e], o), T());
+                mn[e] = packed_min(mn[e], __shfl_xor_sync(0xffffffffu, mn[e], o), T());
+            }
+        }
+    }
+    __device__ __forceinline__ void store(void* kmax, void* kmin, int aligned, size_t o) const {  // o: in 16-byte chunks
+        const uint4 vx = make_uint4(mx[0], mx[1], mx[2], mx[3]), vn = make_uint4(mn[0], mn[1], mn[2], mn[3]);
+        if (aligned) {
+            reinterpret_cast<uint4*>(kmax)[o] = vx;
+            reinterpret_cast<uint4*>(kmin)[o] = vn;
+        } else {
+            constexpr int kChunk = 16 / (int)sizeof(T);
+#pragma unroll
+            for (int e = 0; e < kChunk; ++e) {
+                reinterpret_cast<T*>(kmax)[o * kChunk + e] = reinterpret_cast<const T*>(&vx)[e];
+                reinterpret_cast<T*>(kmin)[o * kChunk + e] = reinterpret_cast<const T*>(&vn)[e];
+            }
+        }
+    }
+};
+
 template <typename T>
 __global__ void __launch_bounds__(32 * kSumWarps) summaries_kernel(SummaryParams p) {
     pdl_begin(p.pdl);
-    constexpr uint32_t kNegInf = sizeof(T) == 2 ? 0xFF80FF80u : 0xFF800000u;
-    constexpr uint32_t kPosInf = kNegInf & (sizeof(T) == 2 ? 0x7FFF7FFFu : 0x7FFFFFFFu);
     const int lane = threadIdx.x & 31;
     const int h = blockIdx.y * kSumWarps + (threadIdx.x >> 5), lb = blockIdx.z;
     const int b = lb % p.batch, l = lb / p.batch;
-    int seq_len = p.seq_lens[b];
-    if (p.n_appended) {  // summaries of a commit in flight: the lengths are not advanced yet
-        const int n = min(max(p.n_appended[b], 0), p.A_max);
-        if ((size_t)seq_len + n <= (size_t)p.max_blocks * p.bs) seq_len += n;
-    }
+    const int seq_len = p.seq_lens[b];
     const int begin = p.tok_begin ? p.tok_begin[b] : 0;
     const int i = max(begin, 0) / p.bs + blockIdx.x;
     if (h >= p.Hkv || (size_t)i * p.bs >= (size_t)seq_len || i >= p.max_blocks) return;
@@ -67,46 +100,18 @@ __global__ void __launch_bounds__(32 * kSumWarps) summaries_kernel(SummaryParams
     const int chunk = lane % chunks, tl = lane / chunks;
     const uint4* k = reinterpret_cast<const uint4*>(reinterpret_cast<const T*>(p.k_pool) +
                                                     (((size_t)(p.layer0 + l) * p.n_pages + page) * p.Hkv + h) * p.bs * p.d) + chunk;
-    uint32_t mx[4], mn[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) { mx[e] = kNegInf; mn[e] = kPosInf; }
+    SummaryAcc<T> acc;
     for (int t0 = 0; t0 < n_valid; t0 += kSumLoads * tok_lanes) {
         uint4 buf[kSumLoads];
 #pragma unroll
         for (int u = 0; u < kSumLoads; ++u)  // past the last valid token: that token again, which changes nothing
             buf[u] = k[(size_t)min(t0 + u * tok_lanes + tl, n_valid - 1) * chunks];
 #pragma unroll
-        for (int u = 0; u < kSumLoads; ++u) {
-            const uint32_t w[4] = {buf[u].x, buf[u].y, buf[u].z, buf[u].w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                mx[e] = packed_max(mx[e], w[e], T());
-                mn[e] = packed_min(mn[e], w[e], T());
-            }
-        }
+        for (int u = 0; u < kSumLoads; ++u) acc.take(buf[u]);
     }
-    for (int o = 16; o >= chunks; o >>= 1) {
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            mx[e] = packed_max(mx[e], __shfl_xor_sync(0xffffffffu, mx[e], o), T());
-            mn[e] = packed_min(mn[e], __shfl_xor_sync(0xffffffffu, mn[e], o), T());
-        }
-    }
-    if (tl == 0) {
-        const size_t o = ((((size_t)(p.layer0 + l) * p.batch + b) * p.Hkv + h) * p.max_blocks + i) * chunks + chunk;
-        const uint4 vx = make_uint4(mx[0], mx[1], mx[2], mx[3]), vn = make_uint4(mn[0], mn[1], mn[2], mn[3]);
-        if (p.aligned) {
-            reinterpret_cast<uint4*>(p.kmax)[o] = vx;
-            reinterpret_cast<uint4*>(p.kmin)[o] = vn;
-        } else {
-            constexpr int kChunk = 16 / (int)sizeof(T);
-#pragma unroll
-            for (int e = 0; e < kChunk; ++e) {
-                reinterpret_cast<T*>(p.kmax)[o * kChunk + e] = reinterpret_cast<const T*>(&vx)[e];
-                reinterpret_cast<T*>(p.kmin)[o * kChunk + e] = reinterpret_cast<const T*>(&vn)[e];
-            }
-        }
-    }
+    acc.combine(chunks);
+    if (tl == 0)
+        acc.store(p.kmax, p.kmin, p.aligned, ((((size_t)(p.layer0 + l) * p.batch + b) * p.Hkv + h) * p.max_blocks + i) * chunks + chunk);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -223,31 +228,35 @@ __global__ void __launch_bounds__(32 * kScoreWarps) scores_simt_kernel(ScorePara
 }
 
 // ---------------------------------------------------------------------------------------------
-// Selection: one CTA per (layer, sequence, KV head).  The candidates' (score, index) pairs become
-// unique 64-bit keys whose unsigned order is "score descending, then index ascending, NaN last";
-// an 8-pass most-significant-digit radix select finds the k-th largest key exactly, and a
-// block-wide ordered compaction writes sink | kept candidates | local in ascending order.
+// Selection: one CTA per (layer, sequence, KV head).  A candidate's score becomes a 32-bit key whose unsigned order is
+// "score ascending, NaN first"; a most-significant-digit radix select in digits of 11, 11 and 10 bits finds the key T of the
+// k-th best candidate and how many candidates of that very key are still to be taken (the ones of lowest index), and an
+// ordered compaction writes sink | kept candidates | local in ascending order.  Bound by its barriers and by shared-memory
+// atomics: eight passes of 8 bits over (key, index) pairs, the first of which met two or three crowded bins, took 16.2 us for 2045
+// candidates x 256 lists against 13.1, and 9.7 against 6.6 for 29 x 2.
 // ---------------------------------------------------------------------------------------------
 constexpr int kSelectThreads = 256;
+constexpr int kSelectBins = 2048;
 
-__device__ __forceinline__ uint64_t select_key(float score, int index) {
-    uint32_t bits = __float_as_uint(score);
-    uint32_t ord;
-    if (score != score) ord = 0u;                         // NaN ranks below every number
-    else if (score == 0.f) ord = 0x80000000u;             // -0 and +0 tie
-    else ord = (bits & 0x80000000u) ? ~bits : (bits | 0x80000000u);
-    return ((uint64_t)ord << 32) | (uint64_t)(0xFFFFFFFFu - (uint32_t)index);
+__device__ __forceinline__ uint32_t select_key(float score) {
+    const uint32_t bits = __float_as_uint(score);
+    if (score != score) return 0u;              // NaN ranks below every number
+    if (score == 0.f) return 0x80000000u;       // -0 and +0 tie
+    return (bits & 0x80000000u) ? ~bits : (bits | 0x80000000u);
 }
 
 __global__ void __launch_bounds__(kSelectThreads) select_kernel(SelectParams p) {
     pdl_begin(p.pdl);
-    __shared__ unsigned int hist[256];
-    __shared__ uint64_t s_prefix;
+    __shared__ unsigned int hist[kSelectBins];
+    __shared__ uint32_t s_prefix;
     __shared__ int s_remaining;
     __shared__ int s_warp_counts[kSelectThreads / 32];
-    __shared__ int s_running;
-    __shared__ int s_round_counts[16 * (kSelectThreads / 32)];  // kept candidates per (round, warp)
-    const int h = blockIdx.x, b = blockIdx.y, l = blockIdx.z, tid = threadIdx.x;
+    constexpr int kWarps = kSelectThreads / 32;
+    constexpr int kKeysPerThread = 16;                   // a thread's first keys stay in registers (4096 candidates)
+    __shared__ int s_above[kKeysPerThread * kWarps];     // candidates above T per (round, warp), then their exclusive prefix
+    __shared__ int s_tied[kKeysPerThread * kWarps];      // ... and those equal to T
+    __shared__ int s_run_above, s_run_tied;
+    const int h = blockIdx.x, b = blockIdx.y, l = blockIdx.z, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int seq_len = p.seq_lens[b];
     const int nb = min((seq_len + p.bs - 1) / p.bs, p.max_blocks);
     const float* scores = p.scores + (((size_t)l * p.batch + b) * p.Hkv + h) * p.max_blocks;
@@ -271,78 +280,91 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(SelectParams p) 
     const int lo = p.sink_blocks, hi = nb - p.local_blocks;
     const int k = p.budget_blocks - p.sink_blocks - p.local_blocks;
 
+    // a thread's candidates lo + tid, lo + tid + 256, ...: the first kKeysPerThread keys stay in registers, any further ones
+    // are recomputed from the scores
+    uint32_t keys[kKeysPerThread];
+    const int rounds = min((hi - lo + kSelectThreads - 1) / kSelectThreads, kKeysPerThread);
+#pragma unroll
+    for (int e = 0; e < kKeysPerThread; ++e) {
+        const int i = lo + tid + e * kSelectThreads;
+        keys[e] = i < hi ? select_key(score_at(i)) : 0u;
+    }
+    const int tail0 = lo + tid + kKeysPerThread * kSelectThreads;
     if (tid == 0) {
         s_prefix = 0;
         s_remaining = k;
     }
-    // a thread's candidates lo + tid, lo + tid + 256, ...: the first kKeysPerThread keys stay in registers for
-    // all eight passes (enough for 4096 candidate blocks), any further ones are recomputed from the scores
-    constexpr int kKeysPerThread = 16;
-    uint64_t keys[kKeysPerThread];
+    uint32_t known = 0;  // bits of T found so far
+    for (int pass = 0; pass < 3; ++pass) {
+        const int shift = pass == 0 ? 21 : pass == 1 ? 10 : 0;
+        const uint32_t digit = pass == 2 ? 1023u : 2047u;
 #pragma unroll
-    for (int e = 0; e < kKeysPerThread; ++e) {
-        const int i = lo + tid + e * kSelectThreads;
-        keys[e] = i < hi ? select_key(score_at(i), i) : 0ull;  // key 0 cannot occur: the index part of a real key is > 0
-    }
-    const int tail0 = lo + tid + kKeysPerThread * kSelectThreads;
-    uint64_t known_mask = 0;
-    const int lane = tid & 31, warp = tid >> 5;
-    for (int pass = 7; pass >= 0; --pass) {
-        hist[tid] = 0;  // kSelectThreads == 256 bins
+        for (int u = 0; u < kSelectBins / kSelectThreads; ++u) hist[tid + u * kSelectThreads] = 0;
         __syncthreads();
-        const uint64_t prefix = s_prefix;
+        const uint32_t prefix = s_prefix;
         const int remaining = s_remaining;
 #pragma unroll
-        for (int e = 0; e < kKeysPerThread; ++e) {
-            const uint64_t key = keys[e];
-            if (key != 0ull && (key & known_mask) == prefix) atomicAdd(&hist[(unsigned)(key >> (8 * pass)) & 255u], 1u);
-        }
+        for (int e = 0; e < kKeysPerThread; ++e)
+            if (lo + tid + e * kSelectThreads < hi && (keys[e] & known) == prefix) atomicAdd(&hist[(keys[e] >> shift) & digit], 1u);
         for (int i = tail0; i < hi; i += kSelectThreads) {
-            const uint64_t key = select_key(score_at(i), i);
-            if ((key & known_mask) == prefix) atomicAdd(&hist[(unsigned)(key >> (8 * pass)) & 255u], 1u);
+            const uint32_t key = select_key(score_at(i));
+            if ((key & known) == prefix) atomicAdd(&hist[(key >> shift) & digit], 1u);
         }
         __syncthreads();
-        // thread <-> bin: the digit of the k-th largest key is the bin whose suffix count (this bin and all higher
-        // ones) first reaches `remaining`; found in parallel from a block-wide suffix sum
-        const unsigned c = hist[tid];
-        unsigned v = c;
+        // thread <-> eight bins: the digit of T is the bin whose suffix count (this bin and all higher ones) first reaches
+        // `remaining`; found in parallel from a block-wide suffix sum
+        unsigned c[kSelectBins / kSelectThreads], mine = 0;
+#pragma unroll
+        for (int u = 0; u < kSelectBins / kSelectThreads; ++u) {
+            c[u] = hist[tid * (kSelectBins / kSelectThreads) + u];
+            mine += c[u];
+        }
+        unsigned v = mine;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const unsigned up = __shfl_down_sync(0xffffffffu, v, o);
             if (lane + o < 32) v += up;
         }
-        if (lane == 0) s_warp_counts[warp] = (int)v;  // count of this warp's 32 bins
+        if (lane == 0) s_warp_counts[warp] = (int)v;
         __syncthreads();
-        unsigned above = 0;
-        for (int w2 = warp + 1; w2 < kSelectThreads / 32; ++w2) above += (unsigned)s_warp_counts[w2];
-        const unsigned suffix = v + above, higher = suffix - c;
-        if (suffix >= (unsigned)remaining && higher < (unsigned)remaining) {  // true for exactly one bin
-            s_remaining = remaining - (int)higher;
-            s_prefix = prefix | ((uint64_t)tid << (8 * pass));
+        unsigned higher = v - mine;  // candidates in the bins above this thread's
+        for (int w2 = warp + 1; w2 < kWarps; ++w2) higher += (unsigned)s_warp_counts[w2];
+#pragma unroll
+        for (int u = kSelectBins / kSelectThreads - 1; u >= 0; --u) {
+            if (higher < (unsigned)remaining && higher + c[u] >= (unsigned)remaining) {  // true for exactly one bin
+                s_remaining = remaining - (int)higher;
+                s_prefix = prefix | ((uint32_t)(tid * (kSelectBins / kSelectThreads) + u) << shift);
+            }
+            higher += c[u];
         }
-        known_mask |= 0xFFull << (8 * pass);
+        known |= digit << shift;
         __syncthreads();
     }
-    const uint64_t threshold = s_prefix;  // the k-th largest key; keys are unique
+    const uint32_t T = s_prefix;       // key of the k-th best candidate
+    const int ties = s_remaining;      // candidates of that key to take
 
     for (int i = tid; i < p.sink_blocks; i += kSelectThreads) idx[i] = i;
     for (int i = tid; i < p.local_blocks; i += kSelectThreads) idx[p.sink_blocks + k + i] = hi + i;
-    // Ordered compaction of the kept candidates (ascending block index = round e, then thread).  Register part:
-    // one ballot per round, the (round, warp) counts scanned once by warp 0.
-    constexpr int kWarps = kSelectThreads / 32;
-    unsigned ballots[kKeysPerThread];
+    // Ordered compaction (ascending block index = round e, then thread).  Register part: two ballots per round, the
+    // (round, warp) counts scanned once by warps 0 and 1.
+    unsigned above[kKeysPerThread], tied[kKeysPerThread];
 #pragma unroll
     for (int e = 0; e < kKeysPerThread; ++e) {
-        const bool keep = keys[e] != 0ull && keys[e] >= threshold;
-        ballots[e] = __ballot_sync(0xffffffffu, keep);
-        if (lane == 0) s_round_counts[e * kWarps + warp] = __popc(ballots[e]);
+        const bool in = lo + tid + e * kSelectThreads < hi;
+        above[e] = __ballot_sync(0xffffffffu, in && keys[e] > T);
+        tied[e] = __ballot_sync(0xffffffffu, in && keys[e] == T);
+        if (lane == 0) {
+            s_above[e * kWarps + warp] = __popc(above[e]);
+            s_tied[e * kWarps + warp] = __popc(tied[e]);
+        }
     }
     __syncthreads();
-    if (warp == 0) {  // exclusive scan of the 128 counts: four per lane, then across lanes
+    if (warp < 2) {  // exclusive scan of 128 counts: four per lane, then across lanes
+        int* counts = warp == 0 ? s_above : s_tied;
         int c4[4], sum = 0;
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            c4[u] = s_round_counts[lane * 4 + u];
+            c4[u] = counts[lane * 4 + u];
             sum += c4[u];
         }
         int incl = sum;
@@ -354,37 +376,45 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(SelectParams p) 
         int run = incl - sum;
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            s_round_counts[lane * 4 + u] = run;
+            counts[lane * 4 + u] = run;
             run += c4[u];
         }
-        if (lane == 31) s_running = incl;  // kept so far
+        if (lane == 31) (warp == 0 ? s_run_above : s_run_tied) = incl;
     }
     __syncthreads();
+    const unsigned below_me = (1u << lane) - 1u;
+    auto place = [&](int i, bool is_above, bool is_tied, int n_above, int n_tied) {  // counts of candidates before this one
+        if (is_above) idx[p.sink_blocks + n_above + min(n_tied, ties)] = i;
+        if (is_tied && n_tied < ties) idx[p.sink_blocks + n_above + n_tied] = i;
+    };
 #pragma unroll
-    for (int e = 0; e < kKeysPerThread; ++e) {
-        if ((ballots[e] >> lane) & 1u) {
-            const int offset = s_round_counts[e * kWarps + warp] + __popc(ballots[e] & ((1u << lane) - 1u));
-            if (offset < k) idx[p.sink_blocks + offset] = lo + tid + e * kSelectThreads;
-        }
-    }
+    for (int e = 0; e < kKeysPerThread; ++e)
+        if (e < rounds)
+            place(lo + tid + e * kSelectThreads, (above[e] >> lane) & 1u, (tied[e] >> lane) & 1u,
+                  s_above[e * kWarps + warp] + __popc(above[e] & below_me), s_tied[e * kWarps + warp] + __popc(tied[e] & below_me));
     // candidates beyond the register part (more than 4096 of them): round by round
     for (int base = lo + kKeysPerThread * kSelectThreads; base < hi; base += kSelectThreads) {
         const int i = base + tid;
-        const bool keep = i < hi && select_key(score_at(i), i) >= threshold;
-        const unsigned ballot = __ballot_sync(0xffffffffu, keep);
-        __syncthreads();  // s_running of the previous round has been read by everyone
-        if (lane == 0) s_warp_counts[warp] = __popc(ballot);
-        __syncthreads();
-        int offset = s_running;
-        for (int w = 0; w < warp; ++w) offset += s_warp_counts[w];
-        offset += __popc(ballot & ((1u << lane) - 1u));
-        if (keep && offset < k) idx[p.sink_blocks + offset] = i;
-        __syncthreads();
-        if (tid == 0) {
-            int total = 0;
-            for (int w = 0; w < kWarps; ++w) total += s_warp_counts[w];
-            s_running += total;
+        const uint32_t key = i < hi ? select_key(score_at(i)) : 0u;
+        const unsigned ab = __ballot_sync(0xffffffffu, i < hi && key > T), ti = __ballot_sync(0xffffffffu, i < hi && key == T);
+        __syncthreads();  // the counts of the previous round have been read by everyone
+        if (lane == 0) {
+            s_above[warp] = __popc(ab);
+            s_tied[warp] = __popc(ti);
         }
+        __syncthreads();
+        int n_above = s_run_above, n_tied = s_run_tied;
+        for (int w = 0; w < warp; ++w) {
+            n_above += s_above[w];
+            n_tied += s_tied[w];
+        }
+        place(i, (ab >> lane) & 1u, (ti >> lane) & 1u, n_above + __popc(ab & below_me), n_tied + __popc(ti & below_me));
+        __syncthreads();
+        if (tid == 0)
+            for (int w = 0; w < kWarps; ++w) {
+                s_run_above += s_above[w];
+                s_run_tied += s_tied[w];
+            }
     }
 }
 
@@ -449,51 +479,118 @@ __global__ void __launch_bounds__(128) gather_kernel(GatherParams p) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// Commit: grid = (A_max, Hkv, layers x seqs); a CTA appends one accepted token's K and V row.
+// Commit: grid = (blocks touched, Hkv, layers x seqs); a CTA appends the accepted tokens' K and V rows that fall into one
+// block (a warp per row) and recomputes the block's summary, the appended tokens taken from the step's tensors.  The CTA
+// that finishes last advances the lengths (an arrival counter behind the status word, left at zero): every CTA has read
+// them by then.  One launch where rows, summaries and lengths took three: 4-5 us
+// less host time per call, and on the device 12.5 us against 15.2 for the 46 rows of a refresh (36 layers), 7.5 against 6.9 for
+// four rows (the arrival).
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(32) commit_rows_kernel(CommitParams p) {
+constexpr int kCommitWarps = 4;
+
+template <typename T>
+__global__ void __launch_bounds__(32 * kCommitWarps) commit_kernel(CommitParams p) {
     pdl_begin(p.pdl);
-    const int a = blockIdx.x, h = blockIdx.y, lb = blockIdx.z;
+    __shared__ int s_last;
+    const int h = blockIdx.y, lb = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int b = lb % p.batch, l = lb / p.batch;
     const int n = min(max(p.n_accepted[b], 0), p.A_max);
-    if (a >= n) return;
     const int seq_len = p.seq_lens[b];
-    if ((size_t)seq_len + n > (size_t)p.max_blocks * p.bs) {
-        if (threadIdx.x == 0 && a == 0 && h == 0) record_fault(p.workspace, SPECPV_ERR_CAPACITY, b, seq_len, n, l);
-        return;
+    const bool fits = (size_t)seq_len + n <= (size_t)p.max_blocks * p.bs;
+    const int i = max(seq_len, 0) / p.bs + blockIdx.x;  // logical block
+    if (!fits) {
+        if (threadIdx.x == 0 && blockIdx.x == 0 && h == 0 && n > 0) record_fault(p.workspace, SPECPV_ERR_CAPACITY, b, seq_len, n, l);
+    } else {
+        const int t0 = max(seq_len, i * p.bs), t1 = min(seq_len + n, (i + 1) * p.bs);  // tokens appended to this block
+        const bool summarise = p.kmax && (size_t)i * p.bs < (size_t)(seq_len + n) && i < p.max_blocks;
+        int page = -1;
+        if (t0 < t1 || summarise) {
+            page = p.block_table[(size_t)b * p.max_blocks + i];
+            if (page < 0 || page >= p.n_pages) {
+                if (threadIdx.x == 0) record_fault(p.workspace, SPECPV_ERR_BAD_BLOCK_TABLE, b, i, page, l);
+                page = -1;
+            }
+        }
+        const int chunks = p.d * (int)sizeof(T) / 16;  // 16-byte chunks per row: 8, 16 or 32
+        const size_t page0 = (((size_t)(p.layer0 + l) * p.n_pages + max(page, 0)) * p.Hkv + h) * p.bs;
+        const uint4* k_new = reinterpret_cast<const uint4*>(p.k_new);
+        const uint4* v_new = reinterpret_cast<const uint4*>(p.v_new);
+        uint4* k_pool = reinterpret_cast<uint4*>(p.k_pool);
+        uint4* v_pool = reinterpret_cast<uint4*>(p.v_pool);
+        const int tok_lanes = 32 / chunks, chunk = lane % chunks, tl = lane / chunks;  // rows side by side in a warp
+        // row of the step's tensors that token t takes, -1 if there is none
+        auto source_row = [&](int t) {
+            const int row = p.accepted[(size_t)b * p.A_max + t - seq_len];
+            return row >= 0 && row < p.M_max ? row : -1;
+        };
+        if (page >= 0) {
+            constexpr int kAhead = 4;  // rows in flight per lane
+            const int step = kCommitWarps * tok_lanes;
+            for (int t = t0 + warp * tok_lanes + tl; t < t1; t += kAhead * step) {
+                uint4 kb[kAhead], vb[kAhead];
+                int row[kAhead];
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u) {
+                    row[u] = t + u * step < t1 ? source_row(t + u * step) : -1;
+                    if (row[u] >= 0) {
+                        const size_t src = (((size_t)lb * p.M_max + row[u]) * p.Hkv + h) * chunks + chunk;
+                        kb[u] = k_new[src];
+                        vb[u] = v_new[src];
+                    } else if (t + u * step < t1 && chunk == 0) {
+                        const int a = t + u * step - seq_len;
+                        record_fault(p.workspace, SPECPV_ERR_INVALID_ARG, b, a, p.accepted[(size_t)b * p.A_max + a], l);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u)
+                    if (row[u] >= 0) {
+                        const size_t dst = (page0 + (t + u * step) % p.bs) * chunks + chunk;
+                        k_pool[dst] = kb[u];
+                        v_pool[dst] = vb[u];
+                    }
+            }
+        }
+        if (summarise && page >= 0 && warp == 0) {
+            // as summaries_kernel, with the tokens of this commit read where they come from
+            const int n_valid = min(p.bs, seq_len + n - i * p.bs);
+            SummaryAcc<T> acc;
+            for (int u0 = 0; u0 < n_valid; u0 += kSumLoads * tok_lanes) {
+                uint4 buf[kSumLoads];
+#pragma unroll
+                for (int u = 0; u < kSumLoads; ++u) {
+                    const int in = min(u0 + u * tok_lanes + tl, n_valid - 1), t = i * p.bs + in;
+                    const uint4* src = k_pool + (page0 + in) * chunks;
+                    if (t >= seq_len) {
+                        const int row = source_row(t);
+                        if (row >= 0) src = k_new + (((size_t)lb * p.M_max + row) * p.Hkv + h) * chunks;
+                    }
+                    buf[u] = src[chunk];
+                }
+#pragma unroll
+                for (int u = 0; u < kSumLoads; ++u) acc.take(buf[u]);
+            }
+            acc.combine(chunks);
+            if (tl == 0)
+                acc.store(p.kmax, p.kmin, p.aligned,
+                          ((((size_t)(p.layer0 + l) * p.batch + b) * p.Hkv + h) * p.max_blocks + i) * chunks + chunk);
+        }
     }
-    const int row = p.accepted[(size_t)b * p.A_max + a];
-    if (row < 0 || row >= p.M_max) {
-        if (threadIdx.x == 0) record_fault(p.workspace, SPECPV_ERR_INVALID_ARG, b, a, row, l);
-        return;
+    if (!p.advance) return;
+    __syncthreads();  // the whole CTA has read the lengths
+    if (threadIdx.x == 0) {
+        int32_t* arrived = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(p.workspace) + kCommitCounterOffset);
+        __threadfence();
+        const int total = (int)(gridDim.x * gridDim.y * gridDim.z);
+        s_last = atomicAdd(arrived, 1) == total - 1;
+        if (s_last) *arrived = 0;
     }
-    const int t = seq_len + a;
-    const int page = p.block_table[(size_t)b * p.max_blocks + t / p.bs];
-    if (page < 0 || page >= p.n_pages) {
-        if (threadIdx.x == 0) record_fault(p.workspace, SPECPV_ERR_BAD_BLOCK_TABLE, b, t / p.bs, page, l);
-        return;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    for (int bb = threadIdx.x; bb < p.batch; bb += 32 * kCommitWarps) {
+        const int nn = min(max(p.n_accepted[bb], 0), p.A_max);
+        if ((size_t)p.seq_lens[bb] + nn <= (size_t)p.max_blocks * p.bs) p.seq_lens[bb] += nn;
     }
-    const size_t row_bytes = (size_t)p.d * p.es;
-    const size_t src = (((size_t)lb * p.M_max + row) * p.Hkv + h) * row_bytes;
-    const size_t dst = ((((size_t)(p.layer0 + l) * p.n_pages + page) * p.Hkv + h) * p.bs + t % p.bs) * row_bytes;
-    const uint4* ks = reinterpret_cast<const uint4*>(reinterpret_cast<const char*>(p.k_new) + src);
-    const uint4* vs = reinterpret_cast<const uint4*>(reinterpret_cast<const char*>(p.v_new) + src);
-    uint4* kd = reinterpret_cast<uint4*>(reinterpret_cast<char*>(p.k_pool) + dst);
-    uint4* vd = reinterpret_cast<uint4*>(reinterpret_cast<char*>(p.v_pool) + dst);
-    for (int i = threadIdx.x; i < (int)(row_bytes / 16); i += 32) {
-        kd[i] = ks[i];
-        vd[i] = vs[i];
-    }
-}
-
-__global__ void commit_lens_kernel(int32_t* seq_lens, const int32_t* n_accepted, int batch, int A_max,
-                                   int capacity_tokens) {
-    pdl_trigger();
-    pdl_wait();
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= batch) return;
-    const int n = min(max(n_accepted[b], 0), A_max);
-    if ((size_t)seq_lens[b] + n <= (size_t)capacity_tokens) seq_lens[b] += n;
 }
 
 }  // namespace
@@ -552,20 +649,11 @@ specpv_status launch_gather(const GatherParams& p, int n_layers, cudaStream_t st
     return SPECPV_OK;
 }
 
-specpv_status launch_commit(const CommitParams& p, int n_layers, int32_t* seq_lens, cudaStream_t stream) {
-    if (p.A_max > 0 && n_layers > 0) {
-        dim3 grid(p.A_max, p.Hkv, n_layers * p.batch);
-        SPECPV_LAUNCH(commit_rows_kernel, grid, 32, 0, stream, p);
-    }
-    (void)seq_lens;
-    return SPECPV_OK;
-}
-
-specpv_status launch_commit_lens(int32_t* seq_lens, const int32_t* n_accepted, int batch, int A_max,
-                                 int capacity_tokens, cudaStream_t stream) {
-    if (launch_pdl(commit_lens_kernel, (batch + 63) / 64, 64, 0, stream, seq_lens, n_accepted, batch, A_max, capacity_tokens) != cudaSuccess)
-        return SPECPV_ERR_CUDA;
-    count_launch();
+specpv_status launch_commit(const CommitParams& params, int n_layers, int dtype, cudaStream_t stream) {
+    CommitParams p = params;
+    p.aligned = aligned16(p.kmax) && aligned16(p.kmin);
+    dim3 grid((p.A_max + p.bs - 1) / p.bs + 1, p.Hkv, n_layers * p.batch);
+    SPECPV_LAUNCH(dtype == SPECPV_DTYPE_F32 ? commit_kernel<float> : commit_kernel<__nv_bfloat16>, grid, 32 * kCommitWarps, 0, stream, p);
     return SPECPV_OK;
 }
 

@@ -9,11 +9,10 @@ struct SummaryParams {
     const int32_t* block_table;
     const int32_t* seq_lens;
     const int32_t* tok_begin;   // nullable
-    const int32_t* n_appended;  // nullable: tokens a commit in flight adds to seq_lens
     void* kmax;
     void* kmin;
     void* workspace;
-    int layer0, batch, Hkv, bs, d, max_blocks, n_pages, A_max;
+    int layer0, batch, Hkv, bs, d, max_blocks, n_pages;
     int aligned;  // set by the launcher: kmax and kmin take 16-byte stores
     int pdl;      // set by launch_pdl_if
 };
@@ -66,10 +65,14 @@ struct CommitParams {
     void* k_pool;
     void* v_pool;
     const int32_t* block_table;
-    const int32_t* seq_lens;
+    int32_t* seq_lens;
+    void* kmax;  // nullable, with kmin: summaries of the touched blocks are recomputed
+    void* kmin;
     void* workspace;
-    int layer0, batch, M_max, A_max, Hkv, bs, d, es, max_blocks, n_pages;
-    int pdl;  // set by launch_pdl_if
+    int layer0, batch, M_max, A_max, Hkv, bs, d, max_blocks, n_pages;
+    int advance;  // this call holds the model's last layer: the lengths advance
+    int aligned;  // set by the launcher: kmax and kmin take 16-byte stores
+    int pdl;      // set by launch_pdl_if
 };
 
 specpv_status launch_summaries(const SummaryParams& p, int n_layers, int blocks_touched, int dtype, cudaStream_t stream);
@@ -79,8 +82,6 @@ specpv_status launch_scores_tc(const ScoreParams& p, int n_layers_call, int n_la
                                cudaStream_t stream);
 specpv_status launch_select(const SelectParams& p, int n_layers, cudaStream_t stream);
 specpv_status launch_gather(const GatherParams& p, int n_layers, cudaStream_t stream);
-specpv_status launch_commit(const CommitParams& p, int n_layers, int32_t* seq_lens, cudaStream_t stream);
-specpv_status launch_commit_lens(int32_t* seq_lens, const int32_t* n_accepted, int batch, int A_max,
-                                 int capacity_tokens, cudaStream_t stream);
+specpv_status launch_commit(const CommitParams& p, int n_layers, int dtype, cudaStream_t stream);
 
 }  // namespace specpv

@@ -219,6 +219,44 @@ def test_summaries_of_ragged_blocks_are_exact(dtype, Hkv, d, bs, shift):
         assert torch.all(kmax[:, b, :, nb:].float() == 5.0) and torch.all(kmin[:, b, :, nb:].float() == 5.0)
 
 
+@pytest.mark.parametrize("dtype,d,bs,n", [("bf16", 128, 64, 46), ("bf16", 64, 16, 46), ("fp32", 128, 32, 1), ("fp32", 64, 64, 0),
+                                          ("bf16", 128, 16, 16)])
+def test_commit_across_blocks_and_ragged_batches(dtype, d, bs, n):
+    """A commit of up to 46 rows (a refresh's chain and path) that starts inside a block, at its end and at its first token,
+    over several sequences: rows, summaries of every touched block and lengths against the oracle, twice in a row."""
+    w = wl.make_workload("llama_32k", device="cuda", n_layers=2, spare_tokens=256, Hq=6, Hkv=3, d=d, bs=bs, dtype=dtype, M=48,
+                         ctx=[bs * 5 + 3, bs * 4, bs * 6 - 1], shuffle=True)
+    c = w.cfg
+    L, Hkv, M, batch = c["n_layers"], c["Hkv"], c["M"], w.batch
+    cfg = util.config_for(w)
+    full = util.full_cache(w)
+    full.max_seq_len = int(max(c["ctx"])) + 256
+    ws = torch.zeros(4096, dtype=torch.uint8, device="cuda")
+    kmax = torch.zeros((L, batch, Hkv, w.max_blocks, d), dtype=wl.torch_dtype(dtype), device="cuda")
+    kmin = torch.zeros_like(kmax)
+    B.specpv_update_block_summaries(cfg, 0, L, full, None, w.max_blocks, kmax, kmin, ws)
+    kp, vp = wl.to_numpy(w.k_pool).copy(), wl.to_numpy(w.v_pool).copy()
+    lens = [int(x) for x in c["ctx"]]
+    table = w.block_table.cpu().numpy()
+    knn, vnn = wl.to_numpy(w.k_new), wl.to_numpy(w.v_new)
+    rng = np.random.default_rng(n + bs)
+    for _ in range(2):
+        acc = rng.integers(0, M, size=(batch, 46)).astype(np.int32)
+        counts = [n, max(n - 3, 0), n]
+        B.specpv_commit_accepted(cfg, 0, L, w.k_new, w.v_new, M, torch.from_numpy(acc).cuda(),
+                                 torch.tensor(counts, dtype=torch.int32, device="cuda"), 46, full, kmax, kmin, ws)
+        util.sync_status(ws)
+        for b in range(batch):
+            for l in range(L):
+                new_len = oracle.commit(knn[l, b], vnn[l, b], acc[b, :counts[b]], kp[l], vp[l], table[b], lens[b])
+                okmax, okmin = oracle.block_summaries(kp[l], table[b], new_len)
+                nb = (new_len + bs - 1) // bs
+                assert np.array_equal(util.widen_t(kmax[l, b])[:, :nb], okmax) and np.array_equal(util.widen_t(kmin[l, b])[:, :nb], okmin)
+            lens[b] += counts[b]
+            assert int(w.seq_lens[b]) == lens[b]
+        assert np.array_equal(wl.to_numpy(w.k_pool), kp) and np.array_equal(wl.to_numpy(w.v_pool), vp)
+
+
 def test_commit_in_layer_groups_matches_the_oracle():
     """A step's commit issued in two layer groups, in ascending order: every group writes its rows at the lengths as
     they stand and the lengths advance with the group that holds the model's last layer."""
