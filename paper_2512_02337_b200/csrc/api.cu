@@ -431,34 +431,40 @@ SPECPV_EXPORT specpv_status specpv_verify_host(const specpv_config* cfg, int mod
 
     // The layers go through in groups: while one group's attention runs on `stream`, the next group's inputs arrive
     // on a copy-in stream and the previous group's outputs leave on a copy-out stream (the host link carries both
-    // directions at once).  The two copy streams are created once per device and kept.
+    // directions at once).  The two copy streams are created once per device and kept.  A copy costs some 5 us beside its
+    // bytes (23.6 MB in and 16 MB out: 471 us as one copy each way, 762 as 24), so the groups are few.  The last one is small, its
+    // attention and copy out overlap nothing; where the attention outlasts the copies the first ones are small too, each
+    // copied in while the one before it is worked on.  32 layers, 60 rows: 32768 tokens 1290 -> 1165 us, a 4096-token partial
+    // cache 840 -> 735, against eight equal groups.
     HostCopyStreams* cs = host_copy_streams();
     if (!cs) return SPECPV_ERR_CUDA;
-    constexpr int kMaxGroups = 8;
-    const int n_groups = n_layers < kMaxGroups ? n_layers : kMaxGroups;
-    const int per_group = (n_layers + n_groups - 1) / n_groups;
-    cudaEvent_t begin = nullptr, in_done[kMaxGroups] = {}, run_done[kMaxGroups] = {}, out_done = nullptr;
-    bool ok = cudaEventCreateWithFlags(&begin, cudaEventDisableTiming) == cudaSuccess &&
-              cudaEventCreateWithFlags(&out_done, cudaEventDisableTiming) == cudaSuccess;
-    for (int i = 0; i < n_groups && ok; ++i)
-        ok = cudaEventCreateWithFlags(&in_done[i], cudaEventDisableTiming) == cudaSuccess &&
-             cudaEventCreateWithFlags(&run_done[i], cudaEventDisableTiming) == cudaSuccess;
+    constexpr int kMaxGroups = 4;
+    const double copy_us = (double)n_layers * (q_l + 2.0 * kv_l) / 50.0e3;  // 50 GB/s
+    const double run_us = (double)n_layers * kv->batch * kv->max_seq_len * g.Hkv * 2.0 * g.d * g.es / 4.0e6;  // 4 TB/s
+    static const int kShare[2][kMaxGroups] = {{4, 3, 2, 1}, {1, 2, 5, 2}};  // tenths of the layers
+    const int* share = kShare[run_us > copy_us];
+    int first[kMaxGroups + 1] = {0}, tenths = 0, n_groups = 0;
+    for (int i = 0; i < kMaxGroups; ++i) {
+        tenths += share[i];
+        const int end = i + 1 == kMaxGroups ? n_layers : (n_layers * tenths + 5) / 10;
+        if (end > first[n_groups]) first[++n_groups] = end;
+    }
+    // one event serves every hand-over: a wait refers to the record before it
+    cudaEvent_t event = nullptr;
+    bool ok = cudaEventCreateWithFlags(&event, cudaEventDisableTiming) == cudaSuccess;
     // the staging area may still be in use by earlier work on `stream`
-    ok = ok && cudaEventRecord(begin, s) == cudaSuccess && cudaStreamWaitEvent(cs->in, begin, 0) == cudaSuccess &&
-         cudaStreamWaitEvent(cs->out, begin, 0) == cudaSuccess;
+    ok = ok && cudaEventRecord(event, s) == cudaSuccess && cudaStreamWaitEvent(cs->in, event, 0) == cudaSuccess &&
+         cudaStreamWaitEvent(cs->out, event, 0) == cudaSuccess;
     ok = ok && cudaMemcpyAsync(stage + sp.mask, tree_mask_host, mask_bytes, cudaMemcpyHostToDevice, cs->in) == cudaSuccess;
-    int n_used = 0;
     for (int i = 0; i < n_groups && ok && st == SPECPV_OK; ++i) {
-        const int l0 = i * per_group, nl = n_layers - l0 < per_group ? n_layers - l0 : per_group;
-        if (nl <= 0) break;
-        n_used = i + 1;
+        const int l0 = first[i], nl = first[i + 1] - l0;
         ok = cudaMemcpyAsync(stage + sp.q + l0 * q_l, static_cast<const char*>(q_host) + l0 * q_l, nl * q_l,
                              cudaMemcpyHostToDevice, cs->in) == cudaSuccess &&
              cudaMemcpyAsync(stage + sp.k_new + l0 * kv_l, static_cast<const char*>(k_new_host) + l0 * kv_l, nl * kv_l,
                              cudaMemcpyHostToDevice, cs->in) == cudaSuccess &&
              cudaMemcpyAsync(stage + sp.v_new + l0 * kv_l, static_cast<const char*>(v_new_host) + l0 * kv_l, nl * kv_l,
                              cudaMemcpyHostToDevice, cs->in) == cudaSuccess &&
-             cudaEventRecord(in_done[i], cs->in) == cudaSuccess && cudaStreamWaitEvent(s, in_done[i], 0) == cudaSuccess;
+             cudaEventRecord(event, cs->in) == cudaSuccess && cudaStreamWaitEvent(s, event, 0) == cudaSuccess;
         if (!ok) break;
         st = verify_common(cfg, layer0 + l0, nl, stage + sp.q + l0 * q_l, stage + sp.k_new + l0 * kv_l,
                            stage + sp.v_new + l0 * kv_l, reinterpret_cast<const uint64_t*>(stage + sp.mask), nullptr, M_max, kv,
@@ -466,7 +472,7 @@ SPECPV_EXPORT specpv_status specpv_verify_host(const specpv_config* cfg, int mod
                            lse_host ? reinterpret_cast<float*>(stage + sp.lse + l0 * lse_l) : nullptr, workspace,
                            w.partial_off + w.partial_bytes, stream, mode == SPECPV_MODE_PARTIAL);
         if (st != SPECPV_OK) break;
-        ok = cudaEventRecord(run_done[i], s) == cudaSuccess && cudaStreamWaitEvent(cs->out, run_done[i], 0) == cudaSuccess &&
+        ok = cudaEventRecord(event, s) == cudaSuccess && cudaStreamWaitEvent(cs->out, event, 0) == cudaSuccess &&
              cudaMemcpyAsync(static_cast<char*>(out_host) + l0 * out_l, stage + sp.out + l0 * out_l, nl * out_l,
                              cudaMemcpyDeviceToHost, cs->out) == cudaSuccess;
         if (ok && lse_host)
@@ -474,16 +480,10 @@ SPECPV_EXPORT specpv_status specpv_verify_host(const specpv_config* cfg, int mod
                                  cudaMemcpyDeviceToHost, cs->out) == cudaSuccess;
     }
     // everything is joined back onto `stream` before the call returns (also on the error paths: no copy may outlive it)
-    const bool joined = cudaEventRecord(out_done, cs->out) == cudaSuccess && cudaStreamWaitEvent(s, out_done, 0) == cudaSuccess;
+    const bool joined = event && cudaEventRecord(event, cs->out) == cudaSuccess && cudaStreamWaitEvent(s, event, 0) == cudaSuccess;
     const bool in_idle = cudaStreamSynchronize(cs->in) == cudaSuccess;
     const bool synced = cudaStreamSynchronize(s) == cudaSuccess && (joined || cudaStreamSynchronize(cs->out) == cudaSuccess);
-    (void)n_used;
-    if (begin) cudaEventDestroy(begin);
-    if (out_done) cudaEventDestroy(out_done);
-    for (int i = 0; i < kMaxGroups; ++i) {
-        if (in_done[i]) cudaEventDestroy(in_done[i]);
-        if (run_done[i]) cudaEventDestroy(run_done[i]);
-    }
+    if (event) cudaEventDestroy(event);
     if (st != SPECPV_OK) return st;
     return ok && in_idle && synced ? SPECPV_OK : SPECPV_ERR_CUDA;
 }
