@@ -1,4 +1,5 @@
-"""Thin ctypes binding of libspecpv.so: the same names as include/specpv.h, argument marshalling only.
+"""Thin binding of libspecpv.so: the same names as include/specpv.h, argument marshalling only (in native code for the
+calls of a step, `csrc/pycalls.c`; through ctypes for the others).
 
 Every step of the verification path runs in the library's CUDA kernels; this module converts
 torch tensors to raw pointers and raises :class:`SpecPVError` on a non-zero status.  There is no
@@ -7,6 +8,8 @@ fallback: if the shared library is missing, importing the symbols fails loudly.
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 from ctypes import POINTER, byref, c_double, c_float, c_int, c_int32, c_size_t, c_void_p
 from dataclasses import dataclass
 from pathlib import Path
@@ -15,6 +18,7 @@ import numpy as np
 import torch
 
 LIB_PATH = Path(__file__).resolve().parent / "lib" / "libspecpv.so"
+PYCALLS_PATH = LIB_PATH.with_name("pycalls.so")
 
 STATUS_NAMES = ["OK", "INVALID_ARG", "SHAPE", "BUDGET", "CAPACITY", "BAD_TREE", "BAD_BLOCK_TABLE",
                 "UNSUPPORTED", "CUDA", "TIMEOUT"]
@@ -105,6 +109,24 @@ def _ptr(t) -> int | None:
     raise TypeError(type(t))
 
 
+_pycalls = None
+
+
+def _native():
+    """The native argument conversion (raises like lib() if it has not been built)."""
+    global _pycalls
+    if _pycalls is None:
+        lib()
+        if not PYCALLS_PATH.exists():
+            raise ImportError(f"{PYCALLS_PATH} is missing: run `python -m paper_2512_02337_b200.build`")
+        loader = importlib.machinery.ExtensionFileLoader("pycalls", str(PYCALLS_PATH))
+        module = importlib.util.module_from_spec(importlib.util.spec_from_loader("pycalls", loader))
+        loader.exec_module(module)
+        module.init(torch.Tensor, _ptr, _stream, _get_device, _raw_stream if _get_device is not None else None)
+        _pycalls = module
+    return _pycalls
+
+
 # the current stream's handle without building a torch.cuda.Stream (3 us of a call's host time)
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 _get_device = getattr(torch._C, "_cuda_getDevice", None)
@@ -191,43 +213,30 @@ def specpv_select_mode(ctx_len, budget_tokens, n_partially_verified, n_candidate
 
 def specpv_update_block_summaries(cfg, layer0, n_layers, kv: Cache, tok_begin, max_blocks_touched, kmax, kmin,
                                   workspace, stream=None):
-    d = kv.desc()
-    _check(lib().specpv_update_block_summaries(byref(cfg), layer0, n_layers, byref(d), _ptr(tok_begin),
-                                               max_blocks_touched, _ptr(kmax), _ptr(kmin), _ptr(workspace),
-                                               workspace.numel(), _stream(stream)),
-           "specpv_update_block_summaries")
+    _check(_native().specpv_update_block_summaries(cfg, layer0, n_layers, kv, tok_begin, max_blocks_touched, kmax,
+                                                   kmin, workspace, stream), "specpv_update_block_summaries")
 
 
 def specpv_score_blocks(cfg, layer0, n_layers, q, q_lens, M_max, last_query, kmax, kmin, kv: Cache, scores,
                         workspace, stream=None):
-    d = kv.desc()
-    _check(lib().specpv_score_blocks(byref(cfg), layer0, n_layers, _ptr(q), _ptr(q_lens), M_max,
-                                     _ptr(last_query), _ptr(kmax), _ptr(kmin), byref(d), _ptr(scores),
-                                     _ptr(workspace), workspace.numel(), _stream(stream)),
-           "specpv_score_blocks")
+    _check(_native().specpv_score_blocks(cfg, layer0, n_layers, q, q_lens, M_max, last_query, kmax, kmin, kv, scores,
+                                         workspace, stream), "specpv_score_blocks")
 
 
 def specpv_select_partial_kv(cfg, n_layers, scores, seq_lens, batch, max_blocks, idx, count, workspace, stream=None):
-    _check(lib().specpv_select_partial_kv(byref(cfg), n_layers, _ptr(scores), _ptr(seq_lens), batch,
-                                          max_blocks, _ptr(idx), _ptr(count), _ptr(workspace),
-                                          workspace.numel(), _stream(stream)),
-           "specpv_select_partial_kv")
+    _check(_native().specpv_select_partial_kv(cfg, n_layers, scores, seq_lens, batch, max_blocks, idx, count,
+                                              workspace, stream), "specpv_select_partial_kv")
 
 
 def specpv_refresh_partial(cfg, full: Cache, idx, count, partial: Cache, partial_lens, workspace, stream=None):
-    fd, pd = full.desc(), partial.desc()
-    _check(lib().specpv_refresh_partial(byref(cfg), byref(fd), _ptr(idx), _ptr(count), byref(pd),
-                                        _ptr(partial_lens), _ptr(workspace), workspace.numel(),
-                                        _stream(stream)),
+    _check(_native().specpv_refresh_partial(cfg, full, idx, count, partial, partial_lens, workspace, stream),
            "specpv_refresh_partial")
 
 
 def _verify(fn_name, cfg, layer0, n_layers, q, k_new, v_new, tree_mask, q_lens, M_max, kv: Cache, out, lse,
             workspace, stream):
-    d = kv.desc()
-    _check(getattr(lib(), fn_name)(byref(cfg), layer0, n_layers, _ptr(q), _ptr(k_new), _ptr(v_new),
-                                   _ptr(tree_mask), _ptr(q_lens), M_max, byref(d), _ptr(out), _ptr(lse),
-                                   _ptr(workspace), workspace.numel(), _stream(stream)), fn_name)
+    _check(getattr(_native(), fn_name)(cfg, layer0, n_layers, q, k_new, v_new, tree_mask, q_lens, M_max, kv, out, lse,
+                                       workspace, stream), fn_name)
 
 
 def specpv_verify_partial(cfg, layer0, n_layers, q, k_new, v_new, tree_mask, q_lens, M_max, partial: Cache, out,
@@ -245,10 +254,8 @@ def specpv_verify_partial_static(cfg, layer0, n_layers, q, k_new, v_new, tree_ma
     """specpv_verify_partial without a workspace: the scratch is a fixed array inside the library, so the
     call allocates nothing (for callers whose device memory is all spoken for).  ``device_status`` is an
     optional int32 device tensor of 5 words that receives the call's device-side status."""
-    d = partial.desc()
-    _check(lib().specpv_verify_partial_static(byref(cfg), layer0, n_layers, _ptr(q), _ptr(k_new), _ptr(v_new),
-                                              _ptr(tree_mask), _ptr(q_lens), M_max, byref(d), _ptr(out),
-                                              _ptr(lse), _ptr(device_status), _stream(stream)),
+    _check(_native().specpv_verify_partial_static(cfg, layer0, n_layers, q, k_new, v_new, tree_mask, q_lens, M_max,
+                                                  partial, out, lse, device_status, stream),
            "specpv_verify_partial_static")
 
 
@@ -268,20 +275,14 @@ def specpv_verify_full(cfg, layer0, n_layers, q, k_new, v_new, tree_mask, q_lens
 
 def specpv_verify_host(cfg, mode, layer0, n_layers, q_host, k_new_host, v_new_host, tree_mask_host, M_max,
                        kv: Cache, out_host, lse_host, workspace, stream=None):
-    d = kv.desc()
-    _check(lib().specpv_verify_host(byref(cfg), mode, layer0, n_layers, _ptr(q_host), _ptr(k_new_host),
-                                    _ptr(v_new_host), _ptr(tree_mask_host), M_max, byref(d), _ptr(out_host),
-                                    _ptr(lse_host), _ptr(workspace), workspace.numel(), _stream(stream)),
-           "specpv_verify_host")
+    _check(_native().specpv_verify_host(cfg, mode, layer0, n_layers, q_host, k_new_host, v_new_host, tree_mask_host,
+                                        M_max, kv, out_host, lse_host, workspace, stream), "specpv_verify_host")
 
 
 def specpv_commit_accepted(cfg, layer0, n_layers, k_new, v_new, M_max, accepted, n_accepted, A_max, dst: Cache,
                            kmax, kmin, workspace, stream=None):
-    d = dst.desc()
-    _check(lib().specpv_commit_accepted(byref(cfg), layer0, n_layers, _ptr(k_new), _ptr(v_new), M_max,
-                                        _ptr(accepted), _ptr(n_accepted), A_max, byref(d), _ptr(kmax),
-                                        _ptr(kmin), _ptr(workspace), workspace.numel(), _stream(stream)),
-           "specpv_commit_accepted")
+    _check(_native().specpv_commit_accepted(cfg, layer0, n_layers, k_new, v_new, M_max, accepted, n_accepted, A_max,
+                                            dst, kmax, kmin, workspace, stream), "specpv_commit_accepted")
 
 
 # ---- the linear maps either side of the attention ---------------------------------------------------------------
@@ -293,16 +294,13 @@ def specpv_rope_table(cfg, tree_mask, q_lens, base_pos, batch, M_max, rope_theta
 
 def specpv_qkv_rope(cfg, layer0, n_layers, x, hidden, w_qkv, cos_sin, batch, M_max, q, k_new, v_new, workspace,
                     stream=None):
-    _check(lib().specpv_qkv_rope(byref(cfg), layer0, n_layers, _ptr(x), hidden, _ptr(w_qkv), _ptr(cos_sin),
-                                 batch, M_max, _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(workspace),
-                                 workspace.numel(), _stream(stream)),
-           "specpv_qkv_rope")
+    _check(_native().specpv_qkv_rope(cfg, layer0, n_layers, x, hidden, w_qkv, cos_sin, batch, M_max, q, k_new, v_new,
+                                     workspace, stream), "specpv_qkv_rope")
 
 
 def specpv_o_proj(cfg, layer0, n_layers, attn, w_o, hidden, residual, batch, M_max, y, workspace, stream=None):
-    _check(lib().specpv_o_proj(byref(cfg), layer0, n_layers, _ptr(attn), _ptr(w_o), hidden, _ptr(residual),
-                               batch, M_max, _ptr(y), _ptr(workspace), workspace.numel(), _stream(stream)),
-           "specpv_o_proj")
+    _check(_native().specpv_o_proj(cfg, layer0, n_layers, attn, w_o, hidden, residual, batch, M_max, y, workspace,
+                                   stream), "specpv_o_proj")
 
 
 # ---- full KV cache in host memory -------------------------------------------------------------------------------

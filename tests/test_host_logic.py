@@ -7,6 +7,7 @@ from pathlib import Path
 
 import numpy as np
 import pytest
+import torch
 
 import oracle
 from paper_2512_02337_b200 import binding as B
@@ -168,3 +169,21 @@ def test_replica_timings_are_reduced_with_max_over_ranks_gloo():
         p.join(timeout=60)
         assert p.exitcode == 0
     assert results[0] == results[1] == [11.0, 5.0]
+
+
+@pytest.mark.parametrize("bad,error", [("strided", AssertionError), ("list", TypeError), ("word", TypeError),
+                                       ("config", TypeError), ("cache", AttributeError), (None, B.SpecPVError)])
+def test_native_argument_conversion(bad, error):
+    """Tensors, NumPy arrays and None are taken as pointers, everything else is refused before the library is called; the
+    library then refuses the null query tensor (so no CUDA call is made)."""
+    cfg = B.make_config(n_layers=2, n_q_heads=8, n_kv_heads=2, head_dim=64, block_tokens=64, dtype="fp32", sink_blocks=1,
+                        local_blocks=2, budget_blocks=8, buffer_tokens=64)
+    t = torch.zeros(2, 4, 2, 64, 64)
+    cache = B.Cache(t, t, torch.zeros(1, 4, dtype=torch.int32), torch.zeros(1, dtype=torch.int32), 256)
+    args = dict(cfg=cfg, layer0=0, n_layers=1, q=None, k_new=np.zeros(64, np.float32), v_new=t, tree_mask=t, q_lens=None,
+                M_max=16, full=cache, out=t, lse=None, workspace=t, stream=0)
+    args.update({"strided": dict(v_new=t.transpose(0, 1)), "list": dict(v_new=[1.0]), "word": dict(M_max="16"),
+                 "config": dict(cfg=t.numpy()), "cache": dict(full=t), None: {}}[bad])
+    with pytest.raises(error) as e:
+        B.specpv_verify_full(**args)
+    assert bad is not None or e.value.status == 1
