@@ -1,12 +1,12 @@
 // Block scores on the tensor cores (paper Eq. 2-3): s_i = f_r max(q_r . Kmax_i, q_r . Kmin_i) for
-// bfloat16 summaries with head_dim 128, and the channel-wise form s_i = f_r sum_c max(q_rc Kmax_ic, q_rc Kmin_ic).
+// bfloat16 summaries with head_dim 64 or 128, and the channel-wise form s_i = f_r sum_c max(q_rc Kmax_ic, q_rc Kmin_ic).
 // Because Kmax >= Kmin in every channel, the channel-wise maximum takes Kmax where q is positive and Kmin where it
 // is negative, so that form is the single contraction  Kmax . q+  +  Kmin . q-  with q+ = max(q, 0), q- = min(q, 0)
 // (both exact in bfloat16): the CTA splits Q by sign in shared memory and accumulates both products into one
 // accumulator.
 //
 // Per (layer, sequence, KV head) the two products are dense contractions
-//     Dmax[128 blocks x R] = Kmax_tile[128 x 128] * Q^T[128 x R],   Dmin likewise with Kmin,
+//     Dmax[128 blocks x R] = Kmax_tile[128 x d] * Q^T[d x R],   Dmin likewise with Kmin,
 // issued as tcgen05.mma with both operands in shared memory (128-byte swizzle, loaded by TMA) and float32
 // accumulators in tensor memory.
 //
@@ -23,6 +23,10 @@
 //   warps 4-11  epilogue: thread <-> block of the tile (tensor-memory lane) and one half of the query rows; reduces
 //               over its rows (mean, max, or the rows of the "last" query); the two halves meet in shared memory, the
 //               lower half picking the upper half's result up one tile later
+// Bound by HBM on the summaries, and by the tensor pipe above some 192 rows.  Any group size and both head sizes run here, since a
+// pass's query rows are dense in shared memory and columns beyond them are simply not reduced; the plain kernel, on which
+// group sizes that do not divide 128 and head size 64 ran before, is bound by its multiplications (16384 tokens x 24 layers,
+// 60 x 5 rows of 128: 371 -> 23 us, with 16-token blocks 1368 -> 57; 60 x 4 rows of 64: 152 -> 10 us and 534 -> 22).
 // Every wait is bounded; after a wait that gave up the loops end and nothing more is copied or issued.
 #include "aux_kernels.cuh"
 #include "tc_common.cuh"
@@ -36,13 +40,13 @@ using namespace tc;
 constexpr int kScoreThreads = 384;       // 12 warps; the four control warps hand registers to the eight epilogue warps
 constexpr int kScoreCtas = 148;          // one per SM
 constexpr int kTileBlocks = 128;
-constexpr int kSumTileBytes = 32768;     // a ring slot: the Kmax or the Kmin rows of a tile, [2 d-halves][128 blocks][64 d] bf16
+constexpr int kSumTileBytes = 32768;     // a ring slot: the Kmax or the Kmin rows of a tile, [d/64 parts][128 blocks][64 d] bf16
 constexpr int kScoreStages = 5;          // ring slots (the channel-wise form gives two of them to q-)
-constexpr int kScoreQBytes = 65536;      // [2 d-halves][256 rows][64 d] bf16
+constexpr int kScoreQBytes = 65536;      // [d/64 parts][256 rows][64 d] bf16
 constexpr int kScoreSmem = 1024 + kScoreQBytes + kScoreStages * kSumTileBytes;
 
 struct ScoreTcParams {
-    CUtensorMap tm_q;     // (d, Hq, tokens)  box (64, G, 128/G)
+    CUtensorMap tm_q;     // (d, Hq, tokens)  box (64, G, tokens of the pass)
     CUtensorMap tm_kmax;  // (d, rows)        box (64, 128)
     CUtensorMap tm_kmin;
     const int32_t* q_lens;
@@ -124,7 +128,7 @@ struct ScoreIter {
 static_assert(kScoreSmem + sizeof(ScoreBarriers) + 3 * kTileBlocks * sizeof(float) + 64 <= 227 * 1024, "shared memory of scores_tc_kernel");
 
 // kCw: the channel-wise form (a compile-time switch).
-template <bool kCw>
+template <bool kCw, int D>
 __global__ void __launch_bounds__(kScoreThreads, 1) scores_tc_kernel(const __grid_constant__ ScoreTcParams p) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -167,14 +171,13 @@ __global__ void __launch_bounds__(kScoreThreads, 1) scores_tc_kernel(const __gri
     const uint32_t tmem = bars.tmem_base;
     pdl_trigger();
     pdl_wait();
-    const int tok_per_tile = 128 / p.G;
+    constexpr int kParts = D / 64;  // 64-channel parts of a row
 
     // Register budget: 384 threads start with 168 registers each; the control warps keep 48, which is what lets the
     // epilogue warps grow to 224 (128 x 120 released, 256 x 56 taken).
     if (warp == 0) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
         // ---- producer: the whole warp runs the loop (a lone lane of a diverged warp runs slowly), lane 0 copies ----
-        const int n_q_tiles = p.n_cols > 128 ? 2 : 1;
         ScoreIter it;
         it.init(p);
         ScoreSeg s;
@@ -185,11 +188,9 @@ __global__ void __launch_bounds__(kScoreThreads, 1) scores_tc_kernel(const __gri
             if (sidx > 0) ok &= mbar_wait(smem_u32(&bars.q_empty), (sidx - 1) & 1, abort_flag, p.workspace, 27);
             if (lane == 0 && ok) {
                 const uint32_t qbar = smem_u32(&bars.q_full);
-                mbar_expect_tx(qbar, (uint32_t)(n_q_tiles * 32768));
-                for (int t = 0; t < n_q_tiles; ++t)
-                    for (int half = 0; half < 2; ++half)
-                        tma_load_3d(q_smem + half * 32768 + t * 16384, &p.tm_q, half * 64, s.h * p.G,
-                                    s.lb * p.M_max + p.tok0 + t * tok_per_tile, qbar);
+                mbar_expect_tx(qbar, (uint32_t)(p.tok_n * p.G * D * 2));
+                for (int part = 0; part < kParts; ++part)
+                    tma_load_3d(q_smem + part * 32768, &p.tm_q, part * 64, s.h * p.G, s.lb * p.M_max + p.tok0, qbar);
             }
             __syncwarp();
             const int row0 = (((p.layer0 + s.l) * p.batch + s.b) * p.Hkv + s.h) * p.max_blocks;
@@ -200,11 +201,11 @@ __global__ void __launch_bounds__(kScoreThreads, 1) scores_tc_kernel(const __gri
                         ok &= mbar_wait(smem_u32(&bars.sum_empty[slot]), ((u / stages) - 1) & 1, abort_flag, p.workspace, 21);
                     if (lane == 0 && ok) {
                         const uint32_t full = smem_u32(&bars.sum_full[slot]);
-                        mbar_expect_tx(full, kSumTileBytes);
+                        mbar_expect_tx(full, kTileBlocks * D * 2);
                         const uint32_t dst = sum_smem + slot * kSumTileBytes;
                         const int row = row0 + t * kTileBlocks;
-                        for (int half = 0; half < 2; ++half)
-                            tma_load_2d(dst + half * 16384, which ? &p.tm_kmin : &p.tm_kmax, half * 64, row, full);
+                        for (int part = 0; part < kParts; ++part)
+                            tma_load_2d(dst + part * 16384, which ? &p.tm_kmin : &p.tm_kmax, part * 64, row, full);
                     }
                     __syncwarp();
                 }
@@ -254,7 +255,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) scores_tc_kernel(const __gri
                     if (lane == 0) {
                         const uint32_t a0 = sum_lo + s0 * (kSumTileBytes >> 4), a1 = sum_lo + s1 * (kSumTileBytes >> 4);
 #pragma unroll
-                        for (int kk = 0; kk < 8; ++kk) {
+                        for (int kk = 0; kk < 4 * kParts; ++kk) {
                             const uint32_t a_off = (uint32_t)((kk >> 2) * 16384 + (kk & 3) * 32) >> 4;
                             const uint32_t b_off = (uint32_t)((kk >> 2) * 32768 + (kk & 3) * 32) >> 4;
                             mma_ss(d, ((uint64_t)desc_hi << 32) | (a0 + a_off), ((uint64_t)desc_hi << 32) | (q_lo + b_off), idesc, kk > 0);
@@ -315,7 +316,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) scores_tc_kernel(const __gri
                 if (!ok) break;
                 uint4* qp = reinterpret_cast<uint4*>(smem);
                 uint4* qn = reinterpret_cast<uint4*>(smem + kScoreQBytes);
-                for (int v = threadIdx.x - 128; v < kScoreQBytes / 16; v += 256) {
+                for (int v = threadIdx.x - 128; v < kParts * 32768 / 16; v += 256) {
                     const uint4 w = qp[v];
                     const uint32_t in[4] = {w.x, w.y, w.z, w.w};
                     uint32_t pos[4], neg[4];
@@ -467,29 +468,24 @@ __global__ void __launch_bounds__(kScoreThreads, 1) scores_tc_kernel(const __gri
 
 }  // namespace
 
+// More than 1024 rows per KV head (a group of 33 x 33 step tokens) would take more than four passes over the summaries; no
+// configuration comes near, and the plain kernel takes them.
 bool scores_tc_supported(int dtype, int d, int G, int M_max) {
-    return dtype == SPECPV_DTYPE_BF16 && d == 128 && G <= 128 && (128 % G) == 0 && M_max * G <= 4 * 256 &&
+    return dtype == SPECPV_DTYPE_BF16 && (d == 128 || d == 64) && G <= 128 && M_max * G <= 4 * 256 &&
            tc::get_encode_fn() != nullptr;
 }
 
-specpv_status launch_scores_tc(const ScoreParams& sp, int n_layers_call, int n_layers_total, int max_nb,
-                               cudaStream_t stream) {
-    if (!tc::set_smem_limit_once(reinterpret_cast<const void*>(scores_tc_kernel<false>), kScoreSmem) ||
-        !tc::set_smem_limit_once(reinterpret_cast<const void*>(scores_tc_kernel<true>), kScoreSmem))
-        return SPECPV_ERR_CUDA;
+template <int D>
+static specpv_status launch_scores_d(const ScoreParams& sp, int n_layers_call, int n_layers_total, int max_nb, cudaStream_t stream) {
+    const auto kernel = sp.score_mode == 1 ? scores_tc_kernel<true, D> : scores_tc_kernel<false, D>;
+    if (!tc::set_smem_limit_once(reinterpret_cast<const void*>(kernel), kScoreSmem)) return SPECPV_ERR_CUDA;
     if (max_nb <= 0 || n_layers_call <= 0) return SPECPV_OK;
     ScoreTcParams p{};
     const uint64_t step_tokens = (uint64_t)n_layers_call * sp.batch * sp.M_max;
     {
-        uint64_t dims[3] = {128, (uint64_t)sp.Hq, step_tokens};
-        uint64_t strides[2] = {256, (uint64_t)sp.Hq * 256};
-        uint32_t box[3] = {64, (uint32_t)sp.G, (uint32_t)(128 / sp.G)};
-        if (!tc::encode_map(&p.tm_q, sp.q, 3, dims, strides, box)) return SPECPV_ERR_CUDA;
-    }
-    {
-        uint64_t dims[2] = {128, (uint64_t)n_layers_total * sp.batch * sp.Hkv * sp.max_blocks};
+        uint64_t dims[2] = {D, (uint64_t)n_layers_total * sp.batch * sp.Hkv * sp.max_blocks};
         if (dims[1] >= 0x7FFFFF00ull) return SPECPV_ERR_UNSUPPORTED;
-        uint64_t strides[1] = {256};
+        uint64_t strides[1] = {D * 2};
         uint32_t box[2] = {64, 128};
         if (!tc::encode_map(&p.tm_kmax, sp.kmax, 2, dims, strides, box)) return SPECPV_ERR_CUDA;
         if (!tc::encode_map(&p.tm_kmin, sp.kmin, 2, dims, strides, box)) return SPECPV_ERR_CUDA;
@@ -505,18 +501,28 @@ specpv_status launch_scores_tc(const ScoreParams& sp, int n_layers_call, int n_l
     dim3 grid((unsigned)(total < kScoreCtas ? total : kScoreCtas), 1, 1);
     // The accumulator holds 256 query rows; a step with more (the chain and the tree of a refresh) goes through in
     // passes over the step's tokens, each later pass combining with what is there (sum of per-pass means, or max).
+    // A pass's query rows are one box per 64 channels, token * G + head of the KV group, whatever G is; rows that the
+    // contraction covers beyond them (its width is a multiple of 16) are columns that the epilogue leaves out.
     const int tok_per_pass = 256 / sp.G;
     for (int tok0 = 0; tok0 < sp.M_max; tok0 += tok_per_pass) {
         p.tok0 = tok0;
         p.tok_n = sp.M_max - tok0 < tok_per_pass ? sp.M_max - tok0 : tok_per_pass;
         p.accumulate = tok0 > 0;
-        p.n_cols = p.tok_n * sp.G <= 128 ? 128 : 256;  // accumulator columns, padded to whole 128-row Q tiles
-        if (launch_pdl(sp.score_mode == 1 ? scores_tc_kernel<true> : scores_tc_kernel<false>, grid, kScoreThreads, kScoreSmem, stream,
-                       p) != cudaSuccess)
-            return SPECPV_ERR_CUDA;
+        p.n_cols = (p.tok_n * sp.G + 15) / 16 * 16;
+        uint64_t dims[3] = {D, (uint64_t)sp.Hq, step_tokens};
+        uint64_t strides[2] = {D * 2, (uint64_t)sp.Hq * D * 2};
+        uint32_t box[3] = {64, (uint32_t)sp.G, (uint32_t)p.tok_n};
+        if (!tc::encode_map(&p.tm_q, sp.q, 3, dims, strides, box)) return SPECPV_ERR_CUDA;
+        if (launch_pdl(kernel, grid, kScoreThreads, kScoreSmem, stream, p) != cudaSuccess) return SPECPV_ERR_CUDA;
         count_launch();
     }
     return SPECPV_OK;
+}
+
+specpv_status launch_scores_tc(const ScoreParams& sp, int n_layers_call, int n_layers_total, int max_nb, int d,
+                               cudaStream_t stream) {
+    return d == 128 ? launch_scores_d<128>(sp, n_layers_call, n_layers_total, max_nb, stream)
+                    : launch_scores_d<64>(sp, n_layers_call, n_layers_total, max_nb, stream);
 }
 
 }  // namespace specpv

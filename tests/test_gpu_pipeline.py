@@ -351,11 +351,13 @@ def test_verify_host_matches_the_device_call_and_the_oracle(name, L, over):
     np.testing.assert_allclose(lse_h[l, b].numpy(), o_lse, atol=5e-3)
 
 
-@pytest.mark.parametrize("dtype,Hq,d", [("fp32", 8, 64), ("fp32", 8, 128), ("bf16", 10, 128), ("bf16", 8, 64)])
+@pytest.mark.parametrize("dtype,Hq,d", [("fp32", 8, 64), ("fp32", 8, 128), ("bf16", 10, 128), ("bf16", 8, 64),
+                                        ("bf16", 66, 64)])
 @pytest.mark.parametrize("reduce,score_mode", [(B.REDUCE_MEAN, 0), (B.REDUCE_MAX, 1), (B.REDUCE_LAST, 0)])
 def test_scores_of_the_plain_kernel(dtype, Hq, d, reduce, score_mode):
-    """Geometries the tensor-core score kernel does not take: float32, head size 64, five query heads per KV head; block
-    counts around the 32 a CTA takes, row counts that leave warps without rows."""
+    """What the tensor-core score kernel does not take, float32 and more than 1024 rows per KV head (33 x 33), and two
+    shapes that it does take; block counts around the 32 a CTA of the plain kernel takes, row counts that leave warps
+    without rows."""
     w = wl.make_workload("llama_32k", device="cuda", n_layers=2, Hq=Hq, Hkv=2, d=d, dtype=dtype, M=33,
                          ctx=[64 * 31 + 9, 64 * 33, 64])
     c = w.cfg
@@ -381,6 +383,38 @@ def test_scores_of_the_plain_kernel(dtype, Hq, d, reduce, score_mode):
             # products of the stored values summed in float32: d terms per dot product, then up to 165 rows
             np.testing.assert_allclose(scores[l, b, :, :nb].cpu().numpy(), osc, rtol=2e-5, atol=2e-4, err_msg=f"{l} {b}")
             assert torch.isnan(scores[l, b, :, nb:]).all()
+
+
+@pytest.mark.parametrize("Hq,d,M", [(2, 64, 1), (6, 128, 85), (6, 64, 86), (10, 128, 51), (10, 64, 52), (14, 128, 37),
+                                    (8, 64, 64), (96, 128, 6), (256, 64, 5)])
+@pytest.mark.parametrize("reduce,score_mode", [(B.REDUCE_MEAN, 0), (B.REDUCE_MAX, 0), (B.REDUCE_LAST, 1), (B.REDUCE_MEAN, 1)])
+def test_scores_of_any_group_size_on_the_tensor_core_kernel(Hq, d, M, reduce, score_mode):
+    """One to 128 query heads per KV head, both head sizes; rows just below, at and just above the 256 of a pass and the 128
+    of an epilogue half, contractions a little wider than their rows; blocks around the 128 of a tile."""
+    w = wl.make_workload("llama_32k", device="cuda", n_layers=2, Hq=Hq, Hkv=2, d=d, M=M, ctx=[64 * 128, 64 * 129 - 3, 64 * 5])
+    c = w.cfg
+    Hkv, batch, L = c["Hkv"], w.batch, c["n_layers"]
+    cfg = util.config_for(w, reduce=reduce, score_mode=score_mode)
+    full = util.full_cache(w)
+    ws = B.new_workspace(cfg, L, batch, int(max(c["ctx"])), M)
+    kmax = torch.zeros((L, batch, Hkv, w.max_blocks, d), dtype=torch.bfloat16, device="cuda")
+    kmin = torch.zeros_like(kmax)
+    B.specpv_update_block_summaries(cfg, 0, L, full, None, w.max_blocks, kmax, kmin, ws)
+    q_lens = torch.tensor([M, max(M - 3, 1), (M + 1) // 2], dtype=torch.int32, device="cuda")
+    last = torch.tensor([M - 1, 0, 0], dtype=torch.int32, device="cuda")
+    scores = torch.full((L, batch, Hkv, w.max_blocks), float("nan"), dtype=torch.float32, device="cuda")
+    B.specpv_score_blocks(cfg, 0, L, w.q, q_lens, M, last, kmax, kmin, full, scores, ws)
+    util.sync_status(ws)
+    for l in range(L):
+        for b in range(batch):
+            sl, m = int(c["ctx"][b]), int(q_lens[b])
+            nb = (sl + c["bs"] - 1) // c["bs"]
+            okmax, okmin = oracle.block_summaries(wl.to_numpy(w.k_pool[l]), wl.to_numpy(w.block_table[b]), sl)
+            osc = oracle.block_scores(wl.to_numpy(w.q[l, b, :m]), okmax, okmin, Hkv, reduce=reduce, last_query=int(last[b]),
+                                      score_mode=score_mode)
+            # exact products summed in float32, d (twice d in the channel-wise form) to a dot product: as the plain kernel
+            np.testing.assert_allclose(scores[l, b, :, :nb].cpu().numpy(), osc, rtol=2e-5, atol=2e-4, err_msg=f"{l} {b}")
+            assert torch.isnan(scores[l, b, :, nb:]).all()  # blocks past the context are left alone
 
 
 @pytest.mark.parametrize("score_mode", [0, 1])
