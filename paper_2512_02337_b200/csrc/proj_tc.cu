@@ -6,11 +6,11 @@
 // are bound by HBM.  The weights are therefore the M operand of the tensor-core contraction,
 //     D[128 out features x tokens] += W_tile[128 x 64] * X_tile[tokens x 64]^T     (tcgen05.mma, kind::f16),
 // both operands K-major in shared memory (128-byte swizzle, loaded by TMA through a ring of stages), the
-// float32 accumulator in tensor memory.  A CTA owns one 128-feature tile (one head of the QKV map) and a
-// range of the input features; with several ranges per tile (few tiles, one layer) the partial sums go to
+// float32 accumulator in tensor memory.  A CTA owns one 128-feature tile (one head of 128 or two of 64 of the
+// QKV map) and a range of the input features; with several ranges per tile (few tiles, one layer) the partial sums go to
 // the workspace and a second kernel adds them in a fixed order.  The epilogue turns the accumulator
-// through shared memory so that a thread holds channels (2j, 2j+1) and their rotary partners
-// (64+2j, 64+2j+1) of one row, rotates, adds the residual and writes bfloat16.  Every wait is bounded.
+// through shared memory so that a thread holds two channels and their rotary partners, half a head further on, of one row,
+// rotates, adds the residual and writes bfloat16.  Every wait is bounded.
 #include "proj.cuh"
 #include "tc_common.cuh"
 
@@ -48,14 +48,21 @@ struct __align__(8) ProjBarriers {
     int abort_flag;
 };
 
-// Where channels (2j, 2j+1) and (64+2j, 64+2j+1) of feature tile `tile`, row `tok` of layer-in-call `l` go, and what they
-// are rotated by and added to: asked for ahead of the sums, so that the two latencies overlap.
+// A thread of an epilogue owns two channels of a head and the two that they are rotated with, kHalf (half a head) further
+// on: features (f, f+1) and (f+kHalf, f+kHalf+1) of a tile with f = feature_of<kHalf>(j), j the lane.  A tile is one head of
+// 128 channels or two of 64.
+template <int kHalf>
+__device__ __forceinline__ int feature_of(int j) { return j / (kHalf / 2) * (2 * kHalf) + j % (kHalf / 2) * 2; }
+
+// Where those channels of feature tile `tile`, row `tok` of layer-in-call `l` go, and what they are rotated by and added to:
+// asked for ahead of the sums, so that the two latencies overlap.
 struct ProjTarget {
     __nv_bfloat16* dst;
     float4 cs;         // cos, sin, cos, sin
     uint32_t res[2];   // residual of the two channel pairs
     bool rope, add;
 };
+template <int kHalf>
 __device__ __forceinline__ ProjTarget proj_target(const ProjTcParams& p, int tile, int l, int tok, int j) {
     int s = 0;
     for (int i = 1; i < p.n_seg; ++i)
@@ -65,16 +72,17 @@ __device__ __forceinline__ ProjTarget proj_target(const ProjTcParams& p, int til
     t.rope = sg.rope;
     t.add = p.residual && s == 0;
     t.cs = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (t.rope) t.cs = __ldg(reinterpret_cast<const float4*>(p.cos_sin + ((size_t)tok * 64 + 2 * j) * 2));
-    const size_t off = ((size_t)l * p.tokens + tok) * sg.row_stride + (size_t)(tile - sg.first_tile) * kFeatTile + 2 * j;
+    if (t.rope) t.cs = __ldg(reinterpret_cast<const float4*>(p.cos_sin + ((size_t)tok * kHalf + j % (kHalf / 2) * 2) * 2));
+    const size_t off = ((size_t)l * p.tokens + tok) * sg.row_stride + (size_t)(tile - sg.first_tile) * kFeatTile + feature_of<kHalf>(j);
     t.res[0] = t.res[1] = 0;
     if (t.add) {
         t.res[0] = __ldg(reinterpret_cast<const uint32_t*>(p.residual + off));
-        t.res[1] = __ldg(reinterpret_cast<const uint32_t*>(p.residual + off + 64));
+        t.res[1] = __ldg(reinterpret_cast<const uint32_t*>(p.residual + off + kHalf));
     }
     t.dst = reinterpret_cast<__nv_bfloat16*>(sg.base) + off;
     return t;
 }
+template <int kHalf>
 __device__ __forceinline__ void proj_finish(const ProjTarget& t, float2 lo, float2 hi) {
     if (t.rope) {
         const float4 cs = t.cs;
@@ -88,7 +96,7 @@ __device__ __forceinline__ void proj_finish(const ProjTarget& t, float2 lo, floa
         hi.x += __uint_as_float(t.res[1] << 16); hi.y += __uint_as_float(t.res[1] & 0xFFFF0000u);
     }
     *reinterpret_cast<uint32_t*>(t.dst) = pack_bf16(lo.x, lo.y);
-    *reinterpret_cast<uint32_t*>(t.dst + 64) = pack_bf16(hi.x, hi.y);
+    *reinterpret_cast<uint32_t*>(t.dst + kHalf) = pack_bf16(hi.x, hi.y);
 }
 
 __device__ __forceinline__ size_t partial_base(const ProjTcParams& p, int l, int chunk, int n_chunks, int tile, int split) {
@@ -96,6 +104,7 @@ __device__ __forceinline__ size_t partial_base(const ProjTcParams& p, int l, int
     return (unit * p.splits + split) * (size_t)p.n_pad * kFeatTile;
 }
 
+template <int kHalf>
 __global__ void __launch_bounds__(kProjThreads, 2) proj_tc_kernel(const __grid_constant__ ProjTcParams p) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -206,17 +215,17 @@ __global__ void __launch_bounds__(kProjThreads, 2) proj_tc_kernel(const __grid_c
         tc_fence_before();
         asm volatile("bar.sync 1, 128;" ::: "memory");
         if (ok) {
-            const int et = threadIdx.x - 64, j = et & 31;
+            const int et = threadIdx.x - 64, j = et & 31, feat = feature_of<kHalf>(j);
             float* part = p.splits > 1 ? p.partials + partial_base(p, l, chunk, gridDim.y, tile, split) : nullptr;
 #pragma unroll 4
             for (int t = et >> 5; t < valid; t += 4) {
-                const float2 lo = *reinterpret_cast<const float2*>(stage + t * kFeatTile + 2 * j);
-                const float2 hi = *reinterpret_cast<const float2*>(stage + t * kFeatTile + 64 + 2 * j);
+                const float2 lo = *reinterpret_cast<const float2*>(stage + t * kFeatTile + feat);
+                const float2 hi = *reinterpret_cast<const float2*>(stage + t * kFeatTile + feat + kHalf);
                 if (part) {
-                    *reinterpret_cast<float2*>(part + (size_t)t * kFeatTile + 2 * j) = lo;
-                    *reinterpret_cast<float2*>(part + (size_t)t * kFeatTile + 64 + 2 * j) = hi;
+                    *reinterpret_cast<float2*>(part + (size_t)t * kFeatTile + feat) = lo;
+                    *reinterpret_cast<float2*>(part + (size_t)t * kFeatTile + feat + kHalf) = hi;
                 } else {
-                    proj_finish(proj_target(p, tile, l, tok0 + t, j), lo, hi);
+                    proj_finish<kHalf>(proj_target<kHalf>(p, tile, l, tok0 + t, j), lo, hi);
                 }
             }
         }
@@ -232,7 +241,8 @@ __global__ void __launch_bounds__(kProjThreads, 2) proj_tc_kernel(const __grid_c
 }
 
 // Adds the partial sums of a tile's input-feature ranges in range order and finishes the rows: a CTA takes four rows
-// of one tile, a thread one row's channels (2j, 2j+1, 64+2j, 64+2j+1), so that all its loads are in flight together.
+// of one tile, a thread one row's two channel pairs, so that all its loads are in flight together.
+template <int kHalf>
 __global__ void __launch_bounds__(128) proj_reduce_kernel(const __grid_constant__ ProjTcParams p, int n_chunks) {
     pdl_begin(p.pdl);
     const int tile = blockIdx.x, l = blockIdx.z / n_chunks, chunk = blockIdx.z % n_chunks;
@@ -240,15 +250,15 @@ __global__ void __launch_bounds__(128) proj_reduce_kernel(const __grid_constant_
     const int valid = min(p.n_pad, p.tokens - tok0);
     const int j = threadIdx.x & 31, t = blockIdx.y * 4 + (threadIdx.x >> 5);
     if (t >= valid) return;
-    const float* part = p.partials + partial_base(p, l, chunk, n_chunks, tile, 0) + (size_t)t * kFeatTile + 2 * j;
+    const float* part = p.partials + partial_base(p, l, chunk, n_chunks, tile, 0) + (size_t)t * kFeatTile + feature_of<kHalf>(j);
     const size_t split_stride = (size_t)p.n_pad * kFeatTile;
-    const ProjTarget target = proj_target(p, tile, l, tok0 + t, j);
+    const ProjTarget target = proj_target<kHalf>(p, tile, l, tok0 + t, j);
     float2 a[8], b[8];
 #pragma unroll
     for (int s = 0; s < 8; ++s)
         if (s < p.splits) {
             a[s] = __ldg(reinterpret_cast<const float2*>(part + s * split_stride));
-            b[s] = __ldg(reinterpret_cast<const float2*>(part + s * split_stride + 64));
+            b[s] = __ldg(reinterpret_cast<const float2*>(part + s * split_stride + kHalf));
         }
     float2 lo = make_float2(0.f, 0.f), hi = lo;
 #pragma unroll
@@ -256,7 +266,7 @@ __global__ void __launch_bounds__(128) proj_reduce_kernel(const __grid_constant_
         if (s < p.splits) {
             lo.x += a[s].x; lo.y += a[s].y; hi.x += b[s].x; hi.y += b[s].y;
         }
-    proj_finish(target, lo, hi);
+    proj_finish<kHalf>(target, lo, hi);
 }
 
 // ---- plain kernel: any dtype / head size ---------------------------------------------------------------------
@@ -334,14 +344,20 @@ __global__ void rope_table_kernel(const uint64_t* __restrict__ tree_mask, const 
 
 }  // namespace
 
+// Heads of 64 run here two to a tile (the plain kernel reads the weights once per row: 76 rows, 48 heads of 64, hidden 4096,
+// projection, attention and projection of a layer 892 us with it, 44 without).
 bool proj_tc_supported(const ProjArgs& a) {
-    return a.dtype == SPECPV_DTYPE_BF16 && a.tile == kFeatTile && a.n_in % 64 == 0 && a.n_in >= 64 &&
+    if (a.tile != kFeatTile && a.tile != kFeatTile / 2) return false;
+    for (int i = 0; i < a.n_seg; ++i)  // two heads of 64 share a tile: every tensor must begin on one
+        if (a.seg[i].first_tile * a.tile % kFeatTile != 0) return false;
+    return a.dtype == SPECPV_DTYPE_BF16 && a.n_in % 64 == 0 && a.n_in >= 64 &&
            a.n_out % kFeatTile == 0 && (uint64_t)a.n_layers_total * a.n_out < 0x7FFFFF00ull &&
            (uint64_t)a.n_layers_call * a.tokens < 0x7FFFFF00ull && tc::get_encode_fn() != nullptr;
 }
 
-specpv_status launch_proj_tc(const ProjArgs& a, cudaStream_t stream) {
-    if (!tc::set_smem_limit_once(reinterpret_cast<const void*>(proj_tc_kernel), kProjSmem)) return SPECPV_ERR_CUDA;
+template <int kHalf>
+static specpv_status launch_proj(const ProjArgs& a, cudaStream_t stream) {
+    if (!tc::set_smem_limit_once(reinterpret_cast<const void*>(proj_tc_kernel<kHalf>), kProjSmem)) return SPECPV_ERR_CUDA;
     if (a.tokens <= 0 || a.n_layers_call <= 0) return SPECPV_OK;
     ProjTcParams p{};
     p.n_pad = a.tokens >= kMaxTokTile ? kMaxTokTile : (a.tokens + 31) / 32 * 32;
@@ -362,7 +378,10 @@ specpv_status launch_proj_tc(const ProjArgs& a, cudaStream_t stream) {
     p.residual = reinterpret_cast<const __nv_bfloat16*>(a.residual);
     p.workspace = a.workspace;
     p.n_seg = a.n_seg;
-    for (int i = 0; i < a.n_seg; ++i) p.seg[i] = a.seg[i];
+    for (int i = 0; i < a.n_seg; ++i) {
+        p.seg[i] = a.seg[i];
+        p.seg[i].first_tile = a.seg[i].first_tile * a.tile / kFeatTile;
+    }
     p.layer0 = a.layer0; p.n_tiles = a.n_out / kFeatTile; p.n_out = a.n_out; p.tokens = a.tokens;
     p.ksteps = a.n_in / 64;
     const int stage_bytes = kWTileBytes + p.n_pad * 128;
@@ -389,17 +408,21 @@ specpv_status launch_proj_tc(const ProjArgs& a, cudaStream_t stream) {
     p.group = splits > 1 || p.stages < 4 ? 1 : kIssueGroup;
     p.partials = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(a.workspace) + a.scratch_off);
     dim3 grid(p.n_tiles * splits, n_chunks, a.n_layers_call);
-    if (launch_pdl(proj_tc_kernel, grid, kProjThreads, 1024 + ring_bytes, stream, p) != cudaSuccess) return SPECPV_ERR_CUDA;
+    if (launch_pdl(proj_tc_kernel<kHalf>, grid, kProjThreads, 1024 + ring_bytes, stream, p) != cudaSuccess) return SPECPV_ERR_CUDA;
     count_launch();
     if (splits > 1) {
         const dim3 rgrid(p.n_tiles, (p.n_pad + 3) / 4, a.n_layers_call * n_chunks);
         p.pdl = pdl_pays(rgrid);
-        if ((p.pdl ? launch_pdl(proj_reduce_kernel, rgrid, 128, 0, stream, p, n_chunks)
-                   : launch_plain(proj_reduce_kernel, rgrid, 128, 0, stream, p, n_chunks)) != cudaSuccess)
+        if ((p.pdl ? launch_pdl(proj_reduce_kernel<kHalf>, rgrid, 128, 0, stream, p, n_chunks)
+                   : launch_plain(proj_reduce_kernel<kHalf>, rgrid, 128, 0, stream, p, n_chunks)) != cudaSuccess)
             return SPECPV_ERR_CUDA;
         count_launch();
     }
     return SPECPV_OK;
+}
+
+specpv_status launch_proj_tc(const ProjArgs& a, cudaStream_t stream) {
+    return a.tile == kFeatTile ? launch_proj<kFeatTile / 2>(a, stream) : launch_proj<kFeatTile / 4>(a, stream);
 }
 
 specpv_status launch_proj_simt(const ProjArgs& a, cudaStream_t stream) {

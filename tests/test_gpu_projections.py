@@ -115,6 +115,20 @@ def test_qkv_rope_and_o_proj_match_the_oracle(dtype, Hq, Hkv, d, hidden, batch, 
                          f"o + residual layer {l} seq {b}")
 
 
+@pytest.mark.parametrize("Hq,Hkv,hidden,batch,M,L,layer0,n_call", [
+    (32, 8, 4096, 1, 60, 1, 0, 1),     # one layer: several input ranges per tile
+    (8, 2, 448, 1, 37, 3, 1, 2),       # seven 64-wide input steps
+    (8, 4, 512, 2, 64, 16, 0, 16),     # 128 tiles: one range per tile, 128 rows
+    (4, 2, 256, 5, 64, 1, 0, 1),       # 320 rows: two row chunks
+    (2, 2, 64, 1, 1, 1, 0, 1),         # a tile per tensor, one row
+    (5, 1, 256, 2, 9, 2, 0, 2),        # heads that do not fill whole tiles: plain kernel
+])
+def test_projections_with_two_heads_of_64_to_a_tile(Hq, Hkv, hidden, batch, M, L, layer0, n_call):
+    """Rotation inside each half of a 128-feature tile; same tolerances as above (bfloat16 results of exact products summed in
+    float32)."""
+    test_qkv_rope_and_o_proj_match_the_oracle("bf16", Hq, Hkv, 64, hidden, batch, M, L, layer0, n_call)
+
+
 def test_attention_block_of_a_refresh_step_stage_by_stage():
     """rope table -> QKV -> full verification -> output projection on the LLaMA head geometry with a partially
     verified chain in front of the tree; each stage is checked against the oracle run on the previous stage's
