@@ -148,6 +148,13 @@ def test_many_layers_and_one_layer_agree_with_the_oracle(M, n_layers):
     run_case("bf16", 32, 8, 128, 64, ctx=[128 * 6 + 70], Ms=[M], n_layers=1, seed=M + 1)
 
 
+@pytest.mark.parametrize("M,n_layers", [(8, 1), (9, 24), (40, 1), (41, 20)])
+def test_warps_without_rows(M, n_layers):
+    """Row counts at the 32 rows of a warp: warps without a row in the first and in the second row tile, a second row tile
+    that only one sequence uses, one tile of the step's own tokens and several K/V tiles, one and many KV splits."""
+    run_case("bf16", 32, 8, 128, 64, ctx=[128 * 5 + 70, 0, 128 * 3], Ms=[M, max(M - 33, 1), M // 2], n_layers=n_layers, seed=M)
+
+
 def test_partial_entry_point_multi_layer_bf16():
     run_case("bf16", 32, 8, 128, 64, ctx=[64 * 64 + 20, 64 * 70], Ms=[60, 33], depth=6, branch=4, n_layers=3,
              seed=6, partial_entry=True)
