@@ -13,7 +13,7 @@ constexpr float kRescaleThreshold = 8.0f;  // log2 units
 constexpr float kSafeRowSum = 1.1529215e18f;  // 2^60: a tile's row sum below this cannot overflow the float32 sums
 
 struct TcParams {
-    CUtensorMap tm_q;      // (d, Hq, tokens)          box (64, G, floor(128/G))
+    CUtensorMap tm_q;      // (d, Hq, M_max, layers * batch)  box (64, G, floor(128/G), 1); pair kernel: (d, Hq, tokens)
     CUtensorMap tm_knew;   // (d, Hkv, tokens)         box (64, 1, 8)  (pair kernel: 64)
     CUtensorMap tm_vnew;
     CUtensorMap tm_kpool;  // (64, 8, d/64, rows/8)    box (64, 8, d/64, page size / 8)  (pair kernel: (d, rows), box (64, page size))
