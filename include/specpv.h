@@ -106,8 +106,8 @@ typedef struct {
 const char *specpv_status_string(specpv_status s);
 
 /* Bytes of device workspace that any call below needs for the given limits.  The first
- * SPECPV_WORKSPACE_HEAD_BYTES hold the device status word and the arrival counters of KV ranges that
- * several CTAs share; the caller zeroes them once (cudaMemset) before first use and the library
+ * SPECPV_WORKSPACE_HEAD_BYTES hold the device status word and the arrival counters of the commit and
+ * of KV ranges that several CTAs share; the caller zeroes them once (cudaMemset) before first use and the library
  * leaves them zero after every call that completes (after SPECPV_ERR_TIMEOUT zero them again).  The
  * rest is scratch (split-KV partial results, host-call staging) with no state between calls. */
 #define SPECPV_WORKSPACE_HEAD_BYTES (256u << 10)
@@ -177,8 +177,9 @@ specpv_status specpv_refresh_partial(const specpv_config *cfg, const specpv_page
  * the step's tokens over the partial segment (sink | retrieval | local | buffer) followed by the
  * step's own keys under the tree mask.  out (and lse if not NULL) are fully written for rows
  * < q_lens[b].
- * Two tensor-core kernels serve bfloat16 / head_dim 128: by default one CTA per KV range; with the
- * environment variable SPECPV_ATTN_KERNEL=pair (read at every call) shapes with more than 128 query
+ * bfloat16 runs on the tensor cores for both head sizes and up to 128 query heads per KV head, by
+ * default on a kernel with one CTA per KV range.  With the environment variable
+ * SPECPV_ATTN_KERNEL=pair (read at every call) shapes of head_dim 128 with more than 128 query
  * rows per KV head (M_max * Hq / Hkv) run on a kernel that gives a pair of SMs the two halves of
  * those rows.  The results agree within the tolerance of either; the default is the faster one when
  * steps follow one another (see the comment at attention_pair_wanted). */
@@ -276,8 +277,9 @@ specpv_status specpv_commit_accepted(const specpv_config *cfg, int layer0, int n
  *   w_qkv                  [n_layers][(Hq + 2 Hkv) d][hidden]           q heads, then k heads, then v heads
  *   w_o                    [n_layers][hidden][Hq d]
  *   cos_sin                [batch][M_max][d/2][2] float32               (cos, sin) of every row's angles
- * hidden must be a multiple of 16.  bfloat16 with d = 128 and hidden, Hq d multiples of 64 (128 for
- * the output side of specpv_o_proj) runs on the tensor cores, everything else on a plain kernel.
+ * hidden must be a multiple of 16.  bfloat16 with hidden, Hq d multiples of 64 (128 for the output
+ * side of specpv_o_proj; Hq and Hkv even when d = 64) runs on the tensor cores, everything else on a
+ * plain kernel.
  * Rows >= q_lens[b] are computed like any other row (from whatever x holds there); the caller
  * ignores them. */
 
