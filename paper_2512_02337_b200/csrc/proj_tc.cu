@@ -146,8 +146,11 @@ __global__ void __launch_bounds__(kProjThreads, 2) proj_tc_kernel(const __grid_c
         // ---- producer: the whole warp walks the ring, lane 0 issues the copies ----------------------------
         const int w_row = (p.layer0 + l) * p.n_out + tile * kFeatTile;
         const int x_row = l * p.tokens + tok0;
-        // the weights do not wait for the previous kernel: they start on their way to L2 while it ends
-        for (int i = lane; i < n_k; i += 32) tma_prefetch_2d(&p.tm_w, (kb + i) * 64, w_row);
+        // The weights do not wait for the previous kernel: they start on their way to L2 while it ends.  Only where a tile is split,
+        // so that a CTA's range is short and all ranges are under way at once: with whole tiles the CTAs together ask for more
+        // than L2 holds (32 layers in one launch, 60 rows: 417 us with it, 321 without; output projection 292 and 224).
+        if (p.splits > 1)
+            for (int i = lane; i < n_k; i += 32) tma_prefetch_2d(&p.tm_w, (kb + i) * 64, w_row);
         __syncwarp();
         pdl_wait();
         bool ok = true;
