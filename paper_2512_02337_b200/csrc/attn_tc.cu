@@ -23,6 +23,16 @@
 // Tensor memory (512 columns): S0 | S1 | O0 | O1, 128 columns each, P_t aliases S_t.
 // With several KV splits the unnormalised (O, m, l) go to the workspace and merge_kernel combines
 // them by log-sum-exp.  Every wait is bounded; a wait that gives up records SPECPV_ERR_TIMEOUT.
+//
+// Precision of the weights.  With 128 channels and a group size that divides 128, P is rounded to bfloat16 once.  Head size 64 and the
+// other group sizes (kSplit) keep the float32 weights and accurate log-sum-exps of the plain kernel: P goes to the tensor core as two
+// bfloat16 terms, the rounded weight and what rounding took off, side by side over S (64 + 64 columns), the row sum is taken
+// over the float32 weights, and the scale carries a second term (see scale_log2_lo).  Relative 2-norm errors against float64, one
+// bfloat16 term / two / plain kernel: log-sum-exp 4.8e-5 / 3.5e-8 / 4.0e-8, bfloat16 output 1.86e-3 / 1.66e-3 / 1.66e-3 (1.66e-3 is its own
+// rounding), float32 output 8.5e-4 / 3.6e-6 / 6.6e-7 (12345 tokens, 48 x 5 rows of 128; what is left is the tensor core
+// cutting off the sums over the tokens), 5.4e-5 / 3.3e-8 / 3.4e-8, 1.79e-3 / 1.66e-3 / 1.66e-3 and 6.5e-4 / 2.3e-6 / 3.9e-7
+// (4101 tokens, 60 x 4 rows of 64).  It takes half again the contractions of P V and a third more of the softmax: 24.6 -> 32.0 us and
+// 16.1 -> 18.5 us for one layer, where the plain kernel took 1310 and 375.
 #include "attn_tc.cuh"
 
 namespace specpv {
@@ -167,7 +177,7 @@ __device__ __forceinline__ void produce(const TcParams& p, const Job& c, Barrier
 // Barrier instructions do not overlap with queued MMAs (each costs the pipe 30-100 idle cycles),
 // so the loop keeps them to four waits per KV tile, without votes, and four commits behind MMAs.  The whole
 // warp runs the loop, lane 0 issues.
-template <int D, bool kOne>
+template <int D, bool kOne, bool kSplit>
 __device__ __forceinline__ void issue(const TcParams& p, const Job& c, Barriers& bars, int lane) {
     using Sh = Shape<D>;
     constexpr int kStages = Sh::kStages;
@@ -188,8 +198,11 @@ __device__ __forceinline__ void issue(const TcParams& p, const Job& c, Barriers&
     auto issue_pv = [&](int t, uint32_t vb_lo, bool first) {  // O_t (+)= P_t V
         const uint32_t a = tmem + t * 128, d = tmem + 256 + t * 128;
 #pragma unroll
-        for (int kk = 0; kk < 8; ++kk)  // 16 tokens per instruction: two groups
-            mma_ts_lohi(d, a + kk * 8, vb_lo + (uint32_t)kk * (2 * Sh::kGroupBytes >> 4), kv_hi, kIdescPV<D>, (!first || kk > 0) ? 1u : 0u);
+        for (int kk = 0; kk < 8; ++kk) {  // 16 tokens per instruction: two groups
+            const uint32_t b = vb_lo + (uint32_t)kk * (2 * Sh::kGroupBytes >> 4);
+            mma_ts_lohi(d, a + kk * 8, b, kv_hi, kIdescPV<D>, (!first || kk > 0) ? 1u : 0u);
+            if (kSplit) mma_ts_lohi(d, a + 64 + kk * 8, b, kv_hi, kIdescPV<D>, 1u);
+        }
     };
     auto issue_qk = [&](int t, uint32_t a_lo, uint32_t kb_lo) {  // S_t = Q K^T
         const uint32_t d = tmem + t * 128;
@@ -321,6 +334,7 @@ __device__ __forceinline__ void fix_v(const TcParams& p, const Job& c, Barriers&
 // A warp none of whose rows is in use (38 tokens x 4 heads leave three of the eight without) passes zeros on, and leaves the
 // exponentials to the warp that shares its scheduler and the power to the rest: 64K tokens x 36 layers, 38 rows per head
 // 2080 -> 1956 us, 48 rows 2080 -> 2005, 13 rows 1378 -> 1320; 60 rows, which use every warp, 2080 either way.
+template <bool kSplit>
 __device__ __noinline__ void pass_zeros(const TcParams& p, Barriers& bars, int t, int first_tile, int step, int n_tiles,
                                         uint32_t s_addr, int lane) {
     volatile int* abort_flag = &bars.abort_flag;
@@ -335,6 +349,10 @@ __device__ __noinline__ void pass_zeros(const TcParams& p, Barriers& bars, int t
         tc_fence_after();
         TMEM_ST32(s_addr, zero);
         TMEM_ST32(s_addr + 32, zero);
+        if (kSplit) {
+            TMEM_ST32(s_addr + 64, zero);
+            TMEM_ST32(s_addr + 96, zero);
+        }
         tmem_wait_st();
         tc_fence_before();
         __syncwarp();
@@ -343,7 +361,7 @@ __device__ __noinline__ void pass_zeros(const TcParams& p, Barriers& bars, int t
     mbar_wait(smem_u32(&bars.o_done[t]), 0, abort_flag, p.workspace, 8);  // its contractions have ended before the CTA does
 }
 
-template <int D, bool kOne>
+template <int D, bool kOne, bool kSplit>
 __device__ __forceinline__ void softmax(const TcParams& p, const Job& c, Barriers& bars, int warp, int lane) {
     using Sh = Shape<D>;
     volatile int* abort_flag = &bars.abort_flag;
@@ -363,7 +381,7 @@ __device__ __forceinline__ void softmax(const TcParams& p, const Job& c, Barrier
     const uint32_t s_addr = c.tmem + lane_addr + t * 128;
     const uint32_t o_addr = c.tmem + lane_addr + 256 + t * 128;
     if (!__any_sync(0xffffffffu, row_valid)) {
-        pass_zeros(p, bars, t, first_tile, step, n_tiles, s_addr, lane);
+        pass_zeros<kSplit>(p, bars, t, first_tile, step, n_tiles, s_addr, lane);
         if (kOne && n_tiles > 1) asm volatile("bar.sync 1, 256;" ::: "memory");  // where the two streams meet below
         return;
     }
@@ -375,7 +393,7 @@ __device__ __forceinline__ void softmax(const TcParams& p, const Job& c, Barrier
     }
     float m_run = -INFINITY, l_run = 0.f;
     bool ok = true;
-    const float2 sc2 = make_float2(p.scale_log2, p.scale_log2);
+    const float2 sc2 = make_float2(p.scale_log2, p.scale_log2), sc2_lo = make_float2(p.scale_log2_lo, p.scale_log2_lo);
     // One row tile (the form of short calls): the first pass of the loop is a dry run over zeros by the stream whose S comes
     // last, while Q and the first K tile are still on their way: it brings the loop's code (some 20 KB, straight-line) into
     // the instruction cache.  In a model's layer other kernels have run since the last call, and with cold code the first
@@ -423,7 +441,8 @@ __device__ __forceinline__ void softmax(const TcParams& p, const Job& c, Barrier
         // v[i], whose own value was consumed by an earlier pair, so no second register array is needed.
         // The row sum is taken over the ROUNDED weights the tensor core will use, so that O / l is an
         // exact weighted average of V rows (the rounding error of a dominant weight cancels instead of
-        // scaling the output).
+        // scaling the output).  kSplit: over the float32 weights, which the two terms hold to 2^-18.
+        uint32_t rest[kSplit ? 64 : 1];  // kSplit: what rounding took off, as bf16 pairs
         auto exp_row = [&](float m_use) {
             const float2 nm2 = make_float2(-m_use, -m_use);
             float2 sum2[4];  // independent partial sums: one chain of 64 dependent adds would outlast the exponentials
@@ -431,11 +450,18 @@ __device__ __forceinline__ void softmax(const TcParams& p, const Job& c, Barrier
             for (int e = 0; e < 4; ++e) sum2[e] = make_float2(0.f, 0.f);
 #pragma unroll
             for (int i = 0; i < 64; ++i) {
-                const float2 x = __ffma2_rn(make_float2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1])),
-                                            sc2, nm2);
-                const uint32_t w = pack_bf16(ex2(x.x), ex2(x.y));
+                const float2 sv = make_float2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
+                float2 x = __ffma2_rn(sv, sc2, nm2);
+                if constexpr (kSplit) x = __ffma2_rn(sv, sc2_lo, x);
+                const float2 e = make_float2(ex2(x.x), ex2(x.y));
+                const uint32_t w = pack_bf16(e.x, e.y);
                 v[i] = w;
-                add_bf16_pair(sum2[i & 3], w);
+                if constexpr (kSplit) {
+                    rest[i] = pack_bf16(e.x - __uint_as_float(w << 16), e.y - __uint_as_float(w & 0xFFFF0000u));
+                    sum2[i & 3] = __fadd2_rn(sum2[i & 3], e);
+                } else {
+                    add_bf16_pair(sum2[i & 3], w);
+                }
             }
             const float2 s01 = __fadd2_rn(sum2[0], sum2[1]), s23 = __fadd2_rn(sum2[2], sum2[3]);
             return (s01.x + s23.x) + (s01.y + s23.y);
@@ -512,6 +538,10 @@ __device__ __forceinline__ void softmax(const TcParams& p, const Job& c, Barrier
         }
         TMEM_ST32(s_addr, v);
         TMEM_ST32(s_addr + 32, (v + 32));
+        if constexpr (kSplit) {
+            TMEM_ST32(s_addr + 64, rest);
+            TMEM_ST32(s_addr + 96, (rest + 32));
+        }
         l_run += l_add;
         tmem_wait_st();
         tc_fence_before();
@@ -607,19 +637,20 @@ __device__ __forceinline__ void softmax(const TcParams& p, const Job& c, Barrier
     }
     if (row_valid && (!meet || t == 0)) {
         if (direct) {
-            if (p.lse) p.lse[out_row] = m_run * kLn2 + logf(l_run);
+            if (p.lse) p.lse[out_row] = fmaf(m_run, kLn2, logf(l_run));
         } else {
-            p.part_ml[prow * 2] = m_run * kLn2;  // natural-log units for the merge
+            p.part_ml[prow * 2] = m_run;  // log2 units, unrounded: the merge takes differences of them
             p.part_ml[prow * 2 + 1] = l_run;
         }
     }
 }
 
 // =================================================================================================
+// kSplit: P as two bfloat16 terms (head size 64 and group sizes that do not divide 128).
 // kForm: the row groups a launch can meet (a kernel with both forms has twice the code, which a call that follows other
 // kernels pays for in instruction-cache misses).
 enum { kOneTile, kTwoTiles, kBoth };
-template <int D, int kForm>
+template <int D, int kForm, bool kSplit>
 __global__ void __launch_bounds__(kThreadsTc, 1) attn_tc_kernel(const __grid_constant__ TcParams p) {
     using Sh = Shape<D>;
     extern __shared__ uint8_t smem_raw[];
@@ -729,7 +760,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) attn_tc_kernel(const __grid_con
             produce<D>(p, c, bars, one, lane);
         } else if (warp == 1) {
             asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
-            one ? issue<D, true>(p, c, bars, lane) : issue<D, false>(p, c, bars, lane);
+            one ? issue<D, true, kSplit>(p, c, bars, lane) : issue<D, false, kSplit>(p, c, bars, lane);
         } else if (warp == 2) {
             asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
             one ? fix_v<D, true>(p, c, bars, lane) : fix_v<D, false>(p, c, bars, lane);
@@ -737,7 +768,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) attn_tc_kernel(const __grid_con
             asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
         } else {
             asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
-            one ? softmax<D, true>(p, c, bars, warp, lane) : softmax<D, false>(p, c, bars, warp, lane);
+            one ? softmax<D, true, kSplit>(p, c, bars, warp, lane) : softmax<D, false, kSplit>(p, c, bars, warp, lane);
         }
     }
 
@@ -792,7 +823,7 @@ __global__ void __launch_bounds__(kMergeThreads) merge_tc_kernel(const __grid_co
         if (c0 + lane < p.n_splits) {
             const float2 v = ml[(size_t)(c0 + lane) * p.R_pad];
             if (v.x != -INFINITY) {  // an empty split's partial O was never written: weight 0, not used
-                w_mine = __expf(v.x - m_all);
+                w_mine = ex2(v.x - m_all);
                 l_mine = v.y * w_mine;
             }
         }
@@ -825,27 +856,27 @@ __global__ void __launch_bounds__(kMergeThreads) merge_tc_kernel(const __grid_co
         w2.y = pack_bf16(o.z, o.w);
         reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.out) + row * D)[lane] = w2;
     }
-    if (p.lse && lane == 0) p.lse[row] = m_all + logf(l_all);
+    if (p.lse && lane == 0) p.lse[row] = fmaf(m_all, kLn2, logf(l_all));
 }
 
-template <int D, int kForm>
+template <int D, int kForm, bool kSplit>
 specpv_status launch_form(const TcParams& p, int n_lb, cudaStream_t stream) {
     using Sh = Shape<D>;
-    if (!set_smem_limit_once(reinterpret_cast<const void*>(attn_tc_kernel<D, kForm>), Sh::kSmemBytes)) return SPECPV_ERR_CUDA;
-    if (launch_pdl(attn_tc_kernel<D, kForm>, p.n_splits * p.n_row_groups * p.Hkv * n_lb, kThreadsTc, Sh::kSmemBytes, stream, p) !=
+    if (!set_smem_limit_once(reinterpret_cast<const void*>(attn_tc_kernel<D, kForm, kSplit>), Sh::kSmemBytes)) return SPECPV_ERR_CUDA;
+    if (launch_pdl(attn_tc_kernel<D, kForm, kSplit>, p.n_splits * p.n_row_groups * p.Hkv * n_lb, kThreadsTc, Sh::kSmemBytes, stream, p) !=
         cudaSuccess)
         return SPECPV_ERR_CUDA;
     count_launch();
     return SPECPV_OK;
 }
 
-template <int D>
+template <int D, bool kSplit>
 specpv_status launch_kernels(const TcParams& p, int n_lb, cudaStream_t stream) {
     // per-sequence row counts, or a last row group of one tile, can bring both forms into one launch
     const bool both = p.rg_tiles == 2 && (p.q_lens || p.n_full_groups < p.n_row_groups);
-    const specpv_status st = p.rg_tiles == 1 ? launch_form<D, kOneTile>(p, n_lb, stream)
-                             : both          ? launch_form<D, kBoth>(p, n_lb, stream)
-                                             : launch_form<D, kTwoTiles>(p, n_lb, stream);
+    const specpv_status st = p.rg_tiles == 1 ? launch_form<D, kOneTile, kSplit>(p, n_lb, stream)
+                             : both          ? launch_form<D, kBoth, kSplit>(p, n_lb, stream)
+                                             : launch_form<D, kTwoTiles, kSplit>(p, n_lb, stream);
     if (st != SPECPV_OK) return st;
     if (p.n_splits > 1) {
         constexpr int rows = kMergeThreads / (D / 4);
@@ -937,6 +968,11 @@ specpv_status launch_attention_tc(const AttnArgs& a, cudaStream_t stream) {
     p.bs = a.g.bs;
     p.pool_rows = (uint32_t)pool_rows;
     p.scale_log2 = a.g.scale * kLog2e;
+    // kSplit: what the float32 factor leaves out, and the mean of what the tensor core cuts off a dot product of d channels, which it
+    // sums 16 at a time and truncates each time (measured, of the sum: 4.6e-8 to 8.3e-8 at 64 channels, 8.9e-8 to 13.8e-8 at
+    // 128, the more the more alike the terms are).  Without this term every log-sum-exp comes out 5e-8 to 6e-8 of itself too
+    // small: rms error 6.1e-8 and 7.3e-8 at 64 and 128 channels, 3.3e-8 and 3.5e-8 with it.
+    p.scale_log2_lo = (float)((double)a.g.scale * 1.4426950408889634 * (1.0 + 1.0e-9 * a.g.d) - (double)p.scale_log2);
 
     if (pair) {
         p.n_row_groups = (a.M_max * G + 255) / 256;
@@ -982,7 +1018,8 @@ specpv_status launch_attention_tc(const AttnArgs& a, cudaStream_t stream) {
     p.part_ml = reinterpret_cast<float*>(ws + (size_t)n_units * p.n_splits * p.R_pad * a.g.d * sizeof(float));
 
     const int n_lb = a.n_layers * a.batch;
-    return a.g.d == 128 ? launch_kernels<128>(p, n_lb, stream) : launch_kernels<64>(p, n_lb, stream);
+    if (a.g.d == 64) return launch_kernels<64, true>(p, n_lb, stream);
+    return 128 % G == 0 ? launch_kernels<128, false>(p, n_lb, stream) : launch_kernels<128, true>(p, n_lb, stream);
 }
 
 }  // namespace specpv

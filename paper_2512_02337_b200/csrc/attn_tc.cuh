@@ -39,6 +39,7 @@ struct TcParams {
     int bs;          // tokens per page (16, 32 or 64)
     uint32_t pool_rows;  // rows of the pool tensor map (an out-of-range row coordinate reads zeros)
     float scale_log2;
+    float scale_log2_lo;  // kSplit: correction of scale_log2
 };
 
 // tcgen05.mma with the shared-memory descriptors given as (low word, high word); `acc` = 0

@@ -25,8 +25,9 @@ def attention_kernel(request, monkeypatch):
 
 
 def run_case(dtype, Hq, Hkv, d, bs, ctx, Ms, depth=4, branch=3, n_chain=0, n_layers=1, shuffle=True, seed=0,
-             partial_entry=False):
-    """One verify call on random data; Ms lists the tree size of every sequence (ragged q_lens)."""
+             partial_entry=False, float32_weights=False):
+    """One verify call on random data; Ms lists the tree size of every sequence (ragged q_lens).  ``float32_weights``: hold the
+    results to what float32 weights give (see test_weights_keep_their_float32_precision)."""
     rng = np.random.default_rng(seed)
     dev = "cuda"
     batch = len(ctx)
@@ -80,6 +81,10 @@ def run_case(dtype, Hq, Hkv, d, bs, ctx, Ms, depth=4, branch=3, n_chain=0, n_lay
                                                  table[b], ctx[b])
             util.compare(util.widen_t(out[l, b, :m]), o_out, dtype, f"out l{l} b{b}")
             np.testing.assert_allclose(lse[l, b, :m].cpu().numpy(), o_lse, atol=2e-5 if dtype == "fp32" else 5e-3)
+            if float32_weights:
+                err = out[l, b, :m].double().cpu().numpy() - o_out
+                assert np.sqrt((err ** 2).mean() / (o_out ** 2).mean()) < 1.2e-5
+                np.testing.assert_allclose(lse[l, b, :m].cpu().numpy(), o_lse, rtol=3e-7, atol=2e-6)
             # rows past q_lens[b] are not written
             assert torch.all(out[l, b, m:].float() == 77.0)
 
@@ -127,6 +132,21 @@ def test_packed_rows_and_alternating_streams(Hq, Hkv, d, bs, ctx, Ms, n_chain):
     """Group sizes that do not divide 128 (rows of a tile left over), head size 64, and sequences of one row tile,
     whose two streams take alternate K/V tiles: 0 to 5 context tiles, ragged last tiles, row counts at the tile edge."""
     run_case("bf16", Hq, Hkv, d, bs, ctx=ctx, Ms=Ms, n_chain=n_chain, seed=Hq + d + len(ctx))
+
+
+@pytest.mark.parametrize("Hq,Hkv,d", [(8, 2, 64), (1, 1, 64), (10, 2, 128), (7, 1, 128), (130, 1, 64)])
+@pytest.mark.parametrize("bs,ctx,Ms,n_layers", [
+    (64, [0, 129], [9, 7], 1),             # no context; a tile and one token
+    (16, [128 * 11 + 5], [26], 24),        # one and two row tiles, few KV splits
+    (32, [128 * 9, 100], [64, 33], 1),     # one CTA per few tiles, merged
+])
+def test_weights_keep_their_float32_precision(Hq, Hkv, d, bs, ctx, Ms, n_layers):
+    """bfloat16 caches with head size 64 or a group size that does not divide 128 (and, on the plain kernel, more than 128
+    query heads per KV head): weights in float32, or in two bfloat16 terms that hold them to 2^-18 = 3.8e-6.  The tensor core
+    cuts a sum to 2^-24 of itself after every 16 tokens and term, 16 times a tile: for 12 tiles 192 x 6e-8 = 1.1e-5 at most.  (One
+    bfloat16 term is off by 2^-9 / sqrt(3) = 1.1e-3 a weight.)  A log-sum-exp is rounded once, 2^-24 = 6e-8 of itself, and holds the
+    error of the scores, d / 16 cuts of 2^-24 = 4.8e-7 of a score at most, 2.4e-7 on average, before the mean is put back."""
+    run_case("bf16", Hq, Hkv, d, bs, ctx=ctx, Ms=Ms, n_layers=n_layers, seed=Hq + d + len(ctx), float32_weights=True)
 
 
 @pytest.mark.parametrize("Hq,Hkv,d", [(8, 2, 64), (5, 1, 128)])
