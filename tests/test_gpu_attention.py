@@ -160,6 +160,29 @@ def test_float32_kernel_tile_edges(Hq, Hkv, d, bs, ctx, Ms, n_chain):
     run_case("fp32", Hq, Hkv, d, bs, ctx=ctx, Ms=Ms, n_chain=n_chain, seed=Hq + bs)
 
 
+@pytest.mark.parametrize("d,value", [(64, 0.1), (128, 0.7)])
+def test_float32_kernel_sums_over_long_ranges(d, value):
+    """Equal weights and equal values over 4096 tokens that one CTA walks (enough heads that the KV range is not split): the output
+    is that value.  Sums of 64 tokens added up are off by some 64 x 2^-25 = 1.9e-6 at most, 9e-7 when simulated; one chain
+    of 4096 additions drifts by 4e-5 for these values."""
+    dev = "cuda"
+    Hkv, bs, n, batch = 8, 64, 4096, 74
+    cfg = B.make_config(1, Hkv, Hkv, d, bs, "fp32", 1, 1, 3, bs)
+    k_pool = torch.randn((1, n // bs, Hkv, bs, d), generator=torch.Generator().manual_seed(d)).to(dev)
+    v_pool = torch.full_like(k_pool, value)
+    table = torch.arange(n // bs, dtype=torch.int32, device=dev).repeat(batch, 1)
+    cache = B.Cache(k_pool, v_pool, table, torch.full((batch,), n, dtype=torch.int32, device=dev), n)
+    q = torch.zeros((1, batch, 1, Hkv, d), device=dev)  # equal weights
+    kv_new = torch.full((1, batch, 1, Hkv, d), value, device=dev)
+    mask = torch.ones((batch, 1, 1), dtype=torch.int64, device=dev)
+    ws = B.new_workspace(cfg, 1, batch, n, 1)
+    out = torch.zeros_like(q)
+    B.specpv_verify_full(cfg, 0, 1, q, kv_new, kv_new, mask, None, 1, cache, out, None, ws)
+    util.sync_status(ws)
+    want = kv_new[0, 0, 0, 0, 0].double()
+    assert ((out.double() - want).abs().max() / want).item() < 2e-6
+
+
 @pytest.mark.parametrize("M,n_layers", [(60, 20), (90, 12), (26, 24)])
 def test_many_layers_and_one_layer_agree_with_the_oracle(M, n_layers):
     """The row tiles per CTA and the KV splits depend on how many CTAs a launch has: two row tiles without splits, a last
