@@ -41,7 +41,9 @@ constexpr int kMaxSplitCtas = 8 * 148;  // the workspace holds split-KV partial 
 // all earlier work on the stream is complete and visible; every kernel calls it before it reads or writes anything in
 // global memory that a call passes in (L2 prefetches excepted), so the results are those of plain stream order.  A kernel
 // that holds tensor memory triggers after it has allocated it: a later kernel's allocation can only wait for one that is
-// already held, never the other way round.  The attention kernel triggers when it has written its partial results: merge
+// already held, never the other way round.  While such a kernel runs, its predecessor may still be writing what it will read: it uses
+// plain loads behind pdl_wait(), never loads through the read-only path (__ldg, const __restrict__ parameters), which are promised
+// memory that nobody writes during the kernel and which the compiler may move ahead of the wait.  The attention kernel triggers when it has written its partial results: merge
 // CTAs let in earlier pile up on the few SMs that it leaves free and run there one behind the other (one layer, 4096 tokens:
 // 18.5 us against 16.8).  One layer's QKV projection, partial verification and output projection: 49.1 -> 43.7 us at a
 // 4096-token budget, 43.7 -> 38.0 us at 2048.

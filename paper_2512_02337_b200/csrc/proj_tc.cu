@@ -72,12 +72,12 @@ __device__ __forceinline__ ProjTarget proj_target(const ProjTcParams& p, int til
     t.rope = sg.rope;
     t.add = p.residual && s == 0;
     t.cs = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (t.rope) t.cs = __ldg(reinterpret_cast<const float4*>(p.cos_sin + ((size_t)tok * kHalf + j % (kHalf / 2) * 2) * 2));
+    if (t.rope) t.cs = *reinterpret_cast<const float4*>(p.cos_sin + ((size_t)tok * kHalf + j % (kHalf / 2) * 2) * 2);
     const size_t off = ((size_t)l * p.tokens + tok) * sg.row_stride + (size_t)(tile - sg.first_tile) * kFeatTile + feature_of<kHalf>(j);
     t.res[0] = t.res[1] = 0;
     if (t.add) {
-        t.res[0] = __ldg(reinterpret_cast<const uint32_t*>(p.residual + off));
-        t.res[1] = __ldg(reinterpret_cast<const uint32_t*>(p.residual + off + kHalf));
+        t.res[0] = *reinterpret_cast<const uint32_t*>(p.residual + off);
+        t.res[1] = *reinterpret_cast<const uint32_t*>(p.residual + off + kHalf);
     }
     t.dst = reinterpret_cast<__nv_bfloat16*>(sg.base) + off;
     return t;
@@ -219,16 +219,24 @@ __global__ void __launch_bounds__(kProjThreads, 2) proj_tc_kernel(const __grid_c
         asm volatile("bar.sync 1, 128;" ::: "memory");
         if (ok) {
             const int et = threadIdx.x - 64, j = et & 31, feat = feature_of<kHalf>(j);
-            float* part = p.splits > 1 ? p.partials + partial_base(p, l, chunk, gridDim.y, tile, split) : nullptr;
+            auto sums = [&](int t, int at) { return *reinterpret_cast<const float2*>(stage + t * kFeatTile + at); };
+            if (p.splits > 1) {
+                float* part = p.partials + partial_base(p, l, chunk, gridDim.y, tile, split);
 #pragma unroll 4
-            for (int t = et >> 5; t < valid; t += 4) {
-                const float2 lo = *reinterpret_cast<const float2*>(stage + t * kFeatTile + feat);
-                const float2 hi = *reinterpret_cast<const float2*>(stage + t * kFeatTile + feat + kHalf);
-                if (part) {
-                    *reinterpret_cast<float2*>(part + (size_t)t * kFeatTile + feat) = lo;
-                    *reinterpret_cast<float2*>(part + (size_t)t * kFeatTile + feat + kHalf) = hi;
-                } else {
-                    proj_finish<kHalf>(proj_target<kHalf>(p, tile, l, tok0 + t, j), lo, hi);
+                for (int t = et >> 5; t < valid; t += 4) {
+                    *reinterpret_cast<float2*>(part + (size_t)t * kFeatTile + feat) = sums(t, feat);
+                    *reinterpret_cast<float2*>(part + (size_t)t * kFeatTile + feat + kHalf) = sums(t, feat + kHalf);
+                }
+            } else {
+                constexpr int kAhead = 4;  // rows whose angles and residual are in flight together
+                for (int t0 = et >> 5; t0 < valid; t0 += 4 * kAhead) {
+                    ProjTarget target[kAhead];
+#pragma unroll
+                    for (int u = 0; u < kAhead; ++u)
+                        if (t0 + 4 * u < valid) target[u] = proj_target<kHalf>(p, tile, l, tok0 + t0 + 4 * u, j);
+#pragma unroll
+                    for (int u = 0; u < kAhead; ++u)
+                        if (t0 + 4 * u < valid) proj_finish<kHalf>(target[u], sums(t0 + 4 * u, feat), sums(t0 + 4 * u, feat + kHalf));
                 }
             }
         }
@@ -260,8 +268,8 @@ __global__ void __launch_bounds__(128) proj_reduce_kernel(const __grid_constant_
 #pragma unroll
     for (int s = 0; s < 8; ++s)
         if (s < p.splits) {
-            a[s] = __ldg(reinterpret_cast<const float2*>(part + s * split_stride));
-            b[s] = __ldg(reinterpret_cast<const float2*>(part + s * split_stride + kHalf));
+            a[s] = *reinterpret_cast<const float2*>(part + s * split_stride);
+            b[s] = *reinterpret_cast<const float2*>(part + s * split_stride + kHalf);
         }
     float2 lo = make_float2(0.f, 0.f), hi = lo;
 #pragma unroll
@@ -324,9 +332,8 @@ __global__ void __launch_bounds__(128) proj_simt_kernel(const __grid_constant__ 
 }
 
 // ---- positions and rotary angles of a step's rows ------------------------------------------------------------
-__global__ void rope_table_kernel(const uint64_t* __restrict__ tree_mask, const int32_t* __restrict__ q_lens,
-                                  const int32_t* __restrict__ base_pos, int M_max, int d, double theta,
-                                  float* __restrict__ cos_sin) {
+__global__ void rope_table_kernel(const uint64_t* tree_mask, const int32_t* q_lens, const int32_t* base_pos, int M_max, int d,
+                                  double theta, float* cos_sin) {
     pdl_trigger();
     pdl_wait();
     const int row = blockIdx.x, b = row / M_max, j = row % M_max;

@@ -205,3 +205,48 @@ def test_projections_at_full_size_in_the_benchmark_launch(name, layers):
             util.compare(util.widen_t(v_new[l, b]), ov, "bf16", f"v layer {l} seq {b}")
             util.compare(util.widen_t(y[l, b]), oracle.linear(xb, wo, wl.to_numpy(bw.residual[l, b])), "bf16",
                          f"block output layer {l} seq {b}")
+
+
+@pytest.mark.parametrize("M,hidden", [(24, 1024), (70, 512)])
+def test_projections_follow_the_calls_before_them_without_a_pause(M, hidden):
+    """Commit, rope table at the lengths that the commit has just advanced, QKV projection and output projection onto its own last
+    result, forty times back to back: every call reads what the one before it writes while both are resident.  Positions
+    exactly, the projections to the rounding of their bfloat16 results (the sums before it are float32)."""
+    Hq, Hkv, d, steps, theta, dev = 8, 2, 128, 40, 1.0e4, "cuda"
+    dt = torch.bfloat16
+    g = torch.Generator().manual_seed(M)
+    cfg = make_cfg("bf16", Hq, Hkv, d, 1)
+    parents = [wl.make_tree(M, 6, 4, np.random.default_rng(M))]
+    masks = util.device_masks(parents, M)
+    x = rand((steps, 1, 1, M, hidden), dt, g)
+    w_qkv, w_o = rand((1, (Hq + 2 * Hkv) * d, hidden), dt, g, hidden ** -0.5), rand((1, hidden, Hq * d), dt, g, (Hq * d) ** -0.5)
+    n_pages = 8
+    pool = torch.zeros((1, n_pages, Hkv, 64, d), dtype=dt, device=dev)
+    cache = B.Cache(pool, torch.zeros_like(pool), torch.arange(n_pages, dtype=torch.int32, device=dev)[None],
+                    torch.tensor([5], dtype=torch.int32, device=dev), n_pages * 64)
+    ws = B.new_workspace(cfg, 1, 1, n_pages * 64, M)
+    accepted = torch.zeros((1, 4), dtype=torch.int32, device=dev)
+    n_acc = torch.tensor([3], dtype=torch.int32, device=dev)
+    k_new, v_new = torch.zeros((2, 1, 1, M, Hkv, d), dtype=dt, device=dev)
+    cos_sin = torch.zeros((steps, 1, M, d // 2, 2), dtype=torch.float32, device=dev)
+    q = torch.zeros((steps, 1, 1, M, Hq, d), dtype=dt, device=dev)
+    y = torch.zeros((steps + 1, 1, 1, M, hidden), dtype=dt, device=dev)
+    for i in range(steps):
+        B.specpv_commit_accepted(cfg, 0, 1, k_new, v_new, M, accepted, n_acc, 4, cache, None, None, ws)
+        B.specpv_rope_table(cfg, masks, None, cache.seq_lens, 1, M, theta, cos_sin[i])
+        B.specpv_qkv_rope(cfg, 0, 1, x[i], hidden, w_qkv, cos_sin[i], 1, M, q[i], k_new, v_new, ws)
+        B.specpv_o_proj(cfg, 0, 1, q[i], w_o, hidden, y[i], 1, M, y[i + 1], ws)
+    util.sync_status(ws)
+    for i in range(steps):
+        c, s = oracle_cos_sin(oracle.step_positions(parents[0], 0, 5 + 3 * (i + 1)), d, theta)
+        np.testing.assert_allclose(cos_sin[i, 0, :, :, 0].cpu().numpy(), c, atol=1e-7, err_msg=f"step {i}")
+        np.testing.assert_allclose(cos_sin[i, 0, :, :, 1].cpu().numpy(), s, atol=1e-7, err_msg=f"step {i}")
+        proj = (x[i, 0, 0].double() @ w_qkv[0, :Hq * d].double().T).view(M, Hq, d)
+        lo, hi = proj[..., :d // 2], proj[..., d // 2:]
+        cos, sin = cos_sin[i, 0].double()[:, None].unbind(-1)
+        want = {"q": (torch.cat([lo * cos - hi * sin, hi * cos + lo * sin], -1), q[i, 0, 0]),
+                "y": (q[i, 0, 0].double().reshape(M, -1) @ w_o[0].double().T + y[i, 0, 0].double(), y[i + 1, 0, 0])}
+        for name, (exact, got) in want.items():
+            # half a unit in the last place of a bfloat16 with its 8 significant bits is at most 2^-8 of the value (just above a
+            # power of two); the float32 sums of up to 1024 terms below 16 before it: 1e-5
+            assert ((got.double() - exact).abs() <= exact.abs() * 2.0 ** -8 + 1e-5).all(), (name, i)

@@ -187,3 +187,13 @@ def test_native_argument_conversion(bad, error):
     with pytest.raises(error) as e:
         B.specpv_verify_full(**args)
     assert bad is not None or e.value.status == 1
+
+
+def test_overlapped_kernels_load_nothing_through_the_read_only_path():
+    """A kernel launched as a programmatic dependent runs while its predecessor may still be writing what it will read, so no
+    source that launches one holds a non-coherent load: __ldg, ld.global.nc, or const __restrict__ kernel parameters."""
+    sources = {p.name: re.sub(r"//[^\n]*", "", p.read_text()) for p in sorted((ROOT / "paper_2512_02337_b200" / "csrc").glob("*.cu"))}
+    overlapped = {n: s for n, s in sources.items() if re.search(r"\blaunch_pdl(_if)?\(|SPECPV_LAUNCH\(", s)}
+    assert {"attn_tc.cu", "attn_simt.cu", "aux_kernels.cu", "proj_tc.cu", "score_tc.cu"} <= set(overlapped)
+    for name, text in overlapped.items():
+        assert not re.findall(r"__ldg\s*\(|ld\.global\.nc|__restrict__", text), name
