@@ -992,11 +992,16 @@ specpv_status launch_attention_tc(const AttnArgs& a, cudaStream_t stream) {
     const int positions = (a.max_seq_len + kTileTokens - 1) / kTileTokens + 1;  // context tiles + the tile of the step's own tokens
     const double row_bytes = (double)n_units * a.M_max * G * (a.g.d + 2) * sizeof(float);  // partial results of a split
     const double tile_bytes = (double)n_units * 128 * (a.g.d + 2) * sizeof(float);
+    // The partial rows are stored 32 bytes at a time and a workspace need only be 16-byte aligned: they start at the next multiple of
+    // 32, and the 16 bytes before it are not counted as scratch.
+    char* ws = reinterpret_cast<char*>(a.workspace) + a.partial_off;
+    const size_t skip = (32 - (reinterpret_cast<uintptr_t>(ws) & 31)) & 31;
+    const double scratch = (double)a.partial_bytes - (double)skip;
     double best_cost = 1e30;
     for (int rg_tiles = row_tiles > 1 ? 2 : 1; rg_tiles >= 1; --rg_tiles) {
         const int groups = (row_tiles + rg_tiles - 1) / rg_tiles, full = row_tiles / rg_tiles;
         for (int s = 1; s <= 64 && s <= positions; ++s) {
-            if (s > 1 && tile_bytes * s * groups * rg_tiles > (double)a.partial_bytes) break;
+            if (s > 1 && tile_bytes * s * groups * rg_tiles > scratch) break;
             const int tiles = (positions + s - 1) / s;
             const double t1 = 7.0 + 0.9 * tiles + (s > 1 ? 1.5 : 0.0), t2 = 7.0 + 1.5 * tiles + (s > 1 ? 4.0 : 0.0);
             const long long n_long = (long long)n_units * s * full, n_short = (long long)n_units * s * (groups - full);
@@ -1013,9 +1018,8 @@ specpv_status launch_attention_tc(const AttnArgs& a, cudaStream_t stream) {
     p.n_full_groups = row_tiles / p.rg_tiles;
     p.n_full_units = n_units * p.n_full_groups;
     p.R_pad = p.n_row_groups * p.rg_tiles * 128;
-    char* ws = reinterpret_cast<char*>(a.workspace) + a.partial_off;
-    p.part_o = reinterpret_cast<float*>(ws);
-    p.part_ml = reinterpret_cast<float*>(ws + (size_t)n_units * p.n_splits * p.R_pad * a.g.d * sizeof(float));
+    p.part_o = reinterpret_cast<float*>(ws + skip);
+    p.part_ml = reinterpret_cast<float*>(ws + skip + (size_t)n_units * p.n_splits * p.R_pad * a.g.d * sizeof(float));
 
     const int n_lb = a.n_layers * a.batch;
     if (a.g.d == 64) return launch_kernels<64, true>(p, n_lb, stream);

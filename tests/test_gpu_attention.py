@@ -160,6 +160,36 @@ def test_float32_kernel_tile_edges(Hq, Hkv, d, bs, ctx, Ms, n_chain):
     run_case("fp32", Hq, Hkv, d, bs, ctx=ctx, Ms=Ms, n_chain=n_chain, seed=Hq + bs)
 
 
+@pytest.mark.parametrize("Hq,Hkv,d,ctx,n_layers", [(8, 2, 64, 3000, 1), (10, 2, 128, 3000, 1), (32, 8, 128, 700, 1),
+                                                   (32, 8, 128, 6000, 4)])
+def test_workspace_off_a_32_byte_boundary(Hq, Hkv, d, ctx, n_layers):
+    """A workspace needs 16-byte alignment and no more: 16 bytes past a multiple of 32, as large as the call asks for and not a
+    byte larger, gives what an aligned one gives, and nothing before or behind it is written."""
+    dev, bs, M = "cuda", 64, 20
+    g = torch.Generator().manual_seed(ctx + d)
+    bf = lambda *shape: torch.randn(shape, generator=g).to(torch.bfloat16).to(dev)  # noqa: E731
+    n_pages = (ctx + bs - 1) // bs
+    pools, q = bf(2, n_layers, n_pages, Hkv, bs, d), bf(n_layers, 1, M, Hq, d)
+    k_new, v_new = bf(2, n_layers, 1, M, Hkv, d)
+    cache = B.Cache(pools[0], pools[1], torch.arange(n_pages, dtype=torch.int32, device=dev)[None],
+                    torch.tensor([ctx], dtype=torch.int32, device=dev), ctx)
+    mask = util.device_masks([wl.make_tree(M, 5, 4, np.random.default_rng(1))], M)
+    cfg = B.make_config(n_layers, Hq, Hkv, d, bs, "bf16", 1, 1, 3, bs, out_f32=1)
+    n = B.specpv_workspace_bytes(cfg, n_layers, 1, ctx, M)
+    results = []
+    for offset in (0, 16):
+        buf = torch.full((n + 4096,), 0x5A, dtype=torch.uint8, device=dev)
+        ws = buf[1024 + offset:1024 + offset + n]
+        assert ws.data_ptr() % 32 == offset
+        ws.zero_()
+        out, lse = torch.zeros_like(q, dtype=torch.float32), torch.zeros((n_layers, 1, M, Hq), device=dev)
+        B.specpv_verify_full(cfg, 0, n_layers, q, k_new, v_new, mask, None, M, cache, out, lse, ws)
+        util.sync_status(ws)
+        assert (buf[:1024 + offset] == 0x5A).all() and (buf[1024 + offset + n:] == 0x5A).all()
+        results.append((out, lse))
+    assert torch.equal(results[0][0], results[1][0]) and torch.equal(results[0][1], results[1][1])
+
+
 @pytest.mark.parametrize("d,value", [(64, 0.1), (128, 0.7)])
 def test_float32_kernel_sums_over_long_ranges(d, value):
     """Equal weights and equal values over 4096 tokens that one CTA walks (enough heads that the KV range is not split): the output
