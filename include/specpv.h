@@ -106,10 +106,13 @@ typedef struct {
 const char *specpv_status_string(specpv_status s);
 
 /* Bytes of device workspace that any call below needs for the given limits.  The first
- * SPECPV_WORKSPACE_HEAD_BYTES hold the device status word and the arrival counters of the commit and
- * of KV ranges that several CTAs share; the caller zeroes them once (cudaMemset) before first use and the library
+ * SPECPV_WORKSPACE_HEAD_BYTES hold the device status word and the arrival counters of KV ranges that
+ * several CTAs share; the caller zeroes them once (cudaMemset) before first use and the library
  * leaves them zero after every call that completes (after SPECPV_ERR_TIMEOUT zero them again).  The
- * rest is scratch (split-KV partial results, host-call staging) with no state between calls. */
+ * rest is scratch (split-KV partial results, partial sums of the projections, host-call staging) with no state between
+ * calls.  Calls whose work can overlap on the GPU (different streams without an ordering between them) need a workspace
+ * each if they are verify or projection calls; the others (summaries, scores, selection, refresh, commit) touch
+ * the status word only and may share one. */
 #define SPECPV_WORKSPACE_HEAD_BYTES (256u << 10)
 size_t specpv_workspace_bytes(const specpv_config *cfg, int n_layers_per_call, int max_batch,
                               int max_seq_len, int M_max);

@@ -510,8 +510,7 @@ SPECPV_EXPORT specpv_status specpv_commit_accepted(const specpv_config* cfg, int
     p.kmax = kmax; p.kmin = kmin; p.workspace = workspace;
     p.layer0 = layer0; p.batch = dst->batch; p.M_max = M_max; p.A_max = A_max; p.Hkv = g.Hkv; p.bs = g.bs; p.d = g.d;
     p.max_blocks = dst->max_blocks; p.n_pages = dst->n_pages;
-    p.advance = layer0 + n_layers == g.n_layers;
-    return launch_commit(p, n_layers, g.dtype, s);
+    return launch_commit(p, n_layers, g.dtype, layer0 + n_layers == g.n_layers, s);
 }
 
 // ---- the linear maps either side of the attention --------------------------------------------------------------

@@ -477,18 +477,17 @@ __global__ void __launch_bounds__(128) gather_kernel(GatherParams p) {
 
 // ---------------------------------------------------------------------------------------------
 // Commit: grid = (blocks touched, Hkv, layers x seqs); a CTA appends the accepted tokens' K and V rows that fall into one
-// block (a warp per row) and recomputes the block's summary, the appended tokens taken from the step's tensors.  The CTA
-// that finishes last advances the lengths (an arrival counter behind the status word, left at zero): every CTA has read
-// them by then.  One launch where rows, summaries and lengths took three: 4-5 us
-// less host time per call, and on the device 12.5 us against 15.2 for the 46 rows of a refresh (36 layers), 7.5 against 6.9 for
-// four rows (the arrival).
+// block (a warp per row) and recomputes the block's summary, the appended tokens taken from the step's tensors.  The lengths
+// advance in a launch behind it: every CTA reads them, and a commit keeps nothing in the workspace but the status word, so that
+// commits of two caches on two streams may share one (an arrival counter there made the launch unnecessary, 9.3 us a call against
+// 11.4, but mixed the arrivals of two such commits).  Bound by launches: rows, summaries and lengths in three took 14 us of host
+// time a call.
 // ---------------------------------------------------------------------------------------------
 constexpr int kCommitWarps = 4;
 
 template <typename T>
 __global__ void __launch_bounds__(32 * kCommitWarps) commit_kernel(CommitParams p) {
     pdl_begin(p.pdl);
-    __shared__ int s_last;
     const int h = blockIdx.y, lb = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int b = lb % p.batch, l = lb / p.batch;
     const int n = min(max(p.n_accepted[b], 0), p.A_max);
@@ -572,22 +571,15 @@ __global__ void __launch_bounds__(32 * kCommitWarps) commit_kernel(CommitParams 
                           ((((size_t)(p.layer0 + l) * p.batch + b) * p.Hkv + h) * p.max_blocks + i) * chunks + chunk);
         }
     }
-    if (!p.advance) return;
-    __syncthreads();  // the whole CTA has read the lengths
-    if (threadIdx.x == 0) {
-        int32_t* arrived = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(p.workspace) + kCommitCounterOffset);
-        __threadfence();
-        const int total = (int)(gridDim.x * gridDim.y * gridDim.z);
-        s_last = atomicAdd(arrived, 1) == total - 1;
-        if (s_last) *arrived = 0;
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    for (int bb = threadIdx.x; bb < p.batch; bb += 32 * kCommitWarps) {
-        const int nn = min(max(p.n_accepted[bb], 0), p.A_max);
-        if ((size_t)p.seq_lens[bb] + nn <= (size_t)p.max_blocks * p.bs) p.seq_lens[bb] += nn;
-    }
+}
+
+constexpr int kLensThreads = 128;
+__global__ void __launch_bounds__(kLensThreads) commit_lens_kernel(CommitParams p) {
+    pdl_begin(p.pdl);
+    const int b = blockIdx.x * kLensThreads + threadIdx.x;
+    if (b >= p.batch) return;
+    const int n = min(max(p.n_accepted[b], 0), p.A_max);
+    if ((size_t)p.seq_lens[b] + n <= (size_t)p.max_blocks * p.bs) p.seq_lens[b] += n;
 }
 
 }  // namespace
@@ -646,11 +638,12 @@ specpv_status launch_gather(const GatherParams& p, int n_layers, cudaStream_t st
     return SPECPV_OK;
 }
 
-specpv_status launch_commit(const CommitParams& params, int n_layers, int dtype, cudaStream_t stream) {
+specpv_status launch_commit(const CommitParams& params, int n_layers, int dtype, bool advance, cudaStream_t stream) {
     CommitParams p = params;
     p.aligned = aligned16(p.kmax) && aligned16(p.kmin);
     dim3 grid((p.A_max + p.bs - 1) / p.bs + 1, p.Hkv, n_layers * p.batch);
     SPECPV_LAUNCH(dtype == SPECPV_DTYPE_F32 ? commit_kernel<float> : commit_kernel<__nv_bfloat16>, grid, 32 * kCommitWarps, 0, stream, p);
+    if (advance) SPECPV_LAUNCH(commit_lens_kernel, dim3((p.batch + kLensThreads - 1) / kLensThreads), kLensThreads, 0, stream, p);
     return SPECPV_OK;
 }
 

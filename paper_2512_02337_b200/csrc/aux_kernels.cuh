@@ -70,7 +70,6 @@ struct CommitParams {
     void* kmin;
     void* workspace;
     int layer0, batch, M_max, A_max, Hkv, bs, d, max_blocks, n_pages;
-    int advance;  // this call holds the model's last layer: the lengths advance
     int aligned;  // set by the launcher: kmax and kmin take 16-byte stores
     int pdl;      // set by launch_pdl_if
 };
@@ -82,6 +81,7 @@ specpv_status launch_scores_tc(const ScoreParams& p, int n_layers_call, int n_la
                                cudaStream_t stream);
 specpv_status launch_select(const SelectParams& p, int n_layers, cudaStream_t stream);
 specpv_status launch_gather(const GatherParams& p, int n_layers, cudaStream_t stream);
-specpv_status launch_commit(const CommitParams& p, int n_layers, int dtype, cudaStream_t stream);
+// advance: this call holds the model's last layer, the lengths advance
+specpv_status launch_commit(const CommitParams& p, int n_layers, int dtype, bool advance, cudaStream_t stream);
 
 }  // namespace specpv

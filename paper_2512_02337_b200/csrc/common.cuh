@@ -28,7 +28,6 @@ __device__ __forceinline__ void record_fault(void* workspace, int code, int i0, 
 }
 
 constexpr size_t kStatusBytes = 256;
-constexpr size_t kCommitCounterOffset = 128;  // arrival counter of the commit kernel, zero between launches
 // Head of every workspace: the status word, then arrival counters of KV ranges shared between CTAs (two per (layer,
 // sequence, KV head, group of 256 rows) of a call; zero between launches).  All scratch starts behind it.
 constexpr size_t kHeaderBytes = 256 * 1024;

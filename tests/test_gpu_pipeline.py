@@ -285,6 +285,35 @@ def test_commit_in_layer_groups_matches_the_oracle():
     assert np.array_equal(wl.to_numpy(w.k_pool), kp0) and np.array_equal(wl.to_numpy(w.v_pool), vp0)
 
 
+def test_commits_of_two_caches_on_two_streams_share_a_workspace():
+    """A commit keeps nothing in the workspace but the status word: commits of the full cache on one stream and of the partial
+    cache on another, unordered, over one workspace, advance either cache's lengths by what was accepted, every time, and
+    leave the workspace as it was."""
+    dev, L, Hkv, d, bs, M, steps = "cuda", 36, 8, 128, 64, 8, 25
+    cfg = B.make_config(L, 32, Hkv, d, bs, "bf16", 1, 2, 8, bs)
+    k_new, v_new = (torch.randn((L, 1, M, Hkv, d), device=dev).to(torch.bfloat16) for _ in range(2))
+    caches = []
+    for n_pages in (12, 6):
+        pool = torch.zeros((2, L, n_pages, Hkv, bs, d), dtype=torch.bfloat16, device=dev)
+        caches.append(B.Cache(pool[0], pool[1], torch.arange(n_pages, dtype=torch.int32, device=dev)[None],
+                              torch.tensor([3], dtype=torch.int32, device=dev), n_pages * bs))
+    acc = torch.tensor([[4, 0, 6, 1]], dtype=torch.int32, device=dev)
+    counts = [torch.tensor([n], dtype=torch.int32, device=dev) for n in (4, 2)]
+    ws = torch.zeros(B.WORKSPACE_HEAD_BYTES, dtype=torch.uint8, device=dev)
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    torch.cuda.synchronize()
+    for _ in range(steps):
+        for s, cache, n in zip(streams, caches, counts):
+            B.specpv_commit_accepted(cfg, 0, L, k_new, v_new, M, acc, n, 4, cache, None, None, ws, stream=s)
+    torch.cuda.synchronize()
+    assert not ws.any()
+    for cache, n in zip(caches, (4, 2)):
+        assert int(cache.seq_lens[0]) == 3 + steps * n
+        for pool, new in ((cache.k_pool, k_new), (cache.v_pool, v_new)):
+            flat = pool.permute(0, 1, 3, 2, 4).reshape(L, -1, Hkv, d)
+            assert torch.equal(flat[:, 3:3 + steps * n], new[:, 0][:, acc[0, :n].long()].repeat(1, steps, 1, 1))
+
+
 @pytest.mark.parametrize("nb,budget", [(300, 40), (2048, 64), (4099, 128), (9000, 1000)])
 def test_selection_alone_on_synthetic_scores_with_ties_and_nan(nb, budget):
     """The selection kernel on its own: more candidate blocks than it keeps in registers (nb > 4096), repeated
