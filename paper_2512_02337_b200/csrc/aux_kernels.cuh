@@ -76,7 +76,7 @@ struct CommitParams {
 
 specpv_status launch_summaries(const SummaryParams& p, int n_layers, int blocks_touched, int dtype, cudaStream_t stream);
 specpv_status launch_scores(const ScoreParams& p, int n_layers, int max_nb, int dtype, int d, cudaStream_t stream);
-bool scores_tc_supported(int dtype, int d, int G, int M_max);
+bool scores_tc_supported(const ScoreParams& p, int dtype, int d);
 specpv_status launch_scores_tc(const ScoreParams& p, int n_layers_call, int n_layers_total, int max_nb, int d,
                                cudaStream_t stream);
 specpv_status launch_select(const SelectParams& p, int n_layers, cudaStream_t stream);

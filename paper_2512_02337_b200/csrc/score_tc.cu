@@ -23,10 +23,11 @@
 //   warps 4-11  epilogue: thread <-> block of the tile (tensor-memory lane) and one half of the query rows; reduces
 //               over its rows (mean, max, or the rows of the "last" query); the two halves meet in shared memory, the
 //               lower half picking the upper half's result up one tile later
-// Bound by HBM on the summaries, and by the tensor pipe above some 192 rows.  Any group size and both head sizes run here, since a
-// pass's query rows are dense in shared memory and columns beyond them are simply not reduced; the plain kernel, on which
-// group sizes that do not divide 128 and head size 64 ran before, is bound by its multiplications (16384 tokens x 24 layers,
-// 60 x 5 rows of 128: 371 -> 23 us, with 16-token blocks 1368 -> 57; 60 x 4 rows of 64: 152 -> 10 us and 534 -> 22).
+// Bound by HBM on the summaries, and by the tensor pipe above some 192 rows.  Any group size and both head sizes can run here, since a
+// pass's query rows are dense in shared memory and columns beyond them are simply not reduced; the plain kernel, which
+// takes group sizes that do not divide 128 and head size 64 where it is the more exact one (scores_tc_supported), is bound by its
+// multiplications (16384 tokens x 24 layers, 60 x 5 rows of 128: 371 us there, 23 here, with 16-token blocks 1368 and 57; 60 x 4
+// rows of 64: 152 and 10, 534 and 22).
 // Every wait is bounded; after a wait that gave up the loops end and nothing more is copied or issued.
 #include "aux_kernels.cuh"
 #include "tc_common.cuh"
@@ -470,9 +471,17 @@ __global__ void __launch_bounds__(kScoreThreads, 1) scores_tc_kernel(const __gri
 
 // More than 1024 rows per KV head (a group of 33 x 33 step tokens) would take more than four passes over the summaries; no
 // configuration comes near, and the plain kernel takes them.
-bool scores_tc_supported(int dtype, int d, int G, int M_max) {
-    return dtype == SPECPV_DTYPE_BF16 && (d == 128 || d == 64) && G <= 128 && M_max * G <= 4 * 256 &&
-           tc::get_encode_fn() != nullptr;
+// The tensor core truncates its sums, which makes a score 4.6e-8 to 14e-8 of itself too small; the plain kernel rounds, but adds a mean
+// over many rows up in one chain.  Head size 64 and group sizes that do not divide 128 run here where that makes the more exact
+// result: means of the full dot products over 32 rows or more (relative 2-norm errors against float64, here / plain: 240 rows of 128
+// 7.3e-8 / 2.3e-7, 32 rows of 64 4.8e-8 / 8.5e-8, 10 rows of 128 7.3e-8 / 5.8e-8; maxima, 240 rows of 128, 7.6e-8 / 4.9e-8;
+// channel-wise, one row of 128, 1.6e-7 / 5.7e-8).  Also left to the plain kernel, for what it makes of them: per-sequence row
+// counts, of which one may be 0 (the mean over no rows is NaN), and channel-wise scores of infinite keys (0 x infinity here).
+bool scores_tc_supported(const ScoreParams& p, int dtype, int d) {
+    if (dtype != SPECPV_DTYPE_BF16 || (d != 128 && d != 64) || p.G > 128 || p.M_max * p.G > 4 * 256) return false;
+    const bool few_or_other = p.reduce != SPECPV_REDUCE_MEAN || p.score_mode != 0 || p.q_lens != nullptr || p.M_max * p.G < 32;
+    if ((d == 64 || 128 % p.G != 0) && few_or_other) return false;
+    return tc::get_encode_fn() != nullptr;
 }
 
 template <int D>

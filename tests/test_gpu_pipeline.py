@@ -384,9 +384,9 @@ def test_verify_host_matches_the_device_call_and_the_oracle(name, L, over):
                                         ("bf16", 66, 64)])
 @pytest.mark.parametrize("reduce,score_mode", [(B.REDUCE_MEAN, 0), (B.REDUCE_MAX, 1), (B.REDUCE_LAST, 0)])
 def test_scores_of_the_plain_kernel(dtype, Hq, d, reduce, score_mode):
-    """What the tensor-core score kernel does not take, float32 and more than 1024 rows per KV head (33 x 33), and two
-    shapes that it does take; block counts around the 32 a CTA of the plain kernel takes, row counts that leave warps
-    without rows."""
+    """What the tensor-core score kernel does not take: float32, more than 1024 rows per KV head (33 x 33), and head size 64 or a
+    group size that does not divide 128 with per-sequence row counts; block counts around the 32 a CTA of the plain
+    kernel takes, row counts that leave warps without rows."""
     w = wl.make_workload("llama_32k", device="cuda", n_layers=2, Hq=Hq, Hkv=2, d=d, dtype=dtype, M=33,
                          ctx=[64 * 31 + 9, 64 * 33, 64])
     c = w.cfg
@@ -418,8 +418,10 @@ def test_scores_of_the_plain_kernel(dtype, Hq, d, reduce, score_mode):
                                     (8, 64, 64), (96, 128, 6), (256, 64, 5)])
 @pytest.mark.parametrize("reduce,score_mode", [(B.REDUCE_MEAN, 0), (B.REDUCE_MAX, 0), (B.REDUCE_LAST, 1), (B.REDUCE_MEAN, 1)])
 def test_scores_of_any_group_size_on_the_tensor_core_kernel(Hq, d, M, reduce, score_mode):
-    """One to 128 query heads per KV head, both head sizes; rows just below, at and just above the 256 of a pass and the 128
-    of an epilogue half, contractions a little wider than their rows; blocks around the 128 of a tile."""
+    """One to 128 query heads per KV head, both head sizes, ragged row counts: rows just below, at and just above the 256 of a
+    pass and the 128 of an epilogue half, contractions a little wider than their rows; blocks around the 128 of a tile.  (With
+    per-sequence row counts these shapes run on the plain kernel; test_mean_scores_on_the_tensor_core_kernel has such
+    shapes without.)"""
     w = wl.make_workload("llama_32k", device="cuda", n_layers=2, Hq=Hq, Hkv=2, d=d, M=M, ctx=[64 * 128, 64 * 129 - 3, 64 * 5])
     c = w.cfg
     Hkv, batch, L = c["Hkv"], w.batch, c["n_layers"]
@@ -444,6 +446,100 @@ def test_scores_of_any_group_size_on_the_tensor_core_kernel(Hq, d, M, reduce, sc
             # exact products summed in float32, d (twice d in the channel-wise form) to a dot product: as the plain kernel
             np.testing.assert_allclose(scores[l, b, :, :nb].cpu().numpy(), osc, rtol=2e-5, atol=2e-4, err_msg=f"{l} {b}")
             assert torch.isnan(scores[l, b, :, nb:]).all()  # blocks past the context are left alone
+
+
+def score_call(Hq, Hkv, d, M, kmax, kmin, q, lens, bs=64, q_lens=None, reduce=0, score_mode=0):
+    """Scores of one layer for given summaries [batch][Hkv][blocks][d] and queries; -7 where nothing was written."""
+    batch, blocks = kmax.shape[0], kmax.shape[2]
+    cfg = B.make_config(1, Hq, Hkv, d, bs, "bf16", 1, 2, 4, bs, reduce=reduce, score_mode=score_mode)
+    pool = torch.zeros((1, 1, Hkv, bs, d), dtype=torch.bfloat16, device="cuda")
+    cache = B.Cache(pool, pool, torch.zeros((batch, blocks), dtype=torch.int32, device="cuda"),
+                    torch.tensor(lens, dtype=torch.int32, device="cuda"), max(lens))
+    ws = torch.zeros(B.WORKSPACE_HEAD_BYTES, dtype=torch.uint8, device="cuda")
+    scores = torch.full((1, batch, Hkv, blocks), -7.0, device="cuda")
+    rows = None if q_lens is None else torch.tensor(q_lens, dtype=torch.int32, device="cuda")
+    B.specpv_score_blocks(cfg, 0, 1, q, rows, M, None, kmax, kmin, cache, scores, ws)
+    util.sync_status(ws)
+    return scores[0]
+
+
+def score_reference(kmax, kmin, q, Hkv, reduce, score_mode):
+    """[Hkv][blocks] float64 scores of one sequence: kmax, kmin [Hkv][blocks][d], q [rows][Hq][d]."""
+    d = q.shape[-1]
+    rows = q.double().reshape(q.shape[0], Hkv, -1, d)
+    if reduce == B.REDUCE_LAST:
+        rows = rows[:1]
+    rows = rows.permute(1, 0, 2, 3).reshape(Hkv, -1, d)
+    a, z = kmax.double().transpose(1, 2), kmin.double().transpose(1, 2)
+    s = torch.maximum(rows @ a, rows @ z) if score_mode == 0 else rows.clamp(min=0) @ a + rows.clamp(max=0) @ z
+    return s.amax(1) if reduce == B.REDUCE_MAX else s.mean(1)
+
+
+@pytest.mark.parametrize("Hq,Hkv,d,M", [(8, 2, 64, 8), (8, 2, 64, 64), (10, 2, 128, 51), (10, 2, 128, 52), (14, 2, 128, 37),
+                                        (256, 2, 64, 5), (2, 2, 64, 32), (7, 1, 128, 90), (96, 2, 128, 6)])
+def test_mean_scores_on_the_tensor_core_kernel(Hq, Hkv, d, M):
+    """Head size 64 and group sizes that do not divide 128 without per-sequence row counts: 32 rows and just above, just below
+    and above the 256 of a pass, three passes; blocks around the 128 of a tile."""
+    lens = [64 * 128, 64 * 129 - 3, 64 * 5]
+    g = torch.Generator().manual_seed(Hq + M)
+    key = torch.randn((2, 3, Hkv, 129, d), generator=g)
+    kmax, kmin = (t.to(torch.bfloat16).cuda() for t in (key.amax(0), key.amin(0)))
+    q = torch.randn((1, 3, M, Hq, d), generator=g).to(torch.bfloat16).cuda()
+    got = score_call(Hq, Hkv, d, M, kmax, kmin, q, lens)
+    for b, n in enumerate(lens):
+        nb = (n + 63) // 64
+        want = score_reference(kmax[b, :, :nb], kmin[b, :, :nb], q[0, b], Hkv, 0, 0)
+        torch.testing.assert_close(got[b, :, :nb].double(), want, rtol=2e-5, atol=2e-4)
+        assert (got[b, :, nb:] == -7.0).all()
+
+
+@pytest.mark.parametrize("Hq,Hkv,d", [(8, 2, 64), (10, 2, 128), (3, 1, 128)])
+@pytest.mark.parametrize("M,reduce,score_mode", [(60, B.REDUCE_MAX, 0), (60, B.REDUCE_LAST, 0), (60, B.REDUCE_MEAN, 1),
+                                                 (1, B.REDUCE_MEAN, 0), (40, B.REDUCE_MEAN, 0)])
+def test_scores_are_rounded_not_truncated(Hq, Hkv, d, M, reduce, score_mode):
+    """Head size 64 and group sizes that do not divide 128: float32 products, rounded sums.  Rounding errors have either sign, at
+    2^-24 sqrt(d) = 6.7e-7 a score at most over 4000 scores they leave 1e-8 between the scores' mean size and the exact one; truncated
+    sums are 4.6e-8 (d = 64) to 14e-8 (d = 128) too small.  The mean of the full dot products over 32 rows or more stays on the tensor
+    cores, whose error there is below that of the plain kernel's long sums: 1.6e-7 bounds both."""
+    blocks = 2048
+    g = torch.Generator().manual_seed(d + M + reduce)
+    u = torch.randn((Hkv, 1, d), generator=g)
+    u = 6.0 * u / u.norm(dim=-1, keepdim=True)
+    key = torch.randn((2, 1, Hkv, blocks, d), generator=g) + u * torch.rand((Hkv, blocks, 1), generator=g)
+    kmax, kmin = (t.to(torch.bfloat16).cuda() for t in (key.amax(0), key.amin(0)))
+    q = (torch.randn((1, 1, M, Hq, d), generator=g) + u[:, 0].repeat_interleave(Hq // Hkv, 0)).to(torch.bfloat16).cuda()
+    got = score_call(Hq, Hkv, d, M, kmax, kmin, q, [blocks * 64], reduce=reduce, score_mode=score_mode)[0].double()
+    want = score_reference(kmax[0], kmin[0], q[0, 0], Hkv, reduce, score_mode)
+    drift = (((got - want) * want).sum() / (want * want).sum()).abs().item()
+    assert drift < (1.6e-7 if reduce == B.REDUCE_MEAN and score_mode == 0 and M > 1 else 2.5e-8)
+
+
+@pytest.mark.parametrize("Hq,Hkv,d", [(8, 2, 64), (10, 2, 128)])
+def test_scores_without_rows_and_with_infinite_keys(Hq, Hkv, d):
+    """Head size 64 and group sizes that do not divide 128: a sequence with no rows in this step has a mean of NaN, a maximum of
+    -infinity and row 0 as its last row; a channel whose maximum is infinite counts, channel-wise, for the queries that are positive
+    there and for no others."""
+    g = torch.Generator().manual_seed(d)
+    key = torch.randn((2, 2, Hkv, 40, d), generator=g)
+    kmax, kmin = (t.to(torch.bfloat16).cuda() for t in (key.amax(0), key.amin(0)))
+    q = torch.randn((1, 2, 6, Hq, d), generator=g).to(torch.bfloat16).cuda()
+    lens = [64 * 40, 64 * 39 + 1]
+    for reduce in (B.REDUCE_MEAN, B.REDUCE_MAX, B.REDUCE_LAST):
+        got = score_call(Hq, Hkv, d, 6, kmax, kmin, q, lens, q_lens=[0, 6], reduce=reduce)
+        if reduce == B.REDUCE_MEAN:
+            assert got[0].isnan().all()
+        elif reduce == B.REDUCE_MAX:
+            assert (got[0] == -float("inf")).all()
+        else:
+            torch.testing.assert_close(got[0].double(), score_reference(kmax[0], kmin[0], q[0, 0], Hkv, reduce, 0), rtol=2e-5, atol=2e-4)
+        torch.testing.assert_close(got[1].double(), score_reference(kmax[1], kmin[1], q[0, 1], Hkv, reduce, 0), rtol=2e-5, atol=2e-4)
+    q[..., 3] = -q[..., 3].abs() - 0.1
+    plain = score_call(Hq, Hkv, d, 6, kmax, kmin, q, lens, score_mode=1)
+    kmax[:, :, 5, 3] = float("inf")
+    assert torch.equal(score_call(Hq, Hkv, d, 6, kmax, kmin, q, lens, score_mode=1), plain)
+    q[:, :, 0, :, 3] = 1.0
+    got = score_call(Hq, Hkv, d, 6, kmax, kmin, q, lens, score_mode=1)
+    assert (got[:, :, 5] == float("inf")).all() and got[:, :, :5].isfinite().all()
 
 
 @pytest.mark.parametrize("score_mode", [0, 1])
