@@ -187,8 +187,9 @@ specpv_status specpv_refresh_partial(const specpv_config *cfg, const specpv_page
  * those rows.  The results agree within the tolerance of either; the default is the faster one when
  * steps follow one another (see the comment at attention_pair_wanted).
  * Precision: the attention weights of a float32 cache are float32 throughout.  Over a bfloat16 cache they are rounded to bfloat16
- * where head_dim is 128 and Hq / Hkv divides 128; for head_dim 64 and the other group sizes they are held to 2^-18 (two
- * bfloat16 terms), which leaves the log-sum-exp accurate to float32 and out, with cfg->out_f32, to about 5e-6. */
+ * where head_dim is 128 and Hq / Hkv divides 128; for head_dim 64 and the other group sizes they are held to 2^-16 (two
+ * bfloat16 terms), which leaves the log-sum-exp accurate to float32 and out, with cfg->out_f32, to about 5e-6 of itself
+ * (the plain kernel: 6e-7). */
 specpv_status specpv_verify_partial(const specpv_config *cfg, int layer0, int n_layers, const void *q,
                                     const void *k_new, const void *v_new, const uint64_t *tree_mask,
                                     const int32_t *q_lens, int M_max, const specpv_paged_kv *partial,

@@ -26,13 +26,13 @@
 //
 // Precision of the weights.  With 128 channels and a group size that divides 128, P is rounded to bfloat16 once.  Head size 64 and the
 // other group sizes (kSplit) keep the float32 weights and accurate log-sum-exps of the plain kernel: P goes to the tensor core as two
-// bfloat16 terms, the rounded weight and what rounding took off, side by side over S (64 + 64 columns), the row sum is taken
+// bfloat16 terms, the weight's upper half and what that leaves out, side by side over S (64 + 64 columns), the row sum is taken
 // over the float32 weights, and the scale carries a second term (see scale_log2_lo).  Relative 2-norm errors against float64, one
 // bfloat16 term / two / plain kernel: log-sum-exp 4.8e-5 / 3.5e-8 / 4.0e-8, bfloat16 output 1.86e-3 / 1.66e-3 / 1.66e-3 (1.66e-3 is its own
-// rounding), float32 output 8.5e-4 / 3.6e-6 / 6.6e-7 (12345 tokens, 48 x 5 rows of 128; what is left is the tensor core
-// cutting off the sums over the tokens), 5.4e-5 / 3.3e-8 / 3.4e-8, 1.79e-3 / 1.66e-3 / 1.66e-3 and 6.5e-4 / 2.3e-6 / 3.9e-7
-// (4101 tokens, 60 x 4 rows of 64).  It takes half again the contractions of P V and a third more of the softmax: 24.6 -> 32.0 us and
-// 16.1 -> 18.5 us for one layer, where the plain kernel took 1310 and 375.
+// rounding), float32 output 8.5e-4 / 5.5e-6 / 6.6e-7 (12345 tokens, 48 x 5 rows of 128; what is left is the tensor core
+// cutting off the sums over the tokens), 5.4e-5 / 3.3e-8 / 3.4e-8, 1.79e-3 / 1.66e-3 / 1.66e-3 and 6.5e-4 / 4.5e-6 / 3.9e-7
+// (4101 tokens, 60 x 4 rows of 64).  It takes half again the contractions of P V and a third more of the softmax: 24.6 -> 31.4 us and
+// 16.1 -> 18.7 us for one layer, where the plain kernel took 1310 and 375.
 #include "attn_tc.cuh"
 
 namespace specpv {
@@ -441,8 +441,12 @@ __device__ __forceinline__ void softmax(const TcParams& p, const Job& c, Barrier
         // v[i], whose own value was consumed by an earlier pair, so no second register array is needed.
         // The row sum is taken over the ROUNDED weights the tensor core will use, so that O / l is an
         // exact weighted average of V rows (the rounding error of a dominant weight cancels instead of
-        // scaling the output).  kSplit: over the float32 weights, which the two terms hold to 2^-18.
-        uint32_t rest[kSplit ? 64 : 1];  // kSplit: what rounding took off, as bf16 pairs
+        // scaling the output).  kSplit: over the float32 weights, which the two terms hold to 2^-16.
+        // kSplit: the first term is the weight cut to its upper half, the second what that took off, as bf16 pairs.  Neither term of a
+        // weight is ever negative or zero (the second has 2^-23 of the weight added), so that a weight times an infinite
+        // value stays infinite.
+        constexpr float kOnePlus = 1.f + 1.1920929e-7f;
+        uint32_t rest[kSplit ? 64 : 1];
         auto exp_row = [&](float m_use) {
             const float2 nm2 = make_float2(-m_use, -m_use);
             float2 sum2[4];  // independent partial sums: one chain of 64 dependent adds would outlast the exponentials
@@ -454,12 +458,17 @@ __device__ __forceinline__ void softmax(const TcParams& p, const Job& c, Barrier
                 float2 x = __ffma2_rn(sv, sc2, nm2);
                 if constexpr (kSplit) x = __ffma2_rn(sv, sc2_lo, x);
                 const float2 e = make_float2(ex2(x.x), ex2(x.y));
-                const uint32_t w = pack_bf16(e.x, e.y);
-                v[i] = w;
                 if constexpr (kSplit) {
-                    rest[i] = pack_bf16(e.x - __uint_as_float(w << 16), e.y - __uint_as_float(w & 0xFFFF0000u));
+                    const uint32_t ex = __float_as_uint(e.x), ey = __float_as_uint(e.y);
+                    v[i] = __byte_perm(ex, ey, 0x7632);  // the upper halves
+                    const float2 minus_upper = make_float2(__uint_as_float((ex & 0xFFFF0000u) | 0x80000000u),
+                                                           __uint_as_float((ey & 0xFFFF0000u) | 0x80000000u));
+                    const float2 r = __ffma2_rn(e, make_float2(kOnePlus, kOnePlus), minus_upper);
+                    rest[i] = pack_bf16(r.x, r.y);
                     sum2[i & 3] = __fadd2_rn(sum2[i & 3], e);
                 } else {
+                    const uint32_t w = pack_bf16(e.x, e.y);
+                    v[i] = w;
                     add_bf16_pair(sum2[i & 3], w);
                 }
             }

@@ -142,7 +142,7 @@ def test_packed_rows_and_alternating_streams(Hq, Hkv, d, bs, ctx, Ms, n_chain):
 ])
 def test_weights_keep_their_float32_precision(Hq, Hkv, d, bs, ctx, Ms, n_layers):
     """bfloat16 caches with head size 64 or a group size that does not divide 128 (and, on the plain kernel, more than 128
-    query heads per KV head): weights in float32, or in two bfloat16 terms that hold them to 2^-18 = 3.8e-6.  The tensor core
+    query heads per KV head): weights in float32, or in two bfloat16 terms that hold them to 2^-16, 2.6e-6 rms.  The tensor core
     cuts a sum to 2^-24 of itself after every 16 tokens and term, 16 times a tile: for 12 tiles 192 x 6e-8 = 1.1e-5 at most.  (One
     bfloat16 term is off by 2^-9 / sqrt(3) = 1.1e-3 a weight.)  A log-sum-exp is rounded once, 2^-24 = 6e-8 of itself, and holds the
     error of the scores, d / 16 cuts of 2^-24 = 4.8e-7 of a score at most, 2.4e-7 on average, before the mean is put back."""
@@ -158,6 +158,35 @@ def test_weights_keep_their_float32_precision(Hq, Hkv, d, bs, ctx, Ms, n_layers)
 def test_float32_kernel_tile_edges(Hq, Hkv, d, bs, ctx, Ms, n_chain):
     """The plain kernel's 64-row and 64-token tiles at their edges, one and many KV splits."""
     run_case("fp32", Hq, Hkv, d, bs, ctx=ctx, Ms=Ms, n_chain=n_chain, seed=Hq + bs)
+
+
+@pytest.mark.parametrize("Hq,Hkv,d", [(8, 2, 64), (10, 2, 128), (8, 2, 128)])
+def test_infinite_values_stay_infinite(Hq, Hkv, d):
+    """A channel in which a visible token's value is infinite is infinite in the output (the weight is positive, however it is held),
+    NaN where infinities of both signs meet, and the other channels know nothing of it."""
+    dev, bs, M, ctx = "cuda", 64, 30, 900
+    g = torch.Generator().manual_seed(d + Hq)
+    bf = lambda *shape: torch.randn(shape, generator=g).to(torch.bfloat16).to(dev)  # noqa: E731
+    pools, q = bf(2, 1, 15, Hkv, bs, d), bf(1, 1, M, Hq, d)
+    k_new, v_new = bf(2, 1, 1, M, Hkv, d)
+    cache = B.Cache(pools[0], pools[1], torch.arange(15, dtype=torch.int32, device=dev)[None],
+                    torch.tensor([ctx], dtype=torch.int32, device=dev), ctx)
+    mask = util.device_masks([wl.make_tree(M, 5, 4, np.random.default_rng(1))], M)
+    cfg = B.make_config(1, Hq, Hkv, d, bs, "bf16", 1, 1, 3, bs, out_f32=1)
+    ws = B.new_workspace(cfg, 1, 1, ctx, M)
+    out = torch.zeros_like(q, dtype=torch.float32)
+    call = lambda: B.specpv_verify_full(cfg, 0, 1, q, k_new, v_new, mask, None, M, cache, out, None, ws)  # noqa: E731
+    call()
+    plain, inf = out.clone(), float("inf")
+    for t in range(0, 128, 3):  # whatever bits the weights have
+        cache.v_pool[0, t // bs, :, t % bs, 1] = inf
+    cache.v_pool[0, 5, :, 7, 2] = -inf
+    cache.v_pool[0, 5, :, 8, 3], cache.v_pool[0, 6, :, 8, 3] = inf, -inf
+    v_new[0, 0, 0, :, 4] = inf  # the root, which every row sees
+    call()
+    util.sync_status(ws)
+    assert (out[..., 1] == inf).all() and (out[..., 2] == -inf).all() and out[..., 3].isnan().all() and (out[..., 4] == inf).all()
+    assert torch.equal(out[..., 5:], plain[..., 5:]) and torch.equal(out[..., 0], plain[..., 0])
 
 
 @pytest.mark.parametrize("Hq,Hkv,d,ctx,n_layers", [(8, 2, 64, 3000, 1), (10, 2, 128, 3000, 1), (32, 8, 128, 700, 1),
