@@ -1,5 +1,5 @@
 """Thin binding of libspecpv.so: the same names as include/specpv.h, argument marshalling only (in native code for the
-calls of a step, `csrc/pycalls.c`; through ctypes for the others).
+calls of a step, `csrc/pycalls.c`, where that has been built; through ctypes for the others).
 
 Every step of the verification path runs in the library's CUDA kernels; this module converts
 torch tensors to raw pointers and raises :class:`SpecPVError` on a non-zero status.  There is no
@@ -10,6 +10,7 @@ from __future__ import annotations
 import ctypes
 import importlib.machinery
 import importlib.util
+import sysconfig
 from ctypes import POINTER, byref, c_double, c_float, c_int, c_int32, c_size_t, c_void_p
 from dataclasses import dataclass
 from pathlib import Path
@@ -18,7 +19,7 @@ import numpy as np
 import torch
 
 LIB_PATH = Path(__file__).resolve().parent / "lib" / "libspecpv.so"
-PYCALLS_PATH = LIB_PATH.with_name("pycalls.so")
+PYCALLS_PATH = LIB_PATH.with_name("pycalls" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 STATUS_NAMES = ["OK", "INVALID_ARG", "SHAPE", "BUDGET", "CAPACITY", "BAD_TREE", "BAD_BLOCK_TABLE",
                 "UNSUPPORTED", "CUDA", "TIMEOUT"]
@@ -62,17 +63,20 @@ class PagedKV(ctypes.Structure):
                 ("n_pages", c_int32), ("max_seq_len", c_int32)]
 
 
-# Argument kinds of the calls (P pointer, i int32, z size_t, d double): declared, so that plain Python numbers can be passed.
+# The calls of a step by the kinds of their Python arguments, as in pycalls.c: G Config, i int, P tensor or None, C Cache,
+# W workspace tensor (pointer and bytes), S stream.
+_STEP_CALLS = {
+    "specpv_update_block_summaries": "GiiCPiPPWS", "specpv_score_blocks": "GiiPPiPPPCPWS", "specpv_select_partial_kv": "GiPPiiPPWS",
+    "specpv_refresh_partial": "GCPPCPWS", "specpv_verify_partial": "GiiPPPPPiCPPWS", "specpv_verify_full": "GiiPPPPPiCPPWS",
+    "specpv_verify_partial_static": "GiiPPPPPiCPPPS", "specpv_verify_host": "GiiiPPPPiCPPWS",
+    "specpv_commit_accepted": "GiiPPiPPiCPPWS", "specpv_qkv_rope": "GiiPiPPiiPPPWS", "specpv_o_proj": "GiiPPiPiiPWS",
+}
+# C argument kinds (P pointer, i int32, z size_t, d double): declared, so that plain Python numbers can be passed.
 # A call of the step is a few microseconds of device work, and wrapping every argument in a ctypes object cost as much.
 _SIGNATURES = {
-    "specpv_poll_status": "PPP", "specpv_build_tree_mask": "PiiPi", "specpv_select_mode": "iiiiii",
-    "specpv_update_block_summaries": "PiiPPiPPPzP", "specpv_score_blocks": "PiiPPiPPPPPPzP",
-    "specpv_select_partial_kv": "PiPPiiPPPzP", "specpv_refresh_partial": "PPPPPPPzP",
-    "specpv_verify_partial": "PiiPPPPPiPPPPzP", "specpv_verify_full": "PiiPPPPPiPPPPzP",
-    "specpv_verify_host": "PiiiPPPPiPPPPzP", "specpv_commit_accepted": "PiiPPiPPiPPPPzP",
-    "specpv_verify_partial_static": "PiiPPPPPiPPPPP", "specpv_rope_table": "PPPPiidPP",
-    "specpv_qkv_rope": "PiiPiPPiiPPPPzP", "specpv_o_proj": "PiiPPiPiiPPzP",
+    "specpv_poll_status": "PPP", "specpv_build_tree_mask": "PiiPi", "specpv_select_mode": "iiiiii", "specpv_rope_table": "PPPPiidPP",
     "specpv_verify_full_offloaded": "PiiPPPPPiPPPPzPP", "specpv_selftest_wait_timeout": "PziPP",
+    **{name: kinds.translate(str.maketrans({"G": "P", "C": "P", "W": "Pz", "S": "P"})) for name, kinds in _STEP_CALLS.items()},
 }
 _KINDS = {"P": c_void_p, "i": c_int, "z": c_size_t, "d": c_double}
 
@@ -112,13 +116,37 @@ def _ptr(t) -> int | None:
 _pycalls = None
 
 
+class _CtypesCalls:
+    """The calls of a step through ctypes, for an interpreter that pycalls.c has not been built for."""
+
+    def __getattr__(self, name):
+        fn, kinds = getattr(lib(), name), _STEP_CALLS[name]
+
+        def call(*args):
+            values = []
+            for kind, arg in zip(kinds, args, strict=True):
+                if kind == "G":
+                    values.append(byref(arg))
+                elif kind == "C":
+                    values.append(byref(arg.desc()))
+                elif kind == "S":
+                    values.append(_stream(arg))
+                else:
+                    values.append(arg if kind == "i" else _ptr(arg))
+                if kind == "W":
+                    values.append(arg.numel())
+            return fn(*values)
+        return call
+
+
 def _native():
-    """The native argument conversion (raises like lib() if it has not been built)."""
+    """The argument conversion of the step's calls: native, or through ctypes where that has not been built."""
     global _pycalls
     if _pycalls is None:
         lib()
         if not PYCALLS_PATH.exists():
-            raise ImportError(f"{PYCALLS_PATH} is missing: run `python -m paper_2512_02337_b200.build`")
+            _pycalls = _CtypesCalls()
+            return _pycalls
         loader = importlib.machinery.ExtensionFileLoader("pycalls", str(PYCALLS_PATH))
         module = importlib.util.module_from_spec(importlib.util.spec_from_loader("pycalls", loader))
         loader.exec_module(module)

@@ -2,15 +2,17 @@
 from __future__ import annotations
 
 import os
+import shlex
 import subprocess
 import sys
 import sysconfig
+import warnings
 from pathlib import Path
 
 PKG = Path(__file__).resolve().parent
 CSRC = PKG / "csrc"
 LIB = PKG / "lib" / "libspecpv.so"
-PYCALLS = PKG / "lib" / "pycalls.so"
+PYCALLS = PKG / "lib" / ("pycalls" + sysconfig.get_config_var("EXT_SUFFIX"))  # per interpreter: another one builds its own
 SOURCES = ["api.cu", "aux_kernels.cu", "attn_simt.cu", "attn_tc.cu", "attn_pair.cu", "score_tc.cu", "proj_tc.cu", "offload.cu", "selftest.cu"]
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -24,26 +26,39 @@ def _nvcc() -> str:
     return cand if Path(cand).exists() else "nvcc"
 
 
-def needs_build() -> bool:
-    if not LIB.exists() or not PYCALLS.exists():
+def needs_build(target: Path = LIB) -> bool:
+    if not target.exists():
         return True
     newest = max(p.stat().st_mtime for p in list(CSRC.iterdir()) + [PKG.parent / "include" / "specpv.h"])
-    return newest > min(LIB.stat().st_mtime, PYCALLS.stat().st_mtime)
+    return newest > target.stat().st_mtime
 
 
 def _build_pycalls() -> None:
+    """The argument conversion needs a C compiler and Python's headers, which the library itself does without: where they are
+    missing the binding converts through ctypes."""
     tmp = PYCALLS.with_suffix(f".{os.getpid()}.tmp")
-    subprocess.run([os.environ.get("CC") or "gcc", "-O2", "-std=gnu11", "-Wall", "-fPIC", "-fvisibility=hidden", "-shared",
-                    "-I", sysconfig.get_paths()["include"], str(CSRC / "pycalls.c"), "-o", str(tmp),
-                    "-L", str(LIB.parent), "-lspecpv", "-Wl,-rpath,$ORIGIN"], check=True)
-    os.replace(tmp, PYCALLS)
+    try:
+        subprocess.run([*shlex.split(os.environ.get("CC") or "gcc"), "-O2", "-std=gnu11", "-Wall", "-fPIC", "-fvisibility=hidden",
+                        "-shared", "-I", sysconfig.get_paths()["include"], str(CSRC / "pycalls.c"), "-o", str(tmp),
+                        "-L", str(LIB.parent), "-lspecpv", "-Wl,-rpath,$ORIGIN"], check=True)
+    except (OSError, subprocess.CalledProcessError) as e:
+        PYCALLS.unlink(missing_ok=True)  # one of an older source must not be used
+        warnings.warn(f"{PYCALLS.name} was not built ({e}): the binding's calls are converted through ctypes")
+    else:
+        os.replace(tmp, PYCALLS)
 
 
 def build(force: bool = False, verbose: bool = False) -> Path:
-    """Compile every .cu of the library into lib/libspecpv.so (static cudart, no libcuda link), then lib/pycalls.so."""
-    if not force and not needs_build():
-        return LIB
+    """Compile every .cu of the library into lib/libspecpv.so (static cudart, no libcuda link), then the argument conversion."""
     LIB.parent.mkdir(exist_ok=True)
+    if force or needs_build():
+        _build_lib(verbose)
+    if force or needs_build(PYCALLS):
+        _build_pycalls()
+    return LIB
+
+
+def _build_lib(verbose: bool) -> None:
     objdir = PKG / "lib" / "obj"
     objdir.mkdir(exist_ok=True)
     objs = []
@@ -68,8 +83,6 @@ def build(force: bool = False, verbose: bool = False) -> Path:
     subprocess.run([_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-o", str(tmp), *objs,
                     "-cudart", "static"], check=True)
     os.replace(tmp, LIB)
-    _build_pycalls()
-    return LIB
 
 
 if __name__ == "__main__":

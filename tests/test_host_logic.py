@@ -2,6 +2,7 @@
 functions (tree mask, mode rule) agree bit-for-bit with the oracle, and argument validation rejects
 bad requests before anything is launched."""
 import ctypes
+import os
 import re
 from pathlib import Path
 
@@ -171,22 +172,63 @@ def test_replica_timings_are_reduced_with_max_over_ranks_gloo():
     assert results[0] == results[1] == [11.0, 5.0]
 
 
-@pytest.mark.parametrize("bad,error", [("strided", AssertionError), ("list", TypeError), ("word", TypeError),
-                                       ("config", TypeError), ("cache", AttributeError), (None, B.SpecPVError)])
-def test_native_argument_conversion(bad, error):
-    """Tensors, NumPy arrays and None are taken as pointers, everything else is refused before the library is called; the
-    library then refuses the null query tensor (so no CUDA call is made)."""
+@pytest.fixture(params=["native", "ctypes"])
+def conversion(request, monkeypatch, tmp_path):
+    """The step's calls with their arguments converted in native code and, where that has not been built, through ctypes."""
+    monkeypatch.setattr(B, "_pycalls", None)
+    if request.param == "ctypes":
+        monkeypatch.setattr(B, "PYCALLS_PATH", tmp_path / "missing.so")
+    assert isinstance(B._native(), B._CtypesCalls) == (request.param == "ctypes")
+    return request.param
+
+
+def verify_full_args(**over):
+    """Arguments of a call that the library refuses for its null query tensor (so no CUDA call is made)."""
     cfg = B.make_config(n_layers=2, n_q_heads=8, n_kv_heads=2, head_dim=64, block_tokens=64, dtype="fp32", sink_blocks=1,
                         local_blocks=2, budget_blocks=8, buffer_tokens=64)
     t = torch.zeros(2, 4, 2, 64, 64)
     cache = B.Cache(t, t, torch.zeros(1, 4, dtype=torch.int32), torch.zeros(1, dtype=torch.int32), 256)
-    args = dict(cfg=cfg, layer0=0, n_layers=1, q=None, k_new=np.zeros(64, np.float32), v_new=t, tree_mask=t, q_lens=None,
-                M_max=16, full=cache, out=t, lse=None, workspace=t, stream=0)
-    args.update({"strided": dict(v_new=t.transpose(0, 1)), "list": dict(v_new=[1.0]), "word": dict(M_max="16"),
-                 "config": dict(cfg=t.numpy()), "cache": dict(full=t), None: {}}[bad])
-    with pytest.raises(error) as e:
+    return dict(dict(cfg=cfg, layer0=0, n_layers=1, q=None, k_new=np.zeros(64, np.float32), v_new=t, tree_mask=t, q_lens=None,
+                     M_max=16, full=cache, out=t, lse=None, workspace=t, stream=0), **over)
+
+
+@pytest.mark.parametrize("bad,error", [("strided", AssertionError), ("list", TypeError), ("word", TypeError),
+                                       ("config", TypeError), ("cache", AttributeError), (None, B.SpecPVError)])
+def test_native_argument_conversion(bad, error, conversion):
+    """Tensors, NumPy arrays and None are taken as pointers, everything else is refused before the library is called; the
+    library then refuses the null query tensor."""
+    t = torch.zeros(2, 4, 2, 64, 64)
+    args = verify_full_args(**{"strided": dict(v_new=t.transpose(0, 1)), "list": dict(v_new=[1.0]), "word": dict(M_max="16"),
+                               "config": dict(cfg=t.numpy()), "cache": dict(full=t), None: {}}[bad])
+    with pytest.raises((error, ctypes.ArgumentError) if bad == "word" else error) as e:
         B.specpv_verify_full(**args)
     assert bad is not None or e.value.status == 1
+
+
+def test_both_conversions_know_the_same_calls():
+    """The table of pycalls.c and the binding's, and the library's functions of those names."""
+    source = (ROOT / "paper_2512_02337_b200" / "csrc" / "pycalls.c").read_text()
+    assert dict(re.findall(r'X\((specpv_\w+), "(\w+)", call_', source)) == B._STEP_CALLS
+    assert set(B._SIGNATURES) == set(B.EXPORTS[3:] + B.SELFTEST_EXPORTS)
+
+
+def test_build_does_without_a_c_compiler_and_builds_per_interpreter(monkeypatch, tmp_path):
+    """Where the argument conversion cannot be compiled the library is built all the same, a stale one is removed, and the calls
+    go through ctypes; its file name carries the interpreter's ABI, so that another interpreter does not load it."""
+    import sysconfig
+    assert build_mod.PYCALLS == B.PYCALLS_PATH and build_mod.PYCALLS.name == "pycalls" + sysconfig.get_config_var("EXT_SUFFIX")
+    stale = tmp_path / build_mod.PYCALLS.name
+    stale.touch()
+    os.utime(stale, (0, 0))
+    monkeypatch.setattr(build_mod, "PYCALLS", stale)
+    for compiler in ("/nonexistent/cc", "false --some-flag"):
+        monkeypatch.setenv("CC", compiler)
+        with pytest.warns(UserWarning, match="through ctypes"):
+            assert build_mod.build() == build_mod.LIB
+        assert not stale.exists()
+    monkeypatch.setenv("CC", "gcc -g0")  # a command with arguments
+    build_mod.build()
+    assert stale.exists() and not build_mod.needs_build(stale)
 
 
 def test_overlapped_kernels_load_nothing_through_the_read_only_path():
