@@ -150,7 +150,8 @@ def _native():
         loader = importlib.machinery.ExtensionFileLoader("pycalls", str(PYCALLS_PATH))
         module = importlib.util.module_from_spec(importlib.util.spec_from_loader("pycalls", loader))
         loader.exec_module(module)
-        module.init(torch.Tensor, _ptr, _stream, _get_device, _raw_stream if _get_device is not None else None)
+        module.init(torch.Tensor, _ptr, _stream, _get_device, _raw_stream if _get_device is not None else None, Cache,
+                    ctypes.Structure, c_int.__base__)
         _pycalls = module
     return _pycalls
 

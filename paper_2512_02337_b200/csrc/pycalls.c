@@ -12,8 +12,9 @@
 
 #include "../../include/specpv.h"
 
-/* Argument kinds: G specpv_config structure, i int, P tensor or None, C cache (the binding's Cache) -> specpv_paged_kv,
- * W workspace tensor -> pointer and bytes, S stream or None (the current one). */
+/* Argument kinds: G specpv_config structure, i int, P tensor or None, C cache (the binding's Cache, or anything else whose
+ * desc() gives a specpv_paged_kv structure) -> specpv_paged_kv, W workspace tensor -> pointer and bytes, S stream or None (the
+ * current one). */
 typedef struct {
     const char *name, *kinds;
     int (*call)(const uint64_t *v);
@@ -57,8 +58,10 @@ static int call_o_proj(const uint64_t *v) {
     return specpv_o_proj(P(0), I(1), I(2), P(3), P(4), I(5), P(6), I(7), I(8), P(9), P(10), (size_t)v[11], P(12));
 }
 
-static PyObject *tensor_type, *convert, *convert_stream, *get_device, *raw_stream;  /* set once by init() */
-static PyObject *s_data_ptr, *s_is_contiguous, *s_size, *s_numel, *s_k_pool, *s_v_pool, *s_block_table, *s_seq_lens, *s_max_seq_len;
+/* set once by init(): torch.Tensor, the binding's converters, torch's current device and stream, the binding's Cache and
+ * ctypes' structures and simple values */
+static PyObject *tensor_type, *convert, *convert_stream, *get_device, *raw_stream, *cache_type, *structure_type, *simple_type;
+static PyObject *s_data_ptr, *s_is_contiguous, *s_size, *s_numel, *s_k_pool, *s_v_pool, *s_block_table, *s_seq_lens, *s_max_seq_len, *s_desc, *s_value;
 static PyObject *zero, *one;
 
 static int take_u64(PyObject *number, uint64_t *out) {  /* steals the reference */
@@ -94,7 +97,31 @@ static int pointer_of(PyObject *arg, uint64_t *out) {
     return data_ptr(arg, out);
 }
 
+/* The memory of a ctypes structure of at least `size` bytes; it lives as long as the structure does. */
+static int structure_of(PyObject *arg, size_t size, const void **out) {
+    Py_buffer view;
+    if (!PyObject_TypeCheck(arg, (PyTypeObject *)structure_type)) {
+        PyErr_Format(PyExc_TypeError, "a ctypes structure was expected, not %.80s", Py_TYPE(arg)->tp_name);
+        return -1;
+    }
+    if (PyObject_GetBuffer(arg, &view, PyBUF_SIMPLE)) return -1;
+    const int ok = view.len >= (Py_ssize_t)size;
+    *out = view.buf;
+    PyBuffer_Release(&view);
+    if (!ok) PyErr_Format(PyExc_TypeError, "%.80s is too small", Py_TYPE(arg)->tp_name);
+    return ok ? 0 : -1;
+}
+
+/* Read straight from the attributes of a Cache; another type's own desc() is asked. */
 static int cache_of(PyObject *cache, specpv_paged_kv *kv) {
+    if ((PyObject *)Py_TYPE(cache) != cache_type) {
+        const void *desc = NULL;
+        PyObject *d = PyObject_CallMethodNoArgs(cache, s_desc);
+        const int bad = !d || structure_of(d, sizeof *kv, &desc);
+        if (!bad) *kv = *(const specpv_paged_kv *)desc;
+        Py_XDECREF(d);
+        return bad ? -1 : 0;
+    }
     PyObject *k = PyObject_GetAttr(cache, s_k_pool), *v = PyObject_GetAttr(cache, s_v_pool);
     PyObject *table = PyObject_GetAttr(cache, s_block_table), *lens = PyObject_GetAttr(cache, s_seq_lens);
     PyObject *limit = PyObject_GetAttr(cache, s_max_seq_len);
@@ -120,13 +147,22 @@ static int cache_of(PyObject *cache, specpv_paged_kv *kv) {
 }
 
 static int config_of(PyObject *arg, uint64_t *out) {
-    Py_buffer view;
-    if (PyObject_GetBuffer(arg, &view, PyBUF_SIMPLE)) return -1;
-    const int ok = view.len == (Py_ssize_t)sizeof(specpv_config);
-    *out = (uint64_t)(uintptr_t)view.buf;  /* the structure's own memory, which the caller's reference keeps */
-    PyBuffer_Release(&view);
-    if (!ok) PyErr_SetString(PyExc_TypeError, "the first argument must be a Config");
-    return ok ? 0 : -1;
+    const void *cfg = NULL;
+    if (structure_of(arg, sizeof(specpv_config), &cfg)) return -1;
+    *out = (uint64_t)(uintptr_t)cfg;
+    return 0;
+}
+
+static int int_of(PyObject *arg, uint64_t *out) {
+    PyObject *value = NULL;  /* of a c_int and the like */
+    if (PyObject_TypeCheck(arg, (PyTypeObject *)simple_type)) {
+        if (!(value = PyObject_GetAttr(arg, s_value))) return -1;
+        arg = value;
+    }
+    const long x = PyLong_AsLong(arg);
+    Py_XDECREF(value);
+    *out = (uint64_t)x;
+    return x == -1 && PyErr_Occurred() ? -1 : 0;
 }
 
 static int stream_of(PyObject *arg, uint64_t *out) {
@@ -149,12 +185,7 @@ static PyObject *invoke(const Spec *spec, PyObject *const *args, Py_ssize_t n) {
     for (Py_ssize_t i = 0; i < n; ++i) {
         int st = 0;
         switch (spec->kinds[i]) {
-            case 'i': {
-                const long x = PyLong_AsLong(args[i]);
-                st = x == -1 && PyErr_Occurred() ? -1 : 0;
-                v[n_v] = (uint64_t)x;
-                break;
-            }
+            case 'i': st = int_of(args[i], &v[n_v]); break;
             case 'G': st = config_of(args[i], &v[n_v]); break;
             case 'C':
                 st = cache_of(args[i], &caches[n_caches]);
@@ -198,15 +229,14 @@ static PyObject *invoke(const Spec *spec, PyObject *const *args, Py_ssize_t n) {
     }
 CALLS(WRAPPER)
 
-/* init(tensor type, converter of other pointer arguments, converter of streams, current device, raw current stream) */
 static PyObject *py_init(PyObject *self, PyObject *const *args, Py_ssize_t n) {
     (void)self;
-    PyObject **slots[] = {&tensor_type, &convert, &convert_stream, &get_device, &raw_stream};
-    if (n != 5 || !PyType_Check(args[0])) {
-        PyErr_SetString(PyExc_TypeError, "init takes a type and four objects");
+    PyObject **slots[] = {&tensor_type, &convert, &convert_stream, &get_device, &raw_stream, &cache_type, &structure_type, &simple_type};
+    if (n != 8 || !PyType_Check(args[0]) || !PyType_Check(args[6]) || !PyType_Check(args[7])) {
+        PyErr_SetString(PyExc_TypeError, "init takes eight objects, the first and the last two of them types");
         return NULL;
     }
-    for (int i = 0; i < 5; ++i) {
+    for (int i = 0; i < 8; ++i) {
         Py_INCREF(args[i]);
         Py_XSETREF(*slots[i], args[i]);
     }
@@ -224,7 +254,8 @@ PyMODINIT_FUNC PyInit_pycalls(void) {
         const char *text;
     } names[] = {{&s_data_ptr, "data_ptr"},       {&s_is_contiguous, "is_contiguous"}, {&s_size, "size"},
                  {&s_numel, "numel"},             {&s_k_pool, "k_pool"},               {&s_v_pool, "v_pool"},
-                 {&s_block_table, "block_table"}, {&s_seq_lens, "seq_lens"},           {&s_max_seq_len, "max_seq_len"}};
+                 {&s_block_table, "block_table"}, {&s_seq_lens, "seq_lens"},           {&s_max_seq_len, "max_seq_len"},
+                 {&s_desc, "desc"},               {&s_value, "value"}};
     for (size_t i = 0; i < sizeof(names) / sizeof(names[0]); ++i)
         if (!(*names[i].slot = PyUnicode_InternFromString(names[i].text))) return NULL;
     if (!(zero = PyLong_FromLong(0)) || !(one = PyLong_FromLong(1))) return NULL;

@@ -205,6 +205,44 @@ def test_native_argument_conversion(bad, error, conversion):
     assert bad is not None or e.value.status == 1
 
 
+def test_conversion_takes_what_ctypes_takes_and_refuses_the_rest(conversion):
+    """A configuration is a ctypes structure, its own or another that begins alike, and no other buffer of that size; sizes may be
+    c_int; a cache is asked for its own desc() where it has one, a subclass of Cache as well as any other object."""
+    args = verify_full_args()
+    cfg = args["cfg"]
+    for other in (bytes(cfg), bytearray(bytes(cfg)), np.frombuffer(bytes(cfg), dtype=np.uint8)):
+        with pytest.raises(TypeError):
+            B.specpv_verify_full(**dict(args, cfg=other))
+
+    class Longer(ctypes.Structure):
+        _fields_ = B.Config._fields_ + [("more", ctypes.c_int32)]
+    longer = Longer.from_buffer_copy(bytes(cfg) + bytes(4))
+
+    def too_long():  # 257 tokens in a table of 4 pages of 64: SPECPV_ERR_CAPACITY, where the cache itself gives INVALID_ARG
+        kv = B.Cache.desc(args["full"])
+        kv.max_seq_len = 257
+        return kv
+
+    class Subclass(B.Cache):
+        def desc(self):
+            return too_long()
+
+    class Other:
+        desc = staticmethod(too_long)
+
+    class Wrong:
+        def desc(self):
+            return b"0" * ctypes.sizeof(B.PagedKV)
+    sub = Subclass(**vars(args["full"]))
+    for over, status in ((dict(cfg=longer), 1), (dict(M_max=ctypes.c_int(16), layer0=ctypes.c_int32(0)), 1), (dict(full=sub), 4),
+                         (dict(full=Other()), 4)):
+        with pytest.raises(B.SpecPVError) as e:
+            B.specpv_verify_full(**dict(args, **over))
+        assert e.value.status == status, over
+    with pytest.raises(TypeError):
+        B.specpv_verify_full(**dict(args, full=Wrong()))
+
+
 def test_both_conversions_know_the_same_calls():
     """The table of pycalls.c and the binding's, and the library's functions of those names."""
     source = (ROOT / "paper_2512_02337_b200" / "csrc" / "pycalls.c").read_text()
