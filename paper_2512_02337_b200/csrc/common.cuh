@@ -51,7 +51,8 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 
 // The wait costs every CTA a few hundred nanoseconds, so a kernel of many short CTAs is launched the ordinary way (block
 // summaries of 96K tokens x 32 layers, 49152 CTAs: 1040 us with it, 940 without); such kernels take the flag in their
-// parameters.
+// parameters (launch_pdl_if).  Kernels whose CTAs run for many microseconds (attention, block scores, projections) and the rope
+// table, a CTA per row of a step, are always launched as dependents.
 constexpr long long kPdlMaxCtas = 8 * 148;
 inline bool pdl_pays(dim3 grid) { return (long long)grid.x * grid.y * grid.z <= kPdlMaxCtas; }
 __device__ __forceinline__ void pdl_begin(int on) {

@@ -1,7 +1,7 @@
 """GPU parity of the linear maps either side of the attention (QKV projection with rotary embedding, step positions,
-output projection) against the oracle, through the C ABI: the tensor-core path (bfloat16, head size 128) with one
-and several input-feature ranges per tile, several layers, more rows than one accumulator holds, and the plain path
-(float32, head size 64, odd hidden sizes)."""
+output projection) against the oracle, through the C ABI: the tensor-core path (bfloat16, heads of 128 and pairs of
+heads of 64) with one and several input-feature ranges per tile, several layers, more rows than one accumulator holds, and the
+plain path (float32, odd numbers of heads of 64, odd hidden sizes)."""
 import numpy as np
 import pytest
 import torch
@@ -65,7 +65,8 @@ def test_rope_table_positions_and_angles(d, theta):
 CASES = [
     # dtype, Hq, Hkv, d, hidden, batch, M, n_layers (pool), layer0, n_call
     ("fp32", 8, 2, 64, 512, 1, 16, 1, 0, 1),        # plain path, the tiny config's geometry
-    ("bf16", 4, 2, 64, 192, 2, 9, 2, 1, 1),         # plain path in bfloat16, second layer of the pool
+    ("bf16", 4, 2, 64, 192, 2, 9, 2, 1, 1),         # QKV on the tensor cores, output on the plain path, second layer of the pool
+    ("bf16", 3, 1, 64, 80, 2, 9, 2, 1, 1),          # plain path in bfloat16 for both
     ("bf16", 32, 8, 128, 4096, 1, 60, 1, 0, 1),     # tensor cores, one layer: six input ranges per tile
     ("bf16", 8, 2, 128, 448, 1, 37, 3, 1, 2),       # seven 64-wide input steps over seven ranges, layers 1-2 of 3
     ("bf16", 8, 4, 128, 1024, 4, 64, 10, 0, 10),    # 160 tiles: one range per tile, 256 rows per tile
