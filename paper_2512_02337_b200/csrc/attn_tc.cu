@@ -980,8 +980,11 @@ specpv_status launch_attention_tc(const AttnArgs& a, cudaStream_t stream) {
     // kSplit: what the float32 factor leaves out, and the mean of what the tensor core cuts off a dot product of d channels, which it
     // sums 16 at a time and truncates each time (measured, of the sum: 4.6e-8 to 8.3e-8 at 64 channels, 8.9e-8 to 13.8e-8 at
     // 128, the more the more alike the terms are).  Without this term every log-sum-exp comes out 5e-8 to 6e-8 of itself too
-    // small: rms error 6.1e-8 and 7.3e-8 at 64 and 128 channels, 3.3e-8 and 3.5e-8 with it.
+    // small: rms error 6.1e-8 and 7.3e-8 at 64 and 128 channels, 3.3e-8 and 3.5e-8 with it.  The term is positive, as the products
+    // of masked scores, -infinity, need it to be: scale_log2 is at most 2^-24 = 6.0e-8 of itself, less the 1.3e-8 that
+    // kLog2e is too small by, above the exact factor, and 6.4e-8 are added (and where all of this underflows, the smallest float).
     p.scale_log2_lo = (float)((double)a.g.scale * 1.4426950408889634 * (1.0 + 1.0e-9 * a.g.d) - (double)p.scale_log2);
+    if (!(p.scale_log2_lo > 0.f)) p.scale_log2_lo = 1.4e-45f;
 
     if (pair) {
         p.n_row_groups = (a.M_max * G + 255) / 256;

@@ -160,6 +160,31 @@ def test_float32_kernel_tile_edges(Hq, Hkv, d, bs, ctx, Ms, n_chain):
     run_case("fp32", Hq, Hkv, d, bs, ctx=ctx, Ms=Ms, n_chain=n_chain, seed=Hq + bs)
 
 
+@pytest.mark.parametrize("dtype,Hq,Hkv,d", [("bf16", 8, 2, 64), ("bf16", 10, 2, 128), ("bf16", 8, 2, 128), ("fp32", 8, 2, 64)])
+@pytest.mark.parametrize("scale", [0.31, 1.0, 2.0 ** -23 + 2.0 ** -46, 1e-40])
+def test_softmax_scale(dtype, Hq, Hkv, d, scale):
+    """A softmax scale of the caller's, down to one that makes all visible keys count alike: masked keys still count nothing."""
+    dev, bs, M, ctx = "cuda", 64, 21, 333
+    dt = wl.torch_dtype(dtype)
+    g = torch.Generator().manual_seed(d + Hq)
+    mk = lambda *shape: (0.5 * torch.randn(shape, generator=g)).to(dt).to(dev)  # noqa: E731
+    pools, q = mk(2, 1, 6, Hkv, bs, d), mk(1, 1, M, Hq, d)
+    k_new, v_new = mk(2, 1, 1, M, Hkv, d)
+    table = torch.arange(6, dtype=torch.int32, device=dev)[None]
+    cache = B.Cache(pools[0], pools[1], table, torch.tensor([ctx], dtype=torch.int32, device=dev), ctx)
+    parents = wl.make_tree(M, 5, 4, np.random.default_rng(1))
+    cfg = B.make_config(1, Hq, Hkv, d, bs, dtype, 1, 1, 3, bs, softmax_scale=scale, out_f32=1)
+    ws = B.new_workspace(cfg, 1, 1, ctx, M)
+    out, lse = torch.zeros((1, 1, M, Hq, d), device=dev), torch.zeros((1, 1, M, Hq), device=dev)
+    B.specpv_verify_full(cfg, 0, 1, q, k_new, v_new, util.device_masks([parents], M), None, M, cache, out, lse, ws)
+    util.sync_status(ws)
+    o_out, o_lse = oracle.tree_attention(wl.to_numpy(q[0, 0]), wl.to_numpy(k_new[0, 0]), wl.to_numpy(v_new[0, 0]),
+                                         oracle.tree_mask(parents), wl.to_numpy(pools[0, 0]), wl.to_numpy(pools[1, 0]),
+                                         table[0].cpu().numpy(), ctx, float(np.float32(scale)))
+    util.compare(out[0, 0].cpu().numpy(), o_out, dtype, f"scale {scale}")
+    np.testing.assert_allclose(lse[0, 0].cpu().numpy(), o_lse, atol=2e-5 if dtype == "fp32" else 5e-3)
+
+
 @pytest.mark.parametrize("Hq,Hkv,d", [(8, 2, 64), (10, 2, 128), (8, 2, 128)])
 def test_infinite_values_stay_infinite(Hq, Hkv, d):
     """A channel in which a visible token's value is infinite is infinite in the output (the weight is positive, however it is held),
