@@ -57,6 +57,7 @@ struct Shape {
     static constexpr int kSmemBytes = 1024 + kQBytes + kStages * kSlotBytes;
 };
 constexpr int kMaxStages = 10;
+constexpr int kShortWalk = 4;  // tiles per CTA
 
 using namespace tc;
 
@@ -371,7 +372,7 @@ __device__ __forceinline__ void softmax(const TcParams& p, const Job& c, Barrier
     const int n_tiles = c.n_tiles;
     constexpr int step = kOne ? 2 : 1;
     const int first_tile = kOne ? t : 0;     // K/V tiles of this stream: first_tile, first_tile + step, ..
-    if (first_tile >= n_tiles) return;
+    const bool idle = kOne && first_tile >= n_tiles;  // one tile: nothing for stream 1, which still does the dry run below
     const int row_tile = kOne ? 0 : t;
     const int row = row_tile * 128 + row_in_tile;                              // row within the row group
     const int tok = c.tok0 + row_tile * c.tok_per_tile + row_in_tile / p.G;    // step token of this row
@@ -381,6 +382,7 @@ __device__ __forceinline__ void softmax(const TcParams& p, const Job& c, Barrier
     const uint32_t s_addr = c.tmem + lane_addr + t * 128;
     const uint32_t o_addr = c.tmem + lane_addr + 256 + t * 128;
     if (!__any_sync(0xffffffffu, row_valid)) {
+        if (idle) return;
         pass_zeros<kSplit>(p, bars, t, first_tile, step, n_tiles, s_addr, lane);
         if (kOne && n_tiles > 1) asm volatile("bar.sync 1, 256;" ::: "memory");  // where the two streams meet below
         return;
@@ -394,14 +396,16 @@ __device__ __forceinline__ void softmax(const TcParams& p, const Job& c, Barrier
     float m_run = -INFINITY, l_run = 0.f;
     bool ok = true;
     const float2 sc2 = make_float2(p.scale_log2, p.scale_log2), sc2_lo = make_float2(p.scale_log2_lo, p.scale_log2_lo);
-    // One row tile (the form of short calls): the first pass of the loop is a dry run over zeros by the stream whose S comes
-    // last, while Q and the first K tile are still on their way: it brings the loop's code (some 20 KB, straight-line) into
+    // One row tile (the form of short calls): the first pass of the loop is a dry run over zeros by stream 1, whose S comes
+    // last or not at all, while Q and the first K tile are still on their way: it brings the loop's code (straight-line) into
     // the instruction cache.  In a model's layer other kernels have run since the last call, and with cold code the first
-    // tile took 4.6-5 us from S to P instead of 1.5.  (The form with two row tiles walks long contexts, where its loop
-    // ran 8 % slower with the dry run in it.)
-    const bool warm_up = kOne && (t == 1 || n_tiles == 1);
+    // tile took 4.6-5 us from S to P instead of 1.5.  It passes through what a stream's first tile needs, the general path: through
+    // both paths, and by stream 0 in CTAs of one tile, whose S then waited for it, it took twice as long (us per layer: 8 rows x 4,
+    // 1024 tokens 10.5 -> 9.6; 26 rows x 4 of 64 channels, 1500 and 811 tokens 14.0 -> 13.4; 48 rows x 5, 12345 tokens
+    // 32.0 -> 30.4).  (The form with two row tiles walks long contexts, where its loop ran 8 % slower with the dry run in it.)
+    const bool warm_up = kOne && t == 1;
     uint32_t s_par = warm_up ? 1 : 0;
-    for (int j = warm_up ? first_tile - step : first_tile; j < n_tiles && ok; j += step, s_par ^= 1) {
+    for (int j = warm_up ? first_tile - step : first_tile; (j < n_tiles || (kOne && j < first_tile)) && ok; j += step, s_par ^= 1) {
         const bool dry = kOne && j < first_tile;
         const bool is_new = j >= c.n_ctx_tiles;
         const int n_valid = is_new ? c.M : min(kTileTokens, c.seq_len - (c.tile_begin + j) * kTileTokens);
@@ -479,16 +483,16 @@ __device__ __forceinline__ void softmax(const TcParams& p, const Job& c, Barrier
         // is and skip the row maximum.  Weights may then exceed 1; float32 sums and bf16 weights keep
         // their relative precision whatever the exponent, so only overflow has to be ruled out: if a
         // row sum leaves the safe range (or a row has no reference yet), the warp takes the tile again
-        // from tensor memory on the general path, which brings m_run up to date.  (The dry run, without a reference,
-        // passes through both paths.)
+        // from tensor memory on the general path, which brings m_run up to date.  A short walk of the two-term form, whose fast path
+        // would be met with cold code, stays on the general path (40 rows x 4 of 64 channels, 4 tiles per CTA: 17.8 -> 17.3 us).
         float l_add = 0.f;
-        bool general = !dry && (j == first_tile || masked);
+        bool general = j <= first_tile || masked || (kOne && kSplit && n_tiles <= kShortWalk);
         if (!general) {
             l_add = exp_row(m_run);
             const bool bad = !(l_add < kSafeRowSum) || m_run == -INFINITY;
             if (__any_sync(0xffffffffu, bad)) {
                 general = true;
-                if (!dry) load_s();  // S_t is still intact: P has not been stored yet
+                load_s();  // S_t is still intact: P has not been stored yet
             }
         }
         if (general) {
@@ -543,6 +547,7 @@ __device__ __forceinline__ void softmax(const TcParams& p, const Job& c, Barrier
         }
         if (dry) {
             l_run = l_add < 0.f ? l_add : 0.f;  // never negative: zero again, and the dry run's sums are not dead code
+            if (idle) return;
             continue;
         }
         TMEM_ST32(s_addr, v);

@@ -357,3 +357,11 @@ def test_large_score_jumps_take_the_general_path(where):
     assert np.abs(o_lse).max() > 200  # the jump really is beyond what unscaled float32 weights could hold
     util.compare(out[0, 0].cpu().numpy(), o_out, "bf16", f"jump {where}")
     np.testing.assert_allclose(lse[0, 0].cpu().numpy(), o_lse, rtol=2e-5, atol=5e-3)
+
+
+@pytest.mark.parametrize("Hq,Hkv,d", [(8, 8, 128), (40, 8, 128), (32, 8, 64)])
+@pytest.mark.parametrize("tiles", [0, 1, 3, 4, 6])
+def test_short_walks_of_one_cta(Hq, Hkv, d, tiles):
+    """Enough heads that no KV range is split: a CTA walks `tiles` context tiles of 128 tokens (the last one ragged) and the step's
+    own, one tile (nothing for the second stream), as many as the short walk of the two-term form takes, and more."""
+    run_case("bf16", Hq, Hkv, d, 64, ctx=[max(128 * tiles - 27, 0)], Ms=[6], n_layers=19, seed=60 + tiles, float32_weights=d == 64 or Hq == 40)
