@@ -251,3 +251,9 @@ def test_projections_follow_the_calls_before_them_without_a_pause(M, hidden):
             # half a unit in the last place of a bfloat16 with its 8 significant bits is at most 2^-8 of the value (just above a
             # power of two); the float32 sums of up to 1024 terms below 16 before it: 1e-5
             assert ((got.double() - exact).abs() <= exact.abs() * 2.0 ** -8 + 1e-5).all(), (name, i)
+
+
+@pytest.mark.parametrize("M,L", [(15, 1), (16, 1), (17, 1), (33, 1), (48, 1), (49, 12), (16, 12)])
+def test_projection_rows_in_steps_of_sixteen(M, L):
+    """Accumulator widths that are a multiple of 16 rows and not of 32, with the input features split and (12 layers) whole."""
+    test_qkv_rope_and_o_proj_match_the_oracle("bf16", 16, 2, 128, 512, 1, M, L, 0, L)
