@@ -229,15 +229,14 @@ __global__ void __launch_bounds__(32 * kScoreWarps) scores_simt_kernel(ScorePara
 
 // ---------------------------------------------------------------------------------------------
 // Selection: one CTA per (layer, sequence, KV head).  A candidate's score becomes a 32-bit key whose unsigned order is
-// "score ascending, NaN first"; a most-significant-digit radix select in digits of 11, 11 and 10 bits finds the key T of the
-// k-th best candidate and how many candidates of that very key are still to be taken (the ones of lowest index), and an
-// ordered compaction writes sink | kept candidates | local in ascending order.  Bound by its barriers and by shared-memory
-// atomics: eight passes of 8 bits over (key, index) pairs, the first of which met two or three crowded bins, took 16.2 us for 2045
-// candidates x 256 lists against 13.1, and 9.7 against 6.6 for 29 x 2.
+// "score ascending, NaN first"; the key T of the k-th best candidate is found two bits at a time from the top, by counting the keys
+// (in registers) that reach each of three thresholds, until a threshold is met by k candidates exactly or all bits are known; then
+// an ordered compaction writes sink | kept candidates | local in ascending order, the candidates of key T that are still to be
+// taken by lowest index.  Bound by latency: its steps, a count and one barrier each, and the fetch of its code, which follows other
+// kernels: no more keys per thread, each of them code, than the lists need.  From the end of the scores to its own, against a histogram
+// per digit of 11 bits (four barriers a digit, crowded bins): 509 candidates x 256 lists 16.8 -> 12.1 us, 29 x 2 8.4 -> 4.2 (8.2 with
+// sixteen keys per thread).
 // ---------------------------------------------------------------------------------------------
-constexpr int kSelectThreads = 256;
-constexpr int kSelectBins = 2048;
-
 __device__ __forceinline__ uint32_t select_key(float score) {
     const uint32_t bits = __float_as_uint(score);
     if (score != score) return 0u;              // NaN ranks below every number
@@ -245,18 +244,17 @@ __device__ __forceinline__ uint32_t select_key(float score) {
     return (bits & 0x80000000u) ? ~bits : (bits | 0x80000000u);
 }
 
+// kSelectKeys: a thread's first keys stay in registers, any further ones are formed again from the scores.
+template <int kSelectThreads, int kSelectKeys>
 __global__ void __launch_bounds__(kSelectThreads) select_kernel(SelectParams p) {
     pdl_begin(p.pdl);
-    __shared__ unsigned int hist[kSelectBins];
-    __shared__ uint32_t s_prefix;
-    __shared__ int s_remaining;
-    __shared__ int s_warp_counts[kSelectThreads / 32];
     constexpr int kWarps = kSelectThreads / 32;
-    constexpr int kKeysPerThread = 16;                   // a thread's first keys stay in registers (4096 candidates)
-    __shared__ int s_above[kKeysPerThread * kWarps];     // candidates above T per (round, warp), then their exclusive prefix
-    __shared__ int s_tied[kKeysPerThread * kWarps];      // ... and those equal to T
+    __shared__ int4 s_reach[3];                     // candidates that reach the thresholds of a step
+    __shared__ int s_above[kSelectKeys * kWarps];   // candidates above T per (round, warp), then their exclusive prefix
+    __shared__ int s_tied[kSelectKeys * kWarps];    // ... and those equal to T
     __shared__ int s_run_above, s_run_tied;
     const int h = blockIdx.x, b = blockIdx.y, l = blockIdx.z, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int32_t* idx = p.idx + (((size_t)l * p.batch + b) * p.Hkv + h) * p.budget_blocks;
     const int seq_len = p.seq_lens[b];
     const int nb = min((seq_len + p.bs - 1) / p.bs, p.max_blocks);
     const float* scores = p.scores + (((size_t)l * p.batch + b) * p.Hkv + h) * p.max_blocks;
@@ -270,7 +268,6 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(SelectParams p) 
         for (int hh = 0; hh < p.Hkv; ++hh) acc += scores_h0[(size_t)hh * p.max_blocks + i];
         return acc * inv_heads;
     };
-    int32_t* idx = p.idx + (((size_t)l * p.batch + b) * p.Hkv + h) * p.budget_blocks;
     const int count = min(nb, p.budget_blocks);
     if (l == 0 && h == 0 && tid == 0) p.count[b] = count;
     if (nb <= p.budget_blocks) {
@@ -280,76 +277,75 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(SelectParams p) 
     const int lo = p.sink_blocks, hi = nb - p.local_blocks;
     const int k = p.budget_blocks - p.sink_blocks - p.local_blocks;
 
-    // a thread's candidates lo + tid, lo + tid + 256, ...: the first kKeysPerThread keys stay in registers, any further ones
-    // are recomputed from the scores
-    uint32_t keys[kKeysPerThread];
-    const int rounds = min((hi - lo + kSelectThreads - 1) / kSelectThreads, kKeysPerThread);
+    // a thread's candidates: lo + tid, lo + tid + kSelectThreads, ...
+    uint32_t keys[kSelectKeys];
+    const int rounds = min((hi - lo + kSelectThreads - 1) / kSelectThreads, kSelectKeys);
 #pragma unroll
-    for (int e = 0; e < kKeysPerThread; ++e) {
+    for (int e = 0; e < kSelectKeys; ++e) {
         const int i = lo + tid + e * kSelectThreads;
-        keys[e] = i < hi ? select_key(score_at(i)) : 0u;
+        keys[e] = i < hi ? select_key(score_at(i)) : 0u;  // 0 reaches no threshold
     }
-    const int tail0 = lo + tid + kKeysPerThread * kSelectThreads;
-    if (tid == 0) {
-        s_prefix = 0;
-        s_remaining = k;
-    }
-    uint32_t known = 0;  // bits of T found so far
-    for (int pass = 0; pass < 3; ++pass) {
-        const int shift = pass == 0 ? 21 : pass == 1 ? 10 : 0;
-        const uint32_t digit = pass == 2 ? 1023u : 2047u;
+    const int tail0 = lo + tid + kSelectKeys * kSelectThreads;
+    if (tid < 3) s_reach[tid] = make_int4(0, 0, 0, 0);
+    __syncthreads();
+    uint32_t T = 0;    // its bits found so far
+    int n_above = 0;   // candidates whose bits found so far are above T's
+    int ties = -1;     // candidates of key T to take
+#pragma unroll 1
+    for (int shift = 30, at = 0; shift >= 0; shift -= 2, at = at == 2 ? 0 : at + 1) {
+        const uint32_t t1 = T + (1u << shift), t2 = T + (2u << shift), t3 = T + (3u << shift);
+        int c1 = 0, c2 = 0, c3 = 0;
 #pragma unroll
-        for (int u = 0; u < kSelectBins / kSelectThreads; ++u) hist[tid + u * kSelectThreads] = 0;
-        __syncthreads();
-        const uint32_t prefix = s_prefix;
-        const int remaining = s_remaining;
-#pragma unroll
-        for (int e = 0; e < kKeysPerThread; ++e)
-            if (lo + tid + e * kSelectThreads < hi && (keys[e] & known) == prefix) atomicAdd(&hist[(keys[e] >> shift) & digit], 1u);
+        for (int e = 0; e < kSelectKeys; ++e)
+            if (e < rounds) {
+                c1 += keys[e] >= t1;
+                c2 += keys[e] >= t2;
+                c3 += keys[e] >= t3;
+            }
         for (int i = tail0; i < hi; i += kSelectThreads) {
             const uint32_t key = select_key(score_at(i));
-            if ((key & known) == prefix) atomicAdd(&hist[(key >> shift) & digit], 1u);
+            c1 += key >= t1;
+            c2 += key >= t2;
+            c3 += key >= t3;
         }
+        c1 = __reduce_add_sync(0xffffffffu, c1);
+        c2 = __reduce_add_sync(0xffffffffu, c2);
+        c3 = __reduce_add_sync(0xffffffffu, c3);
+        if (lane < 3) atomicAdd(&s_reach[at].x + lane, lane == 0 ? c1 : lane == 1 ? c2 : c3);
         __syncthreads();
-        // thread <-> eight bins: the digit of T is the bin whose suffix count (this bin and all higher ones) first reaches
-        // `remaining`; found in parallel from a block-wide suffix sum
-        unsigned c[kSelectBins / kSelectThreads], mine = 0;
-#pragma unroll
-        for (int u = 0; u < kSelectBins / kSelectThreads; ++u) {
-            c[u] = hist[tid * (kSelectBins / kSelectThreads) + u];
-            mine += c[u];
+        const int4 reach = s_reach[at];
+        if (tid == 0) s_reach[at == 0 ? 2 : at - 1] = make_int4(0, 0, 0, 0);  // read before this step's barrier, used behind the next one
+        int reached;
+        if (reach.z >= k) {
+            T = t3;
+            reached = reach.z;
+        } else if (reach.y >= k) {
+            T = t2;
+            reached = reach.y;
+            n_above = reach.z;
+        } else if (reach.x >= k) {
+            T = t1;
+            reached = reach.x;
+            n_above = reach.y;
+        } else {
+            reached = 0;  // T stays as it is
+            n_above = reach.x;
         }
-        unsigned v = mine;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned up = __shfl_down_sync(0xffffffffu, v, o);
-            if (lane + o < 32) v += up;
+        if (reached == k) {  // exactly the candidates from T on
+            --T;
+            ties = 0;
+            break;
         }
-        if (lane == 0) s_warp_counts[warp] = (int)v;
-        __syncthreads();
-        unsigned higher = v - mine;  // candidates in the bins above this thread's
-        for (int w2 = warp + 1; w2 < kWarps; ++w2) higher += (unsigned)s_warp_counts[w2];
-#pragma unroll
-        for (int u = kSelectBins / kSelectThreads - 1; u >= 0; --u) {
-            if (higher < (unsigned)remaining && higher + c[u] >= (unsigned)remaining) {  // true for exactly one bin
-                s_remaining = remaining - (int)higher;
-                s_prefix = prefix | ((uint32_t)(tid * (kSelectBins / kSelectThreads) + u) << shift);
-            }
-            higher += c[u];
-        }
-        known |= digit << shift;
-        __syncthreads();
     }
-    const uint32_t T = s_prefix;       // key of the k-th best candidate
-    const int ties = s_remaining;      // candidates of that key to take
+    if (ties < 0) ties = k - n_above;
 
     for (int i = tid; i < p.sink_blocks; i += kSelectThreads) idx[i] = i;
     for (int i = tid; i < p.local_blocks; i += kSelectThreads) idx[p.sink_blocks + k + i] = hi + i;
     // Ordered compaction (ascending block index = round e, then thread).  Register part: two ballots per round, the
     // (round, warp) counts scanned once by warps 0 and 1.
-    unsigned above[kKeysPerThread], tied[kKeysPerThread];
+    unsigned above[kSelectKeys], tied[kSelectKeys];
 #pragma unroll
-    for (int e = 0; e < kKeysPerThread; ++e) {
+    for (int e = 0; e < kSelectKeys; ++e) {
         const bool in = lo + tid + e * kSelectThreads < hi;
         above[e] = __ballot_sync(0xffffffffu, in && keys[e] > T);
         tied[e] = __ballot_sync(0xffffffffu, in && keys[e] == T);
@@ -359,13 +355,14 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(SelectParams p) 
         }
     }
     __syncthreads();
-    if (warp < 2) {  // exclusive scan of 128 counts: four per lane, then across lanes
+    if (warp < 2) {  // exclusive scan of the counts: some per lane, then across lanes
+        constexpr int kEach = kSelectKeys * kWarps / 32;
         int* counts = warp == 0 ? s_above : s_tied;
-        int c4[4], sum = 0;
+        int each[kEach], sum = 0;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            c4[u] = counts[lane * 4 + u];
-            sum += c4[u];
+        for (int u = 0; u < kEach; ++u) {
+            each[u] = counts[lane * kEach + u];
+            sum += each[u];
         }
         int incl = sum;
 #pragma unroll
@@ -375,9 +372,9 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(SelectParams p) 
         }
         int run = incl - sum;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            counts[lane * 4 + u] = run;
-            run += c4[u];
+        for (int u = 0; u < kEach; ++u) {
+            counts[lane * kEach + u] = run;
+            run += each[u];
         }
         if (lane == 31) (warp == 0 ? s_run_above : s_run_tied) = incl;
     }
@@ -388,12 +385,12 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(SelectParams p) 
         if (is_tied && n_tied < ties) idx[p.sink_blocks + n_above + n_tied] = i;
     };
 #pragma unroll
-    for (int e = 0; e < kKeysPerThread; ++e)
+    for (int e = 0; e < kSelectKeys; ++e)
         if (e < rounds)
             place(lo + tid + e * kSelectThreads, (above[e] >> lane) & 1u, (tied[e] >> lane) & 1u,
                   s_above[e * kWarps + warp] + __popc(above[e] & below_me), s_tied[e * kWarps + warp] + __popc(tied[e] & below_me));
-    // candidates beyond the register part (more than 4096 of them): round by round
-    for (int base = lo + kKeysPerThread * kSelectThreads; base < hi; base += kSelectThreads) {
+    // candidates beyond the register part: round by round
+    for (int base = lo + kSelectKeys * kSelectThreads; base < hi; base += kSelectThreads) {
         const int i = base + tid;
         const uint32_t key = i < hi ? select_key(score_at(i)) : 0u;
         const unsigned ab = __ballot_sync(0xffffffffu, i < hi && key > T), ti = __ballot_sync(0xffffffffu, i < hi && key == T);
@@ -627,8 +624,13 @@ specpv_status launch_scores(const ScoreParams& p, int n_layers, int max_nb, int 
 
 specpv_status launch_select(const SelectParams& p, int n_layers, cudaStream_t stream) {
     if (n_layers <= 0 || p.batch <= 0) return SPECPV_OK;
-    dim3 grid(p.Hkv, p.batch, n_layers);
-    SPECPV_LAUNCH(select_kernel, grid, kSelectThreads, 0, stream, p);
+    const dim3 grid(p.Hkv, p.batch, n_layers);
+    if (p.max_blocks <= 1024)
+        SPECPV_LAUNCH(select_kernel<256, 4>, grid, 256, 0, stream, p);
+    else if (p.max_blocks <= 4096)
+        SPECPV_LAUNCH(select_kernel<512, 8>, grid, 512, 0, stream, p);
+    else
+        SPECPV_LAUNCH(select_kernel<1024, 16>, grid, 1024, 0, stream, p);
     return SPECPV_OK;
 }
 

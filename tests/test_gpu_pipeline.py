@@ -574,3 +574,10 @@ def test_scores_of_a_refresh_step_with_more_rows_than_one_accumulator(reduce, sc
             assert np.isfinite(got).all()
             np.testing.assert_allclose(got, osc, rtol=2e-3, atol=2e-2, err_msg=f"layer {l} seq {b}")
             assert torch.isnan(scores[l, b, :, nb:]).all()  # blocks past the context are left alone
+
+
+@pytest.mark.parametrize("nb,budget", [(7, 5), (259, 100), (1024, 5), (1025, 64), (4096, 4095), (4097, 64), (16387, 128), (16500, 64)])
+def test_selection_at_the_edges_of_its_register_forms(nb, budget):
+    """Candidate counts either side of what the forms of the selection kernel keep in registers, one candidate to choose,
+    and all but one."""
+    test_selection_alone_on_synthetic_scores_with_ties_and_nan(nb, budget)
