@@ -115,28 +115,27 @@ __global__ void __launch_bounds__(32 * kSumWarps) summaries_kernel(SummaryParams
 }
 
 // ---------------------------------------------------------------------------------------------
-// Eq. 2-3 (SIMT form): lane <-> block, the CTA's 32 blocks' summaries staged in shared memory as float32; the warps share
-// the group's query rows out in turns of kScoreRowTile rows, which they read as broadcasts, and their partial results are
-// added in warp order.  Bound by latency on the small shapes it serves (2048 tokens, 64 rows: 40 -> 6 us against a warp
-// per 32 blocks that took all rows by itself).  grid = (block groups, Hkv, layers x seqs).
+// Eq. 2-3 (SIMT form): a warp owns kBlocks blocks, whose summaries are staged in shared memory as float32 and read as broadcasts, a
+// lane the query rows lane, lane + 32, .. of the group, staged kScoreRows at a time; a block's results are added over the lanes by
+// shuffles.  Bound by latency on the small shapes it serves: one block per warp spreads 75 blocks of two heads over 20 CTAs (a lane
+// per block and 32 blocks per CTA left them on 6: 128 rows of 64 channels 18.6 -> 6.6 us, 33 blocks and 64 rows 10.3 -> 4.1); four
+// blocks per warp read the rows once for four where the launch has CTAs enough.  grid = (block groups, Hkv, layers x seqs).
 // ---------------------------------------------------------------------------------------------
 constexpr int kScoreWarps = 8;
-constexpr int kScoreBlocksPerCta = 32;
-constexpr int kScoreRowTile = 4;
+constexpr int kScoreRows = 64;
 
-template <typename T, int D>
+template <typename T, int D, int kBlocks>
 __global__ void __launch_bounds__(32 * kScoreWarps) scores_simt_kernel(ScoreParams p) {
     pdl_begin(p.pdl);
-    extern __shared__ float smem[];
-    float* Smax = smem;                                   // [blocks][D + 1]
-    float* Smin = Smax + kScoreBlocksPerCta * (D + 1);    // [blocks][D + 1]
-    __shared__ float s_q[kScoreWarps][kScoreRowTile][D];
-    __shared__ float s_red[kScoreWarps][32];
+    constexpr int kPitch = D + 4, kCtaBlocks = kScoreWarps * kBlocks;  // pitch: a warp's 16-byte reads of 32 rows meet no bank twice
+    extern __shared__ __align__(16) float smem[];
+    float* rows_s = smem;                              // [kScoreRows][kPitch]
+    float* sums_s = rows_s + kScoreRows * kPitch;      // [blocks][2][D]: Kmax, Kmin
     const int h = blockIdx.y, lb = blockIdx.z, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = lb % p.batch, l = lb / p.batch;
     const int seq_len = p.seq_lens[b];
     const int nb = (seq_len + p.bs - 1) / p.bs;
-    const int blk0 = blockIdx.x * kScoreBlocksPerCta;
+    const int blk0 = blockIdx.x * kCtaBlocks;
     if (blk0 >= nb) return;
     int M = p.q_lens ? p.q_lens[b] : p.M_max;
     M = min(max(M, 0), p.M_max);
@@ -150,80 +149,81 @@ __global__ void __launch_bounds__(32 * kScoreWarps) scores_simt_kernel(ScorePara
     const size_t sum_base = ((((size_t)(p.layer0 + l) * p.batch + b) * p.Hkv + h) * p.max_blocks) * D;
     const T* kmax = reinterpret_cast<const T*>(p.kmax) + sum_base;
     const T* kmin = reinterpret_cast<const T*>(p.kmin) + sum_base;
-    for (int e = tid; e < kScoreBlocksPerCta * D; e += blockDim.x) {
-        int bi = e / D, c = e % D;
-        int i = blk0 + bi;
-        float vmax = 0.f, vmin = 0.f;
-        if (i < nb) {
-            vmax = to_float(kmax[(size_t)i * D + c]);
-            vmin = to_float(kmin[(size_t)i * D + c]);
-        }
-        Smax[bi * (D + 1) + c] = vmax;
-        Smin[bi * (D + 1) + c] = vmin;
+#pragma unroll
+    for (int e = tid; e < kCtaBlocks * D; e += 32 * kScoreWarps) {
+        const int bi = e / D, c = e % D, i = blk0 + bi;
+        sums_s[(bi * 2) * D + c] = i < nb ? to_float(kmax[(size_t)i * D + c]) : 0.f;
+        sums_s[(bi * 2 + 1) * D + c] = i < nb ? to_float(kmin[(size_t)i * D + c]) : 0.f;
     }
     const T* q = reinterpret_cast<const T*>(p.q) + (size_t)lb * p.M_max * p.Hq * D;
-    __syncthreads();
-    const float* my_max = Smax + lane * (D + 1);
-    const float* my_min = Smin + lane * (D + 1);
-    float red = p.reduce == SPECPV_REDUCE_MAX ? -INFINITY : 0.f;
-    for (int r0 = row_begin + warp * kScoreRowTile; r0 < row_end; r0 += kScoreWarps * kScoreRowTile) {
-        __syncwarp();
-        float (*Qs)[D] = s_q[warp];
-        for (int e = lane; e < kScoreRowTile * D; e += 32) {
-            int r = r0 + e / D, c = e % D;
-            float v = 0.f;
-            if (r < row_end) {
-                int j = r / p.G, g = r % p.G;
-                v = to_float(q[((size_t)j * p.Hq + h * p.G + g) * D + c]);
-            }
-            Qs[e / D][c] = v;
-        }
-        __syncwarp();
-        float dmax[kScoreRowTile], dmin[kScoreRowTile];
+    const bool reduce_max = p.reduce == SPECPV_REDUCE_MAX;
+    float red[kBlocks];
 #pragma unroll
-        for (int i = 0; i < kScoreRowTile; ++i) dmax[i] = dmin[i] = 0.f;
-        if (p.score_mode == 0) {
+    for (int k = 0; k < kBlocks; ++k) red[k] = reduce_max ? -INFINITY : 0.f;
+    for (int r0 = row_begin; r0 < row_end; r0 += kScoreRows) {
+        if (r0 != row_begin) __syncthreads();  // the rows before these have been read
+        const int n_rows = min(kScoreRows, row_end - r0);
 #pragma unroll 4
-            for (int c = 0; c < D; ++c) {
-                float a = my_max[c], bb = my_min[c];
+        for (int r = warp; r < n_rows; r += kScoreWarps) {
+            const T* src = q + ((size_t)((r0 + r) / p.G) * p.Hq + h * p.G + (r0 + r) % p.G) * D;
 #pragma unroll
-                for (int i = 0; i < kScoreRowTile; ++i) {
-                    float qc = Qs[i][c];
-                    dmax[i] = fmaf(qc, a, dmax[i]);
-                    dmin[i] = fmaf(qc, bb, dmin[i]);
-                }
-            }
-        } else {
-            // channel-wise form: a channel with q_c >= 0 takes Kmax_c, one with q_c < 0 takes Kmin_c
-            // (Kmax_c >= Kmin_c), so the score is one dot product with a per-channel choice of operand
-#pragma unroll 4
-            for (int c = 0; c < D; ++c) {
-                float a = my_max[c], bb = my_min[c];
-#pragma unroll
-                for (int i = 0; i < kScoreRowTile; ++i) {
-                    float qc = Qs[i][c];
-                    dmax[i] = fmaf(qc, qc < 0.f ? bb : a, dmax[i]);
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < kScoreRowTile; ++i) dmin[i] = dmax[i];
+            for (int c = lane; c < D; c += 32) rows_s[r * kPitch + c] = to_float(src[c]);
         }
+        __syncthreads();
+        for (int r = lane; r < n_rows; r += 32) {
+            const float* row = rows_s + r * kPitch;
+            const float* sums = sums_s + warp * kBlocks * 2 * D;
+            float dmax[kBlocks], dmin[kBlocks];
 #pragma unroll
-        for (int i = 0; i < kScoreRowTile; ++i) {
-            if (r0 + i >= row_end) continue;
-            float s = fmaxf(dmax[i], dmin[i]);
-            red = p.reduce == SPECPV_REDUCE_MAX ? fmaxf(red, s) : red + s;
+            for (int k = 0; k < kBlocks; ++k) dmax[k] = dmin[k] = 0.f;
+            if (p.score_mode == 0) {
+#pragma unroll 4
+                for (int c = 0; c < D; c += 4) {
+                    const float4 qv = *reinterpret_cast<const float4*>(row + c);
+#pragma unroll
+                    for (int k = 0; k < kBlocks; ++k) {
+                        const float4 a = *reinterpret_cast<const float4*>(sums + k * 2 * D + c);
+                        const float4 bb = *reinterpret_cast<const float4*>(sums + (k * 2 + 1) * D + c);
+                        dmax[k] = fmaf(qv.w, a.w, fmaf(qv.z, a.z, fmaf(qv.y, a.y, fmaf(qv.x, a.x, dmax[k]))));
+                        dmin[k] = fmaf(qv.w, bb.w, fmaf(qv.z, bb.z, fmaf(qv.y, bb.y, fmaf(qv.x, bb.x, dmin[k]))));
+                    }
+                }
+            } else {
+                // channel-wise form: a channel with q_c >= 0 takes Kmax_c, one with q_c < 0 takes Kmin_c
+                // (Kmax_c >= Kmin_c), so the score is one dot product with a per-channel choice of operand
+#pragma unroll 4
+                for (int c = 0; c < D; c += 4) {
+                    const float4 qv = *reinterpret_cast<const float4*>(row + c);
+#pragma unroll
+                    for (int k = 0; k < kBlocks; ++k) {
+                        const float4 a = *reinterpret_cast<const float4*>(sums + k * 2 * D + c);
+                        const float4 bb = *reinterpret_cast<const float4*>(sums + (k * 2 + 1) * D + c);
+                        dmax[k] = fmaf(qv.x, qv.x < 0.f ? bb.x : a.x, dmax[k]);
+                        dmax[k] = fmaf(qv.y, qv.y < 0.f ? bb.y : a.y, dmax[k]);
+                        dmax[k] = fmaf(qv.z, qv.z < 0.f ? bb.z : a.z, dmax[k]);
+                        dmax[k] = fmaf(qv.w, qv.w < 0.f ? bb.w : a.w, dmax[k]);
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < kBlocks; ++k) dmin[k] = dmax[k];
+            }
+#pragma unroll
+            for (int k = 0; k < kBlocks; ++k) {
+                const float s = fmaxf(dmax[k], dmin[k]);
+                red[k] = reduce_max ? fmaxf(red[k], s) : red[k] + s;
+            }
         }
     }
-    s_red[warp][lane] = red;
-    __syncthreads();
-    const int i = blk0 + tid;
-    if (tid < 32 && i < nb) {
-        red = s_red[0][tid];
 #pragma unroll
-        for (int w = 1; w < kScoreWarps; ++w) red = p.reduce == SPECPV_REDUCE_MAX ? fmaxf(red, s_red[w][tid]) : red + s_red[w][tid];
-        if (p.reduce != SPECPV_REDUCE_MAX) red /= (float)(row_end - row_begin);
-        p.scores[(((size_t)lb * p.Hkv + h) * p.max_blocks) + i] = red;
+    for (int k = 0; k < kBlocks; ++k) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float other = __shfl_xor_sync(0xffffffffu, red[k], o);
+            red[k] = reduce_max ? fmaxf(red[k], other) : red[k] + other;
+        }
+        const int i = blk0 + warp * kBlocks + k;
+        if (lane == 0 && i < nb)
+            p.scores[((size_t)lb * p.Hkv + h) * p.max_blocks + i] = reduce_max ? red[k] : red[k] / (float)(row_end - row_begin);
     }
 }
 
@@ -601,13 +601,21 @@ specpv_status launch_summaries(const SummaryParams& params, int n_layers, int bl
     return SPECPV_OK;
 }
 
+template <typename T, int D, int kBlocks>
+static specpv_status launch_scores_form(const ScoreParams& p, int n_layers, int max_nb, cudaStream_t stream) {
+    constexpr int kCtaBlocks = kScoreWarps * kBlocks;
+    const size_t smem = (size_t)(kScoreRows * (D + 4) + kCtaBlocks * 2 * D) * sizeof(float);
+    if (!tc::set_smem_limit_once(reinterpret_cast<const void*>(scores_simt_kernel<T, D, kBlocks>), (int)smem)) return SPECPV_ERR_CUDA;
+    dim3 grid((max_nb + kCtaBlocks - 1) / kCtaBlocks, p.Hkv, n_layers * p.batch);
+    SPECPV_LAUNCH(scores_simt_kernel<T, D, kBlocks>, grid, 32 * kScoreWarps, smem, stream, p);
+    return SPECPV_OK;
+}
+
 template <typename T, int D>
 static specpv_status launch_scores_typed(const ScoreParams& p, int n_layers, int max_nb, cudaStream_t stream) {
-    const size_t smem = (size_t)(2 * kScoreBlocksPerCta * (D + 1)) * sizeof(float);
-    if (!tc::set_smem_limit_once(reinterpret_cast<const void*>(scores_simt_kernel<T, D>), (int)smem)) return SPECPV_ERR_CUDA;
-    dim3 grid((max_nb + kScoreBlocksPerCta - 1) / kScoreBlocksPerCta, p.Hkv, n_layers * p.batch);
-    SPECPV_LAUNCH(scores_simt_kernel<T, D>, grid, 32 * kScoreWarps, smem, stream, p);
-    return SPECPV_OK;
+    // four blocks per warp once that still gives two CTAs to every SM
+    const long long ctas = (long long)((max_nb + 4 * kScoreWarps - 1) / (4 * kScoreWarps)) * p.Hkv * n_layers * p.batch;
+    return ctas >= 2 * 148 ? launch_scores_form<T, D, 4>(p, n_layers, max_nb, stream) : launch_scores_form<T, D, 1>(p, n_layers, max_nb, stream);
 }
 
 specpv_status launch_scores(const ScoreParams& p, int n_layers, int max_nb, int dtype, int d, cudaStream_t stream) {

@@ -581,3 +581,25 @@ def test_selection_at_the_edges_of_its_register_forms(nb, budget):
     """Candidate counts either side of what the forms of the selection kernel keep in registers, one candidate to choose,
     and all but one."""
     test_selection_alone_on_synthetic_scores_with_ties_and_nan(nb, budget)
+
+
+@pytest.mark.parametrize("blocks,layers", [(1, 1), (8, 1), (9, 1), (31, 75), (33, 75)])
+@pytest.mark.parametrize("M,d", [(16, 64), (17, 128), (33, 64)])
+def test_plain_scores_in_both_forms(blocks, layers, M, d):
+    """One block per warp and, with CTAs enough (75 layers x 2 heads x 2 groups of 32 blocks), four; 64, 68 and 132 rows around
+    the 64 that are staged at a time."""
+    w = wl.make_workload("tiny_fp32", device="cuda", n_layers=layers, Hq=8, Hkv=2, d=d, M=M, ctx=[64 * blocks - 5])
+    cfg, full = util.config_for(w, reduce=B.REDUCE_MEAN), util.full_cache(w)
+    ws = B.new_workspace(cfg, layers, 1, 64 * blocks, M)
+    kmax = torch.zeros((layers, 1, 2, w.max_blocks, d), dtype=torch.float32, device="cuda")
+    kmin = torch.zeros_like(kmax)
+    B.specpv_update_block_summaries(cfg, 0, layers, full, None, w.max_blocks, kmax, kmin, ws)
+    scores = torch.full((layers, 1, 2, w.max_blocks), float("nan"), dtype=torch.float32, device="cuda")
+    B.specpv_score_blocks(cfg, 0, layers, w.q, None, M, torch.zeros(1, dtype=torch.int32, device="cuda"), kmax, kmin, full, scores, ws)
+    util.sync_status(ws)
+    for l in {0, layers - 1}:
+        want = oracle.block_scores(wl.to_numpy(w.q[l, 0]), wl.to_numpy(kmax[l, 0])[:, :blocks],
+                                   wl.to_numpy(kmin[l, 0])[:, :blocks], 2, reduce=B.REDUCE_MEAN)
+        # products of the stored values summed in float32: d terms per dot product, then up to 132 rows
+        np.testing.assert_allclose(scores[l, 0, :, :blocks].cpu().numpy(), want, rtol=2e-5, atol=2e-4)
+        assert torch.isnan(scores[l, 0, :, blocks:]).all()
