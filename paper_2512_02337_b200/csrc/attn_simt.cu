@@ -11,8 +11,8 @@
 // a log-sum-exp merge.
 // Short calls are bound by latency: the form before this one (a warp per four rows, a lane per token, 256 tokens per CTA)
 // left a 2048-token call on 16 CTAs.  8 query heads of 64, 2 KV heads, 16 rows, float32: 2048 tokens 119 -> 18 us.
-// Larger ones are bound by shared-memory reads, two 16-byte loads per 16 multiplications (32 rows, 8192 tokens x 4 layers:
-// 283 -> 108 us).
+// Larger ones are bound by shared-memory reads, two 16-byte loads per 16 multiplications, which are done in packed pairs (32 rows,
+// 8192 tokens x 4 layers: 283 -> 108 us, one layer at a time 28.8 -> 26.7 by the packing).
 #include <math.h>
 
 #include "common.cuh"
@@ -84,6 +84,7 @@ __global__ void __launch_bounds__(kThreads) attn_simt_kernel(SimtParams p) {
     float* Vs = Kt + D * kPitch;
     float* Ps = Vs + kTok * D;
     __shared__ uint64_t s_mask[kRows][2];  // step tokens each row sees
+    __shared__ __align__(4) unsigned char s_exists[kTok];  // whether the tile has this token (one behind a bad page id is skipped)
 
     const int split = blockIdx.x % p.n_splits, row0 = blockIdx.x / p.n_splits * kRows;
     const int h = blockIdx.y, lb = blockIdx.z;
@@ -130,6 +131,7 @@ __global__ void __launch_bounds__(kThreads) attn_simt_kernel(SimtParams p) {
     }
     // K and V rows of tile `tile` for this thread's token, in flight while the previous tile is worked on
     float4 kbuf[kLoads], vbuf[kLoads];
+    bool exists = false;
     auto fetch = [&](int tile) {
         const T *ks = nullptr, *vs = nullptr;
         if (tile < ctx_tiles) {
@@ -140,6 +142,8 @@ __global__ void __launch_bounds__(kThreads) attn_simt_kernel(SimtParams p) {
                     const size_t off = (((size_t)page * p.Hkv + h) * p.bs + t % p.bs) * D;
                     ks = k_pool + off;
                     vs = v_pool + off;
+                } else if (sc == 0 && row0 == 0) {
+                    record_fault(p.workspace, SPECPV_ERR_BAD_BLOCK_TABLE, b, t / p.bs, page, l);
                 }
             }
         } else if ((tile - ctx_tiles) * kTok + st < M) {
@@ -147,6 +151,7 @@ __global__ void __launch_bounds__(kThreads) attn_simt_kernel(SimtParams p) {
             ks = k_new + off;
             vs = v_new + off;
         }
+        exists = ks != nullptr;
 #pragma unroll
         for (int i = 0; i < kLoads; ++i) {
             const int c = (sc + 4 * i) * 4;
@@ -176,50 +181,45 @@ __global__ void __launch_bounds__(kThreads) attn_simt_kernel(SimtParams p) {
             Kt[(c + 3) * kPitch + st] = kbuf[i].w;
             *reinterpret_cast<float4*>(Vs + st * D + c) = vbuf[i];
         }
+        if (sc == 0) s_exists[st] = exists;
         __syncthreads();
         if (tile + 1 < tile_end) fetch(tile + 1);
         // S = Q K^T: rows 4 ty .. + 3, tokens 4 tx .. + 3.  Channels are summed in runs of 16, the runs then added: the
         // rounding of a long serial sum would show in the weights of the largest logits.
-        float sv[4][4];
+        float2 sp[4][2];  // tokens (0, 1) and (2, 3)
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) sv[i][j] = 0.f;
+        for (int i = 0; i < 4; ++i) sp[i][0] = sp[i][1] = make_float2(0.f, 0.f);
 #pragma unroll 1
         for (int c0 = 0; c0 < D; c0 += 16) {
-            float part[4][4];
+            float2 part[4][2];
 #pragma unroll
             for (int cc = 0; cc < 16; ++cc) {
                 const float4 a = *reinterpret_cast<const float4*>(Qt + (c0 + cc) * kPitch + 4 * ty);
                 const float4 k4 = *reinterpret_cast<const float4*>(Kt + (c0 + cc) * kPitch + 4 * tx);
-                const float av[4] = {a.x, a.y, a.z, a.w}, kv[4] = {k4.x, k4.y, k4.z, k4.w};
+                const float av[4] = {a.x, a.y, a.z, a.w};
+                const float2 kv[2] = {make_float2(k4.x, k4.y), make_float2(k4.z, k4.w)};
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) part[i][j] = cc == 0 ? av[i] * kv[j] : fmaf(av[i], kv[j], part[i][j]);
+                    for (int j = 0; j < 2; ++j)
+                        part[i][j] = cc == 0 ? __fmul2_rn(make_float2(av[i], av[i]), kv[j]) : __ffma2_rn(make_float2(av[i], av[i]), kv[j], part[i][j]);
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) sv[i][j] += part[i][j];
+                for (int j = 0; j < 2; ++j) sp[i][j] = __fadd2_rn(sp[i][j], part[i][j]);
         }
-        // which of the thread's tokens exist (a token behind a bad page id is skipped)
-        unsigned exists = 0;
+        float sv[4][4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int t = tok0 + 4 * tx + j;
-            bool ok = t < (is_new ? M : seq_len);
-            if (ok && !is_new) {
-                const int page = table[t / p.bs];
-                ok = page >= 0 && page < p.n_pages;
-                if (!ok && ty == 0 && row0 == 0) record_fault(p.workspace, SPECPV_ERR_BAD_BLOCK_TABLE, b, t / p.bs, page, l);
-            }
-            exists |= (unsigned)ok << j;
+        for (int i = 0; i < 4; ++i) {
+            sv[i][0] = sp[i][0].x; sv[i][1] = sp[i][0].y; sv[i][2] = sp[i][1].x; sv[i][3] = sp[i][1].y;
         }
+        const uchar4 e4 = *reinterpret_cast<const uchar4*>(s_exists + 4 * tx);
+        const unsigned in_tile = (unsigned)e4.x | (unsigned)e4.y << 1 | (unsigned)e4.z << 2 | (unsigned)e4.w << 3;
         float corr[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            unsigned vis = exists;
+            unsigned vis = in_tile;
             if (is_new) vis &= (unsigned)(s_mask[4 * ty + i][(tok0 + 4 * tx) >> 6] >> ((4 * tx) & 63)) & 15u;
             float mx = -INFINITY;
 #pragma unroll
@@ -244,11 +244,11 @@ __global__ void __launch_bounds__(kThreads) attn_simt_kernel(SimtParams p) {
         // O = O corr + P V, channels c * 16 + 4 tx + ..: the tile's 64 products are summed apart and then added, because one chain
         // over a CTA's whole share (2112 tokens of 8192 with 240 rows x 8 heads x 2 layers) loses digits (8.9e-7 against 8.2e-7
         // with 432 tokens to a chain).
-        float tile_acc[4][CPT];
+        float2 tile_acc[4][CPT / 2];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int c = 0; c < CPT; ++c) tile_acc[i][c] = 0.f;
+            for (int c = 0; c < CPT / 2; ++c) tile_acc[i][c] = make_float2(0.f, 0.f);
 #pragma unroll 2
         for (int t = 0; t < kTok; t += 4) {
             float4 pr[4];
@@ -256,24 +256,25 @@ __global__ void __launch_bounds__(kThreads) attn_simt_kernel(SimtParams p) {
             for (int i = 0; i < 4; ++i) pr[i] = *reinterpret_cast<const float4*>(Ps + (4 * ty + i) * kPitch + t);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                float vv[CPT];
+                float2 vv[CPT / 2];
 #pragma unroll
                 for (int c = 0; c < CPT; c += 4) {
                     const float4 v4 = *reinterpret_cast<const float4*>(Vs + (t + u) * D + c * 16 + 4 * tx);
-                    vv[c] = v4.x; vv[c + 1] = v4.y; vv[c + 2] = v4.z; vv[c + 3] = v4.w;
+                    vv[c / 2] = make_float2(v4.x, v4.y);
+                    vv[c / 2 + 1] = make_float2(v4.z, v4.w);
                 }
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const float w = u == 0 ? pr[i].x : u == 1 ? pr[i].y : u == 2 ? pr[i].z : pr[i].w;
 #pragma unroll
-                    for (int c = 0; c < CPT; ++c) tile_acc[i][c] = fmaf(w, vv[c], tile_acc[i][c]);
+                    for (int c = 0; c < CPT / 2; ++c) tile_acc[i][c] = __ffma2_rn(make_float2(w, w), vv[c], tile_acc[i][c]);
                 }
             }
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int c = 0; c < CPT; ++c) acc[i][c] = fmaf(acc[i][c], corr[i], tile_acc[i][c]);
+            for (int c = 0; c < CPT; ++c) acc[i][c] = fmaf(acc[i][c], corr[i], c % 2 ? tile_acc[i][c / 2].y : tile_acc[i][c / 2].x);
     }
     // acc[i][c .. c + 3] are channels 16 c + 4 tx .. + 3 of row 4 ty + i
 #pragma unroll
@@ -302,59 +303,79 @@ __global__ void __launch_bounds__(kThreads) attn_simt_kernel(SimtParams p) {
     }
 }
 
-// Log-sum-exp merge of the per-split partial results: D/4 threads per row, four channels each, eight partial rows in flight
-// per thread; grid = (row groups, KV heads, layers x seqs).
+// Log-sum-exp merge of the per-split partial results: D/4 threads per row and group of D/4 splits, four channels each, eight
+// partial rows in flight per thread; a row's groups (up to 64 splits in all) meet in shared memory and are added in order.  Bound by
+// latency: 64 splits one group of lanes after the other took 8.1 us a call, side by side 4.6; 33 splits 5.9 and 3.5.  grid = (row groups, KV heads, layers x seqs).
 constexpr int kMergeThreads = 128;
 constexpr int kMergeAhead = 8;
 template <typename TO, int D>
 __global__ void __launch_bounds__(kMergeThreads) merge_splits_kernel(SimtParams p) {
     pdl_begin(p.pdl);
-    constexpr int kRowThreads = D / 4;
-    const int r = blockIdx.x * (kMergeThreads / kRowThreads) + threadIdx.x / kRowThreads;
-    const int h = blockIdx.y, lb = blockIdx.z, lane = threadIdx.x % kRowThreads;
+    constexpr int kRowThreads = D / 4, kGroups = 64 / kRowThreads, kRowsAtOnce = kMergeThreads / 64;
+    __shared__ float4 s_o[kMergeThreads];
+    __shared__ float s_l[kMergeThreads];
+    const int r = blockIdx.x * kRowsAtOnce + threadIdx.x / 64;
+    const int h = blockIdx.y, lb = blockIdx.z, lane = threadIdx.x % kRowThreads, group = threadIdx.x % 64 / kRowThreads;
     const int b = lb % p.batch;
     int M = p.q_lens ? p.q_lens[b] : p.M_max;
     M = min(max(M, 0), p.M_max);
-    if (r >= M * p.G) return;
+    const bool row_valid = r < M * p.G;
     const unsigned members = kRowThreads == 32 ? 0xffffffffu : 0xffffu << (threadIdx.x & 16);
     const int R_max = p.M_max * p.G;
-    const size_t row0 = ((size_t)lb * p.Hkv + h) * p.n_splits * R_max + r;
+    const size_t row0 = ((size_t)lb * p.Hkv + h) * p.n_splits * R_max + (row_valid ? r : 0);
+    const int c0 = group * kRowThreads, n = min(kRowThreads, p.n_splits - c0);  // this group's splits
     const float4* po = reinterpret_cast<const float4*>(p.part_o + row0 * D) + lane;
     const float2* ml = reinterpret_cast<const float2*>(p.part_ml) + row0;
     const size_t po_stride = (size_t)R_max * kRowThreads;
+    float4 buf[kMergeAhead];
+    auto fetch = [&](int s0) {
+#pragma unroll
+        for (int u = 0; u < kMergeAhead; ++u)
+            if (s0 + u < n) buf[u] = po[(size_t)(c0 + s0 + u) * po_stride];
+    };
+    fetch(0);
     float m_all = -INFINITY;
-    for (int s = lane; s < p.n_splits; s += kRowThreads) m_all = fmaxf(m_all, ml[(size_t)s * R_max].x);
+    float2 mine = make_float2(-INFINITY, 0.f);  // of split c0 + lane
+#pragma unroll
+    for (int g = 0; g < kGroups; ++g)
+        if (g * kRowThreads + lane < p.n_splits) {
+            const float2 v = ml[(size_t)(g * kRowThreads + lane) * R_max];
+            m_all = fmaxf(m_all, v.x);
+            if (g == group) mine = v;
+        }
 #pragma unroll
     for (int o = kRowThreads / 2; o > 0; o >>= 1) m_all = fmaxf(m_all, __shfl_xor_sync(members, m_all, o));
+    float w_mine = 0.f, l_mine = 0.f;
+    if (mine.x != -INFINITY) {  // a split that saw no token weighs nothing
+        w_mine = expf(mine.x - m_all);
+        l_mine = mine.y * w_mine;
+    }
     float l_all = 0.f;
     float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int c0 = 0; c0 < p.n_splits; c0 += kRowThreads) {  // a lane per split of this chunk
-        const int n = min(kRowThreads, p.n_splits - c0);
-        float w_mine = 0.f, l_mine = 0.f;
-        if (lane < n) {
-            const float2 v = ml[(size_t)(c0 + lane) * R_max];
-            if (v.x != -INFINITY) {  // a split that saw no token weighs nothing
-                w_mine = expf(v.x - m_all);
-                l_mine = v.y * w_mine;
-            }
-        }
-        for (int s0 = 0; s0 < n; s0 += kMergeAhead) {
-            float4 buf[kMergeAhead];
+    for (int s0 = 0; s0 < n; s0 += kMergeAhead) {
+        if (s0) fetch(s0);
 #pragma unroll
-            for (int u = 0; u < kMergeAhead; ++u) buf[u] = po[(size_t)(c0 + min(s0 + u, n - 1)) * po_stride];
-#pragma unroll
-            for (int u = 0; u < kMergeAhead; ++u) {
-                // lanes past the last split hold weight 0; beyond the row's lanes the shuffle would wrap
-                const float w = __shfl_sync(members, w_mine, min(s0 + u, kRowThreads - 1), kRowThreads);
-                const float lw = __shfl_sync(members, l_mine, min(s0 + u, kRowThreads - 1), kRowThreads);
-                if (s0 + u >= n || w == 0.f) continue;
-                l_all += lw;
-                o.x = fmaf(buf[u].x, w, o.x);
-                o.y = fmaf(buf[u].y, w, o.y);
-                o.z = fmaf(buf[u].z, w, o.z);
-                o.w = fmaf(buf[u].w, w, o.w);
-            }
+        for (int u = 0; u < kMergeAhead; ++u) {  // (D/4 is a multiple of kMergeAhead: the shuffles stay among the row's lanes)
+            const float w = __shfl_sync(members, w_mine, s0 + u, kRowThreads);
+            const float lw = __shfl_sync(members, l_mine, s0 + u, kRowThreads);
+            if (s0 + u >= n || w == 0.f) continue;
+            l_all += lw;
+            o.x = fmaf(buf[u].x, w, o.x);
+            o.y = fmaf(buf[u].y, w, o.y);
+            o.z = fmaf(buf[u].z, w, o.z);
+            o.w = fmaf(buf[u].w, w, o.w);
         }
+    }
+    s_o[threadIdx.x] = o;
+    s_l[threadIdx.x] = l_all;
+    __syncthreads();
+    if (!row_valid || group) return;
+#pragma unroll
+    for (int g = 1; g < kGroups; ++g) {
+        if (g * kRowThreads >= p.n_splits) break;
+        const float4 v = s_o[threadIdx.x + g * kRowThreads];
+        o.x += v.x; o.y += v.y; o.z += v.z; o.w += v.w;
+        l_all += s_l[threadIdx.x + g * kRowThreads];
     }
     const int j = r / p.G, g = r % p.G;
     const size_t row = ((size_t)lb * p.M_max + j) * p.Hq + h * p.G + g;
@@ -375,7 +396,7 @@ specpv_status launch_typed(const AttnArgs& a, SimtParams& p, cudaStream_t stream
     if (launch_pdl_if(attn_simt_kernel<T, TO, D>, grid, kThreads, smem, stream, p) != cudaSuccess) return SPECPV_ERR_CUDA;
     count_launch();
     if (p.n_splits > 1) {
-        constexpr int rows = kMergeThreads / (D / 4);
+        constexpr int rows = kMergeThreads / 64;
         dim3 mgrid((a.M_max * a.g.G + rows - 1) / rows, a.g.Hkv, a.n_layers * a.batch);
         if (launch_pdl_if(merge_splits_kernel<TO, D>, mgrid, kMergeThreads, 0, stream, p) != cudaSuccess) return SPECPV_ERR_CUDA;
         count_launch();

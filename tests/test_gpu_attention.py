@@ -365,3 +365,10 @@ def test_short_walks_of_one_cta(Hq, Hkv, d, tiles):
     """Enough heads that no KV range is split: a CTA walks `tiles` context tiles of 128 tokens (the last one ragged) and the step's
     own, one tile (nothing for the second stream), as many as the short walk of the two-term form takes, and more."""
     run_case("bf16", Hq, Hkv, d, 64, ctx=[max(128 * tiles - 27, 0)], Ms=[6], n_layers=19, seed=60 + tiles, float32_weights=d == 64 or Hq == 40)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("splits", [2, 15, 16, 17, 32, 33, 63, 64])
+def test_float32_merge_around_its_groups_of_splits(d, splits):
+    """One tile of 64 tokens per split (64 of them at most): counts around the 16 (32 with 128 channels) that a group of lanes merges."""
+    run_case("fp32", 8, 2, d, 64, ctx=[64 * (splits - 1) - 7], Ms=[5], seed=90 + splits)
