@@ -473,26 +473,26 @@ __global__ void __launch_bounds__(128) gather_kernel(GatherParams p) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// Commit: grid = (blocks touched, Hkv, layers x seqs); a CTA appends the accepted tokens' K and V rows that fall into one
-// block (a warp per row) and recomputes the block's summary, the appended tokens taken from the step's tensors.  The lengths
-// advance in a launch behind it: every CTA reads them, and a commit keeps nothing in the workspace but the status word, so that
-// commits of two caches on two streams may share one (an arrival counter there made the launch unnecessary, 9.3 us a call against
-// 11.4, but mixed the arrivals of two such commits).  Bound by launches: rows, summaries and lengths in three took 14 us of host
-// time a call.
+// Commit: four warps append the accepted tokens' K and V rows that fall into one block (a warp per row) and recompute the block's
+// summary, the appended tokens taken from the step's tensors; a unit of work is (block touched, KV head, layer x seq).  All units
+// read the lengths.  Where they fit into two turns of one CTA (one float32 layer, short steps), that CTA advances the lengths
+// itself; else a CTA takes a unit, and the lengths advance in a launch behind it: a commit keeps nothing in the workspace but the
+// status word, so that commits of two caches on two streams may share one (an arrival counter there made the launch unnecessary,
+// 9.3 us a call against 11.4, but mixed the arrivals of two such commits).  Bound by launches: rows, summaries and lengths in
+// three took 14 us of host time a call, in two 6.7; in one a float32 step with two commits takes 67.7 us instead of 74.4.
 // ---------------------------------------------------------------------------------------------
 constexpr int kCommitWarps = 4;
+constexpr int kCommitUnits = 4;  // of one CTA at a time
 
 template <typename T>
-__global__ void __launch_bounds__(32 * kCommitWarps) commit_kernel(CommitParams p) {
-    pdl_begin(p.pdl);
-    const int h = blockIdx.y, lb = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__device__ __forceinline__ void commit_unit(const CommitParams& p, int touched, int h, int lb, int warp, int lane) {
     const int b = lb % p.batch, l = lb / p.batch;
     const int n = min(max(p.n_accepted[b], 0), p.A_max);
     const int seq_len = p.seq_lens[b];
     const bool fits = (size_t)seq_len + n <= (size_t)p.max_blocks * p.bs;
-    const int i = max(seq_len, 0) / p.bs + blockIdx.x;  // logical block
+    const int i = max(seq_len, 0) / p.bs + touched;  // logical block
     if (!fits) {
-        if (threadIdx.x == 0 && blockIdx.x == 0 && h == 0 && n > 0) record_fault(p.workspace, SPECPV_ERR_CAPACITY, b, seq_len, n, l);
+        if (warp == 0 && lane == 0 && touched == 0 && h == 0 && n > 0) record_fault(p.workspace, SPECPV_ERR_CAPACITY, b, seq_len, n, l);
     } else {
         const int t0 = max(seq_len, i * p.bs), t1 = min(seq_len + n, (i + 1) * p.bs);  // tokens appended to this block
         const bool summarise = p.kmax && (size_t)i * p.bs < (size_t)(seq_len + n) && i < p.max_blocks;
@@ -500,7 +500,7 @@ __global__ void __launch_bounds__(32 * kCommitWarps) commit_kernel(CommitParams 
         if (t0 < t1 || summarise) {
             page = p.block_table[(size_t)b * p.max_blocks + i];
             if (page < 0 || page >= p.n_pages) {
-                if (threadIdx.x == 0) record_fault(p.workspace, SPECPV_ERR_BAD_BLOCK_TABLE, b, i, page, l);
+                if (warp == 0 && lane == 0) record_fault(p.workspace, SPECPV_ERR_BAD_BLOCK_TABLE, b, i, page, l);
                 page = -1;
             }
         }
@@ -570,13 +570,33 @@ __global__ void __launch_bounds__(32 * kCommitWarps) commit_kernel(CommitParams 
     }
 }
 
+__device__ __forceinline__ void advance_length(const CommitParams& p, int b) {
+    const int n = min(max(p.n_accepted[b], 0), p.A_max);
+    if ((size_t)p.seq_lens[b] + n <= (size_t)p.max_blocks * p.bs) p.seq_lens[b] += n;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(32 * kCommitWarps) commit_kernel(CommitParams p) {
+    pdl_begin(p.pdl);
+    commit_unit<T>(p, blockIdx.x, blockIdx.y, blockIdx.z, threadIdx.x >> 5, threadIdx.x & 31);
+}
+
 constexpr int kLensThreads = 128;
 __global__ void __launch_bounds__(kLensThreads) commit_lens_kernel(CommitParams p) {
     pdl_begin(p.pdl);
     const int b = blockIdx.x * kLensThreads + threadIdx.x;
-    if (b >= p.batch) return;
-    const int n = min(max(p.n_accepted[b], 0), p.A_max);
-    if ((size_t)p.seq_lens[b] + n <= (size_t)p.max_blocks * p.bs) p.seq_lens[b] += n;
+    if (b < p.batch) advance_length(p, b);
+}
+
+// One CTA: units (x, y, z) of a grid of `units`, at most twice kCommitUnits of them, and the lengths behind a barrier.
+template <typename T>
+__global__ void __launch_bounds__(32 * kCommitWarps * kCommitUnits) commit_small_kernel(CommitParams p, dim3 units) {
+    pdl_begin(1);
+    const int n = units.x * units.y * units.z;
+    for (int u = threadIdx.x / (32 * kCommitWarps); u < n; u += kCommitUnits)
+        commit_unit<T>(p, u % units.x, u / units.x % units.y, u / (units.x * units.y), (threadIdx.x >> 5) % kCommitWarps, threadIdx.x & 31);
+    __syncthreads();  // every unit has read the lengths
+    if ((int)threadIdx.x < p.batch) advance_length(p, threadIdx.x);
 }
 
 }  // namespace
@@ -652,6 +672,14 @@ specpv_status launch_commit(const CommitParams& params, int n_layers, int dtype,
     CommitParams p = params;
     p.aligned = aligned16(p.kmax) && aligned16(p.kmin);
     dim3 grid((p.A_max + p.bs - 1) / p.bs + 1, p.Hkv, n_layers * p.batch);
+    // at most two turns of the one CTA: each is a chain of three loads, some 2 us, against a launch
+    if (advance && (long long)grid.x * grid.y * grid.z <= 2 * kCommitUnits) {
+        if (launch_pdl(dtype == SPECPV_DTYPE_F32 ? commit_small_kernel<float> : commit_small_kernel<__nv_bfloat16>, 1,
+                       32 * kCommitWarps * kCommitUnits, 0, stream, p, grid) != cudaSuccess)
+            return SPECPV_ERR_CUDA;
+        count_launch();
+        return SPECPV_OK;
+    }
     SPECPV_LAUNCH(dtype == SPECPV_DTYPE_F32 ? commit_kernel<float> : commit_kernel<__nv_bfloat16>, grid, 32 * kCommitWarps, 0, stream, p);
     if (advance) SPECPV_LAUNCH(commit_lens_kernel, dim3((p.batch + kLensThreads - 1) / kLensThreads), kLensThreads, 0, stream, p);
     return SPECPV_OK;

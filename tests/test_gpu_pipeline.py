@@ -603,3 +603,39 @@ def test_plain_scores_in_both_forms(blocks, layers, M, d):
         # products of the stored values summed in float32: d terms per dot product, then up to 132 rows
         np.testing.assert_allclose(scores[l, 0, :, :blocks].cpu().numpy(), want, rtol=2e-5, atol=2e-4)
         assert torch.isnan(scores[l, 0, :, blocks:]).all()
+
+
+@pytest.mark.parametrize("dtype,Hkv,batch,bs,A", [("fp32", 1, 1, 64, 4), ("fp32", 2, 2, 64, 4), ("bf16", 1, 4, 16, 16), ("bf16", 4, 1, 32, 5),
+                                                  ("fp32", 3, 1, 16, 17)])
+def test_commit_of_few_units_in_one_launch(dtype, Hkv, batch, bs, A):
+    """Up to eight units of work (block touched, KV head, sequence) go through one CTA that advances the lengths itself; nine, the last
+    case, through two launches.  Three commits in a row, of which the second appends nothing to the first sequence."""
+    d, M = 64, 24
+    w = wl.make_workload("tiny_fp32", device="cuda", n_layers=1, spare_tokens=256, Hq=2 * Hkv, Hkv=Hkv, d=d, bs=bs, dtype=dtype, M=M,
+                         ctx=[bs * 3 + 5 * b - 1 for b in range(batch)])
+    cfg, full = B.make_config(1, 2 * Hkv, Hkv, d, bs, dtype, 1, 1, 3, bs), util.full_cache(w)
+    full.max_seq_len = int(max(w.cfg["ctx"])) + 256
+    ws = torch.zeros(4096, dtype=torch.uint8, device="cuda")
+    kmax = torch.zeros((1, batch, Hkv, w.max_blocks, d), dtype=wl.torch_dtype(dtype), device="cuda")
+    kmin = torch.zeros_like(kmax)
+    B.specpv_update_block_summaries(cfg, 0, 1, full, None, w.max_blocks, kmax, kmin, ws)
+    kp, vp = wl.to_numpy(w.k_pool).copy(), wl.to_numpy(w.v_pool).copy()
+    lens, table = [int(x) for x in w.cfg["ctx"]], w.block_table.cpu().numpy()
+    knn, vnn = wl.to_numpy(w.k_new), wl.to_numpy(w.v_new)
+    rng = np.random.default_rng(bs + A)
+    for turn in range(3):
+        acc = rng.integers(0, M, size=(batch, A)).astype(np.int32)
+        counts = [0 if turn == 1 and b == 0 else A - b % 2 for b in range(batch)]
+        before = B.specpv_kernel_launches()
+        B.specpv_commit_accepted(cfg, 0, 1, w.k_new, w.v_new, M, torch.from_numpy(acc).cuda(),
+                                 torch.tensor(counts, dtype=torch.int32, device="cuda"), A, full, kmax, kmin, ws)
+        assert B.specpv_kernel_launches() - before == (2 if Hkv == 3 else 1)
+        util.sync_status(ws)
+        for b in range(batch):
+            new_len = oracle.commit(knn[0, b], vnn[0, b], acc[b, :counts[b]], kp[0], vp[0], table[b], lens[b])
+            okmax, okmin = oracle.block_summaries(kp[0], table[b], new_len)
+            nb = (new_len + bs - 1) // bs
+            assert np.array_equal(util.widen_t(kmax[0, b])[:, :nb], okmax) and np.array_equal(util.widen_t(kmin[0, b])[:, :nb], okmin)
+            lens[b] += counts[b]
+            assert int(w.seq_lens[b]) == lens[b]
+        assert np.array_equal(wl.to_numpy(w.k_pool), kp) and np.array_equal(wl.to_numpy(w.v_pool), vp)
