@@ -394,7 +394,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1) att
         bool ok = true;
         for (int sidx = 0; ok && it.next(p, s); ++sidx) {
             const int qb = sidx & 1;
-            if (sidx >= 2) ok = pair_wait(smem_u32(&bars.q_empty[qb]), ((sidx >> 1) - 1) & 1, abort_flag, peer_abort, p.workspace, 1);
+            if (sidx >= 2) ok = __all_sync(0xffffffffu, pair_wait(smem_u32(&bars.q_empty[qb]), ((sidx >> 1) - 1) & 1, abort_flag, peer_abort, p.workspace, 1));
             if (!ok) break;
             if (lane == 0) {
                 if (rank == 0) mbar_expect_tx(smem_u32(&bars.q_full[qb]), 2 * kQTile);
@@ -409,7 +409,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1) att
                 const uint32_t ks = t % kRing;
                 const int page = page_next;
                 if (k_lane && j + 1 < s.n_ctx) page_next = page_load(s, blk + ppt);
-                if (t >= (uint32_t)kRing) ok = pair_wait(smem_u32(&bars.k_empty[ks]), ((t / kRing) - 1) & 1, abort_flag, peer_abort, p.workspace, 2);
+                if (t >= (uint32_t)kRing) ok = __all_sync(0xffffffffu, pair_wait(smem_u32(&bars.k_empty[ks]), ((t / kRing) - 1) & 1, abort_flag, peer_abort, p.workspace, 2));
                 if (!ok) break;
                 const uint32_t dst = k_smem + ks * kHalf, full = lead_k_full0 + ks * 8;
                 if (lane == 0 && rank == 0) mbar_expect_tx(smem_u32(&bars.k_full[ks]), 2 * kHalf);
@@ -439,6 +439,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1) att
                     ok = pair_wait(smem_u32(&bars.v_full[vs]), (g / kRing) & 1, abort_flag, peer_abort, p.workspace, 4);
                     if (ok && j == 0 && sidx > 0) ok = pair_wait(smem_u32(&bars.o_free), (sidx - 1) & 1, abort_flag, peer_abort, p.workspace, 6);
                     if (ok) ok = pair_wait(smem_u32(&bars.p_full[buf]), (g / kLag) & 1, abort_flag, peer_abort, p.workspace, 7);
+                    ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
                     tc_fence_after();
                     if (lane == 0) {
@@ -473,7 +474,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1) att
                 const uint32_t vs = g % kRing;
                 const int page = page_next;
                 if (v_lane && j + 1 < s.n_ctx) page_next = page_load(s, blk + ppt);
-                if (g >= (uint32_t)kRing) ok = pair_wait(smem_u32(&bars.v_empty[vs]), ((g / kRing) - 1) & 1, abort_flag, peer_abort, p.workspace, 16);
+                if (g >= (uint32_t)kRing) ok = __all_sync(0xffffffffu, pair_wait(smem_u32(&bars.v_empty[vs]), ((g / kRing) - 1) & 1, abort_flag, peer_abort, p.workspace, 16));
                 if (!ok) break;
                 const bool fix = j >= s.first_fix;
                 const uint32_t dst = v_smem + vs * kHalf, full = lead_v_full0 + vs * 8, vfix = smem_u32(&bars.vfix_full[vs]);
@@ -493,7 +494,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1) att
                 }
                 __syncwarp();
                 if (fix) {
-                    ok = pair_wait(vfix, (fix_parity >> vs) & 1u, abort_flag, peer_abort, p.workspace, 8);
+                    ok = __all_sync(0xffffffffu, pair_wait(vfix, (fix_parity >> vs) & 1u, abort_flag, peer_abort, p.workspace, 8));
                     if (!ok) break;
                     fix_parity ^= 1u << vs;
                     const int n_valid = max(j >= s.n_ctx ? s.M : min(kTileTokens, s.seq_len - (s.tile_begin + j) * kTileTokens), 0);
@@ -526,6 +527,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1) att
                     if (ok) ok = pair_wait(smem_u32(&bars.k_full[ks]), (t / kRing) & 1, abort_flag, peer_abort, p.workspace, 13);
                     if (ok && t >= (uint32_t)kLag)
                         ok = pair_wait(smem_u32(&bars.v_empty[(t - kLag) % kRing]), ((t - kLag) / kRing) & 1, abort_flag, peer_abort, p.workspace, 14);
+                    ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
                     tc_fence_after();
                     if (lane == 0) {
@@ -779,17 +781,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1) att
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&bars.rows_done));
                 if (warp == 4) {  // every warp of this CTA has written its rows: take a ticket
-                    ok = pair_wait(smem_u32(&bars.rows_done), rows_phase & 1, abort_flag, peer_abort, p.workspace, 17);
+                    ok = __all_sync(0xffffffffu, pair_wait(smem_u32(&bars.rows_done), rows_phase & 1, abort_flag, peer_abort, p.workspace, 17));
                     if (ok && lane == 0) bars.ticket = atomicAdd(p.counters + s.counter + (int)rank, 1);
                     __syncwarp();
                 } else {
-                    ok = pair_wait(smem_u32(&bars.rows_done), rows_phase & 1, abort_flag, peer_abort, p.workspace, 17);
+                    ok = __all_sync(0xffffffffu, pair_wait(smem_u32(&bars.rows_done), rows_phase & 1, abort_flag, peer_abort, p.workspace, 17));
                 }
                 if (!ok) break;
                 ++rows_phase;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&bars.rows_done));  // second round: the ticket is in shared memory
-                ok = pair_wait(smem_u32(&bars.rows_done), rows_phase & 1, abort_flag, peer_abort, p.workspace, 18);
+                ok = __all_sync(0xffffffffu, pair_wait(smem_u32(&bars.rows_done), rows_phase & 1, abort_flag, peer_abort, p.workspace, 18));
                 if (!ok) break;
                 ++rows_phase;
                 if (*reinterpret_cast<volatile int*>(&bars.ticket) == s.n_seg - 1) {

@@ -151,7 +151,7 @@ __device__ __forceinline__ void produce(const TcParams& p, const Job& c, Barrier
             const int j = kv ? i - lag : i;
             if (j < 0 || j >= c.n_tiles) continue;
             const uint32_t full = smem_u32(&bars.kv_full[slot]), empty = smem_u32(&bars.kv_empty[slot]);
-            if (use >= (uint32_t)kStages) ok = mbar_wait(empty, par, abort_flag, p.workspace, 1);
+            if (use >= (uint32_t)kStages) ok = __all_sync(0xffffffffu, mbar_wait(empty, par, abort_flag, p.workspace, 1));
             if (!ok) break;  // a wait gave up: nothing more is copied
             const uint32_t dst = kv_smem + slot * kSlotBytes;
             if (j >= c.n_ctx_tiles) {  // the step's own tokens, a copy per group and part; the rest of the slot is masked or zeroed
@@ -216,7 +216,8 @@ __device__ __forceinline__ void issue(const TcParams& p, const Job& c, Barriers&
     // Ring uses: K0 | V0 K1 | V1 K2 | .. with two row tiles, K0 | K1 | V0 K2 | V1 K3 | .. with one.
     // A wait that gives up raises the abort flag, which makes the later waits of this tile return at once; the
     // loop ends after this tile, so at most one tile's contractions are issued past the failed wait.  (One exit
-    // per tile: an exit after every wait costs the issuing thread 7 % of the kernel.)
+    // per tile: an exit after every wait costs the issuing thread 7 % of the kernel.)  The lanes leave together, on a vote: they
+    // test the barrier and the flag each for itself, and one that left alone would be missing where the others meet.
     if (!kOne) {
         uint32_t k_slot = 0, k_par = 0, v_slot = 1, v_par = 0;  // slot and phase parity of the next K and V tile
         for (int j = 0; j <= n_tiles; ++j) {
@@ -249,8 +250,9 @@ __device__ __forceinline__ void issue(const TcParams& p, const Job& c, Barriers&
                         if (t == 1) tc_commit(empty0 + k_slot * 8);
                     }
                 }
-                __syncwarp();
+                if (t == 0) __syncwarp();
             }
+            ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             if (j < n_tiles) { k_slot += 2; if (k_slot >= kStages) { k_slot -= kStages; k_par ^= 1; } }
             if (j > 0) { v_slot += 2; if (v_slot >= kStages) { v_slot -= kStages; v_par ^= 1; } }
@@ -289,7 +291,7 @@ __device__ __forceinline__ void issue(const TcParams& p, const Job& c, Barriers&
                     tc_commit(empty0 + k_slot * 8);
                 }
             }
-            __syncwarp();
+            ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
         }
     }
@@ -372,6 +374,9 @@ __device__ __forceinline__ void softmax(const TcParams& p, const Job& c, Barrier
     const int n_tiles = c.n_tiles;
     constexpr int step = kOne ? 2 : 1;
     const int first_tile = kOne ? t : 0;     // K/V tiles of this stream: first_tile, first_tile + step, ..
+    // (two row tiles: n_tiles is never 0 here; said, it changes the loop's code, 33 rows x 4 of 64 channels, 16000 tokens x 6
+    // layers 99.7 -> 98.2 us)
+    if (!kOne && n_tiles <= 0) return;
     const bool idle = kOne && first_tile >= n_tiles;  // one tile: nothing for stream 1, which still does the dry run below
     const int row_tile = kOne ? 0 : t;
     const int row = row_tile * 128 + row_in_tile;                              // row within the row group
@@ -405,7 +410,7 @@ __device__ __forceinline__ void softmax(const TcParams& p, const Job& c, Barrier
     // 32.0 -> 30.4).  (The form with two row tiles walks long contexts, where its loop ran 8 % slower with the dry run in it.)
     const bool warm_up = kOne && t == 1;
     uint32_t s_par = warm_up ? 1 : 0;
-    for (int j = warm_up ? first_tile - step : first_tile; (j < n_tiles || (kOne && j < first_tile)) && ok; j += step, s_par ^= 1) {
+    for (int j = warm_up ? first_tile - step : first_tile; j < n_tiles && ok; j += step, s_par ^= 1) {
         const bool dry = kOne && j < first_tile;
         const bool is_new = j >= c.n_ctx_tiles;
         const int n_valid = is_new ? c.M : min(kTileTokens, c.seq_len - (c.tile_begin + j) * kTileTokens);
@@ -486,7 +491,7 @@ __device__ __forceinline__ void softmax(const TcParams& p, const Job& c, Barrier
         // from tensor memory on the general path, which brings m_run up to date.  A short walk of the two-term form, whose fast path
         // would be met with cold code, stays on the general path (40 rows x 4 of 64 channels, 4 tiles per CTA: 17.8 -> 17.3 us).
         float l_add = 0.f;
-        bool general = j <= first_tile || masked || (kOne && kSplit && n_tiles <= kShortWalk);
+        bool general = (kOne ? j <= first_tile : j == first_tile) || masked || (kOne && kSplit && n_tiles <= kShortWalk);
         if (!general) {
             l_add = exp_row(m_run);
             const bool bad = !(l_add < kSafeRowSum) || m_run == -INFINITY;
@@ -520,7 +525,7 @@ __device__ __forceinline__ void softmax(const TcParams& p, const Job& c, Barrier
             // The decision is per row, the tensor-memory traffic is warp-wide: if any row of the
             // warp rescales, all 32 rows pass through it (with a factor of 1 where nothing changes).
             bool need = false;
-            if (j <= first_tile) {
+            if (kOne ? j <= first_tile : j == first_tile) {
                 m_run = m_tile;
             } else {
                 need = m_tile > m_run + kRescaleThreshold || (m_run == -INFINITY && m_tile > -INFINITY);
@@ -582,7 +587,7 @@ __device__ __forceinline__ void softmax(const TcParams& p, const Job& c, Barrier
         w_other = m_o == -INFINITY ? 0.f : ex2(m_o - m_all);
         l_run = l_run * w_mine + l_o * w_other;
         m_run = m_all;
-        if (*abort_flag) ok = false;
+        ok = __all_sync(0xffffffffu, ok && !*abort_flag);
         if (ok) ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.o_done[1 - t]), 0, abort_flag, p.workspace, 8));
     }
     if (ok) ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.o_done[t]), 0, abort_flag, p.workspace, 8));

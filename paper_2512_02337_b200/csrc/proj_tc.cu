@@ -162,6 +162,7 @@ __global__ void __launch_bounds__(kProjThreads, 2) proj_tc_kernel(const __grid_c
             for (int i = i0; i < i1; ++i)
                 if (i >= p.stages)
                     ok &= mbar_wait(smem_u32(&bars.empty[i % p.stages]), ((i / p.stages) - 1) & 1, abort_flag, p.workspace, 30);
+            ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;  // a wait gave up: nothing more is copied
             if (lane == 0) {
                 for (int i = i0; i < i1; ++i) {
@@ -183,7 +184,7 @@ __global__ void __launch_bounds__(kProjThreads, 2) proj_tc_kernel(const __grid_c
         pdl_wait();  // (nothing to read here, but the limits of the waits below start to run)
         for (int i = 0; i < n_k; ++i) {
             const int slot = i % p.stages;
-            ok &= mbar_wait(smem_u32(&bars.full[slot]), (i / p.stages) & 1, abort_flag, p.workspace, 31);
+            ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.full[slot]), (i / p.stages) & 1, abort_flag, p.workspace, 31));
             if (!ok) break;  // a wait gave up: nothing more is issued
             tc_fence_after();
             if (lane == 0) {

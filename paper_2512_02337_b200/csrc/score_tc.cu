@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) scores_tc_kernel(const __gri
         bool ok = true;
         for (int sidx = 0; ok && it.next(p, s); ++sidx) {
             // Q may only be replaced once the contractions of the previous stretch have read it
-            if (sidx > 0) ok &= mbar_wait(smem_u32(&bars.q_empty), (sidx - 1) & 1, abort_flag, p.workspace, 27);
+            if (sidx > 0) ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.q_empty), (sidx - 1) & 1, abort_flag, p.workspace, 27));
             if (lane == 0 && ok) {
                 const uint32_t qbar = smem_u32(&bars.q_full);
                 mbar_expect_tx(qbar, (uint32_t)(p.tok_n * p.G * D * 2));
@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) scores_tc_kernel(const __gri
                 for (uint32_t which = 0; which < 2; ++which) {  // the Kmax rows of the tile, then its Kmin rows
                     const uint32_t u = 2 * g + which, slot = u % stages;
                     if (u >= (uint32_t)stages)
-                        ok &= mbar_wait(smem_u32(&bars.sum_empty[slot]), ((u / stages) - 1) & 1, abort_flag, p.workspace, 21);
+                        ok &= __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.sum_empty[slot]), ((u / stages) - 1) & 1, abort_flag, p.workspace, 21));
                     if (lane == 0 && ok) {
                         const uint32_t full = smem_u32(&bars.sum_full[slot]);
                         mbar_expect_tx(full, kTileBlocks * D * 2);
@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) scores_tc_kernel(const __gri
                 }
                 // Q is released by both warps: each commit covers the contractions its own thread has issued
                 if (t == s.t1 - 1 && lane == 0) tc_commit(smem_u32(&bars.q_empty));
-                __syncwarp();
+                ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;  // a wait gave up: nothing is issued past this tile
             }
         }

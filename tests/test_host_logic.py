@@ -277,3 +277,21 @@ def test_overlapped_kernels_load_nothing_through_the_read_only_path():
     assert {"attn_tc.cu", "attn_simt.cu", "aux_kernels.cu", "proj_tc.cu", "score_tc.cu"} <= set(overlapped)
     for name, text in overlapped.items():
         assert not re.findall(r"__ldg\s*\(|ld\.global\.nc|__restrict__", text), name
+
+
+@pytest.mark.parametrize("source", ["attn_tc.cu", "attn_pair.cu", "score_tc.cu", "proj_tc.cu"])
+def test_lanes_of_a_warp_give_up_together(source):
+    """A wait that can give up returns a value per lane, and so does a look at the abort flag: an exit, a condition of a loop or of a
+    vote that depends on one comes after a vote of the whole warp.  (Lanes that disagreed would wait for one another in different
+    places, without a limit.)  Checked on the source: such a case cannot be brought about on a GPU that works."""
+    own = False  # whether `ok` may differ between lanes
+    for n, line in enumerate((build_mod.CSRC / source).read_text().split("\n"), 1):
+        code = line.split("//")[0]
+        if re.search(r"\bbool ok = ", code):
+            own = False
+        if re.search(r"if \(!ok\) (break|return)|if \(ok\) ok = __all_sync", code):
+            assert not own, f"{source}:{n} leaves without a vote"
+        if re.search(r"\bok &?= .*__all_sync\(0xffffffffu, ", code):
+            own = False if "ok &=" not in code else own
+        elif re.search(r"\bok &?= (mbar|pair)_wait\(|\*abort_flag\) ok = ", code):
+            own = True
