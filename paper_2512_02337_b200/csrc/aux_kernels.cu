@@ -229,13 +229,16 @@ __global__ void __launch_bounds__(32 * kScoreWarps) scores_simt_kernel(ScorePara
 
 // ---------------------------------------------------------------------------------------------
 // Selection: one CTA per (layer, sequence, KV head).  A candidate's score becomes a 32-bit key whose unsigned order is
-// "score ascending, NaN first"; the key T of the k-th best candidate is found two bits at a time from the top, by counting the keys
-// (in registers) that reach each of three thresholds, until a threshold is met by k candidates exactly or all bits are known; then
-// an ordered compaction writes sink | kept candidates | local in ascending order, the candidates of key T that are still to be
-// taken by lowest index.  Bound by latency: its steps, a count and one barrier each, and the fetch of its code, which follows other
-// kernels: no more keys per thread, each of them code, than the lists need.  From the end of the scores to its own, against a histogram
-// per digit of 11 bits (four barriers a digit, crowded bins): 509 candidates x 256 lists 16.8 -> 12.1 us, 29 x 2 8.4 -> 4.2 (8.2 with
-// sixteen keys per thread).
+// "score ascending, NaN first".  The key T of the k-th best candidate starts with the bits that all keys share (those of the smallest
+// and the largest) and is found two bits at a time from there, by counting the keys (in registers) that reach each of three
+// thresholds, until a threshold is met by k candidates exactly or all bits are known; after kSelectSteps steps the range of the keys
+// that are still undecided is looked at again, which ends the search among equal scores.  Then an ordered compaction writes
+// sink | kept candidates | local in ascending order, the candidates of key T that are still to be taken by lowest index.
+// Bound by latency: a count and one barrier per step, and the fetch of its code, which follows other kernels: no more keys per
+// thread, each of them code, than the lists need.  us per call, repeated calls, scores of one sign, against a histogram per digit of
+// 11 bits / this search from the top bit, without a second look and with more code: 29 candidates x 2 lists 6.5 / 5.1 -> 3.3, 509 x 256
+// 11.4 / 8.4 -> 6.0, 2045 x 256 13.2 / 12.9 -> 9.2 (with many ties 13.3 / 15.6 -> 7.7), 3837 x 128 11.5 / 13.9 -> 9.0, 4090 x 256
+// 15.6 / 16.4 -> 13.9, 8189 x 256 31.8 / 38.3 -> 20.2, 16300 x 64 44.8 / 27.0 -> 22.5, 65000 x 32 223 / 140 -> 139.
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t select_key(float score) {
     const uint32_t bits = __float_as_uint(score);
@@ -244,24 +247,32 @@ __device__ __forceinline__ uint32_t select_key(float score) {
     return (bits & 0x80000000u) ? ~bits : (bits | 0x80000000u);
 }
 
-// kSelectKeys: a thread's first keys stay in registers, any further ones are formed again from the scores.
-template <int kSelectThreads, int kSelectKeys>
-__global__ void __launch_bounds__(kSelectThreads) select_kernel(SelectParams p) {
+// Steps between two looks at the range of the undecided keys: most lists are decided after ten from the top bit.  (2045 x 256, one sign /
+// many ties, measured with more code: 4 steps 11.2 / 9.5 us, 8 10.9 / 9.0, 16 10.4 / 13.2.)  Where keys are formed again for each step a look costs as much
+// as a step: none at the start, and later than most lists need.
+constexpr int kSelectSteps = 8, kSelectStepsTail = 12;
+
+// kSelectKeys: a thread's keys stay in registers; those that the largest form has no room for are formed again from the scores.
+// Registers: without a minimum of one CTA per SM the compiler stops at 32 and the loads wait for one another (2045 x 256: 9.2 -> 11.9 us);
+// 16 keys in 512 threads leave room for two (8189 x 256: 26.3 -> 20.2).
+template <int kSelectThreads, int kSelectKeys, bool kTail = false>
+__global__ void __launch_bounds__(kSelectThreads, kSelectThreads == 512 && kSelectKeys == 16 ? 2 : 1) select_kernel(SelectParams p) {
     pdl_begin(p.pdl);
-    constexpr int kWarps = kSelectThreads / 32;
-    __shared__ int4 s_reach[3];                     // candidates that reach the thresholds of a step
-    __shared__ int s_above[kSelectKeys * kWarps];   // candidates above T per (round, warp), then their exclusive prefix
-    __shared__ int s_tied[kSelectKeys * kWarps];    // ... and those equal to T
-    __shared__ int s_run_above, s_run_tied;
+    constexpr int kWarps = kSelectThreads / 32, kCounts = kSelectKeys * kWarps;
+    static_assert(32 * kSelectKeys < 1024 && kCounts % 32 == 0 && kCounts * 32 < 65536, "packed counts");
+    __shared__ int4 s_reach[3];         // candidates that reach the thresholds of a step
+    __shared__ uint2 s_range[kWarps];   // smallest and largest undecided key of each warp
+    __shared__ unsigned s_counts[kCounts];  // per (round, warp): candidates above T | of key T << 16, then the sums of those before
+    __shared__ unsigned s_total;        // ... and of all of them
     const int h = blockIdx.x, b = blockIdx.y, l = blockIdx.z, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int32_t* idx = p.idx + (((size_t)l * p.batch + b) * p.Hkv + h) * p.budget_blocks;
     const int seq_len = p.seq_lens[b];
     const int nb = min((seq_len + p.bs - 1) / p.bs, p.max_blocks);
     const float* scores = p.scores + (((size_t)l * p.batch + b) * p.Hkv + h) * p.max_blocks;
-    // head-shared selection ranks the blocks on the mean of the layer's KV heads' scores, summed in float32 in
-    // head order (the ranking is a pure function of these bits, the same in every head's CTA)
-    const float* scores_h0 = p.scores + (((size_t)l * p.batch + b) * p.Hkv) * p.max_blocks;
-    const float inv_heads = 1.0f / (float)p.Hkv;
+    // share_heads: the score of a block is the float32 sum over the KV heads in head order, scaled by 1/Hkv (every CTA
+    // of a layer computes the same sums and therefore the same list)
+    const float* scores_h0 = p.scores + ((size_t)l * p.batch + b) * p.Hkv * p.max_blocks;
+    const float inv_heads = 1.f / (float)p.Hkv;
     auto score_at = [&](int i) {
         if (!p.share_heads) return scores[i];
         float acc = 0.f;
@@ -271,7 +282,7 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(SelectParams p) 
     const int count = min(nb, p.budget_blocks);
     if (l == 0 && h == 0 && tid == 0) p.count[b] = count;
     if (nb <= p.budget_blocks) {
-        for (int i = tid; i < p.budget_blocks; i += kSelectThreads) idx[i] = i < nb ? i : -1;
+        for (int i = tid; i < nb; i += kSelectThreads) idx[i] = i;
         return;
     }
     const int lo = p.sink_blocks, hi = nb - p.local_blocks;
@@ -279,139 +290,197 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(SelectParams p) 
 
     // a thread's candidates: lo + tid, lo + tid + kSelectThreads, ...
     uint32_t keys[kSelectKeys];
-    const int rounds = min((hi - lo + kSelectThreads - 1) / kSelectThreads, kSelectKeys);
+    const int rounds = min((hi - lo + kSelectThreads - 1) / kSelectThreads, kSelectKeys);  // (no test of it where most keys are used)
+    const int tail0 = lo + kSelectKeys * kSelectThreads;  // candidates from here on are not in registers
+    uint32_t smallest = 0xffffffffu, largest = 0u;        // of this thread's undecided keys
+    float own[kSelectKeys];  // their scores: as score_at, all loads of a head in flight together
+    if (!p.share_heads) {
+#pragma unroll
+        for (int e = 0; e < kSelectKeys; ++e) {
+            const int i = lo + tid + e * kSelectThreads;
+            own[e] = i < hi ? scores[i] : 0.f;
+        }
+    } else {
+#pragma unroll
+        for (int e = 0; e < kSelectKeys; ++e) own[e] = 0.f;
+#pragma unroll 2
+        for (int hh = 0; hh < p.Hkv; ++hh)
+#pragma unroll
+            for (int e = 0; e < kSelectKeys; ++e) {
+                const int i = lo + tid + e * kSelectThreads;
+                own[e] += i < hi ? scores_h0[(size_t)hh * p.max_blocks + i] : 0.f;
+            }
+#pragma unroll
+        for (int e = 0; e < kSelectKeys; ++e) own[e] *= inv_heads;
+    }
 #pragma unroll
     for (int e = 0; e < kSelectKeys; ++e) {
-        const int i = lo + tid + e * kSelectThreads;
-        keys[e] = i < hi ? select_key(score_at(i)) : 0u;  // 0 reaches no threshold
+        const bool in = lo + tid + e * kSelectThreads < hi;
+        keys[e] = in ? select_key(own[e]) : 0u;  // 0 reaches no threshold
+        smallest = in ? min(smallest, keys[e]) : smallest;
+        largest = max(largest, keys[e]);
     }
-    const int tail0 = lo + tid + kSelectKeys * kSelectThreads;
+    const bool has_tail = kTail && tail0 < hi;
+    if (has_tail) {
+        smallest = 0u;
+        largest = 0xffffffffu;
+    }
     if (tid < 3) s_reach[tid] = make_int4(0, 0, 0, 0);
-    __syncthreads();
-    uint32_t T = 0;    // its bits found so far
+    uint32_t T;        // key of the k-th best candidate, the bits found so far
     int n_above = 0;   // candidates whose bits found so far are above T's
     int ties = -1;     // candidates of key T to take
+    int at = 0;
 #pragma unroll 1
-    for (int shift = 30, at = 0; shift >= 0; shift -= 2, at = at == 2 ? 0 : at + 1) {
-        const uint32_t t1 = T + (1u << shift), t2 = T + (2u << shift), t3 = T + (3u << shift);
-        int c1 = 0, c2 = 0, c3 = 0;
+    for (;;) {
+        // the bits that all undecided keys share are T's
+        smallest = __reduce_min_sync(0xffffffffu, smallest);
+        largest = __reduce_max_sync(0xffffffffu, largest);
+        if (lane == 0) s_range[warp] = make_uint2(smallest, largest);
+        __syncthreads();
+        const uint2 range = s_range[lane % kWarps];
+        smallest = __reduce_min_sync(0xffffffffu, range.x);
+        largest = __reduce_max_sync(0xffffffffu, range.y);
+        T = smallest;
+        if (smallest >= largest) break;  // one key is left
+        int shift = (31 - __clz(smallest ^ largest)) & ~1;
+        T &= ~((4u << shift) - 1u);
+        const int stop = max(shift - 2 * (has_tail ? kSelectStepsTail : kSelectSteps), -2);
+#pragma unroll 1
+        for (; shift > stop; shift -= 2, at = at == 2 ? 0 : at + 1) {
+            const uint32_t t1 = T + (1u << shift), t2 = T + (2u << shift), t3 = T + (3u << shift);
+            unsigned c = 0;  // three counts of ten bits
+#pragma unroll
+            for (int e = 0; e < kSelectKeys; ++e)
+                if (kSelectKeys > 8 || e < rounds) c += (keys[e] >= t1 ? 1u : 0u) + (keys[e] >= t2 ? 1u << 10 : 0u) + (keys[e] >= t3 ? 1u << 20 : 0u);
+            c = __reduce_add_sync(0xffffffffu, c);
+            int mine = lane < 3 ? (c >> (10 * lane)) & 1023u : 0;  // lane j: candidates of this warp that reach threshold j
+            if (has_tail) {
+                int c1 = 0, c2 = 0, c3 = 0;
+#pragma unroll 4
+                for (int i = tail0 + tid; i < hi; i += kSelectThreads) {
+                    const uint32_t key = select_key(score_at(i));
+                    c1 += key >= t1;
+                    c2 += key >= t2;
+                    c3 += key >= t3;
+                }
+                c1 = __reduce_add_sync(0xffffffffu, c1);
+                c2 = __reduce_add_sync(0xffffffffu, c2);
+                c3 = __reduce_add_sync(0xffffffffu, c3);
+                mine += lane == 0 ? c1 : lane == 1 ? c2 : c3;
+            }
+            if (lane < 3 && mine) atomicAdd(&s_reach[at].x + lane, mine);
+            __syncthreads();
+            const int4 reach = s_reach[at];
+            if (tid == 0) s_reach[at == 0 ? 2 : at - 1] = make_int4(0, 0, 0, 0);  // read before this step's barrier, used behind the next one
+            int reached;
+            if (reach.z >= k) {
+                T = t3;
+                reached = reach.z;
+            } else if (reach.y >= k) {
+                T = t2;
+                reached = reach.y;
+                n_above = reach.z;
+            } else if (reach.x >= k) {
+                T = t1;
+                reached = reach.x;
+                n_above = reach.y;
+            } else {
+                reached = 0;  // T stays as it is
+                n_above = reach.x;
+            }
+            if (reached == k) {  // exactly the candidates from T on
+                --T;
+                ties = 0;
+                break;
+            }
+        }
+        if (ties == 0 || shift < 0) break;
+        const uint32_t width = 4u << shift;  // the undecided keys are T .. T + width - 1
+        smallest = 0xffffffffu;
+        largest = 0u;
+        auto look_at = [&](uint32_t key) {
+            if (key - T < width) {
+                smallest = min(smallest, key);
+                largest = max(largest, key);
+            }
+        };
 #pragma unroll
         for (int e = 0; e < kSelectKeys; ++e)
-            if (e < rounds) {
-                c1 += keys[e] >= t1;
-                c2 += keys[e] >= t2;
-                c3 += keys[e] >= t3;
-            }
-        for (int i = tail0; i < hi; i += kSelectThreads) {
-            const uint32_t key = select_key(score_at(i));
-            c1 += key >= t1;
-            c2 += key >= t2;
-            c3 += key >= t3;
-        }
-        c1 = __reduce_add_sync(0xffffffffu, c1);
-        c2 = __reduce_add_sync(0xffffffffu, c2);
-        c3 = __reduce_add_sync(0xffffffffu, c3);
-        if (lane < 3) atomicAdd(&s_reach[at].x + lane, lane == 0 ? c1 : lane == 1 ? c2 : c3);
-        __syncthreads();
-        const int4 reach = s_reach[at];
-        if (tid == 0) s_reach[at == 0 ? 2 : at - 1] = make_int4(0, 0, 0, 0);  // read before this step's barrier, used behind the next one
-        int reached;
-        if (reach.z >= k) {
-            T = t3;
-            reached = reach.z;
-        } else if (reach.y >= k) {
-            T = t2;
-            reached = reach.y;
-            n_above = reach.z;
-        } else if (reach.x >= k) {
-            T = t1;
-            reached = reach.x;
-            n_above = reach.y;
-        } else {
-            reached = 0;  // T stays as it is
-            n_above = reach.x;
-        }
-        if (reached == k) {  // exactly the candidates from T on
-            --T;
-            ties = 0;
-            break;
-        }
+            if (kSelectKeys > 8 || e < rounds) look_at(keys[e]);
+        if (has_tail)
+            for (int i = tail0 + tid; i < hi; i += kSelectThreads) look_at(select_key(score_at(i)));
     }
     if (ties < 0) ties = k - n_above;
 
     for (int i = tid; i < p.sink_blocks; i += kSelectThreads) idx[i] = i;
     for (int i = tid; i < p.local_blocks; i += kSelectThreads) idx[p.sink_blocks + k + i] = hi + i;
     // Ordered compaction (ascending block index = round e, then thread).  Register part: two ballots per round, the
-    // (round, warp) counts scanned once by warps 0 and 1.
-    unsigned above[kSelectKeys], tied[kSelectKeys];
+    // (round, warp) counts scanned once by warp 0.
 #pragma unroll
     for (int e = 0; e < kSelectKeys; ++e) {
         const bool in = lo + tid + e * kSelectThreads < hi;
-        above[e] = __ballot_sync(0xffffffffu, in && keys[e] > T);
-        tied[e] = __ballot_sync(0xffffffffu, in && keys[e] == T);
-        if (lane == 0) {
-            s_above[e * kWarps + warp] = __popc(above[e]);
-            s_tied[e * kWarps + warp] = __popc(tied[e]);
-        }
+        const unsigned above = __ballot_sync(0xffffffffu, in && keys[e] > T), tied = __ballot_sync(0xffffffffu, in && keys[e] == T);
+        if (lane == 0) s_counts[e * kWarps + warp] = (unsigned)__popc(above) | (unsigned)__popc(tied) << 16;
     }
     __syncthreads();
-    if (warp < 2) {  // exclusive scan of the counts: some per lane, then across lanes
-        constexpr int kEach = kSelectKeys * kWarps / 32;
-        int* counts = warp == 0 ? s_above : s_tied;
-        int each[kEach], sum = 0;
+    if (warp == 0) {  // exclusive scan of the counts: some per lane, then across lanes
+        constexpr int kEach = kCounts / 32;
+        unsigned each[kEach], sum = 0;
 #pragma unroll
         for (int u = 0; u < kEach; ++u) {
-            each[u] = counts[lane * kEach + u];
+            each[u] = s_counts[lane * kEach + u];
             sum += each[u];
         }
-        int incl = sum;
+        unsigned incl = sum;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const int up = __shfl_up_sync(0xffffffffu, incl, o);
+            const unsigned up = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += up;
         }
-        int run = incl - sum;
+        unsigned run = incl - sum;
 #pragma unroll
         for (int u = 0; u < kEach; ++u) {
-            counts[lane * kEach + u] = run;
+            s_counts[lane * kEach + u] = run;
             run += each[u];
         }
-        if (lane == 31) (warp == 0 ? s_run_above : s_run_tied) = incl;
+        if (lane == 31) s_total = incl;
     }
     __syncthreads();
     const unsigned below_me = (1u << lane) - 1u;
-    auto place = [&](int i, bool is_above, bool is_tied, int n_above, int n_tied) {  // counts of candidates before this one
-        if (is_above) idx[p.sink_blocks + n_above + min(n_tied, ties)] = i;
-        if (is_tied && n_tied < ties) idx[p.sink_blocks + n_above + n_tied] = i;
+    // candidate i: above T, or of key T; `above` and `tied` of either before it
+    auto place = [&](int i, bool is_above, bool is_tied, int above, int tied) {
+        if (is_above) idx[p.sink_blocks + above + min(tied, ties)] = i;
+        if (is_tied && tied < ties) idx[p.sink_blocks + above + tied] = i;
     };
 #pragma unroll
     for (int e = 0; e < kSelectKeys; ++e)
-        if (e < rounds)
-            place(lo + tid + e * kSelectThreads, (above[e] >> lane) & 1u, (tied[e] >> lane) & 1u,
-                  s_above[e * kWarps + warp] + __popc(above[e] & below_me), s_tied[e * kWarps + warp] + __popc(tied[e] & below_me));
+        if (e < rounds) {
+            const bool in = lo + tid + e * kSelectThreads < hi, is_above = in && keys[e] > T, is_tied = in && keys[e] == T;
+            const unsigned above = __ballot_sync(0xffffffffu, is_above), tied = __ballot_sync(0xffffffffu, is_tied);
+            const unsigned before = s_counts[e * kWarps + warp];
+            place(lo + tid + e * kSelectThreads, is_above, is_tied, (int)(before & 0xffffu) + __popc(above & below_me),
+                  (int)(before >> 16) + __popc(tied & below_me));
+        }
+    if (!has_tail) return;
     // candidates beyond the register part: round by round
-    for (int base = lo + kSelectKeys * kSelectThreads; base < hi; base += kSelectThreads) {
+    int run_above = (int)(s_total & 0xffffu), run_tied = (int)(s_total >> 16);
+    for (int base = tail0; base < hi; base += kSelectThreads) {
         const int i = base + tid;
         const uint32_t key = i < hi ? select_key(score_at(i)) : 0u;
-        const unsigned ab = __ballot_sync(0xffffffffu, i < hi && key > T), ti = __ballot_sync(0xffffffffu, i < hi && key == T);
+        const bool is_above = i < hi && key > T, is_tied = i < hi && key == T;
+        const unsigned above = __ballot_sync(0xffffffffu, is_above), tied = __ballot_sync(0xffffffffu, is_tied);
         __syncthreads();  // the counts of the previous round have been read by everyone
-        if (lane == 0) {
-            s_above[warp] = __popc(ab);
-            s_tied[warp] = __popc(ti);
-        }
+        if (lane == 0) s_counts[warp] = (unsigned)__popc(above) | (unsigned)__popc(tied) << 16;
         __syncthreads();
-        int n_above = s_run_above, n_tied = s_run_tied;
-        for (int w = 0; w < warp; ++w) {
-            n_above += s_above[w];
-            n_tied += s_tied[w];
+        unsigned before = 0, all = 0;
+        for (int w = 0; w < kWarps; ++w) {
+            if (w == warp) before = all;
+            all += s_counts[w];
         }
-        place(i, (ab >> lane) & 1u, (ti >> lane) & 1u, n_above + __popc(ab & below_me), n_tied + __popc(ti & below_me));
-        __syncthreads();
-        if (tid == 0)
-            for (int w = 0; w < kWarps; ++w) {
-                s_run_above += s_above[w];
-                s_run_tied += s_tied[w];
-            }
+        place(i, is_above, is_tied, run_above + (int)(before & 0xffffu) + __popc(above & below_me),
+              run_tied + (int)(before >> 16) + __popc(tied & below_me));
+        run_above += (int)(all & 0xffffu);
+        run_tied += (int)(all >> 16);
     }
 }
 
@@ -653,12 +722,24 @@ specpv_status launch_scores(const ScoreParams& p, int n_layers, int max_nb, int 
 specpv_status launch_select(const SelectParams& p, int n_layers, cudaStream_t stream) {
     if (n_layers <= 0 || p.batch <= 0) return SPECPV_OK;
     const dim3 grid(p.Hkv, p.batch, n_layers);
-    if (p.max_blocks <= 1024)
-        SPECPV_LAUNCH(select_kernel<256, 4>, grid, 256, 0, stream, p);
-    else if (p.max_blocks <= 4096)
-        SPECPV_LAUNCH(select_kernel<512, 8>, grid, 512, 0, stream, p);
+    // By the most candidates a list can have; up to a list per SM, twice the threads with half the keys each (3837 x 128: 13.0 -> 10.4 us,
+    // 8189 x 8: 16.7 -> 14.6, both with more code), above that they only crowd (4090 x 256: 15.6 -> 21.0).
+    const int n = p.max_blocks - p.sink_blocks - p.local_blocks;
+    const bool few = (long long)grid.x * grid.y * grid.z <= 148;
+    if (n <= 1024)
+        SPECPV_LAUNCH((select_kernel<256, 4>), grid, 256, 0, stream, p);
+    else if (n <= 2048)
+        SPECPV_LAUNCH((select_kernel<512, 4>), grid, 512, 0, stream, p);
+    else if (n <= 4096 && few)
+        SPECPV_LAUNCH((select_kernel<1024, 4>), grid, 1024, 0, stream, p);
+    else if (n <= 4096)
+        SPECPV_LAUNCH((select_kernel<512, 8>), grid, 512, 0, stream, p);
+    else if (n <= 8192 && few)
+        SPECPV_LAUNCH((select_kernel<1024, 8>), grid, 1024, 0, stream, p);
+    else if (n <= 8192)
+        SPECPV_LAUNCH((select_kernel<512, 16>), grid, 512, 0, stream, p);
     else
-        SPECPV_LAUNCH(select_kernel<1024, 16>, grid, 1024, 0, stream, p);
+        SPECPV_LAUNCH((select_kernel<1024, 16, true>), grid, 1024, 0, stream, p);
     return SPECPV_OK;
 }
 

@@ -316,8 +316,8 @@ def test_commits_of_two_caches_on_two_streams_share_a_workspace():
 
 @pytest.mark.parametrize("nb,budget", [(300, 40), (2048, 64), (4099, 128), (9000, 1000)])
 def test_selection_alone_on_synthetic_scores_with_ties_and_nan(nb, budget):
-    """The selection kernel on its own: more candidate blocks than it keeps in registers (nb > 4096), repeated
-    scores (ties go to the lower index), NaN (ranks last), -0 / +0; bit-exact against the oracle."""
+    """The selection kernel on its own: several of its forms, repeated scores (ties go to the lower index), NaN (ranks last),
+    -0 / +0; bit-exact against the oracle."""
     dev = "cuda"
     rng = np.random.default_rng(nb)
     Hkv, L, batch, bs = 3, 2, 2, 64
@@ -578,8 +578,8 @@ def test_scores_of_a_refresh_step_with_more_rows_than_one_accumulator(reduce, sc
 
 @pytest.mark.parametrize("nb,budget", [(7, 5), (259, 100), (1024, 5), (1025, 64), (4096, 4095), (4097, 64), (16387, 128), (16500, 64)])
 def test_selection_at_the_edges_of_its_register_forms(nb, budget):
-    """Candidate counts either side of what the forms of the selection kernel keep in registers, one candidate to choose,
-    and all but one."""
+    """Candidate counts either side of 1024, 4096 and 16384, around which the forms of the selection kernel change, few candidates to
+    choose, and all but one."""
     test_selection_alone_on_synthetic_scores_with_ties_and_nan(nb, budget)
 
 
@@ -639,3 +639,36 @@ def test_commit_of_few_units_in_one_launch(dtype, Hkv, batch, bs, A):
             lens[b] += counts[b]
             assert int(w.seq_lens[b]) == lens[b]
         assert np.array_equal(wl.to_numpy(w.k_pool), kp) and np.array_equal(wl.to_numpy(w.v_pool), vp)
+
+
+@pytest.mark.parametrize("n,L", [(33, 1), (1024, 2), (1025, 1), (2048, 2), (2049, 2), (2049, 20), (4096, 20), (4097, 2), (4097, 20), (8192, 20),
+                                 (8193, 1), (16384, 1), (16385, 1)])
+@pytest.mark.parametrize("shared", [0, 1])
+def test_selection_of_one_and_of_tied_candidates(n, L, shared):
+    """Either side of every form's most candidates, on fewer lists than SMs and on more (20 layers x 8 heads), with k = 1 and 61 of them to
+    choose: the search from the keys' common bits, past its second look, and the one key that is left.  Scores are multiples of 1/4, so that
+    the mean over the 8 heads is exact and many tie; layer 0 has one value everywhere, layer 1 NaN throughout its first list but
+    for one score, and one that is larger than the rest by far."""
+    dev, Hkv, bs = "cuda", 8, 16
+    rng = np.random.default_rng(n + L)
+    nb = n + 3  # 1 sink and 2 local blocks beside the candidates
+    sc = np.round(rng.standard_normal((L, 1, Hkv, nb)) * 16).astype(np.float32) / 4
+    sc[0] = -1.25
+    if L > 1:
+        sc[1, 0, 0] = np.nan
+        sc[1, 0, :, n // 2 + 1] = 1e30
+    scores = torch.from_numpy(sc).to(dev)
+    lens = torch.tensor([nb * bs], dtype=torch.int32, device=dev)
+    ws = torch.zeros(4096, dtype=torch.uint8, device=dev)
+    for budget in (4, 64) if n > 61 else (4,):
+        cfg = B.make_config(L, 4 * Hkv, Hkv, 128, bs, "bf16", 1, 2, budget, 64, select_shared=shared)
+        idx = torch.full((L, 1, Hkv, budget), -7, dtype=torch.int32, device=dev)
+        count = torch.zeros(1, dtype=torch.int32, device=dev)
+        B.specpv_select_partial_kv(cfg, L, scores, lens, 1, nb, idx, count, ws)
+        util.sync_status(ws)
+        got = idx.cpu().numpy()
+        for l in {0, min(1, L - 1), L - 1}:
+            mean = sc[l, 0].astype(np.float64).sum(0) / Hkv
+            for h in range(Hkv):
+                want = oracle.select(mean if shared else sc[l, 0, h].astype(np.float64), 1, 2, budget)
+                assert np.array_equal(got[l, 0, h], want), (budget, l, h)
