@@ -542,16 +542,17 @@ __global__ void __launch_bounds__(128) gather_kernel(GatherParams p) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// Commit: four warps append the accepted tokens' K and V rows that fall into one block (a warp per row) and recompute the block's
-// summary, the appended tokens taken from the step's tensors; a unit of work is (block touched, KV head, layer x seq).  All units
-// read the lengths.  Where they fit into two turns of one CTA (one float32 layer, short steps), that CTA advances the lengths
-// itself; else a CTA takes a unit, and the lengths advance in a launch behind it: a commit keeps nothing in the workspace but the
-// status word, so that commits of two caches on two streams may share one (an arrival counter there made the launch unnecessary,
-// 9.3 us a call against 11.4, but mixed the arrivals of two such commits).  Bound by launches: rows, summaries and lengths in
-// three took 14 us of host time a call, in two 6.7; in one a float32 step with two commits takes 67.7 us instead of 74.4.
+// Commit: a CTA's four warps append the accepted tokens' K and V rows that fall into one block (a warp per row) and recompute the
+// block's summary, the appended tokens taken from the step's tensors; grid = (blocks touched, KV heads, layers x seqs).  All CTAs
+// read the lengths.  Where they are no more than a cluster holds (one or two float32 layers, short steps), they are one, which
+// advances the lengths itself once they have all arrived; else the lengths advance in a launch behind it: a commit keeps nothing in
+// the workspace but the status word, so that commits of two caches on two streams may share one (an arrival counter there made the
+// launch unnecessary, 9.3 us a call against 11.4, but mixed the arrivals of two such commits).  Bound by launches.  us with a copy of
+// the lengths, two launches / a CTA that took four of the units side by side and then the rest / cluster: four units of 4 tokens
+// 6.1 / 6.5 / 5.8, eight 6.1 / 10.4 / 6.4 (a launch less for the host), eight of 46 tokens 10.1 / 18.1 / 10.0, of 64 16.7 / 31.9 / 16.5.
 // ---------------------------------------------------------------------------------------------
 constexpr int kCommitWarps = 4;
-constexpr int kCommitUnits = 4;  // of one CTA at a time
+constexpr int kCommitCluster = 8;  // CTAs of a cluster that every launch may ask for
 
 template <typename T>
 __device__ __forceinline__ void commit_unit(const CommitParams& p, int touched, int h, int lb, int warp, int lane) {
@@ -657,15 +658,13 @@ __global__ void __launch_bounds__(kLensThreads) commit_lens_kernel(CommitParams 
     if (b < p.batch) advance_length(p, b);
 }
 
-// One CTA: units (x, y, z) of a grid of `units`, at most twice kCommitUnits of them, and the lengths behind a barrier.
+// One cluster, a CTA per unit, which advances the lengths itself.
 template <typename T>
-__global__ void __launch_bounds__(32 * kCommitWarps * kCommitUnits) commit_small_kernel(CommitParams p, dim3 units) {
+__global__ void __launch_bounds__(32 * kCommitWarps) commit_cluster_kernel(CommitParams p) {
     pdl_begin(1);
-    const int n = units.x * units.y * units.z;
-    for (int u = threadIdx.x / (32 * kCommitWarps); u < n; u += kCommitUnits)
-        commit_unit<T>(p, u % units.x, u / units.x % units.y, u / (units.x * units.y), (threadIdx.x >> 5) % kCommitWarps, threadIdx.x & 31);
-    __syncthreads();  // every unit has read the lengths
-    if ((int)threadIdx.x < p.batch) advance_length(p, threadIdx.x);
+    commit_unit<T>(p, blockIdx.x, blockIdx.y, blockIdx.z, threadIdx.x >> 5, threadIdx.x & 31);
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");  // every unit has read the lengths
+    if (blockIdx.x + blockIdx.y + blockIdx.z == 0 && (int)threadIdx.x < p.batch) advance_length(p, threadIdx.x);
 }
 
 }  // namespace
@@ -753,10 +752,21 @@ specpv_status launch_commit(const CommitParams& params, int n_layers, int dtype,
     CommitParams p = params;
     p.aligned = aligned16(p.kmax) && aligned16(p.kmin);
     dim3 grid((p.A_max + p.bs - 1) / p.bs + 1, p.Hkv, n_layers * p.batch);
-    // at most two turns of the one CTA: each is a chain of three loads, some 2 us, against a launch
-    if (advance && (long long)grid.x * grid.y * grid.z <= 2 * kCommitUnits) {
-        if (launch_pdl(dtype == SPECPV_DTYPE_F32 ? commit_small_kernel<float> : commit_small_kernel<__nv_bfloat16>, 1,
-                       32 * kCommitWarps * kCommitUnits, 0, stream, p, grid) != cudaSuccess)
+    if (advance && (long long)grid.x * grid.y * grid.z <= kCommitCluster) {
+        cudaLaunchAttribute attr[2]{};
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = grid.x;
+        attr[1].val.clusterDim.y = grid.y;
+        attr[1].val.clusterDim.z = grid.z;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = grid;
+        cfg.blockDim = 32 * kCommitWarps;
+        cfg.stream = stream;
+        cfg.attrs = attr;
+        cfg.numAttrs = 2;
+        if (cudaLaunchKernelEx(&cfg, dtype == SPECPV_DTYPE_F32 ? commit_cluster_kernel<float> : commit_cluster_kernel<__nv_bfloat16>, p) != cudaSuccess)
             return SPECPV_ERR_CUDA;
         count_launch();
         return SPECPV_OK;
