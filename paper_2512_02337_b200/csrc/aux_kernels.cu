@@ -117,20 +117,35 @@ __global__ void __launch_bounds__(32 * kSumWarps) summaries_kernel(SummaryParams
 // ---------------------------------------------------------------------------------------------
 // Eq. 2-3 (SIMT form): a warp owns kBlocks blocks, whose summaries are staged in shared memory as float32 and read as broadcasts, a
 // lane the query rows lane, lane + 32, .. of the group, staged kScoreRows at a time; a block's results are added over the lanes by
-// shuffles.  Bound by latency on the small shapes it serves: one block per warp spreads 75 blocks of two heads over 20 CTAs (a lane
-// per block and 32 blocks per CTA left them on 6: 128 rows of 64 channels 18.6 -> 6.6 us, 33 blocks and 64 rows 10.3 -> 4.1); four
-// blocks per warp read the rows once for four where the launch has CTAs enough.  grid = (block groups, Hkv, layers x seqs).
+// shuffles.  Up to kScoreFewRows rows, eight lanes share a row (kParts) and take every eighth four channels.  Bound by latency on
+// the small shapes it serves: one block per warp spreads 75 blocks of two heads over 20 CTAs (a lane per block and 32 blocks per CTA left
+// them on 6: 128 rows of 64 channels 18.6 -> 6.6 us, 33 blocks and 64 rows 10.3 -> 4.1); four blocks per warp read the rows once for
+// four where the launch has CTAs enough.  Larger ones, us, a lane per block / four blocks per warp with a lane per row, summaries loaded
+// 2 or 4 bytes at a time / this form: 240 rows of 128, 512 blocks x 32 lists 110 / 104 / 102; 64 rows of 128, 512 x 256 233 / 204 / 179; 4 rows
+// of 128, 2048 x 128 203 / 217 / 94, 512 x 32 12.6 / 18.1 / 8.8; 5 rows of 128 (bfloat16), 1024 x 64 45 / 56 / 34; 2 rows of 64 (bfloat16),
+// 1000 x 64 17.7 / 25.4 / 16.2.  grid = (block groups, Hkv, layers x seqs).
 // ---------------------------------------------------------------------------------------------
 constexpr int kScoreWarps = 8;
-constexpr int kScoreRows = 64;
+constexpr int kScoreRows = 64;     // query rows staged at a time
+constexpr int kScoreFewRows = 16;  // .. where eight lanes share a row
 
-template <typename T, int D, int kBlocks>
-__global__ void __launch_bounds__(32 * kScoreWarps) scores_simt_kernel(ScoreParams p) {
+// 16 bytes of storage elements as float32
+__device__ __forceinline__ void store_floats(float* dst, uint4 v, float) { *reinterpret_cast<uint4*>(dst) = v; }
+__device__ __forceinline__ void store_floats(float* dst, uint4 v, __nv_bfloat16) {
+    reinterpret_cast<uint4*>(dst)[0] = make_uint4(v.x << 16, v.x & 0xffff0000u, v.y << 16, v.y & 0xffff0000u);
+    reinterpret_cast<uint4*>(dst)[1] = make_uint4(v.z << 16, v.z & 0xffff0000u, v.w << 16, v.w & 0xffff0000u);
+}
+
+// Registers: eight lanes to a row need no unrolling but room for the loads (four blocks: 80; 94 -> 217 us at 64, 114 with two steps unrolled);
+// four blocks of 128 channels get what three CTAs leave each other (64 rows, 512 blocks x 256 lists 205 -> 179 us).
+template <typename T, int D, int kBlocks, int kParts>
+__global__ void __launch_bounds__(32 * kScoreWarps, kParts > 1 ? 1 : kBlocks == 4 && D == 128 ? 3 : 0) scores_simt_kernel(ScoreParams p) {
     pdl_begin(p.pdl);
     constexpr int kPitch = D + 4, kCtaBlocks = kScoreWarps * kBlocks;  // pitch: a warp's 16-byte reads of 32 rows meet no bank twice
     extern __shared__ __align__(16) float smem[];
-    float* rows_s = smem;                              // [kScoreRows][kPitch]
-    float* sums_s = rows_s + kScoreRows * kPitch;      // [blocks][2][D]: Kmax, Kmin
+    constexpr int kRows = kParts == 1 ? kScoreRows : kScoreFewRows;
+    float* rows_s = smem;                          // [kRows][kPitch]
+    float* sums_s = rows_s + kRows * kPitch;       // [blocks][2][D]: Kmax, Kmin
     const int h = blockIdx.y, lb = blockIdx.z, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = lb % p.batch, l = lb / p.batch;
     const int seq_len = p.seq_lens[b];
@@ -149,20 +164,35 @@ __global__ void __launch_bounds__(32 * kScoreWarps) scores_simt_kernel(ScorePara
     const size_t sum_base = ((((size_t)(p.layer0 + l) * p.batch + b) * p.Hkv + h) * p.max_blocks) * D;
     const T* kmax = reinterpret_cast<const T*>(p.kmax) + sum_base;
     const T* kmin = reinterpret_cast<const T*>(p.kmin) + sum_base;
+    if (((reinterpret_cast<uintptr_t>(kmax) | reinterpret_cast<uintptr_t>(kmin)) & 15) == 0) {  // (uniform; summaries may start anywhere)
+        constexpr int kVec = 16 / (int)sizeof(T);
 #pragma unroll
-    for (int e = tid; e < kCtaBlocks * D; e += 32 * kScoreWarps) {
-        const int bi = e / D, c = e % D, i = blk0 + bi;
-        sums_s[(bi * 2) * D + c] = i < nb ? to_float(kmax[(size_t)i * D + c]) : 0.f;
-        sums_s[(bi * 2 + 1) * D + c] = i < nb ? to_float(kmin[(size_t)i * D + c]) : 0.f;
+        for (int e = tid; e < kCtaBlocks * D / kVec; e += 32 * kScoreWarps) {
+            const int bi = e / (D / kVec), c = e % (D / kVec) * kVec, i = blk0 + bi;
+            uint4 hi = make_uint4(0, 0, 0, 0), lo = hi;
+            if (i < nb) {
+                hi = *reinterpret_cast<const uint4*>(kmax + (size_t)i * D + c);
+                lo = *reinterpret_cast<const uint4*>(kmin + (size_t)i * D + c);
+            }
+            store_floats(sums_s + (bi * 2) * D + c, hi, T());
+            store_floats(sums_s + (bi * 2 + 1) * D + c, lo, T());
+        }
+    } else {
+#pragma unroll 4
+        for (int e = tid; e < kCtaBlocks * D; e += 32 * kScoreWarps) {
+            const int bi = e / D, c = e % D, i = blk0 + bi;
+            sums_s[(bi * 2) * D + c] = i < nb ? to_float(kmax[(size_t)i * D + c]) : 0.f;
+            sums_s[(bi * 2 + 1) * D + c] = i < nb ? to_float(kmin[(size_t)i * D + c]) : 0.f;
+        }
     }
     const T* q = reinterpret_cast<const T*>(p.q) + (size_t)lb * p.M_max * p.Hq * D;
     const bool reduce_max = p.reduce == SPECPV_REDUCE_MAX;
     float red[kBlocks];
 #pragma unroll
     for (int k = 0; k < kBlocks; ++k) red[k] = reduce_max ? -INFINITY : 0.f;
-    for (int r0 = row_begin; r0 < row_end; r0 += kScoreRows) {
+    for (int r0 = row_begin; r0 < row_end; r0 += kRows) {
         if (r0 != row_begin) __syncthreads();  // the rows before these have been read
-        const int n_rows = min(kScoreRows, row_end - r0);
+        const int n_rows = min(kRows, row_end - r0);
 #pragma unroll 4
         for (int r = warp; r < n_rows; r += kScoreWarps) {
             const T* src = q + ((size_t)((r0 + r) / p.G) * p.Hq + h * p.G + (r0 + r) % p.G) * D;
@@ -170,15 +200,16 @@ __global__ void __launch_bounds__(32 * kScoreWarps) scores_simt_kernel(ScorePara
             for (int c = lane; c < D; c += 32) rows_s[r * kPitch + c] = to_float(src[c]);
         }
         __syncthreads();
-        for (int r = lane; r < n_rows; r += 32) {
-            const float* row = rows_s + r * kPitch;
+        for (int r = lane / kParts; kParts == 1 ? r < n_rows : r - lane / kParts < n_rows; r += 32 / kParts) {
+            const int c0 = kParts == 1 ? 0 : 4 * (lane % kParts);  // the lane's first channels
+            const float* row = rows_s + (kParts == 1 ? r : min(r, n_rows - 1)) * kPitch;
             const float* sums = sums_s + warp * kBlocks * 2 * D;
             float dmax[kBlocks], dmin[kBlocks];
 #pragma unroll
             for (int k = 0; k < kBlocks; ++k) dmax[k] = dmin[k] = 0.f;
             if (p.score_mode == 0) {
-#pragma unroll 4
-                for (int c = 0; c < D; c += 4) {
+#pragma unroll (kParts == 1 ? 4 : 1)
+                for (int c = c0; c < D; c += 4 * kParts) {
                     const float4 qv = *reinterpret_cast<const float4*>(row + c);
 #pragma unroll
                     for (int k = 0; k < kBlocks; ++k) {
@@ -191,8 +222,8 @@ __global__ void __launch_bounds__(32 * kScoreWarps) scores_simt_kernel(ScorePara
             } else {
                 // channel-wise form: a channel with q_c >= 0 takes Kmax_c, one with q_c < 0 takes Kmin_c
                 // (Kmax_c >= Kmin_c), so the score is one dot product with a per-channel choice of operand
-#pragma unroll 4
-                for (int c = 0; c < D; c += 4) {
+#pragma unroll (kParts == 1 ? 4 : 1)
+                for (int c = c0; c < D; c += 4 * kParts) {
                     const float4 qv = *reinterpret_cast<const float4*>(row + c);
 #pragma unroll
                     for (int k = 0; k < kBlocks; ++k) {
@@ -209,6 +240,12 @@ __global__ void __launch_bounds__(32 * kScoreWarps) scores_simt_kernel(ScorePara
             }
 #pragma unroll
             for (int k = 0; k < kBlocks; ++k) {
+#pragma unroll
+                for (int o = kParts / 2; o > 0; o >>= 1) {
+                    dmax[k] += __shfl_xor_sync(0xffffffffu, dmax[k], o);
+                    dmin[k] += __shfl_xor_sync(0xffffffffu, dmin[k], o);
+                }
+                if (kParts > 1 && (r >= n_rows || c0 != 0)) continue;
                 const float s = fmaxf(dmax[k], dmin[k]);
                 red[k] = reduce_max ? fmaxf(red[k], s) : red[k] + s;
             }
@@ -689,13 +726,13 @@ specpv_status launch_summaries(const SummaryParams& params, int n_layers, int bl
     return SPECPV_OK;
 }
 
-template <typename T, int D, int kBlocks>
+template <typename T, int D, int kBlocks, int kParts>
 static specpv_status launch_scores_form(const ScoreParams& p, int n_layers, int max_nb, cudaStream_t stream) {
     constexpr int kCtaBlocks = kScoreWarps * kBlocks;
-    const size_t smem = (size_t)(kScoreRows * (D + 4) + kCtaBlocks * 2 * D) * sizeof(float);
-    if (!tc::set_smem_limit_once(reinterpret_cast<const void*>(scores_simt_kernel<T, D, kBlocks>), (int)smem)) return SPECPV_ERR_CUDA;
+    const size_t smem = (size_t)((kParts == 1 ? kScoreRows : kScoreFewRows) * (D + 4) + kCtaBlocks * 2 * D) * sizeof(float);
+    if (!tc::set_smem_limit_once(reinterpret_cast<const void*>(scores_simt_kernel<T, D, kBlocks, kParts>), (int)smem)) return SPECPV_ERR_CUDA;
     dim3 grid((max_nb + kCtaBlocks - 1) / kCtaBlocks, p.Hkv, n_layers * p.batch);
-    SPECPV_LAUNCH(scores_simt_kernel<T, D, kBlocks>, grid, 32 * kScoreWarps, smem, stream, p);
+    SPECPV_LAUNCH((scores_simt_kernel<T, D, kBlocks, kParts>), grid, 32 * kScoreWarps, smem, stream, p);
     return SPECPV_OK;
 }
 
@@ -703,7 +740,12 @@ template <typename T, int D>
 static specpv_status launch_scores_typed(const ScoreParams& p, int n_layers, int max_nb, cudaStream_t stream) {
     // four blocks per warp once that still gives two CTAs to every SM
     const long long ctas = (long long)((max_nb + 4 * kScoreWarps - 1) / (4 * kScoreWarps)) * p.Hkv * n_layers * p.batch;
-    return ctas >= 2 * 148 ? launch_scores_form<T, D, 4>(p, n_layers, max_nb, stream) : launch_scores_form<T, D, 1>(p, n_layers, max_nb, stream);
+    const bool four = ctas >= 2 * 148;
+    // eight lanes to a row up to 16 rows, with one block per warp up to 8 (16 rows of 64, 128 blocks x 8 lists: 3.35 -> 3.65 us with them)
+    const int rows = p.reduce == SPECPV_REDUCE_LAST ? p.G : p.M_max * p.G;
+    if (four)
+        return rows <= kScoreFewRows ? launch_scores_form<T, D, 4, 8>(p, n_layers, max_nb, stream) : launch_scores_form<T, D, 4, 1>(p, n_layers, max_nb, stream);
+    return rows <= kScoreFewRows / 2 ? launch_scores_form<T, D, 1, 8>(p, n_layers, max_nb, stream) : launch_scores_form<T, D, 1, 1>(p, n_layers, max_nb, stream);
 }
 
 specpv_status launch_scores(const ScoreParams& p, int n_layers, int max_nb, int dtype, int d, cudaStream_t stream) {

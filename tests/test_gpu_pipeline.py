@@ -385,8 +385,8 @@ def test_verify_host_matches_the_device_call_and_the_oracle(name, L, over):
 @pytest.mark.parametrize("reduce,score_mode", [(B.REDUCE_MEAN, 0), (B.REDUCE_MAX, 1), (B.REDUCE_LAST, 0)])
 def test_scores_of_the_plain_kernel(dtype, Hq, d, reduce, score_mode):
     """What the tensor-core score kernel does not take: float32, more than 1024 rows per KV head (33 x 33), and head size 64 or a
-    group size that does not divide 128 with per-sequence row counts; block counts around the 32 a CTA of the plain
-    kernel takes, row counts that leave warps without rows."""
+    group size that does not divide 128 with per-sequence row counts; a few blocks more or less than the 8 a CTA of the plain
+    kernel takes (fewer than 296 CTAs), row counts that leave lanes without rows."""
     w = wl.make_workload("llama_32k", device="cuda", n_layers=2, Hq=Hq, Hkv=2, d=d, dtype=dtype, M=33,
                          ctx=[64 * 31 + 9, 64 * 33, 64])
     c = w.cfg
@@ -678,3 +678,40 @@ def test_selection_of_one_and_of_tied_candidates(n, L, shared):
 def test_commit_of_clusters_of_any_size(dtype, batch, A):
     """Two to eight units, three, five and seven among them, with up to as many tokens as the touched blocks hold."""
     test_commit_of_few_units_in_one_launch(dtype, 1, batch, 16, A)
+
+
+@pytest.mark.parametrize("dtype,Hq,d,M", [("fp32", 2, 64, 16), ("fp32", 8, 128, 4), ("fp32", 8, 128, 5), ("bf16", 8, 64, 17), ("bf16", 10, 128, 3),
+                                          ("bf16", 10, 128, 13), ("bf16", 2, 64, 1)])
+@pytest.mark.parametrize("reduce,score_mode", [(B.REDUCE_MEAN, 0), (B.REDUCE_MAX, 1), (B.REDUCE_LAST, 0), (B.REDUCE_LAST, 1)])
+@pytest.mark.parametrize("layers,shift", [(1, 0), (75, 0), (75, 1)])
+def test_plain_scores_with_few_rows_and_summaries_anywhere(dtype, Hq, d, M, reduce, score_mode, layers, shift):
+    """Up to 16 rows of a group, of which eight lanes share one, and just more; one block per warp and (75 layers) four; per-sequence row
+    counts, whose last sequence has none; summaries that start on a 16-byte boundary and one element past it."""
+    Hkv, lens, blocks = 2, [64 * 33 - 5, 64 * 8, 64 * 9 - 63], 33
+    dt = wl.torch_dtype(dtype)
+    g = torch.Generator().manual_seed(Hq + M + layers)
+    key = torch.randn((2, layers, 3, Hkv, blocks, d), generator=g)
+    n = key[0].numel()
+    flat = [torch.zeros(n + 8, dtype=dt, device="cuda")[shift:shift + n] for _ in range(2)]
+    kmax, kmin = (f.view(layers, 3, Hkv, blocks, d).copy_(t.to(dt)) for f, t in zip(flat, (key.amax(0), key.amin(0))))
+    q = torch.randn((layers, 3, M, Hq, d), generator=g).to(dt).cuda()
+    cfg = B.make_config(layers, Hq, Hkv, d, 64, dtype, 1, 2, 4, 64, reduce=reduce, score_mode=score_mode)
+    pool = torch.zeros((layers, 1, Hkv, 64, d), dtype=dt, device="cuda")
+    cache = B.Cache(pool, pool, torch.zeros((3, blocks), dtype=torch.int32, device="cuda"), torch.tensor(lens, dtype=torch.int32, device="cuda"), max(lens))
+    ws = torch.zeros(B.WORKSPACE_HEAD_BYTES, dtype=torch.uint8, device="cuda")
+    scores = torch.full((layers, 3, Hkv, blocks), -7.0, device="cuda")
+    rows = [M, (M + 1) // 2, 0]
+    B.specpv_score_blocks(cfg, 0, layers, q, torch.tensor(rows, dtype=torch.int32, device="cuda"), M, torch.zeros(3, dtype=torch.int32, device="cuda"),
+                          kmax, kmin, cache, scores, ws)
+    util.sync_status(ws)
+    for l in {0, layers // 2, layers - 1}:
+        for b in range(3):
+            nb = (lens[b] + 63) // 64
+            got = scores[l, b]
+            assert (got[:, nb:] == -7.0).all()  # blocks past the context are left alone
+            if rows[b] == 0 and reduce != B.REDUCE_LAST:
+                assert got[:, :nb].isnan().all() if reduce == B.REDUCE_MEAN else (got[:, :nb] == -float("inf")).all()
+                continue
+            want = score_reference(kmax[l, b, :, :nb], kmin[l, b, :, :nb], q[l, b, :max(rows[b], 1)], Hkv, reduce, score_mode)
+            # products of the stored values summed in float32: d terms per dot product, then up to 85 rows
+            torch.testing.assert_close(got[:, :nb].double(), want, rtol=2e-5, atol=2e-4)
