@@ -435,17 +435,26 @@ SPECPV_EXPORT specpv_status specpv_verify_host(const specpv_config* cfg, int mod
     // bytes (23.6 MB in and 16 MB out: 471 us as one copy each way, 762 as 24), so the groups are few.  The last one is small, its
     // attention and copy out overlap nothing; where the attention outlasts the copies the first ones are small too, each
     // copied in while the one before it is worked on.  32 layers, 60 rows: 32768 tokens 1290 -> 1165 us, a 4096-token partial
-    // cache 840 -> 735, against eight equal groups.  Where the copies in are what the call takes, the keys and values of all layers
-    // go first, in a copy each, and only the queries in groups (36 layers, 58 rows, 3659 tokens and a 1024-token partial cache, both calls
-    // 1580 -> 1479 us).
+    // cache 840 -> 735, against eight equal groups.  Where the copies in are what the call takes (attention below half of them), the keys and
+    // values of all layers go first, in a copy each, and only the queries in groups: six copies fewer, but the first copy out starts later.
+    // That pays up to a delay of 150 us where the copies out are no longer than the queries' copies in, which they then run beside, and up to
+    // 25 us where they are.  us, groups with their own keys and values / keys and values first, {4, 3, 2, 1} / {2, 3, 3, 2}; 60 rows,
+    // a partial cache: 32 layers, four heads per KV head, bfloat16 output 738 / 718 / 700, float32 (31 us) 924 / 982 / 928; 16 layers of four
+    // sequences 1322 / 1265 / 1254 and (63 us) 1699 / 1814 / 1707; 32 layers, two heads per KV head (126 us) 855 / 827 / 821, one (315 us) 1093 /
+    // 1123 / 1120 and 1250 / 1387 / 1353.  With attention at 0.6 of the copies in (8192 tokens) 709 / 745 / 736.
     HostCopyStreams* cs = host_copy_streams();
     if (!cs) return SPECPV_ERR_CUDA;
     constexpr int kMaxGroups = 4;
     const double copy_us = (double)n_layers * (q_l + 2.0 * kv_l) / 50.0e3;  // 50 GB/s
-    const double run_us = (double)n_layers * kv->batch * kv->max_seq_len * g.Hkv * 2.0 * g.d * g.es / 4.0e6;  // 4 TB/s
-    static const int kShare[2][kMaxGroups] = {{4, 3, 2, 1}, {1, 2, 5, 2}};  // tenths of the layers
-    const bool copy_bound = run_us <= copy_us;
-    const int* share = kShare[!copy_bound];
+    // 4 TB/s with two row tiles per KV head, with one the copy rate (24 rows x 4, 6000 tokens, taken for copy-bound now: 383 -> 343 us)
+    const double rate = (double)M_max * g.G <= 128 ? 6.4e6 : 4.0e6;
+    const double run_us = (double)n_layers * kv->batch * kv->max_seq_len * g.Hkv * 2.0 * g.d * g.es / rate;
+    static const int kShare[3][kMaxGroups] = {{4, 3, 2, 1}, {1, 2, 5, 2}, {2, 3, 3, 2}};  // tenths of the layers
+    const double delay_us = (double)n_layers * (1.2 * kv_l - 0.2 * q_l) / 50.0e3;  // of the first group's inputs
+    const bool kv_first = run_us <= 0.5 * copy_us && delay_us <= (out_l <= q_l ? 150.0 : 25.0);
+    // (a small call, whose groups cost more than their bytes, takes the shares that leave fewer of them: 4 layers of 24 rows of 8 x 64
+    // float32, 94 -> 82 us)
+    const int* share = kShare[kv_first && copy_us >= 30.0 ? 2 : run_us > copy_us ? 1 : 0];
     int first[kMaxGroups + 1] = {0}, tenths = 0, n_groups = 0;
     for (int i = 0; i < kMaxGroups; ++i) {
         tenths += share[i];
@@ -465,12 +474,12 @@ SPECPV_EXPORT specpv_status specpv_verify_host(const specpv_config* cfg, int mod
                cudaMemcpyAsync(stage + sp.v_new + l0 * kv_l, static_cast<const char*>(v_new_host) + l0 * kv_l, nl * kv_l,
                                cudaMemcpyHostToDevice, cs->in) == cudaSuccess;
     };
-    if (copy_bound) ok = ok && copy_kv(0, n_layers);
+    if (kv_first) ok = ok && copy_kv(0, n_layers);
     for (int i = 0; i < n_groups && ok && st == SPECPV_OK; ++i) {
         const int l0 = first[i], nl = first[i + 1] - l0;
         ok = cudaMemcpyAsync(stage + sp.q + l0 * q_l, static_cast<const char*>(q_host) + l0 * q_l, nl * q_l,
                              cudaMemcpyHostToDevice, cs->in) == cudaSuccess &&
-             (copy_bound || copy_kv(l0, nl)) &&
+             (kv_first || copy_kv(l0, nl)) &&
              cudaEventRecord(event, cs->in) == cudaSuccess && cudaStreamWaitEvent(s, event, 0) == cudaSuccess;
         if (!ok) break;
         st = verify_common(cfg, layer0 + l0, nl, stage + sp.q + l0 * q_l, stage + sp.k_new + l0 * kv_l,

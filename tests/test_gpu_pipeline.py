@@ -347,8 +347,8 @@ def test_selection_alone_on_synthetic_scores_with_ties_and_nan(nb, budget):
 @pytest.mark.parametrize("name,L,over", [("tiny_fp32", 1, {}), ("llama_32k", 5, dict(ctx=[5000])),
                                          ("llama_32k", 11, dict(ctx=[1500])), ("stress_b4", 3, dict(ctx=[900, 2100, 64, 1300]))])
 def test_verify_host_matches_the_device_call_and_the_oracle(name, L, over):
-    """The end-to-end entry point (pinned host step tensors in, host outputs back; layers pipelined in groups of
-    1 and 2 with a short last group) against the device-pointer call and, on one layer, the oracle."""
+    """The end-to-end entry point (pinned host step tensors in, host outputs back; layers pipelined in up to four groups, the copies in
+    being what these calls take) against the device-pointer call and, on one layer, the oracle."""
     w = wl.make_workload(name, device="cuda", n_layers=L, spare_tokens=256, **over)  # the bytes of run_pipeline's caches
     c = w.cfg
     Hq, d, M, batch = c["Hq"], c["d"], c["M"], w.batch
@@ -715,3 +715,49 @@ def test_plain_scores_with_few_rows_and_summaries_anywhere(dtype, Hq, d, M, redu
             want = score_reference(kmax[l, b, :, :nb], kmin[l, b, :, :nb], q[l, b, :max(rows[b], 1)], Hkv, reduce, score_mode)
             # products of the stored values summed in float32: d terms per dot product, then up to 85 rows
             torch.testing.assert_close(got[:, :nb].double(), want, rtol=2e-5, atol=2e-4)
+
+
+@pytest.mark.parametrize("mode", [B.MODE_FULL, B.MODE_PARTIAL])
+@pytest.mark.parametrize("Hq,Hkv,M,ctx,L,out_f32", [
+    (32, 8, 2, [3000], 7, 0),      # attention outlasts the copies: groups of 1, 1, 4, 1 layers with their own keys and values
+    (32, 8, 60, [9000], 5, 1),     # attention at 0.6 of the copies in: groups of 2, 2, 1
+    (32, 8, 60, [1500], 7, 0),     # keys and values first: queries in groups of 1, 3, 2, 1
+    (32, 8, 24, [900, 400], 3, 1),  # the same with outputs longer than the queries, a short delay
+    (8, 8, 100, [300], 8, 1),      # and a delay too long for that
+])
+def test_verify_host_in_every_order_of_its_copies(mode, Hq, Hkv, M, ctx, L, out_f32):
+    """Every layer of the host call against the device-pointer call, every sequence of the last layer against the oracle."""
+    w = wl.make_workload("llama_32k", device="cuda", n_layers=L, spare_tokens=256, Hq=Hq, Hkv=Hkv, M=M, ctx=ctx)
+    c, batch, d = w.cfg, w.batch, w.cfg["d"]
+    cfg = util.config_for(w, out_f32=out_f32, budget_blocks=4, buffer_tokens=64)
+    cache = util.full_cache(w)
+    ws = B.new_workspace(cfg, L, batch, int(max(ctx)) + 256, M)
+    mask = util.device_masks(w.parents, M)
+    dt = torch.float32 if out_f32 else torch.bfloat16
+    out_d = torch.zeros((L, batch, M, Hq, d), dtype=dt, device="cuda")
+    lse_d = torch.zeros((L, batch, M, Hq), dtype=torch.float32, device="cuda")
+    verify = B.specpv_verify_full if mode == B.MODE_FULL else B.specpv_verify_partial
+    verify(cfg, 0, L, w.q, w.k_new, w.v_new, mask, None, M, cache, out_d, lse_d, ws)
+    host = [t.cpu().pin_memory() for t in (w.q, w.k_new, w.v_new)]
+    mask_h = mask.cpu().pin_memory()
+    out_h = torch.full((L, batch, M, Hq, d), float("nan"), dtype=dt).pin_memory()
+    lse_h = torch.full((L, batch, M, Hq), float("nan"), dtype=torch.float32).pin_memory()
+    for _ in range(2):  # twice: the staging area and the copy streams are reused
+        out_h.fill_(float("nan"))
+        B.specpv_verify_host(cfg, mode, 0, L, host[0], host[1], host[2], mask_h, M, cache, out_h, lse_h, ws)
+    util.sync_status(ws)
+    # as above: the groups may split the KV range differently from the one launch.  A bfloat16 output adds half a unit in the last place
+    # of values up to 16 on either side, 2 x 2^-5
+    assert torch.isfinite(out_h).all() and torch.isfinite(lse_h).all()
+    assert (out_h.float() - out_d.cpu().float()).abs().max().item() <= (4e-2 if out_f32 else 4e-2 + 2 ** -4)
+    assert (lse_h - lse_d.cpu()).abs().max().item() <= 4e-2
+    l = L - 1
+    for b in range(batch):
+        o_out, o_lse = oracle.tree_attention(wl.to_numpy(w.q[l, b]), wl.to_numpy(w.k_new[l, b]), wl.to_numpy(w.v_new[l, b]),
+                                             oracle.tree_mask(w.parents[b]), wl.to_numpy(w.k_pool[l]),
+                                             wl.to_numpy(w.v_pool[l]), wl.to_numpy(w.block_table[b]), int(ctx[b]))
+        if out_f32:
+            util.compare(out_h[l, b].numpy(), o_out, "bf16", "verify_host")
+        else:
+            assert np.abs(out_h[l, b].float().numpy() - o_out).max() <= 2e-2 + 2 ** -5
+        np.testing.assert_allclose(lse_h[l, b].numpy(), o_lse, atol=5e-3)
