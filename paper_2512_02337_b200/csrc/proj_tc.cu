@@ -162,9 +162,7 @@ __global__ void __launch_bounds__(kProjThreads, 2) proj_tc_kernel(const __grid_c
             for (int i = i0; i < i1; ++i)
                 if (i >= p.stages)
                     ok &= mbar_wait(smem_u32(&bars.empty[i % p.stages]), ((i / p.stages) - 1) & 1, abort_flag, p.workspace, 30);
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;  // a wait gave up: nothing more is copied
-            if (lane == 0) {
+            if (lane == 0 && ok) {  // a wait gave up: nothing more is copied
                 for (int i = i0; i < i1; ++i) {
                     const int slot = i % p.stages;
                     const uint32_t full = smem_u32(&bars.full[slot]);
@@ -174,7 +172,8 @@ __global__ void __launch_bounds__(kProjThreads, 2) proj_tc_kernel(const __grid_c
                     tma_load_2d(dst + kWTileBytes, &p.tm_x, (kb + i) * 64, x_row, full);
                 }
             }
-            __syncwarp();
+            ok = __all_sync(0xffffffffu, ok);  // the lanes leave together
+            if (!ok) break;
         }
     } else if (warp == 1) {
         // ---- MMA issue --------------------------------------------------------------------------------------
@@ -184,10 +183,9 @@ __global__ void __launch_bounds__(kProjThreads, 2) proj_tc_kernel(const __grid_c
         pdl_wait();  // (nothing to read here, but the limits of the waits below start to run)
         for (int i = 0; i < n_k; ++i) {
             const int slot = i % p.stages;
-            ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.full[slot]), (i / p.stages) & 1, abort_flag, p.workspace, 31));
-            if (!ok) break;  // a wait gave up: nothing more is issued
+            ok = mbar_wait(smem_u32(&bars.full[slot]), (i / p.stages) & 1, abort_flag, p.workspace, 31);
             tc_fence_after();
-            if (lane == 0) {
+            if (lane == 0 && ok) {  // a wait gave up: nothing more is issued
                 const uint32_t a_lo = (((data + slot * stage_bytes) >> 4) & 0x3FFFu) | (1u << 16);
                 const uint32_t b_lo = (((data + slot * stage_bytes + kWTileBytes) >> 4) & 0x3FFFu) | (1u << 16);
 #pragma unroll
@@ -197,7 +195,8 @@ __global__ void __launch_bounds__(kProjThreads, 2) proj_tc_kernel(const __grid_c
                 tc_commit(smem_u32(&bars.empty[slot]));
                 if (i == n_k - 1) tc_commit(smem_u32(&bars.d_full));
             }
-            __syncwarp();
+            ok = __all_sync(0xffffffffu, ok);  // (a vote ahead of the contractions: 0.5 % of a layer's block)
+            if (!ok) break;
         }
     } else {
         // ---- epilogue: thread <-> output feature (tensor-memory lane), then thread <-> (row, channel pairs) ---

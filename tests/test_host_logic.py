@@ -282,15 +282,22 @@ def test_overlapped_kernels_load_nothing_through_the_read_only_path():
 @pytest.mark.parametrize("source", ["attn_tc.cu", "attn_pair.cu", "score_tc.cu", "proj_tc.cu"])
 def test_lanes_of_a_warp_give_up_together(source):
     """A wait that can give up returns a value per lane, and so does a look at the abort flag: an exit, a condition of a loop or of a
-    vote that depends on one comes after a vote of the whole warp.  (Lanes that disagreed would wait for one another in different
+    vote that depends on one comes after a vote of the whole warp, or the loop has no place where the lanes meet.  (Lanes that disagreed would wait for one another in different
     places, without a limit.)  Checked on the source: such a case cannot be brought about on a GPU that works."""
-    own = False  # whether `ok` may differ between lanes
-    for n, line in enumerate((build_mod.CSRC / source).read_text().split("\n"), 1):
+    own, loop = False, 0  # whether `ok` may differ between lanes
+    lines = (build_mod.CSRC / source).read_text().split("\n")
+    for n, line in enumerate(lines, 1):
         code = line.split("//")[0]
         if re.search(r"\bbool ok = ", code):
             own = False
+        if re.search(r"\bfor \(", code) and code.startswith("    for ("):
+            loop = n  # the outermost loop of a role
         if re.search(r"if \(!ok\) (break|return)|if \(ok\) ok = __all_sync", code):
-            assert not own, f"{source}:{n} leaves without a vote"
+            if "each lane by itself" in line:  # allowed in loops whose lanes meet nowhere
+                end = next(i for i in range(n, len(lines)) if lines[i] == "    }")
+                assert not re.search(r"_sync\(|__syncwarp", "\n".join(x.split("//")[0] for x in lines[loop - 1:end])), f"{source}:{n}"
+            else:
+                assert not own, f"{source}:{n} leaves without a vote"
         if re.search(r"\bok &?= .*__all_sync\(0xffffffffu, ", code):
             own = False if "ok &=" not in code else own
         elif re.search(r"\bok &?= (mbar|pair)_wait\(|\*abort_flag\) ok = ", code):
