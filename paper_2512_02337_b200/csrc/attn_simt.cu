@@ -305,7 +305,9 @@ __global__ void __launch_bounds__(kThreads) attn_simt_kernel(SimtParams p) {
 
 // Log-sum-exp merge of the per-split partial results: D/4 threads per row and group of D/4 splits, four channels each, eight
 // partial rows in flight per thread; a row's groups (up to 64 splits in all) meet in shared memory and are added in order.  Bound by
-// latency: 64 splits one group of lanes after the other took 8.1 us a call, side by side 4.6; 33 splits 5.9 and 3.5.  grid = (row groups, KV heads, layers x seqs).
+// latency: 64 splits one group of lanes after the other took 8.1 us a call, side by side 4.6; 33 splits 5.9 and 3.5.  Fewer splits, where groups
+// idle, with the attention before the merge (64 rows of 64 channels): 2 splits 12.2 -> 11.0 us, 5 12.4 -> 11.0, 9 12.8 -> 11.6.
+// grid = (row groups, KV heads, layers x seqs).
 constexpr int kMergeThreads = 128;
 constexpr int kMergeAhead = 8;
 template <typename TO, int D>

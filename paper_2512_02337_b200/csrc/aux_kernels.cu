@@ -581,14 +581,16 @@ __global__ void __launch_bounds__(128) gather_kernel(GatherParams p) {
 // ---------------------------------------------------------------------------------------------
 // Commit: a CTA's four warps append the accepted tokens' K and V rows that fall into one block (a warp per row) and recompute the
 // block's summary, the appended tokens taken from the step's tensors; grid = (blocks touched, KV heads, layers x seqs).  All CTAs
-// read the lengths.  Where they are no more than a cluster holds (one or two float32 layers, short steps), they are one, which
-// advances the lengths itself once they have all arrived; else the lengths advance in a launch behind it: a commit keeps nothing in
-// the workspace but the status word, so that commits of two caches on two streams may share one (an arrival counter there made the
-// launch unnecessary, 9.3 us a call against 11.4, but mixed the arrivals of two such commits).  Bound by launches.  us with a copy of
-// the lengths, two launches / a CTA that took four of the units side by side and then the rest / cluster: four units of 4 tokens
-// 6.1 / 6.5 / 5.8, eight 6.1 / 10.4 / 6.4 (a launch less for the host), eight of 46 tokens 10.1 / 18.1 / 10.0, of 64 16.7 / 31.9 / 16.5.
+// read the lengths.  Up to four of them (one float32 layer, short steps) are one CTA that advances the lengths itself behind a barrier,
+// up to eight one cluster that does so once they have all arrived; else the lengths advance in a launch behind them: a commit keeps
+// nothing in the workspace but the status word, so that commits of two caches on two streams may share one (an arrival counter there
+// made the launch unnecessary, 9.3 us a call against 11.4, but mixed the arrivals of two such commits).  Bound by launches.  us with a
+// copy of the lengths, two launches / a CTA that took four units side by side and then the rest / cluster: four units of 4 tokens 6.1 /
+// 6.5 / 5.8, eight 6.1 / 10.4 / 6.4 (a launch less for the host), eight of 46 tokens 10.1 / 18.1 / 10.0, of 64 16.7 / 31.9 / 16.5.  A cluster
+// costs the host more: a float32 step with two commits of four units 65.3 us with clusters, 64.1 with a CTA.
 // ---------------------------------------------------------------------------------------------
 constexpr int kCommitWarps = 4;
+constexpr int kCommitUnits = 4;    // of one CTA, side by side
 constexpr int kCommitCluster = 8;  // CTAs of a cluster that every launch may ask for
 
 template <typename T>
@@ -695,6 +697,17 @@ __global__ void __launch_bounds__(kLensThreads) commit_lens_kernel(CommitParams 
     if (b < p.batch) advance_length(p, b);
 }
 
+// One CTA for up to kCommitUnits units side by side, which advances the lengths itself behind a barrier.
+template <typename T>
+__global__ void __launch_bounds__(32 * kCommitWarps * kCommitUnits) commit_small_kernel(CommitParams p, dim3 units) {
+    pdl_begin(1);
+    const int u = threadIdx.x / (32 * kCommitWarps);
+    if (u < (int)(units.x * units.y * units.z))
+        commit_unit<T>(p, u % units.x, u / units.x % units.y, u / (units.x * units.y), (threadIdx.x >> 5) % kCommitWarps, threadIdx.x & 31);
+    __syncthreads();  // every unit has read the lengths
+    if ((int)threadIdx.x < p.batch) advance_length(p, threadIdx.x);
+}
+
 // One cluster, a CTA per unit, which advances the lengths itself.
 template <typename T>
 __global__ void __launch_bounds__(32 * kCommitWarps) commit_cluster_kernel(CommitParams p) {
@@ -794,7 +807,15 @@ specpv_status launch_commit(const CommitParams& params, int n_layers, int dtype,
     CommitParams p = params;
     p.aligned = aligned16(p.kmax) && aligned16(p.kmin);
     dim3 grid((p.A_max + p.bs - 1) / p.bs + 1, p.Hkv, n_layers * p.batch);
-    if (advance && (long long)grid.x * grid.y * grid.z <= kCommitCluster) {
+    const long long units = (long long)grid.x * grid.y * grid.z;
+    if (advance && units <= kCommitUnits) {
+        if (launch_pdl(dtype == SPECPV_DTYPE_F32 ? commit_small_kernel<float> : commit_small_kernel<__nv_bfloat16>, 1,
+                       32 * kCommitWarps * (int)units, 0, stream, p, grid) != cudaSuccess)
+            return SPECPV_ERR_CUDA;
+        count_launch();
+        return SPECPV_OK;
+    }
+    if (advance && units <= kCommitCluster) {
         cudaLaunchAttribute attr[2]{};
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = 1;

@@ -608,8 +608,8 @@ def test_plain_scores_in_both_forms(blocks, layers, M, d):
 @pytest.mark.parametrize("dtype,Hkv,batch,bs,A", [("fp32", 1, 1, 64, 4), ("fp32", 2, 2, 64, 4), ("bf16", 1, 4, 16, 16), ("bf16", 4, 1, 32, 5),
                                                   ("fp32", 3, 1, 16, 17)])
 def test_commit_of_few_units_in_one_launch(dtype, Hkv, batch, bs, A):
-    """Up to eight units of work (block touched, KV head, sequence) are one cluster that advances the lengths itself; nine, the last
-    case, take two launches.  Three commits in a row, of which the second appends nothing to the first sequence."""
+    """Up to four units of work (block touched, KV head, sequence) share a CTA, up to eight are a cluster, either of which advances the
+    lengths itself; nine, the last case, take two launches.  Three commits in a row, of which the second appends nothing to the first sequence."""
     d, M = 64, 24
     w = wl.make_workload("tiny_fp32", device="cuda", n_layers=1, spare_tokens=256, Hq=2 * Hkv, Hkv=Hkv, d=d, bs=bs, dtype=dtype, M=M,
                          ctx=[bs * 3 + 5 * b - 1 for b in range(batch)])
@@ -674,9 +674,10 @@ def test_selection_of_one_and_of_tied_candidates(n, L, shared):
                 assert np.array_equal(got[l, 0, h], want), (budget, l, h)
 
 
-@pytest.mark.parametrize("dtype,batch,A", [("fp32", 1, 1), ("bf16", 1, 17), ("fp32", 1, 49), ("bf16", 3, 16), ("bf16", 1, 81), ("fp32", 1, 112), ("bf16", 4, 7)])
-def test_commit_of_clusters_of_any_size(dtype, batch, A):
-    """Two to eight units, three, five and seven among them, with up to as many tokens as the touched blocks hold."""
+@pytest.mark.parametrize("dtype,batch,A", [("fp32", 1, 1), ("bf16", 1, 17), ("bf16", 2, 16), ("fp32", 1, 49), ("bf16", 3, 16), ("bf16", 1, 81), ("fp32", 1, 112),
+                                           ("bf16", 4, 7)])
+def test_commit_of_any_number_of_units(dtype, batch, A):
+    """Two to eight units, with up to as many tokens as the touched blocks hold."""
     test_commit_of_few_units_in_one_launch(dtype, 1, batch, 16, A)
 
 
